@@ -15,6 +15,7 @@
 namespace cih {
 
 constexpr int kMaxWords = 4;              // <= 256 orbitals per species
+constexpr int kLevels = 8;                // oscillator levels of a species: Nmax <= 7 with 256 orbitals
 constexpr int kSortTile = 4096;           // longest neighbour list the sort handles
 
 // ---------------------------------------------------------------- device view
@@ -24,14 +25,45 @@ struct DevSpecies {
     const uint64_t *bits;      // n_sd x W words (W = basis word count)
     const int8_t *N;           // oscillator quanta of each sub-det
     const int32_t *cls_end;    // per sub-det: one past the end of its (2M, parity) class
-    const int64_t *fw_off;     // n_sd + 1: forward same-class neighbours (1 or 2 moves)
-    const int32_t *fw;         //   sorted ascending, all > x
+    const int64_t *fw_off;     // n_sd + 1: slots of the forward same-class neighbours (1 or 2 moves)
+    // slot x = [fw_off[x], fw_off[x+1]): the two-moves ascending from its start,
+    // the one-moves ascending from its end backwards (the j-th at end - 1 - j):
+    const int2 *fw_rec;        //   x: neighbour y (protons: its column base rowbase[y] - nb[y]),
+                               //   y: forward neighbours of the other kind before it | level of y << 24
+    const int32_t *fw_tb;      //   two-move: table index << 1 | sign; one-move: ~(b | d << 8 | sign << 16)
+    const int32_t *fw_lev;     // n_sd x NL: two-moves at levels <= l
     const int64_t *n1_off;     // n_sd + 1: every one-move neighbour
     const int32_t *n1;         //   sorted ascending
-    const int64_t *n1_later;   // per sub-det: first one-move entry beyond its own class
+    const int32_t *n1_self;    // per sub-det: one-move entries below it (the next ones are its
+                               //   forward same-class one-moves, then those of later classes)
     int32_t n_sd;
     int32_t n_orb;
     int32_t orb_base;          // combined index of this species' orbital 0
+    int32_t N0;                // quanta of the lowest configuration; a sub-det's level is (N - N0) >> 1
+    int32_t NL;                // levels
+};
+
+// What a row needs of its proton sub-det p, in one record.
+struct alignas(16) ProtonRec {
+    int64_t l1;                // first later one-move: n1_off[p] + n1_self[p]
+    int64_t fw;                // fw_off[p]
+    int64_t g0;                // first group record
+    int32_t fwlen;             // fw_off[p + 1] - fw_off[p]
+    int32_t colb;              // rowbase[p] - nb[p]
+    int32_t nb;                // first neutron partner
+    int32_t ng;                // group records
+    int32_t dirA;              // directory position ending n's same-class one-moves inside p's range
+    int32_t levA;              // highest neutron level inside p's range
+};
+
+// ... and of its neutron sub-det n.
+struct alignas(16) NeutronRec {
+    int64_t n1;                // n1_off[n]
+    int64_t fw;                // fw_off[n]
+    int32_t fwlen;
+    int32_t self;              // n1_self[n]
+    int32_t N;
+    int32_t pad;
 };
 
 // Everything the Hamiltonian kernels read.
@@ -49,48 +81,42 @@ struct DevBasis {
     int32_t ntot;
     int64_t dim;
     int64_t tbme_len;
-    // fast paths
-    const int32_t *fw_tb[2];   // per forward entry: two-move table index << 1 | sign, or -1
-    const uint32_t *n1_info;   // per neutron one-move entry: packed move (see neighbours.cu)
-    const int16_t *pn_S;       // n_orb_p x pn_G
-    const int32_t *pn_gsize;   // pn_G
-    const int32_t *pn_goff;    // pn_G
-    const int8_t *m2p;         // proton orbital 2m
-    const int8_t *Np;          // proton orbital N
-    int32_t pn_G;
-    int32_t pn_m2span;
-    int32_t max_cand;          // largest candidate list of a proton sub-det
-    int *queue;                // work counter (unused by the row kernels)
-    // candidate table: for proton sub-det p, records cand_off[p] .. cand_off[p+1]
-    // (later same-class sub-dets with one or two protons moved, then later-class
-    // sub-dets with one proton moved, ascending), one int4 each:
-    //   x  column base rowbase[q] - nbeg[q]
-    //   y  directory indices of q's neutron range: start | end << 16
-    //   z  one-move: S row bases A_u | A_v << 16; two-move: table index << 1 | sign
-    //   w  bits 0..7 K_a, 8 N_a & 1, 9 sign, 16..23 a, 24..31 c (one-move only)
-    const int64_t *cand_off;
-    const int4 *cand;
-    const uint8_t *cand_self;      // per record: 0 if n can never lie in q's range,
-                                   // else 1 + the largest N of a partner; bit 7 = two-move
-    const int32_t *row_p;          // row -> proton sub-det
-    int32_t A;                     // particles
-    int32_t nZ[2];                 // particles per species
-    // neutron one-move lists packed (neighbour, move info), and their bucket
-    // directory: for neutron n, dir[n * dir_len + 1 + rc * NL + L] = number of
-    // entries of n's one-move list in buckets <= (relative class rc, level L);
-    // dir[n * dir_len] = 0.  rc = ((2M_y - 2M_n + DM) / 2) * 2 + (N_y & 1).
+    int32_t Nlim;              // quanta limit of the basis
+    int32_t A;                 // particles
+    int32_t nZ[2];             // particles per species
+    const int32_t *row_p;      // row -> proton sub-det
+    const ProtonRec *prec;
+    const NeutronRec *nrec;
+    // Groups of p's later one-moves q > p with equal (class, N): every member
+    // has the same neutron segment for a given row.  Per group (own class
+    // first, levels ascending; then the later classes):
+    //   x  first member relative to ProtonRec::l1 | members << 16
+    //   y  directory positions of the segment: start | end << 16
+    //   z  own class: two-moves of the same level (a level without one-moves
+    //      is a group too), else 0
+    //   w  own class: 1 + largest N of a partner of the members (1 + L_q)
+    //      | two-moves of lower levels << 8, else 0
+    const int4 *grp;
+    const int2 *l1;            // per proton one-move entry: column base of q, a | c << 8 | sign << 16 | pn_a[a] << 17
+    // neutron one-move lists packed: neighbour, then r(d) | r(b) << 8 | t(b) << 16 |
+    // t(d) << 21 | sign << 26 (b in n only, d in the neighbour only; r, t below)
     const int2 *n1p;
+    // bucket directory of each list: dir[n * dir_len + 1 + rc * NL + l] = entries
+    // of n's list in buckets <= (relative class rc, level l); dir[n * dir_len] = 0.
+    // rc = ((2M_y - 2M_n + DM) / 2) * 2 + (N_y & 1).
     const int16_t *dir;
-    int32_t dir_len, NL, DM;
-    // count lists: per proton sub-det p, the directory positions its one-move
-    // candidates' segments start and end at, with multiplicities (position,
-    // coefficient), and the number of candidates whose range holds n itself
-    // per N_n
-    const int64_t *clist_off;  // n_p + 1, or null when the count walks the candidates
-    const int2 *clist;
-    const uint16_t *cself_sfx; // n_p x NL
-    const int16_t *self_rel;       // per neutron n: entries of its one-move list below n
-    const uint8_t *occ[2];         // per sub-det: its occupied orbitals, ascending (Z_s each)
+    int32_t dir_len, DM;
+    const uint8_t *occ[2];     // per sub-det: its occupied orbitals, ascending (Z_s each)
+    // pn pairs: u(a, b) = S(a, t(b)) + r(b) inside the group of (a, t(b)), with
+    // t(b) the dense number of b's (2m, N parity) and r(b) b's rank among the
+    // neutron orbitals with the same t.  pn_s[a * pn_T + t] = S; the group's
+    // table offset and pairs are pn_k[(t + 2 m'_a) ^ (N_a & 1)], with m'_a the
+    // dense number of 2m_a and pn_a[a] = N_a & 1 | 2 m'_a << 1.
+    const int2 *pn_k;          // 64 groups
+    const int16_t *pn_s;
+    const uint8_t *pn_a;
+    int32_t pn_T;
+    const uint16_t *orbs;      // per neutron orbital: r(b) | t(b) << 8
     // one-body table layout (see OneBodyLayout)
     const int16_t *ob_grp, *ob_loc;
     const int32_t *ob_gsize, *ob_goff;
@@ -109,12 +135,11 @@ struct SpeciesBuild {
     const int8_t *N;
     const int16_t *M2;
     const int32_t *cls_end;
-    const int32_t *cls_lookup;  // (M2 + moff) * 2 + parity -> class id, -1 if none
     const int32_t *cls_begin;
     const int32_t *cls_endc;    // per class
     const int8_t *oN;           // per orbital
     const int16_t *om2;
-    int32_t n_sd, n_orb, moff, mspan, Nsub_max;
+    int32_t n_sd, n_orb, Nsub_max;
     const int32_t *hash;        // open-addressing table of sub-det indices, -1 = empty
     uint32_t hash_mask;         // capacity - 1 (power of two)
     const uint64_t *bitsT;      // W x n_sd: the bit strings word-major (coalesced scans)

@@ -11,7 +11,6 @@ namespace cih {
 // Table layout caps of the shared-memory copies the kernels keep.
 constexpr int kLayoutCap = 512;   // global table groups
 constexpr int kOrbCap = 512;      // combined orbitals (two species of at most 256)
-constexpr int kGroupCap = 128;    // dense pn group keys
 
 // Table index of V(ab, cd) for combined orbitals in any order; false if the
 // pairs are not one table entry (a bug in the walk: flagged by the caller).
@@ -63,19 +62,20 @@ __device__ __forceinline__ DF df_add(DF a, DF b)
 __device__ __forceinline__ DF df_of(float x) { return DF{x, 0.f}; }
 __device__ __forceinline__ float df_round(DF v) { return v.hi + v.lo; }
 
-// table index of a pn element from the candidate (uv, mv) and neutron move (ni):
-// u(a, b) = S[a][kappa] + r(b), v(c, d) = S[c][kappa] + r(d), kappa the dense
-// (2M_pair, parity) key; sign = proton move sign ^ neutron move sign
-__device__ __forceinline__ int pn_index_at(const int16_t *S, const int32_t *gs, const int32_t *go, uint32_t uv,
-                                           uint32_t mv, uint32_t ni, int &sign)
+// table index of a pn element from the proton move (l1: a | c << 8 | sign << 16
+// | pn_a[a] << 17) and the neutron move (n1: r(d) | r(b) << 8 | t(b) << 16 |
+// t(d) << 21 | sign << 26): u(a, b) = S(a, t(b)) + r(b), v(c, d) = S(c, t(d)) +
+// r(d) in the group of (a, t(b)); sign = proton move sign ^ neutron move sign.
+// KG, S: pn_k, pn_s in shared memory.
+__device__ __forceinline__ int pn_index_at(const int2 *KG, const int16_t *S, int T, int l1, int n1, int &sign)
 {
-    const int t = (int)((ni >> 16) & 0x7F) - 64 + (int)(((mv >> 8) ^ (ni >> 23)) & 1);
-    const int kappa = (int)(mv & 0xFF) + t;
-    int u = S[(int)(uv & 0xFFFF) + t] + (int)((ni >> 8) & 0xFF);
-    int v = S[(int)(uv >> 16) + t] + (int)(ni & 0xFF);
-    if (u > v) { const int x = u; u = v; v = x; }
-    sign = (int)(((mv >> 9) ^ (ni >> 24)) & 1);
-    return go[kappa] + u * gs[kappa] - ((u * (u - 1)) >> 1) + (v - u);
+    const int t = (n1 >> 16) & 0x1F;
+    const int2 g = KG[(t + ((unsigned)l1 >> 18)) ^ ((l1 >> 17) & 1)];
+    int u = S[(l1 & 0xFF) * T + t] + ((n1 >> 8) & 0xFF);
+    int v = S[((l1 >> 8) & 0xFF) * T + ((n1 >> 21) & 0x1F)] + (n1 & 0xFF);
+    if (u > v) { const int s = u; u = v; v = s; }
+    sign = ((l1 >> 16) ^ (n1 >> 26)) & 1;
+    return g.x + u * g.y - ((u * (u - 1)) >> 1) + (v - u);
 }
 
 }  // namespace cih

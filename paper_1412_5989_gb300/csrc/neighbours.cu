@@ -14,6 +14,7 @@
 
 #include <functional>
 #include <mutex>
+#include <type_traits>
 
 #include "cih_internal.h"
 
@@ -27,43 +28,6 @@ __device__ __forceinline__ void load_bits(const uint64_t *base, int64_t i, uint6
 {
 #pragma unroll
     for (int w = 0; w < W; ++w) o[w] = base[i * W + w];
-}
-
-template <int W>
-__device__ __forceinline__ int xor_pop(const uint64_t (&a)[W], const uint64_t *b)
-{
-    int c = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) c += __popcll(a[w] ^ b[w]);
-    return c;
-}
-
-// Same-class forward neighbours (1 or 2 orbitals moved, index > x): count or
-// write, one warp per sub-det, lanes over the later class members.
-template <int W, bool WRITE>
-__global__ void k_forward(SpeciesBuild S, int64_t *cnt, const int64_t *off, int32_t *out)
-{
-    int lane = threadIdx.x & 31;
-    int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t x = warp; x < S.n_sd; x += nwarps) {
-        uint64_t bx[W];
-        load_bits<W>(S.bits, x, bx);
-        int end = S.cls_end[x];
-        int64_t pos = WRITE ? off[x] : 0;
-        for (int y0 = (int)x + 1; y0 < end; y0 += 32) {
-            int y = y0 + lane;
-            bool hit = false;
-            if (y < end) {
-                int d = xor_pop<W>(bx, S.bits + (int64_t)y * W);
-                hit = d <= 4;                          // d == 0 only for y == x
-            }
-            unsigned m = __ballot_sync(0xffffffffu, hit);
-            if (WRITE && hit) out[pos + __popc(m & ((1u << lane) - 1))] = y;
-            pos += __popc(m);
-        }
-        if (!WRITE && lane == 0) cnt[x] = pos;
-    }
 }
 
 template <int W>
@@ -93,10 +57,8 @@ __global__ void k_hash_build(SpeciesBuild S, int32_t *table)
 
 // index of the sub-det with bits `yb`, or -1 (hash lookup; at most capacity probes)
 template <int W>
-__device__ int find_subdet(const SpeciesBuild &S, const uint64_t (&yb)[W], int Ny, int My)
+__device__ int find_subdet(const SpeciesBuild &S, const uint64_t (&yb)[W])
 {
-    (void)Ny;
-    (void)My;
     uint32_t h = hash_bits<W>(yb) & S.hash_mask;
     for (uint32_t probe = 0; probe <= S.hash_mask; ++probe) {
         const int32_t x = S.hash[h];
@@ -109,114 +71,6 @@ __device__ int find_subdet(const SpeciesBuild &S, const uint64_t (&yb)[W], int N
         h = (h + 1) & S.hash_mask;
     }
     return -1;
-}
-
-// index of the sub-det with bits `yb`, quanta Ny and 2M My, or -1 (binary
-// search inside its class; kept for reference)
-template <int W>
-__device__ int find_subdet_sorted(const SpeciesBuild &S, const uint64_t (&yb)[W], int Ny, int My)
-{
-    int key = My + S.moff;
-    if (key < 0 || key >= S.mspan) return -1;
-    int c = S.cls_lookup[key * 2 + (Ny & 1)];
-    if (c < 0) return -1;
-    int lo = S.cls_begin[c], hi = S.cls_endc[c];       // sorted by (N, bits)
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        int Nm = S.N[mid];
-        bool less;
-        if (Nm != Ny) {
-            less = Nm < Ny;
-        } else {
-            less = false;
-            const uint64_t *mb = S.bits + (int64_t)mid * W;
-#pragma unroll
-            for (int w = W - 1; w >= 0; --w) {
-                if (mb[w] != yb[w]) { less = mb[w] < yb[w]; break; }
-            }
-        }
-        if (less) lo = mid + 1; else hi = mid;
-    }
-    if (lo >= S.cls_endc[c] || S.N[lo] != Ny) return -1;
-    const uint64_t *mb = S.bits + (int64_t)lo * W;
-#pragma unroll
-    for (int w = 0; w < W; ++w)
-        if (mb[w] != yb[w]) return -1;
-    return lo;
-}
-
-// One-move neighbours: remove an occupied orbital r, add an empty orbital a;
-// one warp per sub-det, lanes over a.  Written unsorted, sorted afterwards.
-template <int W, bool WRITE>
-__global__ void k_onemove(SpeciesBuild S, int64_t *cnt, const int64_t *off, int32_t *out)
-{
-    int lane = threadIdx.x & 31;
-    int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t x = warp; x < S.n_sd; x += nwarps) {
-        uint64_t bx[W];
-        load_bits<W>(S.bits, x, bx);
-        int Nx = S.N[x];
-        int Mx = S.M2[x];
-        int64_t pos = WRITE ? off[x] : 0;
-        for (int w = 0; w < W; ++w) {
-            uint64_t occ = bx[w];
-            while (occ) {
-                int r = w * 64 + __ffsll((long long)occ) - 1;
-                occ &= occ - 1;
-                int Nr = S.oN[r], Mr = S.om2[r];
-                for (int a0 = 0; a0 < S.n_orb; a0 += 32) {
-                    int a = a0 + lane;
-                    int found = -1;
-                    if (a < S.n_orb && !((bx[a >> 6] >> (a & 63)) & 1)) {
-                        int Ny = Nx - Nr + S.oN[a];
-                        if (Ny <= S.Nsub_max) {
-                            uint64_t yb[W];
-#pragma unroll
-                            for (int v = 0; v < W; ++v) yb[v] = bx[v];
-                            yb[r >> 6] &= ~(1ull << (r & 63));
-                            yb[a >> 6] |= 1ull << (a & 63);
-                            found = find_subdet<W>(S, yb, Ny, Mx - Mr + S.om2[a]);
-                        }
-                    }
-                    unsigned m = __ballot_sync(0xffffffffu, found >= 0);
-                    if (WRITE && found >= 0) out[pos + __popc(m & ((1u << lane) - 1))] = found;
-                    pos += __popc(m);
-                }
-            }
-        }
-        if (!WRITE && lane == 0) cnt[x] = pos;
-    }
-}
-
-// Sort each list [off[x], off[x+1]) ascending: one block per list, bitonic
-// sort in shared memory (lists are at most kSortTile long; checked on the host).
-__global__ void k_sort_lists(const int64_t *off, int32_t *data, int64_t n)
-{
-    __shared__ int32_t s[kSortTile];
-    for (int64_t x = blockIdx.x; x < n; x += gridDim.x) {
-        int64_t b = off[x];
-        int len = (int)(off[x + 1] - b);
-        if (len <= 1) continue;
-        int P = 1;
-        while (P < len) P <<= 1;
-        for (int i = threadIdx.x; i < P; i += blockDim.x) s[i] = i < len ? data[b + i] : INT32_MAX;
-        __syncthreads();
-        for (int k = 2; k <= P; k <<= 1)
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < P; i += blockDim.x) {
-                    int l = i ^ j;
-                    if (l > i) {
-                        bool up = (i & k) == 0;
-                        int32_t a = s[i], c = s[l];
-                        if ((a > c) == up) { s[i] = c; s[l] = a; }
-                    }
-                }
-                __syncthreads();
-            }
-        for (int i = threadIdx.x; i < len; i += blockDim.x) data[b + i] = s[i];
-        __syncthreads();
-    }
 }
 
 template <int W>
@@ -241,13 +95,11 @@ __device__ __forceinline__ int count_below(const uint64_t (&R)[W], int k)
     return c;
 }
 
-// Packed one-move of each neutron list entry, bra x -> ket y:
-//   b = orbital in x only, d = orbital in y only, R = common orbitals;
-//   bits 0..7 r(d), 8..15 r(b), 16..22 2m_b + 64, 23 N_b & 1,
-//   24 sign (-1)^(#R below b + #R below d).
+// Neutron one-move lists packed, bra x -> ket y (DevBasis::n1p): b = orbital
+// in x only, d = orbital in y only, R = common orbitals, sign (-1)^(#R below b
+// + #R below d); orbs[b] = r(b) | t(b) << 8.
 template <int W>
-__global__ void k_n1_info(SpeciesBuild S, const int64_t *off, const int32_t *list, const int32_t *rn,
-                          uint32_t *info)
+__global__ void k_n1_pack(SpeciesBuild S, const int64_t *off, const int32_t *list, const uint16_t *orbs, int2 *packed)
 {
     int lane = threadIdx.x & 31;
     int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -257,147 +109,208 @@ __global__ void k_n1_info(SpeciesBuild S, const int64_t *off, const int32_t *lis
         load_bits<W>(S.bits, x, bx);
         for (int64_t t = off[x] + lane; t < off[x + 1]; t += 32) {
             uint64_t by[W], R[W], dx[W], dy[W];
-            load_bits<W>(S.bits, list[t], by);
+            const int y = list[t];
+            load_bits<W>(S.bits, y, by);
 #pragma unroll
             for (int w = 0; w < W; ++w) { R[w] = bx[w] & by[w]; dx[w] = bx[w] & ~by[w]; dy[w] = by[w] & ~bx[w]; }
-            int b = low_bit<W>(dx), d = low_bit<W>(dy);
-            int sg = (count_below<W>(R, b) + count_below<W>(R, d)) & 1;
-            info[t] = (uint32_t)rn[d] | ((uint32_t)rn[b] << 8) | ((uint32_t)(S.om2[b] + 64) << 16) |
-                      ((uint32_t)(S.oN[b] & 1) << 23) | ((uint32_t)sg << 24);
+            const int b = low_bit<W>(dx), d = low_bit<W>(dy);
+            const uint32_t sg = (count_below<W>(R, b) + count_below<W>(R, d)) & 1, ob = orbs[b], od = orbs[d];
+            packed[t] = make_int2(y, (int)((od & 0xFF) | (ob & 0xFF) << 8 | (ob >> 8) << 16 | (od >> 8) << 21 | sg << 26));
         }
     }
 }
 
-// Table index (<< 1) and sign bit of the two-move of each forward entry,
-// bra x -> ket y; one-moves are stored as ~(b | d << 8 | sign << 16) with b
-// in x only, d in y only.  Orbitals are offset by `base` into the
-// combined index of the pair table.
+// Splits the staged forward list of each sub-det x (one warp each) into its
+// two-moves, ascending from the slot's start, and its one-moves, ascending from
+// the slot's end backwards (DevSpecies::fw_rec, fw_tb), and counts the
+// two-moves per level.  A two-move's table index (<< 1) and sign bit: bra x ->
+// ket y, orbitals offset by `base` into the pair table; a one-move is stored
+// as ~(b | d << 8 | sign << 16) with b in x only, d in y only.  rowbase / nb:
+// the record holds the column base of y (protons), or null: y itself.
 template <int W>
-__global__ void k_fw_tb(SpeciesBuild S, int base, const int64_t *off, const int32_t *list, const int32_t *pid,
-                        const int32_t *gsize, const int64_t *goff, int ntot, int32_t *tb, int *status)
+__global__ void k_split(SpeciesBuild S, int base, int N0, int NL, const int32_t *cls_of, const int64_t *class_stage,
+                        const int64_t *off, const int32_t *stage, const int64_t *rowbase, const int32_t *nb,
+                        const int32_t *pid, const int32_t *gsize, const int64_t *goff, int ntot, int2 *rec, int32_t *tb,
+                        int32_t *lev, int *status)
 {
-    int lane = threadIdx.x & 31;
-    int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t x = warp; x < S.n_sd; x += nwarps) {
         uint64_t bx[W];
         load_bits<W>(S.bits, x, bx);
-        for (int64_t t = off[x] + lane; t < off[x + 1]; t += 32) {
+        const int c = cls_of[x];
+        const int64_t cb = S.cls_begin[c], m = S.cls_endc[c] - cb, r = x - cb;
+        const int32_t *in = stage + class_stage[c] + r * (m - 1) - r * (r - 1) / 2;
+        const int64_t o0 = off[x], o1 = off[x + 1];
+        const int len = (int)(o1 - o0);
+        int n2 = 0, n1 = 0;                                    // two- and one-moves so far
+        int at_lev = 0;                                        // lane l: two-moves at levels <= l
+        for (int t0 = 0; t0 < len; t0 += 32) {
+            const bool on = t0 + lane < len;
+            const int y = on ? in[t0 + lane] : (int)x;
             uint64_t by[W], R[W], dx[W], dy[W];
-            load_bits<W>(S.bits, list[t], by);
+            load_bits<W>(S.bits, y, by);
             int pc = 0;
 #pragma unroll
             for (int w = 0; w < W; ++w) {
                 R[w] = bx[w] & by[w]; dx[w] = bx[w] & ~by[w]; dy[w] = by[w] & ~bx[w];
                 pc += __popcll(dx[w]);
             }
-            if (pc != 2) {                                  // one-move: ~(b | d << 8 | sign << 16)
-                const int b1 = low_bit<W>(dx), d1 = low_bit<W>(dy);
-                const int s1 = (count_below<W>(R, b1) + count_below<W>(R, d1)) & 1;
-                tb[t] = ~(int32_t)(b1 | (d1 << 8) | (s1 << 16));
-                continue;
+            const bool two = on && pc == 2, one = on && pc != 2;
+            const unsigned m2 = __ballot_sync(0xffffffffu, two), m1 = __ballot_sync(0xffffffffu, one);
+            const int lv = (S.N[y] - N0) >> 1;
+            for (int l = 0; l < NL; ++l) {
+                const unsigned ml = __ballot_sync(0xffffffffu, two && lv <= l);
+                if (lane == l) at_lev += __popc(ml);
             }
-            int a1 = low_bit<W>(dx); dx[a1 >> 6] &= ~(1ull << (a1 & 63));
-            int a2 = low_bit<W>(dx);
-            int c1 = low_bit<W>(dy); dy[c1 >> 6] &= ~(1ull << (c1 & 63));
-            int c2 = low_bit<W>(dy);
-            int sg = (count_below<W>(R, a1) + count_below<W>(R, a2) + count_below<W>(R, c1) + count_below<W>(R, c2)) & 1;
-            int32_t e1 = pid[(base + a1) * ntot + base + a2], e2 = pid[(base + c1) * ntot + base + c2];
-            if (e1 < 0 || e2 < 0 || ((e1 ^ e2) & (0xFFF << 16))) { atomicOr(status, 4); tb[t] = -1; continue; }
-            int g = (e1 >> 16) & 0xFFF;
-            int64_t u = e1 & 0xFFFF, v = e2 & 0xFFFF;
-            if (u > v) { int64_t q = u; u = v; v = q; }
-            int64_t n = gsize[g];
-            int64_t idx = goff[g] + u * n - u * (u - 1) / 2 + (v - u);
-            tb[t] = (int32_t)((idx << 1) | sg);
+            if (on) {
+                const int k2 = n2 + __popc(m2 & lt), k1 = n1 + __popc(m1 & lt);
+                const int64_t slot = two ? o0 + k2 : o1 - 1 - k1;
+                rec[slot] = make_int2(rowbase ? (int)(rowbase[y] - nb[y]) : y, (two ? k1 : k2) | lv << 24);
+                if (one) {
+                    const int b1 = low_bit<W>(dx), d1 = low_bit<W>(dy);
+                    const int s1 = (count_below<W>(R, b1) + count_below<W>(R, d1)) & 1;
+                    tb[slot] = ~(int32_t)(b1 | (d1 << 8) | (s1 << 16));
+                } else {
+                    int a1 = low_bit<W>(dx); dx[a1 >> 6] &= ~(1ull << (a1 & 63));
+                    int a2 = low_bit<W>(dx);
+                    int c1 = low_bit<W>(dy); dy[c1 >> 6] &= ~(1ull << (c1 & 63));
+                    int c2 = low_bit<W>(dy);
+                    int sg = (count_below<W>(R, a1) + count_below<W>(R, a2) + count_below<W>(R, c1) + count_below<W>(R, c2)) & 1;
+                    int32_t e1 = pid[(base + a1) * ntot + base + a2], e2 = pid[(base + c1) * ntot + base + c2];
+                    if (e1 < 0 || e2 < 0 || ((e1 ^ e2) & (0xFFF << 16))) {
+                        atomicOr(status, 4);
+                        tb[slot] = 0;
+                    } else {
+                        int g = (e1 >> 16) & 0xFFF;
+                        int64_t u = e1 & 0xFFFF, v = e2 & 0xFFFF;
+                        if (u > v) { int64_t q = u; u = v; v = q; }
+                        int64_t n = gsize[g];
+                        int64_t idx = goff[g] + u * n - u * (u - 1) / 2 + (v - u);
+                        tb[slot] = (int32_t)((idx << 1) | sg);
+                    }
+                }
+            }
+            n2 += __popc(m2);
+            n1 += __popc(m1);
         }
+        if (lane < NL) lev[x * NL + lane] = at_lev;
     }
 }
 
-// first one-move entry of each sub-det beyond its own class, and the size of
-// its candidate list (forward same-class entries + later-class one-moves)
-__global__ void k_later(int64_t n, const int32_t *cls_end, const int64_t *fw_off, const int64_t *n1_off,
-                        const int32_t *n1, int64_t *later, int *max_cand)
+// one-move entries of each sub-det below itself
+__global__ void k_n1_self(int64_t n, const int64_t *n1_off, const int32_t *n1, int32_t *self)
 {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
         int64_t lo = n1_off[x], hi = n1_off[x + 1];
-        int key = cls_end[x];
+        const int64_t a0 = lo;
         while (lo < hi) {
-            int64_t mid = (lo + hi) >> 1;
-            if (n1[mid] < key) lo = mid + 1; else hi = mid;
+            const int64_t mid = (lo + hi) >> 1;
+            if (n1[mid] < x) lo = mid + 1; else hi = mid;
         }
-        later[x] = lo;
-        int64_t c = (fw_off[x + 1] - fw_off[x]) + (n1_off[x + 1] - lo);
-        atomicMax(max_cand, (int)min(c, (int64_t)INT32_MAX));
+        self[x] = (int32_t)(lo - a0);
     }
 }
 
-// Candidate table of proton sub-det p (bra p -> ket q); see DevBasis.
-// The directory indices locate q's neutron range in the one-move list of any
-// row neutron n of p: the range is the prefix N <= L_q of the class
-// (2M - 2M_q, parity of Nlim - N_q), which relative to n's class is
-// 2M_p - 2M_q.
-template <int W>
-__global__ void k_cand(SpeciesBuild S, DevBasis B, const int8_t *Nq, const int16_t *M2q, int Nlim, int64_t *cand_off,
-                       int4 *cand, uint8_t *cself)
+// Group records of each proton sub-det (DevBasis::grp), one warp per p.  PASS
+// 0 counts them; PASS 1 writes them, and the packed one-moves (DevBasis::l1).
+template <int W, int PASS>
+__global__ void k_groups(SpeciesBuild S, DevBasis B, int64_t *gcnt, int4 *grp, int2 *l1)
 {
-    const DevSpecies &SP = B.sp[0];
-    int lane = threadIdx.x & 31;
-    int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int G = B.pn_G, span = B.pn_m2span, NL = B.NL, DM = B.DM;
+    const DevSpecies &SP = B.sp[0], &SN = B.sp[1];
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int NL = SP.NL;
     for (int64_t p = warp; p < S.n_sd; p += nwarps) {
+        const int64_t i0 = SP.n1_off[p] + SP.n1_self[p], i1 = SP.n1_off[p + 1];
+        const int cend = SP.cls_end[p];
+        int64_t mid = i0, hi = i1;                              // first one-move beyond p's class
+        while (mid < hi) {
+            const int64_t h = (mid + hi) >> 1;
+            if (SP.n1[h] < cend) mid = h + 1; else hi = h;
+        }
+        const int64_t later = mid;
+        // directory positions of the segment of q's range in the list of a row neutron of p
+        auto seg = [&](int q) {
+            const int Lq = B.Nlim - S.N[q], dM = S.M2[p] - S.M2[q];
+            if (dM > B.DM || dM < -B.DM || Lq < SN.N0) return 0;       // no neutron one-move reaches it
+            const int rc = ((dM + B.DM) >> 1) * 2 + (Lq & 1), l = min((Lq - SN.N0) >> 1, SN.NL - 1);
+            return rc * SN.NL | (1 + rc * SN.NL + l) << 16;
+        };
+        // own class: lane l holds level l
+        const int par = (S.N[p] - SP.N0) & 1;
+        int t2 = lane < NL ? SP.fw_lev[p * NL + lane] : 0, e = (int)(later - i0);
+        if (lane < NL) {                                        // one-moves of levels <= lane
+            int64_t lo = i0, h2 = later;
+            while (lo < h2) {
+                const int64_t h = (lo + h2) >> 1;
+                if (((S.N[SP.n1[h]] - SP.N0) >> 1) <= lane) lo = h + 1; else h2 = h;
+            }
+            e = (int)(lo - i0);
+        }
+        const int pe = __shfl_up_sync(0xffffffffu, e, 1), pt2 = __shfl_up_sync(0xffffffffu, t2, 1);
+        const int e0 = lane ? pe : 0, t20 = lane ? pt2 : 0;
+        const bool has = lane < NL && (e > e0 || t2 > t20);
+        const unsigned hm = __ballot_sync(0xffffffffu, has);
+        const int64_t g0 = PASS ? gcnt[p] : 0;
+        if (PASS == 1 && has) {
+            const int Nq = SP.N0 + 2 * lane + par, Lq = B.Nlim - Nq;
+            int st = 0;
+            if (Lq >= SN.N0) {
+                const int rc = (B.DM >> 1) * 2 + (Lq & 1), l = min((Lq - SN.N0) >> 1, SN.NL - 1);
+                st = rc * SN.NL | (1 + rc * SN.NL + l) << 16;
+            }
+            grp[g0 + __popc(hm & lt)] = make_int4(e0 | (e - e0) << 16, st, t2 - t20, (1 + Lq) | t20 << 8);
+        }
+        int ng = __popc(hm);
+        const int gl = ng;                                      // first later-class group
+        for (int64_t t0 = later; t0 < i1; t0 += 32) {
+            const int64_t t = t0 + lane;
+            const int q = t < i1 ? SP.n1[t] : 0;
+            const int b = t > later && t < i1 ? SP.n1[t - 1] : -1;
+            const bool first = t < i1 && (b < 0 || SP.cls_end[q] != SP.cls_end[b] || S.N[q] != S.N[b]);
+            const unsigned fm = __ballot_sync(0xffffffffu, first);
+            if (PASS == 1 && first) grp[g0 + ng + __popc(fm & lt)] = make_int4((int)(t - i0), seg(q), 0, 0);
+            ng += __popc(fm);
+        }
+        if (PASS == 0) {
+            if (lane == 0) gcnt[p] = ng;
+            continue;
+        }
+        __syncwarp();
+        for (int j0 = gl; j0 < ng; j0 += 32) {                  // members of the later-class groups
+            const int j = j0 + lane;
+            int a = 0, z = 0;
+            if (j < ng) {
+                a = grp[g0 + j].x & 0xFFFF;
+                z = j + 1 < ng ? grp[g0 + j + 1].x & 0xFFFF : (int)(i1 - i0);
+            }
+            __syncwarp();
+            if (j < ng) grp[g0 + j].x = a | (z - a) << 16;
+            __syncwarp();
+        }
         uint64_t pb[W];
         load_bits<W>(S.bits, p, pb);
-        const int64_t f0 = SP.fw_off[p], nf = SP.fw_off[p + 1] - f0;
-        const int64_t l0 = SP.n1_later[p];
-        const int64_t C = nf + (SP.n1_off[p + 1] - l0);
-        const int64_t base = cand_off[p];
-        const int par_p = (Nlim - Nq[p]) & 1;
-        for (int64_t k = lane; k < C; k += 32) {
-            const int q = k < nf ? SP.fw[f0 + k] : SP.n1[l0 + (k - nf)];
+        for (int64_t t = i0 + lane; t < i1; t += 32) {
+            const int q = SP.n1[t];
             uint64_t qb[W], R[W], dx[W], dy[W];
             load_bits<W>(S.bits, q, qb);
-            int pc = 0;
 #pragma unroll
-            for (int w = 0; w < W; ++w) {
-                R[w] = pb[w] & qb[w]; dx[w] = pb[w] & ~qb[w]; dy[w] = qb[w] & ~pb[w];
-                pc += __popcll(dx[w]);
-            }
-            const int Lq = Nlim - Nq[q];                       // largest N of a partner of q
-            const int par_q = Lq & 1;
-            const int dM = M2q[p] - M2q[q];
-            const int rc = ((dM + DM) >> 1) * 2 + par_q;
-            const int Lc = min(Lq, NL - 1);
-            int st = rc * NL, en = 1 + rc * NL + Lc;
-            if (dM > DM || dM < -DM || Lc < 0) st = en = 0;  // no neutron one-move reaches q's range
-            const bool same = M2q[p] == M2q[q] && par_p == par_q;    // q's range is in n's class
-            int4 r;
-            r.x = (int32_t)(B.rowbase[q] - B.nb[q]);
-            r.y = st | (en << 16);
-            uint8_t sl = same ? (uint8_t)(1 + Lq) : 0;
-            if (pc == 1) {
-                const int a = low_bit<W>(dx), c = low_bit<W>(dy);
-                const int sg = (count_below<W>(R, a) + count_below<W>(R, c)) & 1;
-                const int Ka = (S.om2[a] + span) & 0xFF;       // >= 0 by the choice of span
-                r.z = (int32_t)((uint32_t)(a * G + Ka) | ((uint32_t)(c * G + Ka) << 16));
-                r.w = (int32_t)((uint32_t)Ka | ((uint32_t)(S.oN[a] & 1) << 8) | ((uint32_t)sg << 9) |
-                                ((uint32_t)a << 16) | ((uint32_t)c << 24));
-            } else {
-                r.z = B.fw_tb[0][f0 + k];
-                r.w = 0;
-                sl |= 0x80;
-            }
-            cand[base + k] = r;
-            cself[base + k] = sl;
+            for (int w = 0; w < W; ++w) { R[w] = pb[w] & qb[w]; dx[w] = pb[w] & ~qb[w]; dy[w] = qb[w] & ~pb[w]; }
+            const int a = low_bit<W>(dx), c = low_bit<W>(dy);
+            const int sg = (count_below<W>(R, a) + count_below<W>(R, c)) & 1;
+            l1[t] = make_int2((int)(B.rowbase[q] - B.nb[q]), a | c << 8 | sg << 16 | B.pn_a[a] << 17);
         }
     }
 }
 
-// occupied orbitals of each sub-det, ascending; and for the neutron lists the
-// number of one-move entries below the sub-det itself
+// occupied orbitals of each sub-det, ascending
 template <int W>
-__global__ void k_occ(SpeciesBuild S, int Z, const int64_t *n1_off, const int32_t *n1, uint8_t *occ, int16_t *self_rel)
+__global__ void k_occ(SpeciesBuild S, int Z, uint8_t *occ)
 {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < S.n_sd; x += (int64_t)gridDim.x * blockDim.x) {
         int k = 0;
@@ -408,27 +321,11 @@ __global__ void k_occ(SpeciesBuild S, int Z, const int64_t *n1_off, const int32_
                 m &= m - 1;
             }
         }
-        if (self_rel) {
-            int64_t lo = n1_off[x], hi = n1_off[x + 1];
-            const int64_t a0 = lo;
-            while (lo < hi) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (n1[mid] < x) lo = mid + 1; else hi = mid;
-            }
-            self_rel[x] = (int16_t)(lo - a0);
-        }
     }
 }
 
-// Pack each neutron one-move entry with its move info, and build the bucket
-// directory of each list (see DevBasis).
-__global__ void k_n1_pack(int64_t n, const int64_t *off, const int32_t *list, const uint32_t *info, int2 *packed)
-{
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < off[n]; t += (int64_t)gridDim.x * blockDim.x)
-        packed[t] = make_int2(list[t], (int)info[t]);
-}
-
-__global__ void k_dir(SpeciesBuild S, const int64_t *off, const int32_t *list, int NL, int DM, int dir_len,
+// bucket directory of each neutron one-move list (DevBasis::dir)
+__global__ void k_dir(SpeciesBuild S, const int64_t *off, const int32_t *list, int N0, int NL, int DM, int dir_len,
                       int16_t *dir)
 {
     int lane = threadIdx.x & 31;
@@ -445,7 +342,7 @@ __global__ void k_dir(SpeciesBuild S, const int64_t *off, const int32_t *list, i
             while (lo < hi) {
                 const int64_t mid = (lo + hi) >> 1;
                 const int y = list[mid];
-                const int key = (((int)S.M2[y] - M0 + DM) >> 1) * 2 * NL + (S.N[y] & 1) * NL + S.N[y];
+                const int key = ((((int)S.M2[y] - M0 + DM) >> 1) * 2 + (S.N[y] & 1)) * NL + ((S.N[y] - N0) >> 1);
                 if (key <= b) lo = mid + 1; else hi = mid;
             }
             d[1 + b] = (int16_t)(lo - a0);
@@ -453,11 +350,30 @@ __global__ void k_dir(SpeciesBuild S, const int64_t *off, const int32_t *list, i
     }
 }
 
-__global__ void k_cand_count(int64_t n, const int64_t *fw_off, const int64_t *n1_off, const int64_t *later,
-                             int64_t *cnt)
+// per-sub-det records of the row kernels
+__global__ void k_proton_rec(DevBasis B, const int64_t *goff, ProtonRec *rec)
 {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
-        cnt[x] = (fw_off[x + 1] - fw_off[x]) + (n1_off[x + 1] - later[x]);
+    const DevSpecies &SP = B.sp[0], &SN = B.sp[1];
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < SP.n_sd; p += (int64_t)gridDim.x * blockDim.x) {
+        const int Lp = B.Nlim - SP.N[p], l = min((Lp - SN.N0) >> 1, SN.NL - 1);
+        ProtonRec r;
+        r.l1 = SP.n1_off[p] + SP.n1_self[p];
+        r.fw = SP.fw_off[p];
+        r.g0 = goff[p];
+        r.fwlen = (int32_t)(SP.fw_off[p + 1] - r.fw);
+        r.colb = (int32_t)(B.rowbase[p] - B.nb[p]);
+        r.nb = B.nb[p];
+        r.ng = (int32_t)(goff[p + 1] - r.g0);
+        r.dirA = 1 + ((B.DM >> 1) * 2 + (Lp & 1)) * SN.NL + l;
+        r.levA = l;
+        rec[p] = r;
+    }
+}
+
+__global__ void k_neutron_rec(DevSpecies SN, NeutronRec *rec)
+{
+    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < SN.n_sd; n += (int64_t)gridDim.x * blockDim.x)
+        rec[n] = NeutronRec{SN.n1_off[n], SN.fw_off[n], (int32_t)(SN.fw_off[n + 1] - SN.fw_off[n]), SN.n1_self[n], SN.N[n], 0};
 }
 
 __global__ void k_row_p(int64_t np, const int64_t *rowbase, int32_t *row_p)
@@ -515,21 +431,6 @@ __global__ void k_bits_T(int64_t n, int W, const uint64_t *bits, uint64_t *bitsT
     }
 }
 
-__global__ void k_forward_compact(SpeciesBuild S, const int32_t *cls_of, const int64_t *class_stage,
-                                  const int64_t *off, const int32_t *stage, int32_t *out)
-{
-    int lane = threadIdx.x & 31;
-    int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t x = warp; x < S.n_sd; x += nwarps) {
-        const int c = cls_of[x];
-        const int64_t cb = S.cls_begin[c], m = S.cls_endc[c] - cb, r = x - cb;
-        const int32_t *in = stage + class_stage[c] + r * (m - 1) - r * (r - 1) / 2;
-        const int64_t o = off[x], len = off[x + 1] - o;
-        for (int64_t i = lane; i < len; i += 32) out[o + i] = in[i];
-    }
-}
-
 // Single-pass one-move lists: each sub-det writes its moves (unsorted) into
 // a slot of `cap` entries; cnt[x] gets the count.
 template <int W>
@@ -562,7 +463,7 @@ __global__ void k_onemove_staged(SpeciesBuild S, int cap, int64_t *cnt, int32_t 
                         for (int v = 0; v < W; ++v) yb[v] = bx[v];
                         yb[r >> 6] &= ~(1ull << (r & 63));
                         yb[a >> 6] |= 1ull << (a & 63);
-                        found = find_subdet<W>(S, yb, 0, 0);
+                        found = find_subdet<W>(S, yb);
                     }
                     const unsigned msk = __ballot_sync(0xffffffffu, found >= 0);
                     if (found >= 0) out[pos + __popc(msk & ((1u << lane) - 1))] = found;
@@ -616,57 +517,6 @@ __global__ void k_onemove_compact_sort(int64_t n, int cap, const int64_t *off, c
     }
 }
 
-
-// Count lists (see DevBasis): one warp per proton sub-det accumulates the
-// directory coefficients of its one-move candidates (segment end +1, start
-// -1) and the histogram of its candidates' 1 + L_q in shared memory; pass 0
-// writes the number of non-zero coefficients, pass 1 the list (ascending
-// directory position) and the suffix counts #{c : 1 + L_q(c) > N}.
-constexpr int kClistDirCap = 4096;
-template <int PASS>
-__global__ void k_clists(int64_t np, const int64_t *cand_off, const int4 *cand, const uint8_t *cself, int dir_len,
-                         int NL, int64_t *clen, const int64_t *clist_off, int2 *clist, uint16_t *cself_sfx)
-{
-    extern __shared__ int cl_sh[];                 // per warp: int[dir_len] coefficients, int[64] histogram
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int *coef = cl_sh + wid * (dir_len + 64);
-    int *hist = coef + dir_len;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t p = warp; p < np; p += nw) {
-        for (int i = lane; i < dir_len; i += 32) coef[i] = 0;
-        for (int i = lane; i < 64; i += 32) hist[i] = 0;
-        __syncwarp();
-        for (int64_t c = cand_off[p] + lane; c < cand_off[p + 1]; c += 32) {
-            const uint8_t sl = cself[c];
-            atomicAdd(&hist[min(sl & 0x7F, 63)], 1);              // > N for every N < NL either way
-            if (!(sl >> 7)) {                                  // one-move: a neutron segment
-                const unsigned y = (unsigned)cand[c].y;
-                atomicAdd(&coef[y >> 16], 1);
-                atomicAdd(&coef[y & 0xFFFF], -1);
-            }
-        }
-        __syncwarp();
-        int64_t out = PASS == 1 ? clist_off[p] : 0;
-        int n = 0;
-        for (int i0 = 0; i0 < dir_len; i0 += 32) {
-            const int i = i0 + lane;
-            const int v = i < dir_len ? coef[i] : 0;
-            const unsigned m = __ballot_sync(0xffffffffu, v != 0);
-            if (PASS == 1 && v != 0) clist[out + n + __popc(m & ((1u << lane) - 1))] = make_int2(i, v);
-            n += __popc(m);
-        }
-        if (PASS == 0 && lane == 0) clen[p] = n;
-        if (PASS == 1)
-            for (int N = lane; N < NL; N += 32) {              // candidates with 1 + L_q > N
-                int s = 0;
-                for (int v = N + 1; v < 64; ++v) s += hist[v];
-                cself_sfx[p * NL + N] = (uint16_t)s;
-            }
-        __syncwarp();
-    }
-}
-
 template <class T>
 int dev_alloc(cih_basis &b, T **p, size_t n)
 {
@@ -714,23 +564,28 @@ int grid_for(int64_t warps)
     return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)sms * 16));
 }
 
+// fn(std::integral_constant<int, W>) for the basis' words per bit string
+template <class Fn>
+void with_words(int W, Fn &&fn)
+{
+    if (W == 1) fn(std::integral_constant<int, 1>());
+    else if (W == 2) fn(std::integral_constant<int, 2>());
+    else fn(std::integral_constant<int, 4>());
+}
+
 // Neighbour lists of one species, in three phases so that both species'
 // kernels queue back to back and the host work in between overlaps them:
 //   1. staged forward and one-move passes, their counts scanned, list totals
 //      copied to pinned host memory;
-//   2. (after one synchronisation) exact-size lists: compaction and sort,
-//      later-entry offsets;
-//   3. (once the table layout is on the device) two-move table indices and
-//      the packed neutron move information.
+//   2. (after one synchronisation) exact-size one-move lists: compaction and sort;
+//   3. (once the table layout is on the device) the forward lists split into
+//      one- and two-moves, with table indices.
 struct Lists {
     int64_t n = 0, ns = 0;
     int64_t *cnt_fw = nullptr, *cnt_n1 = nullptr, *scratch = nullptr, *d_class_stage = nullptr;
-    int32_t *d_cls_of = nullptr, *fw_st = nullptr, *n1_st = nullptr, *fw = nullptr, *n1 = nullptr;
-    int64_t *later = nullptr;
-    int *dmax = nullptr;
+    int32_t *d_cls_of = nullptr, *fw_st = nullptr, *n1_st = nullptr, *n1 = nullptr;
     int cap1 = 1, grid = 1;
     int64_t *tot = nullptr;                   // pinned: forward and one-move totals
-    int32_t *rn = nullptr;                    // neutron species: pn split row of each orbital (device)
 };
 
 template <int W>
@@ -774,53 +629,47 @@ int lists_phase2(cih_basis &b, int t, SpeciesBuild &S, Lists &L, cudaStream_t st
 {
     const int64_t n = L.n;
     int rc;
-    if ((rc = dev_alloc(b, &L.fw, L.tot[0])) || (rc = dev_alloc(b, &L.n1, L.tot[1]))) return rc;
+    int32_t *self;
+    if ((rc = dev_alloc(b, &L.n1, L.tot[1])) || (rc = dev_alloc(b, &self, n))) return rc;
     if (n > 0) {
         count_launches(2);
-        k_forward_compact<<<L.grid, 256, 0, st>>>(S, L.d_cls_of, L.d_class_stage, L.cnt_fw, L.fw_st, L.fw);
         k_onemove_compact_sort<<<(int)std::min<int64_t>(n, 65535), 256, 0, st>>>(n, L.cap1, L.cnt_n1, L.n1_st, L.n1);
+        k_n1_self<<<L.grid, 256, 0, st>>>(n, L.cnt_n1, L.n1, self);
     }
-    dev_free(b, L.fw_st);
     dev_free(b, L.n1_st);
-    L.fw_st = L.n1_st = nullptr;
-    if ((rc = dev_alloc(b, &L.later, n)) || (rc = dev_alloc(b, &L.dmax, 1))) return rc;
-    cudaMemsetAsync(L.dmax, 0, sizeof(int), st);
-    if (n > 0) {
-        count_launches(1);
-        k_later<<<L.grid, 256, 0, st>>>(n, S.cls_end, L.cnt_fw, L.cnt_n1, L.n1, L.later, L.dmax);
-    }
+    L.n1_st = nullptr;
     DevSpecies &D = b.dev.sp[t];
     D.fw_off = L.cnt_fw;
-    D.fw = L.fw;
     D.n1_off = L.cnt_n1;
     D.n1 = L.n1;
-    D.n1_later = L.later;
+    D.n1_self = self;
+    (void)S;
     return CIH_OK;
 }
 
-template <int W>
 int lists_phase3(cih_basis &b, int t, SpeciesBuild &S, Lists &L, cudaStream_t st)
 {
     const int64_t n = L.n;
+    DevSpecies &D = b.dev.sp[t];
     int rc;
-    int32_t *tb;
-    if ((rc = dev_alloc(b, &tb, L.tot[0]))) return rc;
+    int32_t *tb, *lev;
+    int2 *rec;
+    if ((rc = dev_alloc(b, &tb, L.tot[0])) || (rc = dev_alloc(b, &rec, L.tot[0])) ||
+        (rc = dev_alloc(b, &lev, (size_t)n * D.NL)))
+        return rc;
     if (n > 0) {
         count_launches(1);
-        k_fw_tb<W><<<L.grid, 256, 0, st>>>(S, t == 0 ? 0 : b.s[0].n_orb, L.cnt_fw, L.fw, b.dev.pid, b.dev.gsize,
-                                           b.dev.goff, b.dev.ntot, tb, b.dev_status);
+        with_words(b.W, [&](auto w) {
+            k_split<decltype(w)::value><<<L.grid, 256, 0, st>>>(
+                S, D.orb_base, D.N0, D.NL, L.d_cls_of, L.d_class_stage, L.cnt_fw, L.fw_st, t == 0 ? b.dev.rowbase : nullptr,
+                t == 0 ? b.dev.nb : nullptr, b.dev.pid, b.dev.gsize, b.dev.goff, b.dev.ntot, rec, tb, lev, b.dev_status);
+        });
     }
-    if (t == 1) {
-        uint32_t *info;
-        if ((rc = dev_alloc(b, &info, L.tot[1]))) return rc;
-        if (n > 0) {
-            count_launches(1);
-            k_n1_info<W><<<L.grid, 256, 0, st>>>(S, L.cnt_n1, L.n1, L.rn, info);
-        }
-        b.dev.n1_info = info;
-    }
-    if (t == 0) cudaMemcpyAsync(&L.tot[2], L.dmax, sizeof(int), cudaMemcpyDeviceToHost, st);
-    b.dev.fw_tb[t] = tb;
+    dev_free(b, L.fw_st);
+    L.fw_st = nullptr;
+    D.fw_rec = rec;
+    D.fw_tb = tb;
+    D.fw_lev = lev;
     return CIH_OK;
 }
 
@@ -830,8 +679,7 @@ struct SpeciesHost {
     std::vector<uint64_t> bits;
     std::vector<int8_t> N, oN;
     std::vector<int16_t> M2, om2;
-    std::vector<int32_t> cls_end, lookup, cb, ce;
-    int moff = 0, mspan = 0;
+    std::vector<int32_t> cls_end, cb, ce;
 };
 
 void species_prep(const cih_basis &b, int t, SpeciesHost &H)
@@ -845,13 +693,6 @@ void species_prep(const cih_basis &b, int t, SpeciesHost &H)
     H.M2.assign(s.M2.begin(), s.M2.end());
     H.cls_end.resize(s.n_sd);
     for (int64_t i = 0; i < s.n_sd; ++i) H.cls_end[i] = s.cls_end[s.cls[i]];
-    int mabs = 0;
-    for (int m : s.cls_M2) mabs = std::max(mabs, std::abs(m));
-    H.mspan = 2 * mabs + 1 + 64;                     // room for moves that leave the table
-    H.moff = mabs + 32;
-    H.lookup.assign((size_t)H.mspan * 2, -1);
-    for (size_t c = 0; c < s.cls_begin.size(); ++c)
-        H.lookup[(size_t)(s.cls_M2[c] + H.moff) * 2 + s.cls_par[c]] = (int32_t)c;
     H.cb.assign(s.cls_begin.begin(), s.cls_begin.end());
     H.ce.assign(s.cls_end.begin(), s.cls_end.end());
     H.oN.assign(s.oN.begin(), s.oN.end());
@@ -863,11 +704,11 @@ int species_upload(cih_basis &b, int t, const SpeciesHost &H, cudaStream_t st)
     const int W = b.W;
     const Species &s = b.s[t];
     int rc;
-    uint64_t *d_bits; int8_t *d_N; int16_t *d_M2; int32_t *d_cls_end, *d_lookup, *d_cb, *d_ce;
+    uint64_t *d_bits; int8_t *d_N; int16_t *d_M2; int32_t *d_cls_end, *d_cb, *d_ce;
     int8_t *d_oN; int16_t *d_om2;
     if ((rc = upload(b, &d_bits, H.bits, st)) || (rc = upload(b, &d_N, H.N, st)) ||
         (rc = upload(b, &d_M2, H.M2, st)) || (rc = upload(b, &d_cls_end, H.cls_end, st)) ||
-        (rc = upload(b, &d_lookup, H.lookup, st)) || (rc = upload(b, &d_cb, H.cb, st)) ||
+        (rc = upload(b, &d_cb, H.cb, st)) ||
         (rc = upload(b, &d_ce, H.ce, st)) || (rc = upload(b, &d_oN, H.oN, st)) ||
         (rc = upload(b, &d_om2, H.om2, st)))
         return rc;
@@ -878,9 +719,11 @@ int species_upload(cih_basis &b, int t, const SpeciesHost &H, cudaStream_t st)
     D.n_sd = (int32_t)s.n_sd;
     D.n_orb = s.n_orb;
     D.orb_base = t == 0 ? 0 : b.s[0].n_orb;
+    D.N0 = s.N0;
+    D.NL = s.Z > 0 ? ((s.Nsub_max - s.N0) >> 1) + 1 : 1;
+    if (D.NL > kLevels) return fail(CIH_ERR_UNSUPPORTED, "internal: more oscillator levels than 256 orbitals give");
 
-    SpeciesBuild S{d_bits, d_N, d_M2, d_cls_end, d_lookup, d_cb, d_ce, d_oN, d_om2,
-                   (int32_t)s.n_sd, s.n_orb, H.moff, H.mspan, s.Nsub_max, nullptr, 0};
+    SpeciesBuild S{d_bits, d_N, d_M2, d_cls_end, d_cb, d_ce, d_oN, d_om2, (int32_t)s.n_sd, s.n_orb, s.Nsub_max};
     uint32_t cap = 64;
     while (cap < 2 * (uint64_t)s.n_sd) cap <<= 1;
     int32_t *table;
@@ -909,9 +752,7 @@ int species_upload(cih_basis &b, int t, const SpeciesHost &H, cudaStream_t st)
     S.maxN = maxN;
     const int hg = (int)std::min<int64_t>((s.n_sd + 255) / 256 + 1, 65535);
     count_launches(1);
-    if (W == 1) k_hash_build<1><<<hg, 256, 0, st>>>(S, table);
-    else if (W == 2) k_hash_build<2><<<hg, 256, 0, st>>>(S, table);
-    else k_hash_build<4><<<hg, 256, 0, st>>>(S, table);
+    with_words(W, [&](auto w) { k_hash_build<decltype(w)::value><<<hg, 256, 0, st>>>(S, table); });
     b.sbuild[t] = S;
     return CIH_OK;
 }
@@ -943,16 +784,43 @@ int basis_tables_upload(cih_basis &b, cudaStream_t st)
     b.dev.ntot = ntot;
     b.dev.dim = b.dim;
     b.dev.tbme_len = b.layout.total;
-    std::vector<int8_t> m2p(std::max(b.s[0].n_orb, 1), 0), Np(std::max(b.s[0].n_orb, 1), 0);
-    for (int a = 0; a < b.s[0].n_orb; ++a) { m2p[a] = (int8_t)b.s[0].om2[a]; Np[a] = (int8_t)b.s[0].oN[a]; }
-    int16_t *d_S; int32_t *d_gs, *d_go; int8_t *d_m2p, *d_Np;
-    if ((rc = upload(b, &d_S, b.pn.S, st)) || (rc = upload(b, &d_gs, b.pn.gsize, st)) ||
-        (rc = upload(b, &d_go, b.pn.goff, st)) || (rc = upload(b, &d_m2p, m2p, st)) ||
-        (rc = upload(b, &d_Np, Np, st)))
+    b.dev.Nlim = b.Nlim;
+    b.dev.A = b.space.Z + b.space.N;
+    b.dev.nZ[0] = b.space.Z;
+    b.dev.nZ[1] = b.space.N;
+    // pn pairs by proton orbital and neutron type t = (2m, N parity)
+    const Species &P = b.s[0], &Q = b.s[1];
+    int mtop = 1;                                              // odd, >= every |2m|
+    for (int c = 0; c < Q.n_orb; ++c) mtop = std::max(mtop, std::abs(Q.om2[c]));
+    const int T = b.dev.pn_T = (mtop + 1) * 2;
+    if (T > 32) return fail(CIH_ERR_UNSUPPORTED, "neutron orbitals with 2m above 15");
+    std::vector<uint16_t> orbs(std::max(Q.n_orb, 1), 0);       // r(b) | t(b) << 8
+    for (int c = 0; c < Q.n_orb; ++c)
+        orbs[c] = (uint16_t)(b.pn.rn[c] | (((Q.om2[c] + mtop) / 2) * 2 + (Q.oN[c] & 1)) << 8);
+    int ptop = 1;
+    for (int a = 0; a < P.n_orb; ++a) ptop = std::max(ptop, std::abs(P.om2[a]));
+    if (ptop > 15) return fail(CIH_ERR_UNSUPPORTED, "proton orbitals with 2m above 15");
+    std::vector<int2> pk(64, make_int2(0, 0));                 // group of (a, t): key (t + 2 m'_a) ^ N_a parity
+    std::vector<int16_t> ps((size_t)std::max(P.n_orb, 1) * T, 0);
+    std::vector<uint8_t> pa(std::max(P.n_orb, 1), 0);          // N_a parity | 2 m'_a << 1, m'_a = (2m_a + ptop) / 2
+    for (int a = 0; a < P.n_orb; ++a) {
+        pa[a] = (uint8_t)((P.oN[a] & 1) | (P.om2[a] + ptop) << 1);
+        for (int t = 0; t < T; ++t) {
+            const int m = 2 * (t >> 1) - mtop, k2 = P.om2[a] + m + b.pn.m2span;
+            if (k2 < 0 || k2 > 2 * b.pn.m2span) continue;
+            const int kappa = (k2 / 2) * 2 + ((P.oN[a] + t) & 1);
+            pk[(t + (pa[a] >> 1)) ^ (pa[a] & 1)] = make_int2(b.pn.goff[kappa], b.pn.gsize[kappa]);
+            ps[(size_t)a * T + t] = b.pn.S[(size_t)a * b.pn.G + kappa];
+        }
+    }
+    int2 *d_pk; int16_t *d_ps; uint16_t *d_orbs; uint8_t *d_pa;
+    if ((rc = upload(b, &d_pk, pk, st)) || (rc = upload(b, &d_ps, ps, st)) || (rc = upload(b, &d_orbs, orbs, st)) ||
+        (rc = upload(b, &d_pa, pa, st)))
         return rc;
-    b.dev.pn_S = d_S; b.dev.pn_gsize = d_gs; b.dev.pn_goff = d_go; b.dev.m2p = d_m2p; b.dev.Np = d_Np;
-    b.dev.pn_G = b.pn.G;
-    b.dev.pn_m2span = b.pn.m2span;
+    b.dev.pn_k = d_pk;
+    b.dev.pn_a = d_pa;
+    b.dev.pn_s = d_ps;
+    b.dev.orbs = d_orbs;
     int16_t *d_obg, *d_obl; int32_t *d_obs, *d_obo;
     if ((rc = upload(b, &d_obg, b.onebody.grp, st)) || (rc = upload(b, &d_obl, b.onebody.loc, st)) ||
         (rc = upload(b, &d_obs, b.onebody.gsize, st)) || (rc = upload(b, &d_obo, b.onebody.goff, st)))
@@ -1035,7 +903,6 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
     if ((rc = device_pool(b.device, &b.pool))) return rc;
     Timer tm("basis device set-up");
     if ((rc = dev_alloc(b, &b.dev_status, 4))) return rc;
-    b.dev.queue = b.dev_status + 1;
     if (cudaMemsetAsync(b.dev_status, 0, 4 * sizeof(int), st) != cudaSuccess) return cuda_fail(cudaGetLastError(), "status");
     PinnedTotals pin;
     pin.st = st;
@@ -1065,9 +932,7 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
     for (int t = 0; t < 2; ++t) {
         AllocOn on(b, ss[t]);
         if ((rc = species_upload(b, t, H[t], ss[t]))) return rc;
-        if (W == 1) rc = lists_phase1<1>(b, t, b.sbuild[t], L[t], ss[t]);
-        else if (W == 2) rc = lists_phase1<2>(b, t, b.sbuild[t], L[t], ss[t]);
-        else rc = lists_phase1<4>(b, t, b.sbuild[t], L[t], ss[t]);
+        with_words(W, [&](auto w) { rc = lists_phase1<decltype(w)::value>(b, t, b.sbuild[t], L[t], ss[t]); });
         if (rc) return rc;
     }
     tm.mark("species queued");
@@ -1079,144 +944,105 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
     if (e != cudaSuccess) return cuda_fail(e, "neighbour counts");
     tm.mark("staged passes done");
     // basis tables while both streams are idle (no upload waits for a kernel)
-    if ((rc = basis_tables_upload(b, st)) || (rc = upload(b, &L[1].rn, b.pn.rn, st))) return rc;
+    if ((rc = basis_tables_upload(b, st))) return rc;
     cudaEventRecord(side.ev[1], st);
-    // 2. exact-size lists, 3. two-move indices and neutron move information,
-    //    again one species per stream; phase 3 reads the basis tables
-    for (int t = 0; t < 2; ++t) {
-        AllocOn on(b, ss[t]);
-        if ((rc = lists_phase2(b, t, b.sbuild[t], L[t], ss[t]))) return rc;
-        if (t == 1) cudaStreamWaitEvent(side.s, side.ev[1], 0);
-        if (W == 1) rc = lists_phase3<1>(b, t, b.sbuild[t], L[t], ss[t]);
-        else if (W == 2) rc = lists_phase3<2>(b, t, b.sbuild[t], L[t], ss[t]);
-        else rc = lists_phase3<4>(b, t, b.sbuild[t], L[t], ss[t]);
-        if (rc) return rc;
-    }
-    b.scan_scratch_len = scan_scratch_needed(b.dim);
-    if ((rc = dev_alloc(b, &b.scan_scratch, b.scan_scratch_len))) return rc;
     {
-        // neutron one-move lists: packed entries and bucket directory, and the
-        // neutron occupied lists, on the second stream; the proton occupied
-        // lists, candidate table and count lists (which read none of these) on st
         const Species &Q = b.s[1];
         int dm = 0;
         for (int x = 0; x < Q.n_orb; ++x)
             for (int y = 0; y < Q.n_orb; ++y) dm = std::max(dm, std::abs(Q.om2[x] - Q.om2[y]));
-        const int NL = Q.Nsub_max + 1, RC = (dm + 1) * 2;
-        const int dir_len = 1 + RC * NL;
-        if (dir_len > 65535) return fail(CIH_ERR_UNSUPPORTED, "neutron bucket directory too long");
-        const int64_t nn = Q.n_sd;
-        const int64_t tot = L[1].tot[1];
+        b.dev.DM = dm;
+        b.dev.dir_len = 1 + (dm + 1) * 2 * b.dev.sp[1].NL;
+        if (b.dev.dir_len > 65535) return fail(CIH_ERR_UNSUPPORTED, "neutron bucket directory too long");
+    }
+    // 2. exact-size lists, 3. forward lists split, with two-move indices (these
+    //    read the basis tables), again one species per stream
+    for (int t = 0; t < 2; ++t) {
+        AllocOn on(b, ss[t]);
+        if ((rc = lists_phase2(b, t, b.sbuild[t], L[t], ss[t]))) return rc;
+        if (t == 1) cudaStreamWaitEvent(side.s, side.ev[1], 0);
+        if ((rc = lists_phase3(b, t, b.sbuild[t], L[t], ss[t]))) return rc;
+    }
+    b.scan_scratch_len = scan_scratch_needed(b.dim);
+    if ((rc = dev_alloc(b, &b.scan_scratch, b.scan_scratch_len))) return rc;
+    {
+        // neutrons: packed one-move lists, their bucket directory, records and
+        // occupied lists, on the second stream
+        const int64_t nn = b.s[1].n_sd, tot = L[1].tot[1];
         int2 *n1p;
-        int16_t *dir, *srel;
-        uint8_t *occp, *occn;
-        const int g0 = (int)std::min<int64_t>((b.s[0].n_sd + 255) / 256 + 1, 65535);
+        int16_t *dir;
+        uint8_t *occn;
+        NeutronRec *nrec;
         const int g1 = (int)std::min<int64_t>((nn + 255) / 256 + 1, 65535);
-        {
-            AllocOn on(b, side.s);
-            if ((rc = dev_alloc(b, &n1p, tot)) || (rc = dev_alloc(b, &dir, (size_t)nn * dir_len)) ||
-                (rc = dev_alloc(b, &srel, nn)) || (rc = dev_alloc(b, &occn, (size_t)nn * std::max(Q.Z, 1))))
-                return rc;
-            if (nn > 0) {
-                count_launches(2);
-                k_n1_pack<<<(int)std::min<int64_t>((tot + 255) / 256 + 1, 65535), 256, 0, side.s>>>(
-                    nn, b.dev.sp[1].n1_off, b.dev.sp[1].n1, b.dev.n1_info, n1p);
-                k_dir<<<grid_for(nn), 256, 0, side.s>>>(b.sbuild[1], b.dev.sp[1].n1_off, b.dev.sp[1].n1, NL, dm,
-                                                        dir_len, dir);
-            }
-            count_launches(1);
-            if (W == 1) k_occ<1><<<g1, 256, 0, side.s>>>(b.sbuild[1], Q.Z, b.dev.sp[1].n1_off, b.dev.sp[1].n1, occn, srel);
-            else if (W == 2) k_occ<2><<<g1, 256, 0, side.s>>>(b.sbuild[1], Q.Z, b.dev.sp[1].n1_off, b.dev.sp[1].n1, occn, srel);
-            else k_occ<4><<<g1, 256, 0, side.s>>>(b.sbuild[1], Q.Z, b.dev.sp[1].n1_off, b.dev.sp[1].n1, occn, srel);
+        AllocOn on(b, side.s);
+        if ((rc = dev_alloc(b, &n1p, tot)) || (rc = dev_alloc(b, &dir, (size_t)nn * b.dev.dir_len)) ||
+            (rc = dev_alloc(b, &nrec, nn)) || (rc = dev_alloc(b, &occn, (size_t)nn * std::max(b.s[1].Z, 1))))
+            return rc;
+        if (nn > 0) {
+            const DevSpecies &D = b.dev.sp[1];
+            const SpeciesBuild &SB = b.sbuild[1];
+            count_launches(4);
+            with_words(W, [&](auto w) {
+                k_n1_pack<decltype(w)::value><<<grid_for(nn), 256, 0, side.s>>>(SB, D.n1_off, D.n1, b.dev.orbs, n1p);
+                k_occ<decltype(w)::value><<<g1, 256, 0, side.s>>>(SB, b.s[1].Z, occn);
+            });
+            k_dir<<<grid_for(nn), 256, 0, side.s>>>(SB, D.n1_off, D.n1, D.N0, D.NL, b.dev.DM, b.dev.dir_len, dir);
+            k_neutron_rec<<<g1, 256, 0, side.s>>>(D, nrec);
         }
-        cudaEventRecord(side.ev[2], side.s);           // the neutron half is complete here
-        if ((rc = dev_alloc(b, &occp, (size_t)b.s[0].n_sd * std::max(b.s[0].Z, 1)))) return rc;
-        count_launches(1);
-        if (W == 1) k_occ<1><<<g0, 256, 0, st>>>(b.sbuild[0], b.s[0].Z, nullptr, nullptr, occp, nullptr);
-        else if (W == 2) k_occ<2><<<g0, 256, 0, st>>>(b.sbuild[0], b.s[0].Z, nullptr, nullptr, occp, nullptr);
-        else k_occ<4><<<g0, 256, 0, st>>>(b.sbuild[0], b.s[0].Z, nullptr, nullptr, occp, nullptr);
-        b.dev.self_rel = srel;
-        b.dev.occ[0] = occp;
         b.dev.occ[1] = occn;
         b.dev.n1p = n1p;
         b.dev.dir = dir;
-        b.dev.dir_len = dir_len;
-        b.dev.NL = NL;
-        b.dev.DM = dm;
+        b.dev.nrec = nrec;
+        cudaEventRecord(side.ev[2], side.s);           // the neutron half is complete here
     }
-    tm.mark("directory + occupied lists queued");
+    tm.mark("neutron lists queued");
     {
+        // protons (which read no neutron list): occupied lists, rows, groups, records
         const int64_t np = b.s[0].n_sd;
-        int64_t *coff;
+        const int g0 = (int)std::min<int64_t>((np + 255) / 256 + 1, 65535);
+        int64_t *goff;
         int32_t *row_p;
-        if ((rc = dev_alloc(b, &coff, np + 1)) || (rc = dev_alloc(b, &row_p, b.dim))) return rc;
-        int grid = grid_for(np);
+        uint8_t *occp;
+        int2 *l1;
+        ProtonRec *prec;
+        if ((rc = dev_alloc(b, &goff, np + 1)) || (rc = dev_alloc(b, &row_p, b.dim)) ||
+            (rc = dev_alloc(b, &occp, (size_t)np * std::max(b.s[0].Z, 1))) || (rc = dev_alloc(b, &l1, L[0].tot[1])) ||
+            (rc = dev_alloc(b, &prec, np)))
+            return rc;
+        const int grid = grid_for(np);
+        const SpeciesBuild &SB = b.sbuild[0];
         if (np > 0) {
-            count_launches(1);
-            k_cand_count<<<grid, 256, 0, st>>>(np, b.dev.sp[0].fw_off, b.dev.sp[0].n1_off, b.dev.sp[0].n1_later, coff);
-        }
-        if ((rc = exclusive_scan_i64(coff, np, b.scan_scratch, b.scan_scratch_len, st))) return rc;
-        int64_t *total_p = pin.p + 6;
-        e = cudaMemcpyAsync(total_p, coff + np, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return cuda_fail(e, "candidate count");
-        const int64_t total = *total_p;
-        int4 *cand;
-        uint8_t *cself;
-        if ((rc = dev_alloc(b, &cand, total)) || (rc = dev_alloc(b, &cself, total))) return rc;
-        if (np > 0) {
-            count_launches(2);
-            const SpeciesBuild &SB = b.sbuild[0];
-            if (W == 1) k_cand<1><<<grid, 256, 0, st>>>(SB, b.dev, SB.N, SB.M2, b.Nlim, coff, cand, cself);
-            else if (W == 2) k_cand<2><<<grid, 256, 0, st>>>(SB, b.dev, SB.N, SB.M2, b.Nlim, coff, cand, cself);
-            else k_cand<4><<<grid, 256, 0, st>>>(SB, b.dev, SB.N, SB.M2, b.Nlim, coff, cand, cself);
+            count_launches(3);
+            with_words(W, [&](auto w) {
+                k_groups<decltype(w)::value, 0><<<grid, 256, 0, st>>>(SB, b.dev, goff, nullptr, nullptr);
+                k_occ<decltype(w)::value><<<g0, 256, 0, st>>>(SB, b.s[0].Z, occp);
+            });
             k_row_p<<<grid, 256, 0, st>>>(np, b.dev.rowbase, row_p);
         }
-        tm.mark("candidate table queued");
-        b.dev.cand_off = coff;
-        b.dev.cand = cand;
-        b.dev.cand_self = cself;
-        b.dev.row_p = row_p;
-        // count lists (the count pass then reads a handful of directory entries per row)
-        b.dev.clist_off = nullptr;
-        b.dev.clist = nullptr;
-        b.dev.cself_sfx = nullptr;
-        if (np > 0 && b.dev.dir_len <= kClistDirCap && b.dev.NL <= 63) {
-            int64_t *clen, *cloff;
-            uint16_t *sfx;
-            if ((rc = dev_alloc(b, &clen, np + 1)) || (rc = dev_alloc(b, &sfx, (size_t)np * b.dev.NL))) return rc;
-            const int wpb = 8;
-            const size_t sh = (size_t)wpb * (b.dev.dir_len + 64) * sizeof(int);
-            if ((e = cudaFuncSetAttribute(k_clists<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh)) != cudaSuccess ||
-                (e = cudaFuncSetAttribute(k_clists<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh)) != cudaSuccess)
-                return cuda_fail(e, "count lists shared memory");
-            const int gcl = (int)std::min<int64_t>((np + wpb - 1) / wpb, 152 * 8);
-            count_launches(1);
-            k_clists<0><<<gcl, 32 * wpb, sh, st>>>(np, coff, cand, cself, b.dev.dir_len, b.dev.NL, clen, nullptr,
-                                                   nullptr, nullptr);
-            if ((rc = exclusive_scan_i64(clen, np, b.scan_scratch, b.scan_scratch_len, st))) return rc;
-            cloff = clen;
-            int64_t *ctot = pin.p + 7;
-            e = cudaMemcpyAsync(ctot, cloff + np, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e != cudaSuccess) return cuda_fail(e, "count list size");
-            int2 *cl;
-            if ((rc = dev_alloc(b, &cl, std::max<int64_t>(*ctot, 1)))) return rc;
-            count_launches(1);
-            k_clists<1><<<gcl, 32 * wpb, sh, st>>>(np, coff, cand, cself, b.dev.dir_len, b.dev.NL, nullptr, cloff,
-                                                   cl, sfx);
-            b.dev.clist_off = cloff;
-            b.dev.clist = cl;
-            b.dev.cself_sfx = sfx;
+        if ((rc = exclusive_scan_i64(goff, np, b.scan_scratch, b.scan_scratch_len, st))) return rc;
+        int64_t *total = pin.p + 6;
+        e = cudaMemcpyAsync(total, goff + np, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_fail(e, "group count");
+        int4 *grp;
+        if ((rc = dev_alloc(b, &grp, *total))) return rc;
+        if (np > 0) {
+            count_launches(2);
+            with_words(W, [&](auto w) {
+                k_groups<decltype(w)::value, 1><<<grid, 256, 0, st>>>(SB, b.dev, goff, grp, l1);
+            });
+            k_proton_rec<<<g0, 256, 0, st>>>(b.dev, goff, prec);
         }
-        b.dev.A = b.space.Z + b.space.N;
-        b.dev.nZ[0] = b.space.Z;
-        b.dev.nZ[1] = b.space.N;
+        tm.mark("groups queued");
+        b.dev.occ[0] = occp;
+        b.dev.row_p = row_p;
+        b.dev.grp = grp;
+        b.dev.l1 = l1;
+        b.dev.prec = prec;
     }
     cudaStreamWaitEvent(st, side.ev[2], 0);            // join: later work on st sees both species
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "basis upload");
-    b.dev.max_cand = (int32_t)L[0].tot[2];
     return CIH_OK;
 }
 
