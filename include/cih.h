@@ -145,6 +145,10 @@ int cih_ham_count(cih_basis_h h, int64_t *rowptr_dev, int64_t *nnz_out, void *st
  * FP32.  For the few dozen terms of one element this is the exact sum in all
  * but pathological cancellations, so the stored value agrees with the FP64
  * sum rounded to FP32 within 1e-5 (|value| + 1) (in practice bit for bit).
+ * With K = 1 and at least 4,096 rows the call takes stream-ordered
+ * scratch from the library's pool for a working copy of the table (87 MB at 4+4
+ * Nmax=6; inside a stream capture the allocation becomes part of the graph);
+ * without it the fill reads the table itself, with the same results.
  * Errors: CIH_ERR_ARG (K < 1, NULL arrays), CIH_ERR_CUDA. */
 int cih_ham_fill(cih_basis_h h, const int64_t *rowptr_dev, int32_t K, double hbar_omega,
                  const float *tbme_dev, const double *e_sp_dev,
@@ -247,11 +251,9 @@ int cih_tbme_interleave(int32_t K, int64_t tbme_len, const float *tbme_dev, floa
 int cih_set_launch(cih_basis_h h, int32_t warps_per_cta, int32_t ctas_per_sm);
 
 /* Which form of the count pass (Sec. 4.1's first pass) cih_ham_count runs for
- * this handle: walk = 0 (default) sums each row's segment lengths from the
- * per-proton count lists where the basis has them (bucket directories of at
- * most 4096 entries and at most 63 oscillator levels) and walks the
- * candidates otherwise; walk = 1 always walks the candidates, the same walk
- * the fill makes.  Both give the same row pointers.  Errors: CIH_ERR_ARG. */
+ * this handle: walk = 0 (default) sums the group terms of several rows per
+ * warp; walk = 1 runs the row kernel's own walk, one warp per row, as the fill
+ * does.  Both give the same row pointers.  Errors: CIH_ERR_ARG. */
 int cih_set_count_mode(cih_basis_h h, int32_t walk);
 
 /* Autotuner: times the fill (cih_ham_fill; cih_ham_fill_interleaved when

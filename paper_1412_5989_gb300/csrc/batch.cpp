@@ -31,10 +31,12 @@ struct WaveMem {
         ptrs.push_back(*p);
         return true;
     }
-    ~WaveMem()
+    void release()
     {
         for (void *p : ptrs) cudaFreeAsync(p, st);
+        ptrs.clear();
     }
+    ~WaveMem() { release(); }
 };
 
 // streams and events of the concurrent branches, created before any capture
@@ -204,7 +206,7 @@ int batch_solve(cih_instance_t *inst, int n, double hw, int nev, int max_iter, d
 
     // 4. per wave: one graph of fills, then Lanczos and the adjoint per instance
     for (const std::vector<int> &w : waves) {
-        WaveMem mem(st, pool);
+        WaveMem mem(st, pool), fills(st, pool);
         std::vector<int32_t *> col(n, nullptr);
         std::vector<float *> val(n, nullptr);
         std::vector<double *> psi(n, nullptr);
@@ -214,10 +216,23 @@ int batch_solve(cih_instance_t *inst, int n, double hw, int nev, int max_iter, d
                 !mem.get((void **)&psi[i], 8 * K * std::max<int64_t>(inst[i].basis->dim, 1)))
                 return fail(CIH_ERR_NOMEM, "batch: wave arrays");
         }
+        // working copies for the one-set fills where the wave leaves room for
+        // them (taken here: an allocation inside the capture would be the graph's)
+        std::vector<float *> work(n, nullptr);
+        int64_t room = avail;
+        for (int i : w) room -= plan[i].resident;
+        for (int i : w) {
+            const size_t f = inst[i].K == 1 ? fill_work_floats(*inst[i].basis) : 0;
+            if (f == 0 || (int64_t)(f * sizeof(float)) > room || !fills.get((void **)&work[i], f * sizeof(float))) continue;
+            room -= (int64_t)(f * sizeof(float));
+        }
         rc = fan_out(st, w, br, true, [&](int i, cudaStream_t s) {
-            return launch_fill(*inst[i].basis, rowptr[i], inst[i].K, hw, inst[i].tbme_dev, false, false, inst[i].e_sp_dev,
-                               col[i], val[i], s);
+            const cih_instance_t &x = inst[i];
+            const int r = work[i] ? fill_prepare(*x.basis, hw, x.tbme_dev, x.e_sp_dev, nullptr, work[i], s) : CIH_OK;
+            return r ? r : launch_fill(*x.basis, rowptr[i], x.K, hw, x.tbme_dev, false, false, x.e_sp_dev, col[i], val[i], s,
+                                       0, -1, false, nullptr, work[i], false);
         });
+        fills.release();
         if (rc) return rc;
         for (int i : w) {
             const cih_basis &b = *inst[i].basis;

@@ -107,12 +107,17 @@ struct DevBasis {
     const int16_t *dir;
     int32_t dir_len, DM;
     const uint8_t *occ[2];     // per sub-det: its occupied orbitals, ascending (Z_s each)
+    const int32_t *code[2];    // per orbital: its move onto itself, coded as in l1 (protons) or n1p (neutrons)
+    const int32_t *occ_code[2];    // the codes of each sub-det's occupied orbitals
     // pn pairs: u(a, b) = S(a, t(b)) + r(b) inside the group of (a, t(b)), with
     // t(b) the dense number of b's (2m, N parity) and r(b) b's rank among the
     // neutron orbitals with the same t.  pn_s[a * pn_T + t] = S; the group's
     // table offset and pairs are pn_k[(t + 2 m'_a) ^ (N_a & 1)], with m'_a the
     // dense number of 2m_a and pn_a[a] = N_a & 1 | 2 m'_a << 1.
     const int2 *pn_k;          // 64 groups
+    const int2 *pn_kq;         // the same groups stored as full squares one after another (FillWork::sq)
+    const int32_t *sqrow;      // n_sqrow rows of the squares: group << 16 | row
+    int32_t n_sqrow;
     const int16_t *pn_s;
     const uint8_t *pn_a;
     int32_t pn_T;
@@ -209,6 +214,9 @@ struct cih_basis {
     cih::Layout layout;
     cih::OneBodyLayout onebody;
     cih::PnSplit pn;
+    int64_t sq_total = 0;                     // entries of the pn groups as full squares
+    int64_t fw_total[2] = {0, 0};             // slots of the forward lists
+    int64_t n1_total[2] = {0, 0};             // entries of the one-move lists
     cih::SpeciesBuild sbuild[2]{};
     cih::DevBasis dev{};
     cih::DevBuffers buffers;
@@ -220,7 +228,7 @@ struct cih_basis {
     cudaStream_t stream = nullptr;            // stream of the build
     int launch_warps = 16;                    // row kernels: warps per CTA (8 or 16)
     int launch_ctas = 0;                      // row kernels: CTAs per SM (0 = as many as fit)
-    int count_walk = 0;                       // count pass: 1 = walk the candidates even with count lists
+    int count_walk = 0;                       // count pass: 1 = the row kernel's walk
 };
 
 namespace cih {
@@ -282,12 +290,22 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
 // kernels (ham.cu)
 int launch_count(const cih_basis &b, int64_t *rowptr, cudaStream_t st);
 int launch_scan(const cih_basis &b, int64_t *rowptr, cudaStream_t st);
+// With one set (set-major) a fill over many rows first prepares a working copy
+// of the table (fill_prepare) in fill_work_floats() floats of device memory:
+// `work` when the caller gives it (already prepared), else allocated for the call
+// on the stream (unless prepare is false); without it (no memory, few rows) the
+// fill reads the table itself, with the same results.  fill_work_floats is 0 where that form does
+// not apply.
+size_t fill_work_floats(const cih_basis &b);
+int fill_prepare(const cih_basis &b, double hw, const float *tbme, const double *esp, const double *t1, float *work,
+                 cudaStream_t st);
 // interleaved: tables element-major (len x K); em: values element-major (nnz x K)
 // sharded: col / val hold only rows r0 .. r1 - 1 (positions relative to rowptr[r0]);
 // t1: a one-body table (OneBodyLayout) in place of the orbital energies, or null
 int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, const float *tbme, bool interleaved, bool em,
                 const double *esp, int32_t *col, float *val, cudaStream_t st, int64_t r0 = 0, int64_t r1 = -1,
-                bool sharded = false, const double *t1 = nullptr);
+                bool sharded = false, const double *t1 = nullptr, const float *work = nullptr,
+                bool prepare = true);
 int launch_interleave(int K, int64_t len, const float *in, float *out, cudaStream_t st);
 // one-time set-up of the row kernels a call with K sets would launch (shared-
 // memory limits), so that launches made during a stream capture only launch

@@ -59,6 +59,20 @@ struct FillArgs {
     const double *t1;         // one-body table (OneBodyLayout) in place of the orbital energies, or null
 };
 
+// One set's table prepared for the fill (k_fill_prep), all in one allocation:
+//   sq      the pn groups as full squares: no ordering of the pair indices, and
+//           a proton move's entries for one neutron orbital are contiguous;
+//   hi, lo  per species and forward slot: a two-move's signed value (hi); a
+//           one-move's sum over its own species (one-body term, then the
+//           spectators ascending) as a pair hi + lo, unsigned;
+//   d       per species and sub-det: its own part of the diagonal.
+// These depend on one sub-det (pair) and are used by every row that holds it:
+// some 40 rows each at 4+4 Nmax=6.
+struct FillWork {
+    float *sq;
+    float *hi[2], *lo[2];
+    float2 *d[2];
+};
 // table index of t_ac for combined orbitals a, c (either order), -1 if they
 // are not one group of the one-body layout
 __device__ __forceinline__ int onebody_at(const DevBasis &B, int a, int c)
@@ -125,6 +139,12 @@ __device__ __forceinline__ long long psi_prod(const long long *psi, int64_t i, i
 // starts at c + j (len + 1) + t, len being the level's segment.
 
 constexpr int kLaneSets = 16;     // from this many sets on, multi-term sums run with lanes over sets
+// A one-set fill prepares a working copy when it covers at least kPrepareMin rows
+// and 1 / kPrepareShare of the basis.  Measured with / without: 800 rows 25 / 21
+// us, 2,104 rows 26 / 23, 7,916 rows 37 / 41, 8,500 rows 35 / 45, 48,917 rows 113
+// / 167; at 4+4 Nmax=6 (2.2 M rows) a 1/15 share 600 / 1,130, 1/32 355 / 515, 1/64
+// 228 / 257, at 4+4 Nmax=4 a 1/17 share 55 / 59, 1/32 44 / 32.
+constexpr int64_t kPrepareShare = 24, kPrepareMin = 4096;
 constexpr int kSlowCap = 64;
 constexpr int kMaxA = 64;
 constexpr int kPairCap = kMaxA * (kMaxA - 1) / 2;
@@ -310,6 +330,52 @@ __device__ __forceinline__ void put_values_coop(const FillArgs &F, const RowOut 
     }
 }
 
+// lanes for one element's sum over the other species' particles (at most 32:
+// with 33 particles of one species there are none of the other)
+__device__ __forceinline__ int term_lanes(int Zp, int Zn)
+{
+    int g = 1;
+    while (g < 32 && (g < Zp || g < Zn)) g <<= 1;
+    return g;
+}
+
+// pair l of Z items -> (i, j), i < j
+__device__ __forceinline__ void pair_of(int l, int Z, int &i, int &j)
+{
+    i = 0;
+    while (l >= Z - 1 - i) { l -= Z - 1 - i; ++i; }
+    j = i + 1 + l;
+}
+
+// One species' part of the diagonal for set k, by the whole warp: the one-body
+// energies and the pairs of its Z occupied orbitals occ(i) (combined), lanes
+// over both, summed as a tree.
+template <class Occ>
+__device__ __forceinline__ DF diag_own(const DevBasis &B, const int2 *lg, const FillArgs &F, int k, int Z, Occ occ, int *status)
+{
+    const int lane = threadIdx.x & 31;
+    DF acc = df_of(0.f);
+    for (int l = lane; l < Z * (Z - 1) / 2; l += 32) {
+        int i, j, sg;
+        int64_t idx;
+        pair_of(l, Z, i, j);
+        const int a = occ(i), c = occ(j);
+        if (!tbme_at(B, lg, a, c, a, c, idx, sg)) {
+            if (atomicOr(status, 1) == 0) { status[2] = a | (c << 16); status[3] = 1; }
+            continue;
+        }
+        const float v = __ldg(F.tbme + (int64_t)k * F.tb_sk + idx * F.tb_si);
+        acc = df_add(acc, df_of(sg < 0 ? -v : v));
+    }
+    for (int i = lane; i < Z; i += 32) {
+        const int a = occ(i), k1 = F.t1 ? onebody_at(B, a, a) : -1;
+        const double e = F.t1 ? (k1 >= 0 ? F.t1[k1] : 0.0) : F.esp ? F.esp[a] : F.hw * ((double)B.orbN[a] + 1.5);
+        const float hi = (float)e;
+        acc = df_add(acc, DF{hi, (float)(e - (double)hi)});
+    }
+    return warp_sum(acc, 32);
+}
+
 // Deferred one-move elements of a row: lanes over (element, spectator)
 // pairs, groups of the next power of two >= A-1 lanes, segmented sum (from
 // kLaneSets sets on: one element at a time, lanes over sets).
@@ -416,6 +482,49 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
             }
             __syncwarp();
         }
+        nslow = 0;
+        return;
+    }
+    if constexpr (MODE == 1 && K1) {
+        // one set: an element's terms over the other species' particles (a lane
+        // each, summed as a tree) and over its own species' spectators (loaded a
+        // lane each, summed ascending after the one-body term): the sums of k_fill1
+        const int Zp = B.nZ[0], Zn = B.nZ[1], gsz = term_lanes(Zp, Zn), per = 32 / gsz;
+        for (int e0 = 0; e0 < ns; e0 += per) {
+            const int e = e0 + lane / gsz, i = lane % gsz;
+            const bool act = e < ns;
+            const uint32_t code = act ? w_scode[e] : 0;
+            const bool neu = (code >> 31) != 0;
+            const int base = neu ? nbase : 0;
+            const int a = base + (int)(code & 0xFF), c = base + (int)((code >> 8) & 0xFF);
+            const int own0 = neu ? Zp : 0, nown = (neu ? Zn : Zp) - 1, oth0 = neu ? 0 : Zp, noth = neu ? Zp : Zn;
+            int ia = 0;                                             // a's place among its species
+            for (int x = 0; x <= nown; ++x) ia += (w_occ[own0 + x] < a);
+            const bool ho = act && i < noth, hs = act && i < nown;
+            const int ko = ho ? w_occ[oth0 + i] : 0, ks = hs ? w_occ[own0 + i + (i >= ia ? 1 : 0)] : 0;
+            int64_t xo = 0, xs = 0;
+            int go = 1, gs = 1;
+            const bool oko = !ho || tbme_at(B, lg, a, ko, c, ko, xo, go), oks = !hs || tbme_at(B, lg, a, ks, c, ks, xs, gs);
+            if ((!oko || !oks) && atomicOr(status, 1) == 0) {
+                status[2] = a | (c << 16);
+                status[3] = 2 | ((oko ? ks : ko) << 8);
+            }
+            float to = 0.f, ts = 0.f;
+            if (ho && oko) { to = __ldg(F.tbme + xo); if (go < 0) to = -to; }
+            if (hs && oks) { ts = __ldg(F.tbme + xs); if (gs < 0) ts = -ts; }
+            const DF v = warp_sum(df_of(to), gsz);
+            DF own = act ? onebody_term(B, F, a, c, status) : df_of(0.f);
+            for (int x = 0; x < gsz; ++x) {
+                const float y = __shfl_sync(0xffffffffu, ts, x, gsz);
+                if (x < nown) own = df_add(own, df_of(y));
+            }
+            if (act && i == 0) {
+                const float r = df_round(df_add(v, own));
+                R.col[w_spos[e]] = w_scol[e];
+                R.val[w_spos[e]] = (code >> 16) & 1 ? -r : r;
+            }
+        }
+        __syncwarp();
         nslow = 0;
         return;
     }
@@ -615,7 +724,31 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
                 if (lane == 0 && rowlen > 0) R.col[0] = (int32_t)row;
                 __syncwarp();
             }
-            for (int k = 0; k < (kset ? 0 : K1 ? 1 : MODE == 1 ? F.K : Gr.K); ++k) {
+            if constexpr (MODE == 1 && K1) {                 // the sums and their order of k_fill1
+                const int P = term_lanes(Zpro, Zneu), sub = lane / P, j = lane % P;
+                DF acc = df_of(0.f);
+                for (int i = sub; i < Zpro; i += 32 / P) {
+                    if (j >= Zneu) continue;
+                    const int a = w_occ[i], c = w_occ[Zpro + j];
+                    int64_t idx;
+                    int sg;
+                    if (tbme_at(B, lg, a, c, a, c, idx, sg)) {
+                        const float v = __ldg(F.tbme + idx * F.tb_si);
+                        acc = df_add(acc, df_of(sg < 0 ? -v : v));
+                    } else if (atomicOr(status, 1) == 0) {
+                        status[2] = a | (c << 16);
+                        status[3] = 1;
+                    }
+                }
+                acc = warp_sum(acc, 32);
+                const DF dp = diag_own(B, lg, F, 0, Zpro, [&](int i) { return (int)w_occ[i]; }, status);
+                const DF dn = diag_own(B, lg, F, 0, Zneu, [&](int i) { return (int)w_occ[Zpro + i]; }, status);
+                if (lane == 0 && rowlen > 0) {
+                    R.col[0] = (int32_t)row;
+                    R.val[0] = df_round(df_add(acc, df_add(dp, dn)));
+                }
+            }
+            for (int k = 0; k < (kset || (MODE == 1 && K1) ? 0 : K1 ? 1 : MODE == 1 ? F.K : Gr.K); ++k) {
                 DF acc = df_of(0.f);
                 for (int l = lane; l < npairs; l += 32) {
                     const int a = w_occ[pi[l]], c = w_occ[pj[l]];
@@ -801,6 +934,295 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
     }
 }
 
+// The working copy of one set's table (FillWork): warps over the rows of the pn
+// squares, then over the sub-dets of both species.  Bound by its scattered
+// reads of the table (L2); it replaces two to seven of them, and the pair
+// lookups, per element of that kind in every row.
+__global__ void __launch_bounds__(256) k_fill_prep(DevBasis B, FillArgs F, FillWork W, int *status)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t n0 = B.n_sqrow, n1 = n0 + B.sp[0].n_sd, n2 = n1 + B.sp[1].n_sd;
+    for (int64_t t = warp; t < n2; t += nw) {
+        if (t < n0) {
+            const int r = B.sqrow[t], k = r >> 16, u = r & 0xFFFF;
+            const int2 g = B.pn_k[k];
+            const int n = g.y;
+            float *out = W.sq + B.pn_kq[k].x + (int64_t)u * n;
+            for (int v = lane; v < n; v += 32) {
+                const int lo = min(u, v), hi = max(u, v);
+                out[v] = __ldg(F.tbme + g.x + lo * n - ((lo * (lo - 1)) >> 1) + (hi - lo));
+            }
+            continue;
+        }
+        const int s = t < n1 ? 0 : 1;
+        const DevSpecies S = s ? B.sp[1] : B.sp[0];
+        float *hi = s ? W.hi[1] : W.hi[0], *lo = s ? W.lo[1] : W.lo[0];
+        float2 *dg = s ? W.d[1] : W.d[0];
+        const int64_t x = t - (s ? n1 : n0), f0 = S.fw_off[x];
+        const int Z = s ? B.nZ[1] : B.nZ[0], len = (int)(S.fw_off[x + 1] - f0), two = S.fw_lev[x * S.NL + S.NL - 1];
+        const uint8_t *occ = (s ? B.occ[1] : B.occ[0]) + x * Z;
+        const DF d = diag_own(B, nullptr, F, 0, Z, [&](int i) { return S.orb_base + (int)occ[i]; }, status);
+        if (lane == 0) dg[x] = make_float2(d.hi, d.lo);
+        for (int i = lane; i < two; i += 32) {
+            const int tb = S.fw_tb[f0 + i];
+            const float v = __ldg(F.tbme + (tb >> 1));
+            hi[f0 + i] = tb & 1 ? -v : v;
+        }
+        for (int i = two + lane; i < len; i += 32) {
+            const int code = ~S.fw_tb[f0 + i];
+            const int a = S.orb_base + (code & 0xFF), c = S.orb_base + ((code >> 8) & 0xFF);
+            DF own = onebody_term(B, F, a, c, status);
+            for (int j = 0; j < Z; ++j) {
+                const int k = S.orb_base + (int)occ[j];
+                if (k == a) continue;
+                int64_t idx;
+                int sg;
+                float v = 0.f;
+                if (tbme_at(B, nullptr, a, k, c, k, idx, sg)) {
+                    v = __ldg(F.tbme + idx);
+                    if (sg < 0) v = -v;
+                } else if (atomicOr(status, 1) == 0) {
+                    status[2] = a | (c << 16);
+                    status[3] = 2 | (k << 8);
+                }
+                own = df_add(own, df_of(v));
+            }
+            hi[f0 + i] = own.hi;
+            lo[f0 + i] = own.lo;
+        }
+    }
+}
+
+// shared memory of k_fill1: pn groups, then per warp, then the pn index table
+namespace f1 {
+constexpr int kg = 0;                                      // int2[64]: pn_kq
+constexpr int warp0 = 64 * 8;
+constexpr int w_seg = 0;                                   // int4[32], int2[32], int4[kLevels] as k_rows
+constexpr int w_ext = w_seg + 32 * 16;
+constexpr int w_lev = w_ext + 32 * 8;
+constexpr int w_op = w_lev + kLevels * 16;                 // int32[32]: codes of the occupied protons
+constexpr int w_on = w_op + 32 * 4;                        // int32[32]: and neutrons
+constexpr int w_size = w_on + 32 * 4;
+template <int WARPS>
+constexpr int S = warp0 + WARPS * w_size;
+}  // namespace f1
+
+// entry at a 32-bit byte offset from a kernel argument (arrays below 4 GiB:
+// one address register instead of two, no 64-bit address arithmetic)
+template <class T>
+__device__ __forceinline__ T at_byte(const void *base, unsigned off)
+{
+    return __ldg(reinterpret_cast<const T *>(reinterpret_cast<const char *>(base) + off));
+}
+
+constexpr int kW = 2;             // pn windows of 32 elements in flight in k_fill1
+
+// The fill of one set from its working copy: the walk of k_rows, every element
+// one read of a value (two-moves: contiguous; pn: one gather from the squares),
+// one-moves and the diagonal the prepared own-species sum plus the terms over
+// the other species.  Reading the table itself in every row (pair lookups, a
+// gather per spectator) took 364 us at 4+4 Nmax=4 and 8.5 ms at 4+4 Nmax=6;
+// this form 298 us and 7.1 ms with its preparation.  At 3+3 Nmax=6 it issues
+// 5.6 warp instructions per stored nonzero (64 % of the issue slots; 10.9 before
+// the groups); the pn loop is 60 % of the time, waiting on L2 for the members,
+// moves and values of its windows.
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
+k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, int64_t r1, int *status)
+{
+    constexpr int kThreads = WARPS * 32;
+    extern __shared__ __align__(16) unsigned char sb[];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const unsigned lt = (1u << lane) - 1;
+    const DevSpecies &SP = B.sp[0], &SN = B.sp[1];
+    const int T = B.pn_T, Zp = B.nZ[0], Zn = B.nZ[1];
+    int2 *KQ = sptr<int2>(sb, f1::kg);
+    int16_t *S = sptr<int16_t>(sb, f1::S<WARPS>);
+    for (int i = tid; i < SP.n_orb * T; i += kThreads) S[i] = B.pn_s[i];
+    for (int i = tid; i < 64; i += kThreads) KQ[i] = B.pn_kq[i];
+    __syncthreads();
+    const int64_t sbase = F.sharded ? rowptr[F.shard_row] : 0;
+    const int64_t nnz = F.sharded ? rowptr[r1] - sbase : rowptr[B.dim];
+    unsigned char *wb = sb + f1::warp0 + wid * f1::w_size;
+    int4 *w_seg = sptr<int4>(wb, f1::w_seg), *w_lev = sptr<int4>(wb, f1::w_lev);
+    int2 *w_ext = sptr<int2>(wb, f1::w_ext);
+    int *w_op = sptr<int>(wb, f1::w_op), *w_on = sptr<int>(wb, f1::w_on);
+    const int P = term_lanes(Zp, Zn), sub = lane / P, li = lane % P, per = 32 / P;
+    const int64_t gw = (blockIdx.x * (int64_t)kThreads + tid) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * kThreads) >> 5;
+
+    for (int64_t row = r0 + gw; row < r1; row += nw) {
+        const int p = B.row_p[row];
+        const ProtonRec PR = B.prec[p];
+        const int n = (int)(row - PR.colb);
+        const NeutronRec NR = B.nrec[n];
+        const int64_t e0 = rowptr[row] - sbase;
+        const int rowlen = (int)(min(rowptr[row + 1] - sbase, nnz) - e0);
+        int32_t *col = F.col + e0;
+        float *val = F.val + e0;
+        const int16_t *dirn = B.dir + (int64_t)n * B.dir_len;
+        const int cA1 = max(0, dirn[PR.dirA] - NR.self), cA2 = SN.fw_lev[(int64_t)n * SN.NL + PR.levA];
+        int pos = 1 + cA1 + cA2;
+        if (pos > rowlen) {
+            if (lane == 0) atomicOr(status, 2);
+            continue;
+        }
+        if (lane < Zp) w_op[lane] = B.occ_code[0][(int64_t)p * Zp + lane];
+        if (lane < Zn) w_on[lane] = B.occ_code[1][(int64_t)n * Zn + lane];
+        const int2 *recn = SN.fw_rec + NR.fw, *recp = SP.fw_rec + PR.fw;
+        const float *vn = W.hi[1] + NR.fw, *vp = W.hi[0] + PR.fw;
+        const int2 *n1row = B.n1p + NR.n1, *l1row = B.l1 + PR.l1;
+        const unsigned l1o = (unsigned)PR.l1 * 8u, n1o = (unsigned)NR.n1 * 8u, fpo = (unsigned)(PR.fw + PR.fwlen) * 8u;
+        __syncwarp();
+
+        // diagonal
+        {
+            DF acc = df_of(0.f);
+            for (int i = sub; i < Zp; i += per)
+                if (li < Zn) acc = df_add(acc, df_of(__ldg(W.sq + pn_square_at(KQ, S, T, w_op[i], w_on[li]))));
+            acc = warp_sum(acc, 32);
+            if (lane == 0) {
+                const float2 dp = W.d[0][p], dn = W.d[1][n];
+                __stcs(col, (int32_t)row);
+                __stcs(val, df_round(df_add(acc, df_add(DF{dp.x, dp.y}, DF{dn.x, dn.y}))));
+            }
+        }
+        // A: neutron two-moves
+        for (int t = lane; t < cA2; t += 32) {
+            const int2 rc = recn[t];
+            const float v = vn[t];
+            const int e = 1 + t + (rc.y & 0xFFFFFF);
+            __stcs(col + e, PR.colb + rc.x);
+            __stcs(val + e, v);
+        }
+        // B: p's groups, a lane each
+        int c1 = 0;                                             // proton one-moves with n kept
+        for (int g0 = 0; g0 < PR.ng; g0 += 32) {
+            int4 gr = make_int4(0, 0, 0, 0);
+            if (g0 + lane < PR.ng) gr = B.grp[PR.g0 + g0 + lane];
+            const int n1c = (unsigned)gr.x >> 16, s0 = dirn[gr.y & 0xFFFF], len = dirn[(unsigned)gr.y >> 16] - s0;
+            const int self = (gr.w & 0xFF) > NR.N ? 1 : 0;                  // own class and N_n <= L_q
+            const int npn = n1c * len, tot = npn + self * (n1c + gr.z);
+            int itot = tot, ipn = npn;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int o1 = __shfl_up_sync(0xffffffffu, itot, d), o2 = __shfl_up_sync(0xffffffffu, ipn, d);
+                if (lane >= d) { itot += o1; ipn += o2; }
+            }
+            const int Tall = __shfl_sync(0xffffffffu, itot, 31), Tpn = __shfl_sync(0xffffffffu, ipn, 31);
+            if (pos + Tall > rowlen) {
+                if (lane == 0) atomicOr(status, 2);
+                break;
+            }
+            const int at0 = pos + itot - tot, st = ipn - npn, m1 = gr.x & 0xFFFF;
+            const int ins = NR.self - s0;                                   // where n sorts in the segment
+            const int c = at0 - m1 * (len + 1) - (gr.w >> 8);
+            const unsigned ne = __ballot_sync(0xffffffffu, npn > 0);
+            if (npn > 0) {
+                const int j = __popc(ne & lt);
+                w_seg[j] = make_int4(st, (int)(0xFFFFFFFFu / (unsigned)len), m1, self ? c : at0 - st);
+                w_ext[j] = make_int2(s0 | len << 16, self ? ins : -1);
+            }
+            int c2 = 0;
+            if (g0 == 0) {                                      // own-class groups come first, at most kLevels
+                if (gr.w) w_lev[((B.Nlim - (gr.w & 0xFF) + 1) - SP.N0) >> 1] = make_int4(c, len + 1, ins, 0);
+                c1 = __reduce_add_sync(0xffffffffu, self * n1c);
+                c2 = __reduce_add_sync(0xffffffffu, self * gr.z);
+            }
+            __syncwarp();
+            for (int t = lane; t < c2; t += 32) {               // pp two-moves: a prefix of p's list
+                const int2 rc = recp[t];
+                const float v = vp[t];
+                const int4 lv = w_lev[rc.y >> 24];
+                const int e = lv.x + t + (rc.y & 0xFFFFFF) * lv.y;
+                __stcs(col + e, rc.x + n);
+                __stcs(val + e, v);
+            }
+            // pn elements of all groups, flattened as in k_rows, kW windows of 32
+            // at a time so that their chains of loads (member and neutron move, then
+            // the value) overlap; lanes past the end repeat the last element's loads
+            const unsigned le = (2u << lane) - 1u;                 // bits 0..lane
+            int before = -1;                                       // pn groups started before the window, less one
+            for (int w0 = 0; w0 < Tpn; w0 += 32 * kW) {
+                int2 q[kW], ent[kW];
+                int at[kW];
+#pragma unroll
+                for (int u = 0; u < kW; ++u) {
+                    const int w = w0 + 32 * u;
+                    const unsigned mk = __reduce_or_sync(0xffffffffu, npn > 0 && (unsigned)(st - w) < 32u ? 1u << (st - w) : 0u);
+                    const int j = before + __popc(mk & le), e = min(w + lane, Tpn - 1);
+                    before += __popc(mk);
+                    const int4 sg4 = w_seg[j];
+                    const int2 sx = w_ext[j];
+                    const int rel = e - sg4.x, ln = (unsigned)sx.x >> 16;
+                    int qi = (int)__umulhi((unsigned)rel, (unsigned)sg4.y), k = rel - qi * ln;   // at most one short
+                    if (k >= ln) { ++qi; k -= ln; }
+                    const unsigned i1 = sg4.z + qi;
+                    q[u] = at_byte<int2>(B.l1, l1o + i1 * 8);
+                    ent[u] = at_byte<int2>(B.n1p, n1o + ((sx.x & 0xFFFF) + k) * 8);
+                    at[u] = sg4.w + e;
+                    if (sx.y >= 0)                                 // n itself is among the partners
+                        at[u] = sg4.w + i1 * (ln + 1) + (at_byte<int2>(SP.fw_rec, fpo - 8 - i1 * 8).y & 0xFFFFFF) + k +
+                                (k >= sx.y ? 1 : 0);
+                }
+                float v[kW];
+#pragma unroll
+                for (int u = 0; u < kW; ++u) v[u] = at_byte<float>(W.sq, (unsigned)pn_square_at(KQ, S, T, q[u].y, ent[u].y) * 4u);
+#pragma unroll
+                for (int u = 0; u < kW; ++u) {
+                    if (w0 + 32 * u + lane >= Tpn) continue;
+                    __stcs(col + at[u], q[u].x + ent[u].x);
+                    __stcs(val + at[u], __int_as_float(__float_as_int(v[u]) ^ (((q[u].y << 15) ^ (ent[u].y << 5)) & 0x80000000)));
+                }
+            }
+            __syncwarp();
+            pos += Tall;
+        }
+        // one-moves of either species: P lanes an element, one per particle of
+        // the other species
+        for (int t0 = 0; t0 < cA1 + c1; t0 += per) {
+            const int t = t0 + sub;
+            const bool act = t < cA1 + c1, neu = t < cA1;
+            int lc = 0, nc = 0, e = 0, j = 0, sgn = 0;
+            int64_t slot = 0;
+            if (act && neu) {
+                const int2 ent = n1row[NR.self + t];
+                slot = NR.fwlen - 1 - t;
+                e = 1 + t + (recn[slot].y & 0xFFFFFF);
+                j = PR.colb + ent.x;
+                sgn = (ent.y >> 26) & 1;
+                nc = ent.y;
+                if (li < Zp) lc = w_op[li];
+            } else if (act) {
+                const int i1 = t - cA1;
+                const int2 q = l1row[i1];
+                slot = PR.fwlen - 1 - i1;
+                const int o = recp[slot].y;
+                const int4 lv = w_lev[o >> 24];
+                e = lv.x + i1 * lv.y + (o & 0xFFFFFF) + lv.z;
+                j = q.x + n;
+                sgn = (q.y >> 16) & 1;
+                lc = q.y;
+                if (li < Zn) nc = w_on[li];
+            }
+            const bool has = act && li < (neu ? Zp : Zn);
+            float v = 0.f;
+            if (has) v = __ldg(W.sq + pn_square_at(KQ, S, T, lc, nc));
+            const DF sum = warp_sum(df_of(v), P);
+            if (act && li == 0) {
+                slot += neu ? NR.fw : PR.fw;
+                const DF own{(neu ? W.hi[1] : W.hi[0])[slot], (neu ? W.lo[1] : W.lo[0])[slot]};
+                const float r = df_round(df_add(sum, own));
+                __stcs(col + e, j);
+                __stcs(val + e, sgn ? -r : r);
+            }
+        }
+        __syncwarp();
+    }
+}
+
 // Count pass: for row (p, n), 1 for the diagonal + n's forward same-class
 // neighbours inside p's range + the sum over p's groups of members x segment
 // length (+ members and two-moves where n itself is a partner).  Equal to the
@@ -888,7 +1310,10 @@ int launch_rows_w(const cih_basis &b, const int64_t *rowptr, int64_t *counts, co
         // element-major K sets: warp-cooperative writes; 64 is the batched configuration's set count
         if (em) return F.K == 64 ? go(k_rows<MODE, false, WARPS, 64>) : go(k_rows<MODE, false, WARPS, 1>);
     }
-    return k1 ? go(k_rows<MODE, true, WARPS, 0>) : go(k_rows<MODE, false, WARPS, 0>);
+    if constexpr (MODE != 0) {
+        if (k1) return go(k_rows<MODE, true, WARPS, 0>);
+    }
+    return go(k_rows<MODE, false, WARPS, 0>);
 }
 
 template <int MODE>
@@ -945,14 +1370,109 @@ int launch_scan(const cih_basis &b, int64_t *rowptr, cudaStream_t st)
     return exclusive_scan_i64(rowptr, b.dim, b.scan_scratch, b.scan_scratch_len, st);
 }
 
+namespace {
+
+// layout of the working copy: the pair arrays first (8-byte aligned)
+FillWork work_at(const cih_basis &b, float *p)
+{
+    FillWork w;
+    for (int s = 0; s < 2; ++s) {
+        w.d[s] = reinterpret_cast<float2 *>(p);
+        p += 2 * b.s[s].n_sd;
+    }
+    for (int s = 0; s < 2; ++s) {
+        w.hi[s] = p;
+        w.lo[s] = p + b.fw_total[s];
+        p += 2 * b.fw_total[s];
+    }
+    w.sq = p;
+    return w;
+}
+
+template <int WARPS>
+int launch_fill1(const cih_basis &b, const int64_t *rowptr, const FillArgs &F, const FillWork &W, cudaStream_t st, bool dry,
+                 int64_t r0, int64_t r1)
+{
+    const size_t smem = (size_t)f1::S<WARPS> + ((size_t)b.dev.sp[0].n_orb * b.dev.pn_T * 2 + 15) / 16 * 16;
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaError_t e = raise_smem_limit((const void *)k_fill1<WARPS>, dev, (int)smem);
+    if (e != cudaSuccess) return cuda_fail(e, "fill shared memory");
+    if (dry) return CIH_OK;
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fill1<WARPS>, WARPS * 32, smem);
+    per_sm = std::max(per_sm, 1);
+    if (b.launch_ctas > 0) per_sm = std::min(per_sm, b.launch_ctas);
+    const int64_t want = (r1 - r0 + WARPS - 1) / WARPS;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm, want));
+    count_launches(1);
+    k_fill1<WARPS><<<grid, WARPS * 32, smem, st>>>(b.dev, rowptr, F, W, r0, r1, b.dev_status);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? CIH_OK : cuda_fail(e, "fill launch");
+}
+
+}  // namespace
+
+size_t fill_work_floats(const cih_basis &b)
+{
+    // k_fill1 takes 32-bit byte offsets and keeps at most 32 particles of a species
+    const int64_t most = (int64_t)1 << 32;
+    for (int s = 0; s < 2; ++s)
+        if (b.fw_total[s] * 8 >= most || b.n1_total[s] * 8 >= most) return 0;
+    if (b.sq_total * 4 >= most || b.dev.A - 1 > 32 || b.dev.nZ[0] > 32 || b.dev.nZ[1] > 32 || b.dim == 0) return 0;
+    return (size_t)(2 * (b.s[0].n_sd + b.s[1].n_sd) + 2 * (b.fw_total[0] + b.fw_total[1]) + b.sq_total);
+}
+
+int fill_prepare(const cih_basis &b, double hw, const float *tbme, const double *esp, const double *t1, float *work,
+                 cudaStream_t st)
+{
+    FillArgs F{};
+    F.K = 1;
+    F.hw = hw;
+    F.tbme = tbme;
+    F.tb_sk = b.layout.total;
+    F.tb_si = 1;
+    F.esp = esp;
+    F.t1 = t1;
+    const int64_t warps = b.dev.n_sqrow + b.s[0].n_sd + b.s[1].n_sd;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8, 152 * 16));
+    count_launches(1);
+    k_fill_prep<<<grid, 256, 0, st>>>(b.dev, F, work_at(b, work), b.dev_status);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? CIH_OK : cuda_fail(e, "fill preparation");
+}
+
 int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, const float *tbme, bool interleaved,
                 bool em, const double *esp, int32_t *col, float *val, cudaStream_t st, int64_t r0, int64_t r1,
-                bool sharded, const double *t1)
+                bool sharded, const double *t1, const float *work, bool prepare)
 {
     const int vec4 = interleaved && K % 4 == 0 && ((uintptr_t)tbme & 15) == 0 && (!em || ((uintptr_t)val & 15) == 0);
     FillArgs F{K, hw, tbme, interleaved ? 1 : b.layout.total, interleaved ? (int64_t)K : 1, vec4, em && K > 1 ? 1 : 0,
                esp, col, val, sharded ? 1 : 0, r0, t1};
-    return launch_rows<1>(b, rowptr, nullptr, F, GradArgs{}, st, false, r0, r1);
+    const int64_t rend = r1 < 0 ? b.dim : r1;
+    float *own = nullptr;
+    if (K == 1 && !work && prepare && rend - r0 >= kPrepareMin && (rend - r0) * kPrepareShare >= b.dim) {
+        const size_t n = fill_work_floats(b);
+        if (n > 0 && cudaMallocFromPoolAsync((void **)&own, n * sizeof(float), b.pool, st) != cudaSuccess) {
+            (void)cudaGetLastError();
+            own = nullptr;
+        }
+        if (own) {
+            const int rc = fill_prepare(b, hw, tbme, esp, t1, own, st);
+            if (rc) { cudaFreeAsync(own, st); return rc; }
+            work = own;
+        }
+    }
+    if (K != 1 || !work) return launch_rows<1>(b, rowptr, nullptr, F, GradArgs{}, st, false, r0, r1);
+    int rc = CIH_OK;
+    if (b.dim > 0 && rend > r0) {
+        const FillWork W = work_at(b, const_cast<float *>(work));
+        rc = b.launch_warps == 8 ? launch_fill1<8>(b, rowptr, F, W, st, false, r0, rend)
+                                 : launch_fill1<16>(b, rowptr, F, W, st, false, r0, rend);
+    }
+    if (own) cudaFreeAsync(own, st);
+    return rc;
 }
 
 int prepare_rows(const cih_basis &b, int K)
@@ -964,6 +1484,9 @@ int prepare_rows(const cih_basis &b, int K)
     int rc = launch_rows<0>(b, nullptr, nullptr, F, G, nullptr, true);
     if (!rc) rc = launch_rows<1>(b, nullptr, nullptr, F, G, nullptr, true);
     if (!rc) rc = launch_rows<2>(b, nullptr, nullptr, F, G, nullptr, true);
+    if (!rc && K == 1 && fill_work_floats(b) > 0)
+        rc = b.launch_warps == 8 ? launch_fill1<8>(b, nullptr, F, FillWork{}, nullptr, true, 0, 0)
+                                 : launch_fill1<16>(b, nullptr, F, FillWork{}, nullptr, true, 0, 0);
     return rc;
 }
 

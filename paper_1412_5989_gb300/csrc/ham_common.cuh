@@ -15,7 +15,7 @@ constexpr int kOrbCap = 512;      // combined orbitals (two species of at most 2
 // Table index of V(ab, cd) for combined orbitals in any order; false if the
 // pairs are not one table entry (a bug in the walk: flagged by the caller).
 // The group sizes and offsets come from shared memory (lg: size and offset
-// per group, int2) when the layout has at most kLayoutCap groups.
+// per group, int2) when given and the layout has at most kLayoutCap groups.
 __device__ __forceinline__ bool tbme_at(const DevBasis &B, const int2 *lg, int a, int b, int c, int d, int64_t &idx,
                                         int &sign)
 {
@@ -30,7 +30,7 @@ __device__ __forceinline__ bool tbme_at(const DevBasis &B, const int2 *lg, int a
     int u = e1 & 0xFFFF, v = e2 & 0xFFFF;
     if (u > v) { const int t = u; u = v; v = t; }
     int64_t n, off;
-    if (B.ngroups <= kLayoutCap) {
+    if (lg && B.ngroups <= kLayoutCap) {
         const int2 q = lg[g];
         n = q.x;
         off = q.y;
@@ -76,6 +76,15 @@ __device__ __forceinline__ int pn_index_at(const int2 *KG, const int16_t *S, int
     if (u > v) { const int s = u; u = v; v = s; }
     sign = ((l1 >> 16) ^ (n1 >> 26)) & 1;
     return g.x + u * g.y - ((u * (u - 1)) >> 1) + (v - u);
+}
+
+// the same element in the pn groups stored as full squares (KQ: pn_kq)
+__device__ __forceinline__ int pn_square_at(const int2 *KQ, const int16_t *S, int T, int l1, int n1)
+{
+    const int t = (n1 >> 16) & 0x1F;
+    const int2 g = KQ[(t + ((unsigned)l1 >> 18)) ^ ((l1 >> 17) & 1)];
+    const int u = S[(l1 & 0xFF) * T + t] + ((n1 >> 8) & 0xFF);
+    return g.x + u * g.y + S[((l1 >> 8) & 0xFF) * T + ((n1 >> 21) & 0x1F)] + (n1 & 0xFF);
 }
 
 }  // namespace cih

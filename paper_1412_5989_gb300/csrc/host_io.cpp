@@ -32,7 +32,7 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
     double *esp_d = nullptr;
     int64_t *rowptr_d = nullptr;
     int32_t *col_d = nullptr;
-    float *val_d = nullptr;
+    float *val_d = nullptr, *work = nullptr;
     int64_t nnz = 0;
     cudaError_t e;
     if (!alloc((void **)&tbme_d, sizeof(float) * (size_t)K * tl) || !alloc((void **)&rowptr_d, sizeof(int64_t) * (dim + 1)) ||
@@ -58,6 +58,10 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
         rc = fail(CIH_ERR_NOMEM, "build_host: device matrix");
         goto done;
     }
+    // one set: the fill's working copy of the table, prepared once for all chunks
+    if (K == 1 && fill_work_floats(b) > 0 && alloc((void **)&work, sizeof(float) * fill_work_floats(b)) &&
+        (rc = fill_prepare(b, hw, tbme_d, esp_d, nullptr, work, st)))
+        goto done;
     tm.mark_sync("device matrix allocated", st);
     e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e != cudaSuccess) { cs = nullptr; rc = cuda_fail(e, "build_host: copy stream"); goto done; }
@@ -70,7 +74,9 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
             rb[c] = std::lower_bound(rowptr_h, rowptr_h + dim + 1, nnz * c / C) - rowptr_h;
         for (int c = 0; c < C && !rc; ++c) {
             const int64_t r0 = std::min(rb[c], dim), r1 = std::max(r0, std::min(rb[c + 1], dim));
-            if ((rc = launch_fill(b, rowptr_d, K, hw, tbme_d, false, false, esp_d, col_d, val_d, st, r0, r1))) break;
+            if ((rc = launch_fill(b, rowptr_d, K, hw, tbme_d, false, false, esp_d, col_d, val_d, st, r0, r1, false,
+                                  nullptr, work)))
+                break;
             cudaEvent_t ev;
             if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) {
                 rc = cuda_fail(e, "build_host: event");

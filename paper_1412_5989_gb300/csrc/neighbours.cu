@@ -308,16 +308,19 @@ __global__ void k_groups(SpeciesBuild S, DevBasis B, int64_t *gcnt, int4 *grp, i
     }
 }
 
-// occupied orbitals of each sub-det, ascending
+// occupied orbitals of each sub-det, ascending, and the move codes of each
+// orbital kept (codes[a]: DevBasis::occ_code)
 template <int W>
-__global__ void k_occ(SpeciesBuild S, int Z, uint8_t *occ)
+__global__ void k_occ(SpeciesBuild S, int Z, const int32_t *codes, uint8_t *occ, int32_t *occ_code)
 {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < S.n_sd; x += (int64_t)gridDim.x * blockDim.x) {
         int k = 0;
         for (int w = 0; w < W; ++w) {
             uint64_t m = S.bits[x * W + w];
             while (m) {
-                occ[x * Z + k++] = (uint8_t)(w * 64 + __ffsll((long long)m) - 1);
+                const int a = w * 64 + __ffsll((long long)m) - 1;
+                occ[x * Z + k] = (uint8_t)a;
+                occ_code[x * Z + k++] = codes[a];
                 m &= m - 1;
             }
         }
@@ -795,8 +798,12 @@ int basis_tables_upload(cih_basis &b, cudaStream_t st)
     const int T = b.dev.pn_T = (mtop + 1) * 2;
     if (T > 32) return fail(CIH_ERR_UNSUPPORTED, "neutron orbitals with 2m above 15");
     std::vector<uint16_t> orbs(std::max(Q.n_orb, 1), 0);       // r(b) | t(b) << 8
-    for (int c = 0; c < Q.n_orb; ++c)
-        orbs[c] = (uint16_t)(b.pn.rn[c] | (((Q.om2[c] + mtop) / 2) * 2 + (Q.oN[c] & 1)) << 8);
+    std::vector<int32_t> pcode(std::max(P.n_orb, 1), 0), ncode(std::max(Q.n_orb, 1), 0);
+    for (int c = 0; c < Q.n_orb; ++c) {
+        const int r = b.pn.rn[c], t = ((Q.om2[c] + mtop) / 2) * 2 + (Q.oN[c] & 1);
+        orbs[c] = (uint16_t)(r | t << 8);
+        ncode[c] = r | r << 8 | t << 16 | t << 21;
+    }
     int ptop = 1;
     for (int a = 0; a < P.n_orb; ++a) ptop = std::max(ptop, std::abs(P.om2[a]));
     if (ptop > 15) return fail(CIH_ERR_UNSUPPORTED, "proton orbitals with 2m above 15");
@@ -805,6 +812,7 @@ int basis_tables_upload(cih_basis &b, cudaStream_t st)
     std::vector<uint8_t> pa(std::max(P.n_orb, 1), 0);          // N_a parity | 2 m'_a << 1, m'_a = (2m_a + ptop) / 2
     for (int a = 0; a < P.n_orb; ++a) {
         pa[a] = (uint8_t)((P.oN[a] & 1) | (P.om2[a] + ptop) << 1);
+        pcode[a] = a | a << 8 | pa[a] << 17;
         for (int t = 0; t < T; ++t) {
             const int m = 2 * (t >> 1) - mtop, k2 = P.om2[a] + m + b.pn.m2span;
             if (k2 < 0 || k2 > 2 * b.pn.m2span) continue;
@@ -813,7 +821,25 @@ int basis_tables_upload(cih_basis &b, cudaStream_t st)
             ps[(size_t)a * T + t] = b.pn.S[(size_t)a * b.pn.G + kappa];
         }
     }
-    int2 *d_pk; int16_t *d_ps; uint16_t *d_orbs; uint8_t *d_pa;
+    // the groups as full squares, one after another (the fill's working copy of the pn channel)
+    std::vector<int2> pq(64, make_int2(0, 0));
+    std::vector<int32_t> sqrow;                                // every row of every square: group << 16 | row
+    int64_t sq = 0;
+    for (int k = 0; k < 64; ++k) {
+        pq[k] = make_int2((int)std::min<int64_t>(sq, INT32_MAX), pk[k].y);
+        sq += (int64_t)pk[k].y * pk[k].y;
+        for (int u = 0; u < pk[k].y; ++u) sqrow.push_back(k << 16 | u);
+    }
+    b.sq_total = sq;
+    b.dev.n_sqrow = (int32_t)sqrow.size();
+    int2 *d_pk, *d_pq; int16_t *d_ps; uint16_t *d_orbs; uint8_t *d_pa; int32_t *d_sqrow, *d_pc, *d_nc2;
+    if ((rc = upload(b, &d_pq, pq, st)) || (rc = upload(b, &d_sqrow, sqrow, st)) || (rc = upload(b, &d_pc, pcode, st)) ||
+        (rc = upload(b, &d_nc2, ncode, st)))
+        return rc;
+    b.dev.pn_kq = d_pq;
+    b.dev.sqrow = d_sqrow;
+    b.dev.code[0] = d_pc;
+    b.dev.code[1] = d_nc2;
     if ((rc = upload(b, &d_pk, pk, st)) || (rc = upload(b, &d_ps, ps, st)) || (rc = upload(b, &d_orbs, orbs, st)) ||
         (rc = upload(b, &d_pa, pa, st)))
         return rc;
@@ -972,11 +998,13 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
         int2 *n1p;
         int16_t *dir;
         uint8_t *occn;
+        int32_t *occc;
         NeutronRec *nrec;
         const int g1 = (int)std::min<int64_t>((nn + 255) / 256 + 1, 65535);
         AllocOn on(b, side.s);
         if ((rc = dev_alloc(b, &n1p, tot)) || (rc = dev_alloc(b, &dir, (size_t)nn * b.dev.dir_len)) ||
-            (rc = dev_alloc(b, &nrec, nn)) || (rc = dev_alloc(b, &occn, (size_t)nn * std::max(b.s[1].Z, 1))))
+            (rc = dev_alloc(b, &nrec, nn)) || (rc = dev_alloc(b, &occn, (size_t)nn * std::max(b.s[1].Z, 1))) ||
+            (rc = dev_alloc(b, &occc, (size_t)nn * std::max(b.s[1].Z, 1))))
             return rc;
         if (nn > 0) {
             const DevSpecies &D = b.dev.sp[1];
@@ -984,12 +1012,13 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
             count_launches(4);
             with_words(W, [&](auto w) {
                 k_n1_pack<decltype(w)::value><<<grid_for(nn), 256, 0, side.s>>>(SB, D.n1_off, D.n1, b.dev.orbs, n1p);
-                k_occ<decltype(w)::value><<<g1, 256, 0, side.s>>>(SB, b.s[1].Z, occn);
+                k_occ<decltype(w)::value><<<g1, 256, 0, side.s>>>(SB, b.s[1].Z, b.dev.code[1], occn, occc);
             });
             k_dir<<<grid_for(nn), 256, 0, side.s>>>(SB, D.n1_off, D.n1, D.N0, D.NL, b.dev.DM, b.dev.dir_len, dir);
             k_neutron_rec<<<g1, 256, 0, side.s>>>(D, nrec);
         }
         b.dev.occ[1] = occn;
+        b.dev.occ_code[1] = occc;
         b.dev.n1p = n1p;
         b.dev.dir = dir;
         b.dev.nrec = nrec;
@@ -1003,10 +1032,12 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
         int64_t *goff;
         int32_t *row_p;
         uint8_t *occp;
+        int32_t *occc;
         int2 *l1;
         ProtonRec *prec;
         if ((rc = dev_alloc(b, &goff, np + 1)) || (rc = dev_alloc(b, &row_p, b.dim)) ||
-            (rc = dev_alloc(b, &occp, (size_t)np * std::max(b.s[0].Z, 1))) || (rc = dev_alloc(b, &l1, L[0].tot[1])) ||
+            (rc = dev_alloc(b, &occp, (size_t)np * std::max(b.s[0].Z, 1))) ||
+            (rc = dev_alloc(b, &occc, (size_t)np * std::max(b.s[0].Z, 1))) || (rc = dev_alloc(b, &l1, L[0].tot[1])) ||
             (rc = dev_alloc(b, &prec, np)))
             return rc;
         const int grid = grid_for(np);
@@ -1015,7 +1046,7 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
             count_launches(3);
             with_words(W, [&](auto w) {
                 k_groups<decltype(w)::value, 0><<<grid, 256, 0, st>>>(SB, b.dev, goff, nullptr, nullptr);
-                k_occ<decltype(w)::value><<<g0, 256, 0, st>>>(SB, b.s[0].Z, occp);
+                k_occ<decltype(w)::value><<<g0, 256, 0, st>>>(SB, b.s[0].Z, b.dev.code[0], occp, occc);
             });
             k_row_p<<<grid, 256, 0, st>>>(np, b.dev.rowbase, row_p);
         }
@@ -1035,6 +1066,11 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
         }
         tm.mark("groups queued");
         b.dev.occ[0] = occp;
+        b.dev.occ_code[0] = occc;
+        for (int t = 0; t < 2; ++t) {
+            b.fw_total[t] = L[t].tot[0];
+            b.n1_total[t] = L[t].tot[1];
+        }
         b.dev.row_p = row_p;
         b.dev.grp = grp;
         b.dev.l1 = l1;
