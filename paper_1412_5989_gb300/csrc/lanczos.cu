@@ -188,7 +188,7 @@ __global__ void k_split(int64_t n, const double *x, const double *sc, float2 *xs
     }
 }
 
-// K >= 32: lanes over sets, two per lane per pass; K < 32 (KS = next power
+// K > 16: lanes over sets, two per lane per pass; K <= 16 (KS = next power
 // of two): 32/KS lane groups split the row's nonzeros, four at a time per
 // group, and the groups' row sums are reduced at the end.  With K < 32 the
 // matrix is read with evict-first loads, so that its stream does not push x
@@ -330,7 +330,7 @@ void launch_spmv(RowRange rr, int K, const int64_t *rowptr, const int32_t *col, 
 {
     count_launches(1);
     if (K == 64) k_spmv<64><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
-    else if (K >= 32) k_spmv<32><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
+    else if (K > 16) k_spmv<32><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
     else if (K == 1) k_spmv<1><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
     else if (K <= 2) k_spmv<2><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
     else if (K <= 4) k_spmv<4><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
