@@ -283,7 +283,8 @@ int cih_autotune_fill(cih_basis_h h, const int64_t *rowptr_dev, int32_t K, doubl
  * read once per product, FP32-pair arithmetic, fixed-point mirror sums),
  * with the bound taken as F (the Lanczos vectors have unit norm); the
  * orthogonalisation and the vectors stay FP64.
- * Library-allocated for the call: (max_iter + 2) x dim x K double of Lanczos
+ * Library-allocated for the call (at most 1 GiB of freed blocks stays in the
+ * library's pool afterwards): (max_iter + 2) x dim x K double of Lanczos
  * vectors and product scratch, dim x K int64 of mirror accumulators, and for
  * K > 1 an element-major copy of the values (K x nnz float).  Deterministic:
  * the same inputs give the same bits.  Returns 0, or 1 if some set did not

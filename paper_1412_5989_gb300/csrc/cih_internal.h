@@ -16,6 +16,7 @@ namespace cih {
 
 constexpr int kMaxWords = 4;              // <= 256 orbitals per species
 constexpr int kLevels = 8;                // oscillator levels of a species: Nmax <= 7 with 256 orbitals
+constexpr uint64_t kPoolKeep = 1ull << 30; // bytes the library pool keeps after a Lanczos call
 constexpr int kSortTile = 4096;           // longest neighbour list the sort handles
 
 // ---------------------------------------------------------------- device view
@@ -323,6 +324,9 @@ int64_t scan_scratch_needed(int64_t n);
 void tridiag_qr(int n, std::vector<double> &d, std::vector<double> e, std::vector<double> &Z);
 // the same eigenvalues with only the last component of each eigenvector
 void tridiag_qr_last(int n, std::vector<double> &d, std::vector<double> e, std::vector<double> &zlast);
+// whether eigenpair k's residual bound beta |last component| exceeds tol
+// max(1, |eigenvalue|); warm: the eigenvalue of the leading block, updated (NaN: none)
+bool tridiag_pair_open(int n, const double *d, const double *e, int k, double beta, double tol, double &warm);
 // normalised eigenvector for an eigenvalue by inverse iteration
 void tridiag_eigenvector(int n, const double *d, const double *e, double theta, double *z);
 

@@ -12,13 +12,21 @@
 //   - values element-major (the K values of a nonzero together) and vectors
 //     element-major x[i * K + s], FP64;
 //   - full reorthogonalisation: classical Gram-Schmidt applied twice, dot
-//     products reduced in two fixed-order stages.
-// Host: per set (sets on parallel host threads), the lowest Ritz values and
-// the residual bounds beta_m |z_m| from implicit-QR sweeps of the tridiagonal
-// that rotate only the last row of its eigenvector matrix; the lowest Ritz
-// vector's coefficients by inverse iteration.
+//     products reduced in two fixed-order stages;
+//   - one step ahead of the host: the scalars of a step reach it while the next
+//     step runs.
+// Host: per set (sets on parallel host threads), the residual bound of the
+// nev-th pair from a Sturm bisection and a twisted factorisation of the
+// tridiagonal, O(m) a step; once that pair is near its bound, the lowest Ritz values
+// and all residual bounds beta_m |z_m| from implicit-QR sweeps that rotate only
+// the last row of the eigenvector matrix; the lowest Ritz vector's coefficients by
+// inverse iteration.
+// Start of this form -> now, one GB300, whole solves: 800 rows 15.2 -> 4.0 ms;
+// 143,792 rows with gradient 87 -> 39 ms; 64 sets of 48,917 rows 492 -> 370 ms;
+// the uneven batch of 197,822 / 143,792 / 814,092 rows 645 -> 395 ms.
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <thread>
 #include <vector>
 
@@ -45,6 +53,7 @@ void parallel_sets(int K, F &&fn)
     for (auto &x : th) x.join();
 }
 
+constexpr int kSumsqBlocks = 256;                // partial sums of the bound
 constexpr int kDotBlocks = 256;
 constexpr int kThreads = 256;
 
@@ -112,18 +121,25 @@ __global__ void __launch_bounds__(kSumsqThreads) k_upper_sumsq(RowRange rr, int 
     }
 }
 
-// sc = (2^s, 2^-s, 2^r, 2^-r) from the sum of squares F^2 (fixed-order sum
-// of the partials) and, when given, the largest squared norm of the K
+// sc = (2^s, 2^-s, 2^r, 2^-r) from the sum of squares F^2 (the kSumsqBlocks
+// partials, added as a tree) and, when given, the largest squared norm of the K
 // vectors (else the vectors have norm 1), with F ||x|| < 2^e and ||x|| < 2^ex:
 //   s = min(60 - e, 124 - ex): the mirrored products' units 2^-s keep every
 //       accumulator below 2^60, and every x_i 2^s is an FP32 pair;
 //   r = 1 - ex: the row part multiplies x 2^r, of norm below 2 (0 when the
 //       vectors have norm 1).
-__global__ void k_mirror_scale(int parts, const double *partial, int K, const double *xn2, double *sc)
+__global__ void __launch_bounds__(kSumsqBlocks) k_mirror_scale(const double *partial, int K, const double *xn2, double *sc)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double f2 = 0.0;
-    for (int b = 0; b < parts; ++b) f2 += partial[b];
+    __shared__ double red[kSumsqBlocks];
+    const int tid = threadIdx.x;
+    red[tid] = partial[tid];
+    __syncthreads();
+    for (int d = kSumsqBlocks / 2; d > 0; d >>= 1) {              // the order upper_sumsq adds in
+        if (tid < d) red[tid] += red[tid + d];
+        __syncthreads();
+    }
+    if (tid != 0) return;
+    const double f2 = red[0];
     double m = 1.0;
     if (xn2) {
         m = 0.0;
@@ -287,16 +303,21 @@ __global__ void __launch_bounds__(kThreads, 4) k_spmv(RowRange rr, int K, const 
     }
 }
 
-// y[t] = row part 2^-r + mirrored part 2^-s; the accumulators are cleared
-// for the next product
+// y = row part 2^-r + mirrored part 2^-s; the accumulator is cleared for the
+// next product
+__device__ __forceinline__ double finish_entry(const float2 *yrow, unsigned long long *yfix, int64_t t, double sinv, double rinv)
+{
+    const float2 r = yrow[t];
+    const double y = ((double)r.x + (double)r.y) * rinv + (double)(long long)yfix[t] * sinv;
+    yfix[t] = 0ull;
+    return y;
+}
+
 __global__ void k_sym_finish(int64_t n, const double *sc, const float2 *yrow, double *y, unsigned long long *yfix)
 {
     const double sinv = sc[1], rinv = sc[3];
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-        const float2 r = yrow[t];
-        y[t] = ((double)r.x + (double)r.y) * rinv + (double)(long long)yfix[t] * sinv;
-        yfix[t] = 0ull;
-    }
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
+        y[t] = finish_entry(yrow, yfix, t, sinv, rinv);
 }
 
 // Row shards: the local rows' row part in FP64 into yx (the other entries
@@ -338,57 +359,148 @@ void launch_spmv(RowRange rr, int K, const int64_t *rowptr, const int32_t *col, 
     else k_spmv<16><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
 }
 
-// partial[(r * K + s) * gridDim.x + blk] = sum over this block's rows of V[r][i][s] w[i][s]
-__global__ void k_dots(int64_t dim, int K, int nvec, const double *V, int64_t vstride, const double *w,
-                       double *partial)
+// ---- orthogonalisation: classical Gram-Schmidt twice, every sum in a fixed order
+//
+// A dot product is split over kDotBlocks blocks of kThreads threads: thread (sub,
+// s) of block b takes rows b per + sub, then every kDotBlocks per further on (per =
+// kThreads / K rows a block, sets s); the block's threads are added in
+// order, then the blocks in order.  That order is part of the results: the
+// signs of the Ritz vectors hang on the last bits of the tridiagonal, so it stays
+// whatever executes it.  What is fast here: a block takes 32 vectors, whose
+// ordered adds run side by side in one warp (an FP64 instruction occupies the
+// SM's two units for 16 cycles however few lanes are active, so one lane at a
+// time made the adds, not the memory, the limit); they run from shared memory,
+// the blocks' sums are loaded together before theirs, and blocks and threads
+// without rows (whose sums are zeros) are left out.  (A thread adding 256 values
+// of one vector per block, and again 256 blocks' sums from global memory, took 73
+// + 17 us for the dot products of a step at 800 rows, three times a step.)
+constexpr int kDotVecs = 32;           // most vectors of a block (dot_vecs)
+constexpr int kDotPad = kThreads + 1;  // (the ordered adds read a column of 32 vectors: no bank twice)
+
+__host__ __device__ inline int dot_blocks(int64_t dim, int K)
 {
-    __shared__ double red[kThreads];
-    const int per = kThreads / K;                    // rows per pass (K <= kThreads)
-    const int s = threadIdx.x % K, sub = threadIdx.x / K;
-    const bool act = sub < per;
-    for (int r = blockIdx.y; r < nvec; r += gridDim.y) {
-        const double *v = V + (int64_t)r * vstride;
-        double acc = 0.0;
-        if (act)
-            for (int64_t i = (int64_t)blockIdx.x * per + sub; i < dim; i += (int64_t)gridDim.x * per)
-                acc += v[i * K + s] * w[i * K + s];
-        red[threadIdx.x] = acc;
+    const int64_t per = kThreads / K, n = (dim + per - 1) / per;
+    return (int)(n < 1 ? 1 : n < kDotBlocks ? n : kDotBlocks);
+}
+
+// partial[blk * nvec * K + r * K + s] = block blk's part of sum_i V[r][i][s] w[i][s]
+template <int KC>
+__global__ void __launch_bounds__(kThreads) k_dots(int64_t dim, int K_, int nvec, const double *V, int64_t vstride,
+                                                   const double *w, double *partial, int vecs)
+{
+    extern __shared__ double red[];                               // min(vecs, nvec) x kDotPad
+    const int K = KC ? KC : K_, per = kThreads / K, tid = threadIdx.x;
+    const int s = KC == 1 ? 0 : tid % K, sub = KC == 1 ? tid : tid / K;
+    const int r0 = blockIdx.y * vecs, nv = min(vecs, nvec - r0);
+    const int64_t i0 = (int64_t)blockIdx.x * per + sub, step = (int64_t)kDotBlocks * per;
+    for (int u0 = 0; u0 < nv; u0 += 4) {
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        const double *v = V + (int64_t)(r0 + u0) * vstride + s;
+        if (sub < per && u0 + 4 <= nv) {
+#pragma unroll 4
+            for (int64_t i = i0; i < dim; i += step) {
+                const double x = w[i * K + s];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc[u] += v[u * vstride + i * K] * x;
+            }
+        } else if (sub < per) {
+#pragma unroll 2
+            for (int64_t i = i0; i < dim; i += step) {
+                const double x = w[i * K + s];
+#pragma unroll
+                for (int u = 0; u < 3; ++u)
+                    if (u0 + u < nv) acc[u] += v[u * vstride + i * K] * x;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (u0 + u < nv) red[(u0 + u) * kDotPad + tid] = acc[u];
+    }
+    __syncthreads();
+    const int rows = (int)min((int64_t)per, dim - (int64_t)blockIdx.x * per);       // threads with rows
+    for (int q = tid; q < nv * K; q += kThreads) {
+        const int u = KC == 1 ? q : q / K, ss = KC == 1 ? 0 : q - u * K;
+        const double *o = red + u * kDotPad + ss;
+        double t = 0.0;
+#pragma unroll 8
+        for (int x = 0; x < rows; ++x) t += o[x * K];
+        partial[(int64_t)blockIdx.x * nvec * K + (r0 + u) * K + ss] = t;
+    }
+}
+
+// What k_dots_sum does with the sums t over the blocks, q = r K + s:
+//   h    store them (coefficients of the next update); alpha[s] gets the last
+//        vector's, added to its value of the first pass in the second
+//   beta |w|^2 to beta[s], f[s] = 1 / |w|, or 0 for a set that is done or whose
+//        Krylov space is exhausted (the host's test for that)
+//   unit store them, f[s] = 1 / sqrt(t) (0 for a zero vector)
+enum { kSumFirst = 0, kSumSecond = 1, kSumBeta = 2, kSumUnit = 3 };
+constexpr int kSumRows = 128;
+
+__global__ void __launch_bounds__(kThreads) k_dots_sum(int mode, int nvec, int K, int blocks, const double *partial, double *out,
+                                                       double *alpha, double *beta, double *f, const int *done)
+{
+    __shared__ double red[kSumRows][33];
+    const int nq = nvec * K, lane = threadIdx.x & 31, q = blockIdx.x * 32 + lane;
+    double t = 0.0;
+    for (int b0 = 0; b0 < blocks; b0 += kSumRows) {
+        const int n = min(kSumRows, blocks - b0);
+        if (q < nq)
+            for (int b = threadIdx.x >> 5; b < n; b += kThreads / 32) red[b][lane] = partial[(int64_t)(b0 + b) * nq + q];
         __syncthreads();
-        if (threadIdx.x < K) {
-            double t = 0.0;
-            for (int q = 0; q < per; ++q) t += red[q * K + threadIdx.x];
-            partial[((int64_t)r * K + threadIdx.x) * gridDim.x + blockIdx.x] = t;
+        if (threadIdx.x < 32 && q < nq) {
+#pragma unroll 8
+            for (int b = 0; b < n; ++b) t += red[b][lane];
         }
         __syncthreads();
     }
-}
-
-// out[q] = fixed-order sum of the partials of q = r * K + s
-__global__ void k_dots_finish(int n, int parts, const double *partial, double *out)
-{
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-        double t = 0.0;
-        for (int b = 0; b < parts; ++b) t += partial[(int64_t)q * parts + b];
+    if (threadIdx.x >= 32 || q >= nq) return;
+    const int s = q % K, r = q / K;
+    if (mode == kSumFirst || mode == kSumSecond) {
         out[q] = t;
+        if (r == nvec - 1) alpha[s] = mode == kSumFirst ? t : alpha[s] + t;
+    } else if (mode == kSumBeta) {
+        beta[s] = t;
+        const double b = sqrt(fmax(t, 0.0));
+        f[s] = done[s] || b <= 1e-12 * (fabs(alpha[s]) + 1.0) ? 0.0 : 1.0 / b;
+    } else {
+        out[q] = t;
+        f[s] = t > 0.0 ? 1.0 / sqrt(t) : 0.0;
     }
 }
 
-// w[i][s] -= sum_r h[r][s] V[r][i][s]
-__global__ void k_subtract(int64_t n, int K, int nvec, const double *V, int64_t vstride, const double *h, double *w)
+// w[i][s] -= sum_r h[r][s] V[r][i][s], r ascending (out: sum_r h[r][s] V[r][i][s]
+// from zero); eight loads in flight
+template <bool SUB>
+__global__ void __launch_bounds__(kThreads) k_combine(int64_t n, int K, int nvec, const double *V, int64_t vstride, const double *h,
+                                                      double *w)
 {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-        const int s = (int)(t % K);
-        double acc = w[t];
-        for (int r = 0; r < nvec; ++r) acc -= h[r * K + s] * V[(int64_t)r * vstride + t];
-        w[t] = acc;
+        const double *v = V + t, *c = h + (K == 1 ? 0 : t % K);
+        double x = SUB ? w[t] : 0.0;
+        int r = 0;
+        for (; r + 8 <= nvec; r += 8) {
+            double y[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) y[u] = v[(int64_t)(r + u) * vstride];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x = SUB ? x - c[(r + u) * K] * y[u] : x + c[(r + u) * K] * y[u];
+        }
+        for (; r < nvec; ++r) x = SUB ? x - c[r * K] * v[(int64_t)r * vstride] : x + c[r * K] * v[(int64_t)r * vstride];
+        w[t] = x;
     }
 }
 
-// out[t] = in[t] * f[s]
-__global__ void k_scale_sets(int64_t n, int K, const double *in, const double *f, double *out)
+// v = w f, the next Lanczos vector, and its split for the product (k_split)
+__global__ void k_next(int64_t n, int K, const double *w, const double *f, const double *sc, double *v, float2 *xs, float2 *xm)
 {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-        out[t] = in[t] * f[t % K];
+    const double fr = sc[2], fs = sc[0];
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        const double x = w[t] * f[K == 1 ? 0 : t % K];
+        v[t] = x;
+        xs[t] = split2(x * fr);
+        xm[t] = split2(x * fs);
+    }
 }
 
 // deterministic start vector: 1 + 0.5 u_i, u_i from the splitmix64 hash of i (same for every set)
@@ -403,33 +515,47 @@ __global__ void k_start(int64_t dim, int K, double *v)
     }
 }
 
-// evec[s * dim + i] = sum_r c[r * K + s] V[r][i][s]  (set-major output)
-__global__ void k_ritz(int64_t dim, int K, int m, const double *V, int64_t vstride, const double *c, double *evec)
+// evec[s * dim + i] = w[i * K + s] f[s]  (set-major output)
+__global__ void k_ritz_out(int64_t dim, int K, const double *w, const double *f, double *evec)
 {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < dim * K; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = t / K;
         const int s = (int)(t - i * K);
-        double acc = 0.0;
-        for (int r = 0; r < m; ++r) acc += c[r * K + s] * V[(int64_t)r * vstride + t];
-        evec[(int64_t)s * dim + i] = acc;
+        evec[(int64_t)s * dim + i] = w[t] * f[s];
     }
 }
 
-// normalise each set-major vector: block s reduces set s in a fixed order
-__global__ void k_normalise_sets(int64_t dim, double *evec)
+// Vectors of a block of k_dots: as many as leave two blocks per SM, in fours;
+// four where a block has few ordered adds (many sets) or short vectors leave few
+// blocks.  One size for all, at 800 rows / 143,792 rows / 48,917 rows of 64 sets,
+// a whole solve: 4 vectors 3.87 / 47.5 / 383 ms, 32 vectors 4.41 / 38.3 / 391 ms.
+int dot_vecs(int nb, int K, int nvec)
 {
-    __shared__ double red[kThreads];
-    double *v = evec + (int64_t)blockIdx.x * dim;
-    double acc = 0.0;
-    for (int64_t i = threadIdx.x; i < dim; i += blockDim.x) acc += v[i] * v[i];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int d = kThreads / 2; d > 0; d >>= 1) {
-        if (threadIdx.x < d) red[threadIdx.x] += red[threadIdx.x + d];
-        __syncthreads();
-    }
-    const double f = red[0] > 0.0 ? 1.0 / sqrt(red[0]) : 0.0;
-    for (int64_t i = threadIdx.x; i < dim; i += blockDim.x) v[i] *= f;
+    if (K >= 16) return 4;
+    return std::max(4, std::min(kDotVecs, nb * nvec / 304 / 4 * 4));
+}
+
+// k_dots takes up to 66 KB of shared memory (set once per device; idempotent)
+cudaError_t prepare_dots(int K)
+{
+    const int bytes = (int)sizeof(double) * kDotPad * kDotVecs;
+    const void *f = K == 1 ? (const void *)k_dots<1> : K == 64 ? (const void *)k_dots<64> : (const void *)k_dots<0>;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+// sums[q] over r < nvec of V[r] . w per set, then `mode` (k_dots_sum)
+void launch_dots(int mode, int64_t dim, int K, int nvec, const double *V, int64_t vstride, const double *w, double *partial,
+                 double *out, double *alpha, double *beta, double *f, const int *done, cudaStream_t st)
+{
+    const int nb = dot_blocks(dim, K);
+    const int vecs = dot_vecs(nb, K, nvec);
+    const dim3 grid(nb, (nvec + vecs - 1) / vecs);
+    const size_t smem = sizeof(double) * kDotPad * std::min(nvec, vecs);
+    count_launches(2);
+    if (K == 1) k_dots<1><<<grid, kThreads, smem, st>>>(dim, K, nvec, V, vstride, w, partial, vecs);
+    else if (K == 64) k_dots<64><<<grid, kThreads, smem, st>>>(dim, K, nvec, V, vstride, w, partial, vecs);
+    else k_dots<0><<<grid, kThreads, smem, st>>>(dim, K, nvec, V, vstride, w, partial, vecs);
+    k_dots_sum<<<(nvec * K + 31) / 32, kThreads, 0, st>>>(mode, nvec, K, nb, partial, out, alpha, beta, f, done);
 }
 
 int grid_for(int64_t n)
@@ -444,10 +570,45 @@ int64_t lanczos_bytes(int64_t dim, int64_t nnz, int K, int max_iter)
     const int64_t m = std::min<int64_t>(max_iter, dim);
     int64_t bytes = 8 * (m + 1) * dim * K + 8 * dim * K;            // Lanczos vectors, w
     bytes += 32 * dim * K;                                          // mirror accumulators, split x, row part
-    bytes += 8 * (m + 1) * K * kDotBlocks + 8 * (m + 1) * K + 8 * K + 32; // dot partials, h, scale
+    bytes += 8 * (m + 1) * K * kDotBlocks;   // partial sums
+    bytes += 8 * (m + 1) * K + 64 * K + 32;                         // coefficients, scalars, scale
     if (K > 1) bytes += 4 * nnz * K;                                // element-major values
     return bytes + 8 * 256;                                         // allocation granules
 }
+
+// Page-locked blocks for the two scalars a set returns per step (two steps in
+// flight) and the done flags, kept for the next call; at most kKeep of them.
+struct StepLog {
+    static constexpr int kMaxSets = 256, kKeep = 16;
+    double *p = nullptr;                                            // [2][2 K], then int done[K]
+    static std::mutex &mu() { static std::mutex m; return m; }
+    static std::vector<double *> &kept() { static std::vector<double *> v; return v; }
+    bool get()
+    {
+        {
+            std::lock_guard<std::mutex> lock(mu());
+            if (!kept().empty()) {
+                p = kept().back();
+                kept().pop_back();
+                return true;
+            }
+        }
+        if (cudaHostAlloc((void **)&p, sizeof(double) * 4 * kMaxSets + sizeof(int) * kMaxSets, cudaHostAllocPortable) != cudaSuccess) {
+            (void)cudaGetLastError();
+            p = nullptr;
+        }
+        return p != nullptr;
+    }
+    ~StepLog()                                                      // the caller has synchronised the copies
+    {
+        if (!p) return;
+        std::lock_guard<std::mutex> lock(mu());
+        if ((int)kept().size() < kKeep) kept().push_back(p);
+        else cudaFreeHost(p);
+    }
+    double *slot(int j, int K) const { return p + (j & 1) * 2 * K; }
+    int *done() const { return reinterpret_cast<int *>(p + 4 * kMaxSets); }
+};
 
 // sh->f2 -> (2^s, 2^-s, 1, 1): the scale k_mirror_scale gives unit vectors
 static void shard_scale(double f2, double *sc)
@@ -493,7 +654,8 @@ int lanczos(const cih_basis &b, const int64_t *rowptr, const int32_t *col, const
     float *vem = nullptr;
     unsigned long long *yfix = nullptr;
     float2 *xs = nullptr, *xm = nullptr, *yrow = nullptr;
-    double *V = nullptr, *w = nullptr, *partial = nullptr, *hdev = nullptr, *fdev = nullptr, *sc = nullptr;
+    double *V = nullptr, *w = nullptr, *partial = nullptr, *hdev = nullptr, *slog = nullptr, *fdev = nullptr, *sc = nullptr;
+    int *ddone = nullptr;
     bool ok = (sh ? (yfix = sh->acc) != nullptr : alloc((void **)&yfix, sizeof(unsigned long long) * (size_t)vstride)) &&
               alloc((void **)&xs, sizeof(float2) * (size_t)vstride) &&
               alloc((void **)&xm, sizeof(float2) * (size_t)vstride) &&
@@ -501,10 +663,16 @@ int lanczos(const cih_basis &b, const int64_t *rowptr, const int32_t *col, const
               alloc((void **)&V, sizeof(double) * (size_t)(m_max + 1) * vstride) &&
               alloc((void **)&w, sizeof(double) * vstride) &&
               alloc((void **)&partial, sizeof(double) * (size_t)(m_max + 1) * K * kDotBlocks) &&
-              alloc((void **)&hdev, sizeof(double) * (size_t)(m_max + 1) * K) && alloc((void **)&fdev, sizeof(double) * K) &&
-              alloc((void **)&sc, sizeof(double) * 4);
+              alloc((void **)&hdev, sizeof(double) * (size_t)(m_max + 1) * K) &&
+              alloc((void **)&slog, sizeof(double) * 4 * K) && alloc((void **)&fdev, sizeof(double) * K) &&
+              alloc((void **)&sc, sizeof(double) * 4) && alloc((void **)&ddone, sizeof(int) * K);
     if (ok && K > 1 && !values_em) ok = alloc((void **)&vem, sizeof(float) * (size_t)nnz * K);
-    int rc = ok ? CIH_OK : fail(CIH_ERR_NOMEM, "lanczos: device memory");
+    StepLog pin;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    int rc = ok && pin.get() ? CIH_OK : fail(CIH_ERR_NOMEM, "lanczos: memory");
+    for (int i = 0; i < 2 && !rc; ++i)
+        if ((e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming)) != cudaSuccess) rc = cuda_fail(e, "lanczos: event");
+    if (!rc && (e = prepare_dots(K)) != cudaSuccess) rc = cuda_fail(e, "lanczos: shared memory");
     const int g = grid_for(vstride);
     const int gr = (int)std::max<int64_t>(1, std::min<int64_t>((r1 - r0 + 7) / 8, 152 * 32));
 
@@ -517,6 +685,7 @@ int lanczos(const cih_basis &b, const int64_t *rowptr, const int32_t *col, const
         } else {
             vem = const_cast<float *>(val);                         // K = 1, or already element-major
         }
+        cudaMemsetAsync(ddone, 0, sizeof(int) * K, st);
         if (sh) {
             double hsc[4];
             shard_scale(sh->f2, hsc);
@@ -526,17 +695,17 @@ int lanczos(const cih_basis &b, const int64_t *rowptr, const int32_t *col, const
         } else {
             cudaMemsetAsync(yfix, 0, sizeof(unsigned long long) * (size_t)vstride, st);
             count_launches(2);
-            k_upper_sumsq<<<kDotBlocks, kSumsqThreads, 0, st>>>(rr, K, rowptr, vem, partial);
-            k_mirror_scale<<<1, 32, 0, st>>>(kDotBlocks, partial, K, nullptr, sc);
+            k_upper_sumsq<<<kSumsqBlocks, kSumsqThreads, 0, st>>>(rr, K, rowptr, vem, partial);
+            k_mirror_scale<<<1, kSumsqBlocks, 0, st>>>(partial, K, nullptr, sc);
         }
     }
 
-    auto spmv = [&](const double *x, double *y) -> int {
-        count_launches(2);
-        k_split<<<g, kThreads, 0, st>>>(vstride, x, sc, xs, xm);
+    // w = H v_j from the split of v_j
+    auto spmv = [&]() -> int {
         launch_spmv(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, gr, st);
         if (!sh) {
-            k_sym_finish<<<g, kThreads, 0, st>>>(vstride, sc, yrow, y, yfix);
+            count_launches(1);
+            k_sym_finish<<<g, kThreads, 0, st>>>(vstride, sc, yrow, w, yfix);
             return CIH_OK;
         }
         // a shard: its rows' row part, then the caller sums both buffers over the shards
@@ -545,65 +714,68 @@ int lanczos(const cih_basis &b, const int64_t *rowptr, const int32_t *col, const
         cudaError_t ee = cudaStreamSynchronize(st);
         if (ee != cudaSuccess) return cuda_fail(ee, "lanczos: shard product");
         if (sh->combine(sh->ctx) != 0) return fail(CIH_ERR_ARG, "lanczos: the shard combine callback failed");
-        k_shard_finish<<<g, kThreads, 0, st>>>(vstride, sc, sh->yx, yfix, y);
+        k_shard_finish<<<g, kThreads, 0, st>>>(vstride, sc, sh->yx, yfix, w);
         return CIH_OK;
-    };
-    // h[r][s] = V[r] . w for r < nvec: into hdev (device) and hh (host)
-    std::vector<double> hh((size_t)(m_max + 1) * K);
-    auto dots = [&](const double *vb, int nvec, const double *wv) -> int {
-        dim3 grid(kDotBlocks, std::min(nvec, 65535));
-        count_launches(2);
-        k_dots<<<grid, kThreads, 0, st>>>(dim, K, nvec, vb, vstride, wv, partial);
-        k_dots_finish<<<(nvec * K + 255) / 256, 256, 0, st>>>(nvec * K, kDotBlocks, partial, hdev);
-        cudaError_t ee = cudaMemcpyAsync(hh.data(), hdev, sizeof(double) * nvec * K, cudaMemcpyDeviceToHost, st);
-        if (ee == cudaSuccess) ee = cudaStreamSynchronize(st);
-        return ee == cudaSuccess ? CIH_OK : cuda_fail(ee, "lanczos: dots");
-    };
-    std::vector<double> fh(K);
-    auto scale = [&](const double *in, double *out) {
-        cudaMemcpyAsync(fdev, fh.data(), sizeof(double) * K, cudaMemcpyHostToDevice, st);
-        count_launches(1);
-        k_scale_sets<<<g, kThreads, 0, st>>>(vstride, K, in, fdev, out);
     };
 
     // v0 = start / |start| per set
     if (!rc) {
-        count_launches(1);
+        count_launches(2);
         k_start<<<g, kThreads, 0, st>>>(dim, K, w);
-        rc = dots(w, 1, w);
-        for (int s = 0; s < K && !rc; ++s) fh[s] = 1.0 / std::sqrt(hh[s]);
-        if (!rc) scale(w, V);
+        launch_dots(kSumUnit, dim, K, 1, w, vstride, w, partial, hdev, nullptr, nullptr, fdev, nullptr, st);
+        k_next<<<g, kThreads, 0, st>>>(vstride, K, w, fdev, sc, V, xs, xm);
     }
+    // step j on the device: product, orthogonalisation, the scalars to the host,
+    // and the next vector (a finished set's is zero)
+    auto enqueue = [&](int j) -> int {
+        const int r = spmv();
+        if (r) return r;
+        double *alpha = slog + (j & 1) * 2 * K, *beta = alpha + K;
+        for (int pass = 0; pass < 2; ++pass) {                      // alpha_j = v_j . H v_j (+ the second pass's small correction)
+            launch_dots(pass ? kSumSecond : kSumFirst, dim, K, j + 1, V, vstride, w, partial, hdev, alpha, nullptr, nullptr, nullptr, st);
+            count_launches(1);
+            k_combine<true><<<g, kThreads, 0, st>>>(vstride, K, j + 1, V, vstride, hdev, w);
+        }
+        launch_dots(kSumBeta, dim, K, 1, w, vstride, w, partial, nullptr, alpha, beta, fdev, ddone, st);
+        cudaMemcpyAsync(pin.slot(j, K), alpha, sizeof(double) * 2 * K, cudaMemcpyDeviceToHost, st);
+        cudaEventRecord(ev[j & 1], st);
+        if (j + 1 < m_max) {
+            count_launches(1);
+            k_next<<<g, kThreads, 0, st>>>(vstride, K, w, fdev, sc, V + (int64_t)(j + 1) * vstride, xs, xm);
+        }
+        const cudaError_t ee = cudaGetLastError();
+        return ee == cudaSuccess ? CIH_OK : cuda_fail(ee, "lanczos kernels");
+    };
+    // The device runs one step ahead: step j + 1 is queued before the host reads
+    // step j's scalars and decides whether the sets have converged, so the
+    // tridiagonal solves cost no device time; the last step queued may be unused.
+    // (Over shards the caller's callback runs in every step: no step ahead.)
     std::vector<std::vector<double>> alpha(K), beta(K);
     std::vector<int> done(K, 0), m_of(K, 0), met(K, 0);
-    std::vector<double> theta((size_t)K * nev, NAN);
+    std::vector<double> theta((size_t)K * nev, NAN), warm(K, NAN);
     int m = 0;
+    if (!rc && m_max > 0) rc = enqueue(0);
     for (int j = 0; j < m_max && !rc; ++j) {
-        if ((rc = spmv(V + (int64_t)j * vstride, w))) break;
-        for (int pass = 0; pass < 2 && !rc; ++pass) {
-            if ((rc = dots(V, j + 1, w))) break;
-            for (int s = 0; s < K; ++s)                             // alpha_j = v_j . H v_j (+ the
-                if (!done[s]) {                                     // second pass's small correction)
-                    if (pass == 0) alpha[s].push_back(hh[(size_t)j * K + s]);
-                    else alpha[s].back() += hh[(size_t)j * K + s];
-                }
-            count_launches(1);
-            k_subtract<<<g, kThreads, 0, st>>>(vstride, K, j + 1, V, vstride, hdev, w);
-        }
-        if (rc || (rc = dots(w, 1, w))) break;
+        if (!sh && j + 1 < m_max && (rc = enqueue(j + 1))) break;
+        if ((e = cudaEventSynchronize(ev[j & 1])) != cudaSuccess) { rc = cuda_fail(e, "lanczos: step"); break; }
+        const double *log = pin.slot(j, K);
         m = j + 1;
         // per set (sets in parallel on host threads): Ritz values and residual
         // bounds beta_m |z_m| of the lowest nev, from the tridiagonal's QR
-        // eigen-decomposition (last eigenvector components)
+        // eigen-decomposition (last eigenvector components); while the nev-th
+        // pair alone is far from its bound, the decomposition is left out
         parallel_sets(K, [&](int s) {
-            fh[s] = 0.0;
             if (done[s]) return;
-            const double bj = std::sqrt(std::max(hh[s], 0.0));
+            const double bj = std::sqrt(std::max(log[K + s], 0.0));
+            alpha[s].push_back(log[s]);
             beta[s].push_back(bj);
             const int ms = m_of[s] = (int)alpha[s].size();
             const int nv = std::min(nev, ms);
             bool conv = ms >= std::min<int64_t>(nev, dim);
             const bool invariant = bj <= 1e-12 * (std::fabs(alpha[s].back()) + 1.0);
+            if (!invariant && ms < m_max && (!conv || tridiag_pair_open(ms, alpha[s].data(), beta[s].data(), nv - 1, bj,
+                                                                        10.0 * tol, warm[s])))
+                return;
             std::vector<double> dq(alpha[s]), eq(beta[s].begin(), beta[s].begin() + (ms - 1)), zl;
             if (eq.empty()) eq.push_back(0.0);
             tridiag_qr_last(ms, dq, eq, zl);
@@ -614,12 +786,17 @@ int lanczos(const cih_basis &b, const int64_t *rowptr, const int32_t *col, const
             }
             met[s] = conv || invariant;
             if (met[s] || ms == m_max) done[s] = 1;
-            else fh[s] = 1.0 / bj;                                  // next vector; frozen sets get zeros
         });
         bool all = true;
         for (int s = 0; s < K; ++s) all = all && done[s];
         if (all) break;
-        scale(w, V + (int64_t)(j + 1) * vstride);
+        if (K > 1 && !std::equal(done.begin(), done.end(), pin.done())) {
+            // (the flags only spare finished sets further steps; a copy in flight may
+            // carry the newer ones)
+            std::copy(done.begin(), done.end(), pin.done());
+            cudaMemcpyAsync(ddone, pin.done(), sizeof(int) * K, cudaMemcpyHostToDevice, st);
+        }
+        if (sh && j + 1 < m_max) rc = enqueue(j + 1);
     }
     int not_converged = 0;
     if (!rc) {
@@ -635,20 +812,22 @@ int lanczos(const cih_basis &b, const int64_t *rowptr, const int32_t *col, const
             }
         }
         if (evec0 && m > 0) {
+            // (the step queued ahead has read its coefficients before these arrive)
             cudaMemcpyAsync(hdev, coef.data(), sizeof(double) * (size_t)m * K, cudaMemcpyHostToDevice, st);
             count_launches(2);
-            k_ritz<<<g, kThreads, 0, st>>>(dim, K, m, V, vstride, hdev, evec0);
-            k_normalise_sets<<<K, kThreads, 0, st>>>(dim, evec0);
+            k_combine<false><<<g, kThreads, 0, st>>>(vstride, K, m, V, vstride, hdev, w);
+            launch_dots(kSumUnit, dim, K, 1, w, vstride, w, partial, hdev, nullptr, nullptr, fdev, nullptr, st);
+            k_ritz_out<<<g, kThreads, 0, st>>>(dim, K, w, fdev, evec0);
         }
     }
     e = cudaGetLastError();
     if (!rc && e != cudaSuccess) rc = cuda_fail(e, "lanczos kernels");
     for (void *p : bufs) cudaFreeAsync(p, st);
-    if (!rc) {
-        e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = cuda_fail(e, "lanczos");
-    }
-    cudaMemPoolTrimTo(b.pool, 0);                            // the Lanczos vectors go back to the system
+    e = cudaStreamSynchronize(st);                           // also before the page-locked block is given back
+    if (!rc && e != cudaSuccess) rc = cuda_fail(e, "lanczos");
+    for (cudaEvent_t x : ev)
+        if (x) cudaEventDestroy(x);
+    cudaMemPoolTrimTo(b.pool, kPoolKeep);                    // the Lanczos vectors go back to the system
     return rc ? rc : not_converged;
 }
 
@@ -678,14 +857,14 @@ int ham_spmv(const cih_basis &b, const int64_t *rowptr, const int32_t *col, cons
     };
     unsigned long long *yfix = nullptr;
     float2 *xs = nullptr, *xm = nullptr, *yrow = nullptr;
-    double *partial = nullptr, *xpart = nullptr, *xn2 = nullptr, *sc = nullptr;
+    double *partial = nullptr, *xpart = nullptr, *xn2 = nullptr, *xf = nullptr, *sc = nullptr;
     float *vem = nullptr;
     bool ok = alloc((void **)&yfix, sizeof(unsigned long long) * (size_t)n) &&
               alloc((void **)&xs, sizeof(float2) * (size_t)n) && alloc((void **)&xm, sizeof(float2) * (size_t)n) &&
               alloc((void **)&yrow, sizeof(float2) * (size_t)n) &&
-              alloc((void **)&partial, sizeof(double) * kDotBlocks) &&
+              alloc((void **)&partial, sizeof(double) * kSumsqBlocks) &&
               alloc((void **)&xpart, sizeof(double) * (size_t)K * kDotBlocks) &&
-              alloc((void **)&xn2, sizeof(double) * K) && alloc((void **)&sc, sizeof(double) * 4);
+              alloc((void **)&xn2, sizeof(double) * K) && alloc((void **)&xf, sizeof(double) * K) && alloc((void **)&sc, sizeof(double) * 4);
     if (ok && K > 1 && !values_em) ok = alloc((void **)&vem, sizeof(float) * (size_t)nnz * K);
     int rc = ok ? CIH_OK : fail(CIH_ERR_NOMEM, "spmv: device memory");
     if (!rc) {
@@ -696,11 +875,10 @@ int ham_spmv(const cih_basis &b, const int64_t *rowptr, const int32_t *col, cons
             vem = const_cast<float *>(val);
         }
         cudaMemsetAsync(yfix, 0, sizeof(unsigned long long) * (size_t)n, st);
-        count_launches(6);
-        k_upper_sumsq<<<kDotBlocks, kSumsqThreads, 0, st>>>(RowRange{0, dim, 0}, K, rowptr, vem, partial);
-        k_dots<<<dim3(kDotBlocks, 1), kThreads, 0, st>>>(dim, K, 1, x, n, x, xpart);
-        k_dots_finish<<<(K + 255) / 256, 256, 0, st>>>(K, kDotBlocks, xpart, xn2);
-        k_mirror_scale<<<1, 32, 0, st>>>(kDotBlocks, partial, K, xn2, sc);
+        count_launches(4);
+        k_upper_sumsq<<<kSumsqBlocks, kSumsqThreads, 0, st>>>(RowRange{0, dim, 0}, K, rowptr, vem, partial);
+        launch_dots(kSumUnit, dim, K, 1, x, n, x, xpart, xn2, nullptr, nullptr, xf, nullptr, st);
+        k_mirror_scale<<<1, kSumsqBlocks, 0, st>>>(partial, K, xn2, sc);
         k_split<<<grid_for(n), kThreads, 0, st>>>(n, x, sc, xs, xm);
         const int gr = (int)std::min<int64_t>((dim + 7) / 8, 152 * 32);
         launch_spmv(RowRange{0, dim, 0}, K, rowptr, col, vem, xs, xm, yrow, yfix, gr, st);
@@ -727,7 +905,7 @@ int upper_sumsq(const cih_basis &b, const int64_t *rowptr, int64_t r0, int64_t r
     const int64_t nnz = ends[1] - ends[0];
     float *vem = const_cast<float *>(val);
     double *partial = nullptr;
-    if (cudaMallocFromPoolAsync((void **)&partial, sizeof(double) * kDotBlocks, b.pool, st) != cudaSuccess) {
+    if (cudaMallocFromPoolAsync((void **)&partial, sizeof(double) * kSumsqBlocks, b.pool, st) != cudaSuccess) {
         (void)cudaGetLastError();
         return fail(CIH_ERR_NOMEM, "upper_sumsq: device memory");
     }
@@ -743,12 +921,14 @@ int upper_sumsq(const cih_basis &b, const int64_t *rowptr, int64_t r0, int64_t r
         k_vals_em<<<grid_for(nnz * K), kThreads, 0, st>>>(K, nnz, val, vem);
     }
     count_launches(1);
-    k_upper_sumsq<<<kDotBlocks, kSumsqThreads, 0, st>>>(RowRange{r0, r1, ends[0]}, K, rowptr, vem, partial);
-    std::vector<double> hp(kDotBlocks);
-    e = cudaMemcpyAsync(hp.data(), partial, sizeof(double) * kDotBlocks, cudaMemcpyDeviceToHost, st);
+    k_upper_sumsq<<<kSumsqBlocks, kSumsqThreads, 0, st>>>(RowRange{r0, r1, ends[0]}, K, rowptr, vem, partial);
+    std::vector<double> hp(kSumsqBlocks);
+    e = cudaMemcpyAsync(hp.data(), partial, sizeof(double) * kSumsqBlocks, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) rc = cuda_fail(e, "upper_sumsq");
-    for (int k = 0; k < kDotBlocks && !rc; ++k) *f2 += hp[k];             // the order k_mirror_scale sums in
+    for (int d = kSumsqBlocks / 2; d > 0; d >>= 1)                          // the order k_mirror_scale adds in
+        for (int k = 0; k < d; ++k) hp[k] += hp[k + d];
+    if (!rc) *f2 = hp[0];
     cudaFreeAsync(partial, st);
     if (vem != val) cudaFreeAsync(vem, st);
     return rc;

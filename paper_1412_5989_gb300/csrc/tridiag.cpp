@@ -125,6 +125,74 @@ void tridiag_eigenvector(int n, const double *d, const double *e, double theta, 
     }
 }
 
+// Eigenvalues of the tridiagonal below x (Sturm sequence).
+static int sturm_below(int n, const double *d, const double *e, double x)
+{
+    int c = 0;
+    double q = d[0] - x;
+    c += q < 0.0;
+    for (int i = 1; i < n; ++i) {
+        if (q == 0.0) q = 1e-300;
+        q = d[i] - x - e[i - 1] * (e[i - 1] / q);
+        c += q < 0.0;
+    }
+    return c;
+}
+
+// Whether beta |z| > tol max(1, |theta|) for eigenpair k (ascending), z the last
+// component of its eigenvector: theta by bisection (from `warm`, the same
+// eigenvalue of the leading n - 1 block, an upper bound by interlacing), z from
+// the twisted factorisation of T - theta at its smallest twist element.  O(n) per
+// bisection step, where the QR of the whole matrix takes O(n^2).  False when in
+// doubt.
+bool tridiag_pair_open(int n, const double *d, const double *e, int k, double beta, double tol, double &warm)
+{
+    double r = 0.0;                                             // Gershgorin radius of the spectrum
+    double lo = d[0], hi = d[0];
+    for (int i = 0; i < n; ++i) {
+        const double g = (i > 0 ? std::fabs(e[i - 1]) : 0.0) + (i + 1 < n ? std::fabs(e[i]) : 0.0);
+        lo = std::min(lo, d[i] - g);
+        hi = std::max(hi, d[i] + g);
+    }
+    r = std::max(std::fabs(lo), std::fabs(hi));
+    const double ulp = 2.220446049250313e-16 * std::max(r, 1e-300);
+    if (warm == warm) {                                         // (not NaN)
+        const double top = std::min(hi, warm + 8 * ulp);
+        if (sturm_below(n, d, e, top) > k) {
+            hi = top;
+            for (double w = 1e-6 * r + ulp; hi - w > lo; w *= 8)
+                if (sturm_below(n, d, e, hi - w) <= k) { lo = hi - w; break; }
+        }
+    }
+    for (int it = 0; it < 200 && hi - lo > 2 * ulp; ++it) {
+        const double x = 0.5 * (lo + hi);
+        if (sturm_below(n, d, e, x) > k) hi = x; else lo = x;
+    }
+    const double th = 0.5 * (lo + hi);
+    warm = th;
+    // forward and backward pivots; twist element gamma_i = f_i + b_i - (d_i - theta)
+    std::vector<double> f(n), b(n);
+    for (int i = 0; i < n; ++i) {
+        f[i] = d[i] - th - (i ? e[i - 1] * (e[i - 1] / f[i - 1]) : 0.0);
+        if (f[i] == 0.0) f[i] = ulp;
+    }
+    for (int i = n - 1; i >= 0; --i) {
+        b[i] = d[i] - th - (i + 1 < n ? e[i] * (e[i] / b[i + 1]) : 0.0);
+        if (b[i] == 0.0) b[i] = ulp;
+    }
+    int at = 0;
+    double best = INFINITY;
+    for (int i = 0; i < n; ++i) {
+        const double g = std::fabs(f[i] + b[i] - (d[i] - th));
+        if (g < best) { best = g; at = i; }
+    }
+    double z = 1.0, sum = 1.0;
+    for (int i = at - 1; i >= 0; --i) { z *= -e[i] / f[i]; sum += z * z; }
+    z = 1.0;
+    for (int i = at + 1; i < n; ++i) { z *= -e[i - 1] / b[i]; sum += z * z; }
+    return beta * std::fabs(z) > tol * std::max(1.0, std::fabs(th)) * std::sqrt(sum);
+}
+
 }  // namespace cih
 
 extern "C" int cih_tridiag_eigen(int32_t n, const double *diag, const double *offdiag, double *evals,
