@@ -59,7 +59,8 @@ struct FillArgs {
     const double *t1;         // one-body table (OneBodyLayout) in place of the orbital energies, or null
 };
 
-// One set's table prepared for the fill (k_fill_prep), all in one allocation:
+// The tables of up to four sets prepared for the fill (k_fill_prep), all in one
+// allocation, every entry the KV values of the sets together (KV = 1, 2 or 4):
 //   sq      the pn groups as full squares: no ordering of the pair indices, and
 //           a proton move's entries for one neutron orbital are contiguous;
 //   hi, lo  per species and forward slot: a two-move's signed value (hi); a
@@ -72,6 +73,13 @@ struct FillWork {
     float *sq;
     float *hi[2], *lo[2];
     float2 *d[2];
+    int k0, ks;               // the sets k0 .. k0 + ks - 1, ks <= KV
+};
+
+// KV values of an entry, loaded and stored together
+template <int KV>
+struct alignas(4 * KV) Vals {
+    float v[KV];
 };
 // table index of t_ac for combined orbitals a, c (either order), -1 if they
 // are not one group of the one-body layout
@@ -144,6 +152,11 @@ constexpr int kLaneSets = 16;     // from this many sets on, multi-term sums run
 // us, 2,104 rows 26 / 23, 7,916 rows 37 / 41, 8,500 rows 35 / 45, 48,917 rows 113
 // / 167; at 4+4 Nmax=6 (2.2 M rows) a 1/15 share 600 / 1,130, 1/32 355 / 515, 1/64
 // 228 / 257, at 4+4 Nmax=4 a 1/17 share 55 / 59, 1/32 44 / 32.
+// Fills of fewer than kFillSets sets go through the working copy, one, two or four
+// sets a pass (three sets at 5+6 Nmax=4 with a one-body table: 2.91 ms, 6.57 ms
+// from the tables, where a one-move gathered ten entries per set and reduced them
+// in a tree).  From eight on the row kernel's element-major paths write whole lines.
+constexpr int kFillSets = 8;
 constexpr int64_t kPrepareShare = 24, kPrepareMin = 4096;
 constexpr int kSlowCap = 64;
 constexpr int kMaxA = 64;
@@ -485,8 +498,8 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
         nslow = 0;
         return;
     }
-    if constexpr (MODE == 1 && K1) {
-        // one set: an element's terms over the other species' particles (a lane
+    if (MODE == 1 && !EM && F.K < kFillSets) {
+        // few sets: an element's terms over the other species' particles (a lane
         // each, summed as a tree) and over its own species' spectators (loaded a
         // lane each, summed ascending after the one-body term): the sums of k_fill1
         const int Zp = B.nZ[0], Zn = B.nZ[1], gsz = term_lanes(Zp, Zn), per = 32 / gsz;
@@ -509,19 +522,23 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
                 status[2] = a | (c << 16);
                 status[3] = 2 | ((oko ? ks : ko) << 8);
             }
-            float to = 0.f, ts = 0.f;
-            if (ho && oko) { to = __ldg(F.tbme + xo); if (go < 0) to = -to; }
-            if (hs && oks) { ts = __ldg(F.tbme + xs); if (gs < 0) ts = -ts; }
-            const DF v = warp_sum(df_of(to), gsz);
-            DF own = act ? onebody_term(B, F, a, c, status) : df_of(0.f);
-            for (int x = 0; x < gsz; ++x) {
-                const float y = __shfl_sync(0xffffffffu, ts, x, gsz);
-                if (x < nown) own = df_add(own, df_of(y));
-            }
-            if (act && i == 0) {
-                const float r = df_round(df_add(v, own));
-                R.col[w_spos[e]] = w_scol[e];
-                R.val[w_spos[e]] = (code >> 16) & 1 ? -r : r;
+            const DF one = act ? onebody_term(B, F, a, c, status) : df_of(0.f);
+            for (int kk = 0; kk < (K1 ? 1 : F.K); ++kk) {
+                const float *tk = F.tbme + (int64_t)kk * F.tb_sk;
+                float to = 0.f, ts = 0.f;
+                if (ho && oko) { to = __ldg(tk + xo * F.tb_si); if (go < 0) to = -to; }
+                if (hs && oks) { ts = __ldg(tk + xs * F.tb_si); if (gs < 0) ts = -ts; }
+                const DF v = warp_sum(df_of(to), gsz);
+                DF own = one;
+                for (int x = 0; x < gsz; ++x) {
+                    const float y = __shfl_sync(0xffffffffu, ts, x, gsz);
+                    if (x < nown) own = df_add(own, df_of(y));
+                }
+                if (act && i == 0) {
+                    const float r = df_round(df_add(v, own));
+                    if (kk == 0) R.col[w_spos[e]] = w_scol[e];
+                    R.val[(int64_t)w_spos[e] * R.es + (int64_t)kk * R.ks] = (code >> 16) & 1 ? -r : r;
+                }
             }
         }
         __syncwarp();
@@ -724,31 +741,34 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
                 if (lane == 0 && rowlen > 0) R.col[0] = (int32_t)row;
                 __syncwarp();
             }
-            if constexpr (MODE == 1 && K1) {                 // the sums and their order of k_fill1
+            const bool split = MODE == 1 && !EM && F.K < kFillSets;
+            if (split) {                                     // the sums and their order of k_fill1
                 const int P = term_lanes(Zpro, Zneu), sub = lane / P, j = lane % P;
-                DF acc = df_of(0.f);
-                for (int i = sub; i < Zpro; i += 32 / P) {
-                    if (j >= Zneu) continue;
-                    const int a = w_occ[i], c = w_occ[Zpro + j];
-                    int64_t idx;
-                    int sg;
-                    if (tbme_at(B, lg, a, c, a, c, idx, sg)) {
-                        const float v = __ldg(F.tbme + idx * F.tb_si);
-                        acc = df_add(acc, df_of(sg < 0 ? -v : v));
-                    } else if (atomicOr(status, 1) == 0) {
-                        status[2] = a | (c << 16);
-                        status[3] = 1;
+                for (int k = 0; k < (K1 ? 1 : F.K); ++k) {
+                    DF acc = df_of(0.f);
+                    for (int i = sub; i < Zpro; i += 32 / P) {
+                        if (j >= Zneu) continue;
+                        const int a = w_occ[i], c = w_occ[Zpro + j];
+                        int64_t idx;
+                        int sg;
+                        if (tbme_at(B, lg, a, c, a, c, idx, sg)) {
+                            const float v = __ldg(F.tbme + (int64_t)k * F.tb_sk + idx * F.tb_si);
+                            acc = df_add(acc, df_of(sg < 0 ? -v : v));
+                        } else if (atomicOr(status, 1) == 0) {
+                            status[2] = a | (c << 16);
+                            status[3] = 1;
+                        }
+                    }
+                    acc = warp_sum(acc, 32);
+                    const DF dp = diag_own(B, lg, F, k, Zpro, [&](int i) { return (int)w_occ[i]; }, status);
+                    const DF dn = diag_own(B, lg, F, k, Zneu, [&](int i) { return (int)w_occ[Zpro + i]; }, status);
+                    if (lane == 0 && rowlen > 0) {
+                        if (k == 0) R.col[0] = (int32_t)row;
+                        R.val[(int64_t)k * R.ks] = df_round(df_add(acc, df_add(dp, dn)));
                     }
                 }
-                acc = warp_sum(acc, 32);
-                const DF dp = diag_own(B, lg, F, 0, Zpro, [&](int i) { return (int)w_occ[i]; }, status);
-                const DF dn = diag_own(B, lg, F, 0, Zneu, [&](int i) { return (int)w_occ[Zpro + i]; }, status);
-                if (lane == 0 && rowlen > 0) {
-                    R.col[0] = (int32_t)row;
-                    R.val[0] = df_round(df_add(acc, df_add(dp, dn)));
-                }
             }
-            for (int k = 0; k < (kset || (MODE == 1 && K1) ? 0 : K1 ? 1 : MODE == 1 ? F.K : Gr.K); ++k) {
+            for (int k = 0; k < (kset || split ? 0 : K1 ? 1 : MODE == 1 ? F.K : Gr.K); ++k) {
                 DF acc = df_of(0.f);
                 for (int l = lane; l < npairs; l += 32) {
                     const int a = w_occ[pi[l]], c = w_occ[pj[l]];
@@ -934,63 +954,79 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
     }
 }
 
-// The working copy of one set's table (FillWork): warps over the rows of the pn
+// The working copy of the tables (FillWork): warps over the rows of the pn
 // squares, then over the sub-dets of both species.  Bound by its scattered
-// reads of the table (L2); it replaces two to seven of them, and the pair
+// reads of the tables (L2); it replaces two to seven of them, and the pair
 // lookups, per element of that kind in every row.
+template <int KV>
 __global__ void __launch_bounds__(256) k_fill_prep(DevBasis B, FillArgs F, FillWork W, int *status)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t n0 = B.n_sqrow, n1 = n0 + B.sp[0].n_sd, n2 = n1 + B.sp[1].n_sd;
+    auto entry = [&](int64_t idx, bool neg) {                  // the sets' values (a set past the last repeats it)
+        Vals<KV> r;
+#pragma unroll
+        for (int u = 0; u < KV; ++u) {
+            const float v = __ldg(F.tbme + (int64_t)(W.k0 + min(u, W.ks - 1)) * F.tb_sk + idx * F.tb_si);
+            r.v[u] = neg ? -v : v;
+        }
+        return r;
+    };
     for (int64_t t = warp; t < n2; t += nw) {
         if (t < n0) {
             const int r = B.sqrow[t], k = r >> 16, u = r & 0xFFFF;
             const int2 g = B.pn_k[k];
             const int n = g.y;
-            float *out = W.sq + B.pn_kq[k].x + (int64_t)u * n;
+            Vals<KV> *out = reinterpret_cast<Vals<KV> *>(W.sq) + B.pn_kq[k].x + (int64_t)u * n;
             for (int v = lane; v < n; v += 32) {
                 const int lo = min(u, v), hi = max(u, v);
-                out[v] = __ldg(F.tbme + g.x + lo * n - ((lo * (lo - 1)) >> 1) + (hi - lo));
+                out[v] = entry(g.x + lo * n - ((lo * (lo - 1)) >> 1) + (hi - lo), false);
             }
             continue;
         }
         const int s = t < n1 ? 0 : 1;
         const DevSpecies S = s ? B.sp[1] : B.sp[0];
-        float *hi = s ? W.hi[1] : W.hi[0], *lo = s ? W.lo[1] : W.lo[0];
+        Vals<KV> *hi = reinterpret_cast<Vals<KV> *>(s ? W.hi[1] : W.hi[0]), *lo = reinterpret_cast<Vals<KV> *>(s ? W.lo[1] : W.lo[0]);
         float2 *dg = s ? W.d[1] : W.d[0];
         const int64_t x = t - (s ? n1 : n0), f0 = S.fw_off[x];
         const int Z = s ? B.nZ[1] : B.nZ[0], len = (int)(S.fw_off[x + 1] - f0), two = S.fw_lev[x * S.NL + S.NL - 1];
         const uint8_t *occ = (s ? B.occ[1] : B.occ[0]) + x * Z;
-        const DF d = diag_own(B, nullptr, F, 0, Z, [&](int i) { return S.orb_base + (int)occ[i]; }, status);
-        if (lane == 0) dg[x] = make_float2(d.hi, d.lo);
+        for (int u = 0; u < W.ks; ++u) {
+            const DF d = diag_own(B, nullptr, F, W.k0 + u, Z, [&](int i) { return S.orb_base + (int)occ[i]; }, status);
+            if (lane == 0) dg[x * KV + u] = make_float2(d.hi, d.lo);
+        }
         for (int i = lane; i < two; i += 32) {
             const int tb = S.fw_tb[f0 + i];
-            const float v = __ldg(F.tbme + (tb >> 1));
-            hi[f0 + i] = tb & 1 ? -v : v;
+            hi[f0 + i] = entry(tb >> 1, tb & 1);
         }
         for (int i = two + lane; i < len; i += 32) {
             const int code = ~S.fw_tb[f0 + i];
             const int a = S.orb_base + (code & 0xFF), c = S.orb_base + ((code >> 8) & 0xFF);
-            DF own = onebody_term(B, F, a, c, status);
+            const DF one = onebody_term(B, F, a, c, status);
+            DF own[KV];
+#pragma unroll
+            for (int u = 0; u < KV; ++u) own[u] = one;
             for (int j = 0; j < Z; ++j) {
                 const int k = S.orb_base + (int)occ[j];
                 if (k == a) continue;
                 int64_t idx;
                 int sg;
-                float v = 0.f;
                 if (tbme_at(B, nullptr, a, k, c, k, idx, sg)) {
-                    v = __ldg(F.tbme + idx);
-                    if (sg < 0) v = -v;
+                    const Vals<KV> v = entry(idx, sg < 0);
+#pragma unroll
+                    for (int u = 0; u < KV; ++u) own[u] = df_add(own[u], df_of(v.v[u]));
                 } else if (atomicOr(status, 1) == 0) {
                     status[2] = a | (c << 16);
                     status[3] = 2 | (k << 8);
                 }
-                own = df_add(own, df_of(v));
             }
-            hi[f0 + i] = own.hi;
-            lo[f0 + i] = own.lo;
+            Vals<KV> h, l;
+#pragma unroll
+            for (int u = 0; u < KV; ++u) { h.v[u] = own[u].hi; l.v[u] = own[u].lo; }
+            hi[f0 + i] = h;
+            lo[f0 + i] = l;
         }
     }
 }
@@ -1009,17 +1045,36 @@ template <int WARPS>
 constexpr int S = warp0 + WARPS * w_size;
 }  // namespace f1
 
+// read-only load of an entry, all its bytes at once
+template <class T>
+__device__ __forceinline__ T ld(const T *p)
+{
+    T r;
+    if constexpr (sizeof(T) == 4) {
+        const int x = __ldg(reinterpret_cast<const int *>(p));
+        memcpy(&r, &x, 4);
+    } else if constexpr (sizeof(T) == 8) {
+        const int2 x = __ldg(reinterpret_cast<const int2 *>(p));
+        memcpy(&r, &x, 8);
+    } else {
+        static_assert(sizeof(T) == 16, "4, 8 or 16 bytes");
+        const int4 x = __ldg(reinterpret_cast<const int4 *>(p));
+        memcpy(&r, &x, 16);
+    }
+    return r;
+}
+
 // entry at a 32-bit byte offset from a kernel argument (arrays below 4 GiB:
 // one address register instead of two, no 64-bit address arithmetic)
 template <class T>
 __device__ __forceinline__ T at_byte(const void *base, unsigned off)
 {
-    return __ldg(reinterpret_cast<const T *>(reinterpret_cast<const char *>(base) + off));
+    return ld(reinterpret_cast<const T *>(reinterpret_cast<const char *>(base) + off));
 }
 
 constexpr int kW = 2;             // pn windows of 32 elements in flight in k_fill1
 
-// The fill of one set from its working copy: the walk of k_rows, every element
+// The fill of up to KV sets from their working copy: the walk of k_rows, every element
 // one read of a value (two-moves: contiguous; pn: one gather from the squares),
 // one-moves and the diagonal the prepared own-species sum plus the terms over
 // the other species.  Reading the table itself in every row (pair lookups, a
@@ -1028,7 +1083,7 @@ constexpr int kW = 2;             // pn windows of 32 elements in flight in k_fi
 // 5.6 warp instructions per stored nonzero (64 % of the issue slots; 10.9 before
 // the groups); the pn loop is 60 % of the time, waiting on L2 for the members,
 // moves and values of its windows.
-template <int WARPS>
+template <int WARPS, int KV>
 __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
 k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, int64_t r1, int *status)
 {
@@ -1049,6 +1104,24 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
     int4 *w_seg = sptr<int4>(wb, f1::w_seg), *w_lev = sptr<int4>(wb, f1::w_lev);
     int2 *w_ext = sptr<int2>(wb, f1::w_ext);
     int *w_op = sptr<int>(wb, f1::w_op), *w_on = sptr<int>(wb, f1::w_on);
+    constexpr int NW = KV == 1 ? kW : 1;                        // windows in flight
+    const int64_t es = F.em ? F.K : 1, kst = F.em ? 1 : nnz;    // value of set k at row position e: val[e * es + k * kst]
+    const Vals<KV> *sq = reinterpret_cast<const Vals<KV> *>(W.sq);
+    const bool cols = W.k0 == 0;                                // (a later pass of the same fill leaves the columns)
+    auto put = [&](int32_t *col, float *val, int e, int c, const Vals<KV> &v, bool neg) {
+        if (cols) __stcs(col + e, c);
+        const int sm = neg ? (int)0x80000000 : 0;
+        if (KV == 4 && F.vec4 && F.em) {                        // four sets, element-major: one store
+            const float4 r = make_float4(__int_as_float(__float_as_int(v.v[0]) ^ sm), __int_as_float(__float_as_int(v.v[KV > 1 ? 1 : 0]) ^ sm),
+                                         __int_as_float(__float_as_int(v.v[KV > 2 ? 2 : 0]) ^ sm),
+                                         __int_as_float(__float_as_int(v.v[KV > 2 ? 3 : 0]) ^ sm));
+            __stcs(reinterpret_cast<float4 *>(val + (int64_t)e * es), r);
+            return;
+        }
+#pragma unroll
+        for (int u = 0; u < KV; ++u)
+            if (KV == 1 || u < W.ks) __stcs(val + e * es + u * kst, __int_as_float(__float_as_int(v.v[u]) ^ sm));
+    };
     const int P = term_lanes(Zp, Zn), sub = lane / P, li = lane % P, per = 32 / P;
     const int64_t gw = (blockIdx.x * (int64_t)kThreads + tid) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * kThreads) >> 5;
@@ -1061,7 +1134,7 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
         const int64_t e0 = rowptr[row] - sbase;
         const int rowlen = (int)(min(rowptr[row + 1] - sbase, nnz) - e0);
         int32_t *col = F.col + e0;
-        float *val = F.val + e0;
+        float *val = F.val + e0 * es + W.k0 * kst;
         const int16_t *dirn = B.dir + (int64_t)n * B.dir_len;
         const int cA1 = max(0, dirn[PR.dirA] - NR.self), cA2 = SN.fw_lev[(int64_t)n * SN.NL + PR.levA];
         int pos = 1 + cA1 + cA2;
@@ -1072,30 +1145,35 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
         if (lane < Zp) w_op[lane] = B.occ_code[0][(int64_t)p * Zp + lane];
         if (lane < Zn) w_on[lane] = B.occ_code[1][(int64_t)n * Zn + lane];
         const int2 *recn = SN.fw_rec + NR.fw, *recp = SP.fw_rec + PR.fw;
-        const float *vn = W.hi[1] + NR.fw, *vp = W.hi[0] + PR.fw;
+        const Vals<KV> *vn = reinterpret_cast<const Vals<KV> *>(W.hi[1]) + NR.fw, *vp = reinterpret_cast<const Vals<KV> *>(W.hi[0]) + PR.fw;
         const int2 *n1row = B.n1p + NR.n1, *l1row = B.l1 + PR.l1;
         const unsigned l1o = (unsigned)PR.l1 * 8u, n1o = (unsigned)NR.n1 * 8u, fpo = (unsigned)(PR.fw + PR.fwlen) * 8u;
         __syncwarp();
 
         // diagonal
         {
-            DF acc = df_of(0.f);
+            DF acc[KV];
+#pragma unroll
+            for (int u = 0; u < KV; ++u) acc[u] = df_of(0.f);
             for (int i = sub; i < Zp; i += per)
-                if (li < Zn) acc = df_add(acc, df_of(__ldg(W.sq + pn_square_at(KQ, S, T, w_op[i], w_on[li]))));
-            acc = warp_sum(acc, 32);
-            if (lane == 0) {
-                const float2 dp = W.d[0][p], dn = W.d[1][n];
-                __stcs(col, (int32_t)row);
-                __stcs(val, df_round(df_add(acc, df_add(DF{dp.x, dp.y}, DF{dn.x, dn.y}))));
+                if (li < Zn) {
+                    const Vals<KV> v = ld(sq + pn_square_at(KQ, S, T, w_op[i], w_on[li]));
+#pragma unroll
+                    for (int u = 0; u < KV; ++u) acc[u] = df_add(acc[u], df_of(v.v[u]));
+                }
+            Vals<KV> r;
+#pragma unroll
+            for (int u = 0; u < KV; ++u) {
+                acc[u] = warp_sum(acc[u], 32);
+                const float2 dp = W.d[0][(int64_t)p * KV + u], dn = W.d[1][(int64_t)n * KV + u];
+                r.v[u] = df_round(df_add(acc[u], df_add(DF{dp.x, dp.y}, DF{dn.x, dn.y})));
             }
+            if (lane == 0) put(col, val, 0, (int32_t)row, r, false);
         }
         // A: neutron two-moves
         for (int t = lane; t < cA2; t += 32) {
-            const int2 rc = recn[t];
-            const float v = vn[t];
-            const int e = 1 + t + (rc.y & 0xFFFFFF);
-            __stcs(col + e, PR.colb + rc.x);
-            __stcs(val + e, v);
+            const int2 rc = ld(recn + t);
+            put(col, val, 1 + t + (rc.y & 0xFFFFFF), PR.colb + rc.x, ld(vn + t), false);
         }
         // B: p's groups, a lane each
         int c1 = 0;                                             // proton one-moves with n kept
@@ -1133,23 +1211,20 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
             }
             __syncwarp();
             for (int t = lane; t < c2; t += 32) {               // pp two-moves: a prefix of p's list
-                const int2 rc = recp[t];
-                const float v = vp[t];
+                const int2 rc = ld(recp + t);
                 const int4 lv = w_lev[rc.y >> 24];
-                const int e = lv.x + t + (rc.y & 0xFFFFFF) * lv.y;
-                __stcs(col + e, rc.x + n);
-                __stcs(val + e, v);
+                put(col, val, lv.x + t + (rc.y & 0xFFFFFF) * lv.y, rc.x + n, ld(vp + t), false);
             }
             // pn elements of all groups, flattened as in k_rows, kW windows of 32
             // at a time so that their chains of loads (member and neutron move, then
             // the value) overlap; lanes past the end repeat the last element's loads
             const unsigned le = (2u << lane) - 1u;                 // bits 0..lane
             int before = -1;                                       // pn groups started before the window, less one
-            for (int w0 = 0; w0 < Tpn; w0 += 32 * kW) {
-                int2 q[kW], ent[kW];
-                int at[kW];
+            for (int w0 = 0; w0 < Tpn; w0 += 32 * NW) {
+                int2 q[NW], ent[NW];
+                int at[NW];
 #pragma unroll
-                for (int u = 0; u < kW; ++u) {
+                for (int u = 0; u < NW; ++u) {
                     const int w = w0 + 32 * u;
                     const unsigned mk = __reduce_or_sync(0xffffffffu, npn > 0 && (unsigned)(st - w) < 32u ? 1u << (st - w) : 0u);
                     const int j = before + __popc(mk & le), e = min(w + lane, Tpn - 1);
@@ -1167,14 +1242,14 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
                         at[u] = sg4.w + i1 * (ln + 1) + (at_byte<int2>(SP.fw_rec, fpo - 8 - i1 * 8).y & 0xFFFFFF) + k +
                                 (k >= sx.y ? 1 : 0);
                 }
-                float v[kW];
+                Vals<KV> v[NW];
 #pragma unroll
-                for (int u = 0; u < kW; ++u) v[u] = at_byte<float>(W.sq, (unsigned)pn_square_at(KQ, S, T, q[u].y, ent[u].y) * 4u);
+                for (int u = 0; u < NW; ++u)
+                    v[u] = at_byte<Vals<KV>>(W.sq, (unsigned)pn_square_at(KQ, S, T, q[u].y, ent[u].y) * (4u * KV));
 #pragma unroll
-                for (int u = 0; u < kW; ++u) {
+                for (int u = 0; u < NW; ++u) {
                     if (w0 + 32 * u + lane >= Tpn) continue;
-                    __stcs(col + at[u], q[u].x + ent[u].x);
-                    __stcs(val + at[u], __int_as_float(__float_as_int(v[u]) ^ (((q[u].y << 15) ^ (ent[u].y << 5)) & 0x80000000)));
+                    put(col, val, at[u], q[u].x + ent[u].x, v[u], ((q[u].y >> 16) ^ (ent[u].y >> 26)) & 1);
                 }
             }
             __syncwarp();
@@ -1208,15 +1283,19 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
                 if (li < Zn) nc = w_on[li];
             }
             const bool has = act && li < (neu ? Zp : Zn);
-            float v = 0.f;
-            if (has) v = __ldg(W.sq + pn_square_at(KQ, S, T, lc, nc));
-            const DF sum = warp_sum(df_of(v), P);
+            Vals<KV> v{};
+            if (has) v = ld(sq + pn_square_at(KQ, S, T, lc, nc));
+            DF sum[KV];
+#pragma unroll
+            for (int u = 0; u < KV; ++u) sum[u] = warp_sum(df_of(v.v[u]), P);
             if (act && li == 0) {
                 slot += neu ? NR.fw : PR.fw;
-                const DF own{(neu ? W.hi[1] : W.hi[0])[slot], (neu ? W.lo[1] : W.lo[0])[slot]};
-                const float r = df_round(df_add(sum, own));
-                __stcs(col + e, j);
-                __stcs(val + e, sgn ? -r : r);
+                const Vals<KV> h = ld(reinterpret_cast<const Vals<KV> *>(neu ? W.hi[1] : W.hi[0]) + slot),
+                               l = ld(reinterpret_cast<const Vals<KV> *>(neu ? W.lo[1] : W.lo[0]) + slot);
+                Vals<KV> r;
+#pragma unroll
+                for (int u = 0; u < KV; ++u) r.v[u] = df_round(df_add(sum[u], DF{h.v[u], l.v[u]}));
+                put(col, val, e, j, r, sgn);
             }
         }
         __syncwarp();
@@ -1305,7 +1384,7 @@ int launch_rows_w(const cih_basis &b, const int64_t *rowptr, int64_t *counts, co
     };
     const bool k1 = (MODE == 1 && F.K == 1) || (MODE == 2 && G.K == 1);   // one set / one vector
     const int L4 = F.K >> 2;
-    const bool em = MODE == 1 && !k1 && F.em && F.vec4 && (L4 > 32 ? L4 % 32 == 0 : 32 % L4 == 0);
+    const bool em = MODE == 1 && F.K >= kFillSets && F.em && F.vec4 && (L4 > 32 ? L4 % 32 == 0 : 32 % L4 == 0);
     if constexpr (MODE == 1) {
         // element-major K sets: warp-cooperative writes; 64 is the batched configuration's set count
         if (em) return F.K == 64 ? go(k_rows<MODE, false, WARPS, 64>) : go(k_rows<MODE, false, WARPS, 1>);
@@ -1372,57 +1451,87 @@ int launch_scan(const cih_basis &b, int64_t *rowptr, cudaStream_t st)
 
 namespace {
 
-// layout of the working copy: the pair arrays first (8-byte aligned)
-FillWork work_at(const cih_basis &b, float *p)
+// Layout of the working copy of kv sets: the squares, the slots, then the pairs of
+// the diagonal, each at a multiple of 16 bytes.
+size_t work_floats(const cih_basis &b, int kv)
 {
+    auto up = [](int64_t n) { return (n + 3) / 4 * 4; };
+    return (size_t)(up(b.sq_total * kv) + 2 * up(b.fw_total[0] * kv) + 2 * up(b.fw_total[1] * kv) +
+                    up(2 * b.s[0].n_sd * kv) + up(2 * b.s[1].n_sd * kv));
+}
+
+FillWork work_at(const cih_basis &b, float *p, int kv, int k0, int ks)
+{
+    auto take = [&](int64_t n) { float *q = p; p += (n + 3) / 4 * 4; return q; };
     FillWork w;
+    w.sq = take(b.sq_total * kv);
     for (int s = 0; s < 2; ++s) {
-        w.d[s] = reinterpret_cast<float2 *>(p);
-        p += 2 * b.s[s].n_sd;
+        w.hi[s] = take(b.fw_total[s] * kv);
+        w.lo[s] = take(b.fw_total[s] * kv);
     }
-    for (int s = 0; s < 2; ++s) {
-        w.hi[s] = p;
-        w.lo[s] = p + b.fw_total[s];
-        p += 2 * b.fw_total[s];
-    }
-    w.sq = p;
+    for (int s = 0; s < 2; ++s) w.d[s] = reinterpret_cast<float2 *>(take(2 * b.s[s].n_sd * kv));
+    w.k0 = k0;
+    w.ks = ks;
     return w;
 }
 
-template <int WARPS>
-int launch_fill1(const cih_basis &b, const int64_t *rowptr, const FillArgs &F, const FillWork &W, cudaStream_t st, bool dry,
-                 int64_t r0, int64_t r1)
+// k_fill1 takes 32-bit byte offsets and keeps at most 32 particles of a species
+bool fill1_fits(const cih_basis &b, int kv)
+{
+    const int64_t most = (int64_t)1 << 32;
+    for (int s = 0; s < 2; ++s)
+        if (b.fw_total[s] * 8 >= most || b.n1_total[s] * 8 >= most) return false;
+    return b.sq_total * 4 * kv < most && b.dev.A - 1 <= 32 && b.dev.nZ[0] <= 32 && b.dev.nZ[1] <= 32 && b.dim > 0;
+}
+
+template <int WARPS, int KV>
+int launch_fill1_w(const cih_basis &b, const int64_t *rowptr, const FillArgs &F, const FillWork &W, cudaStream_t st, bool dry,
+                   int64_t r0, int64_t r1)
 {
     const size_t smem = (size_t)f1::S<WARPS> + ((size_t)b.dev.sp[0].n_orb * b.dev.pn_T * 2 + 15) / 16 * 16;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e = raise_smem_limit((const void *)k_fill1<WARPS>, dev, (int)smem);
+    cudaError_t e = raise_smem_limit((const void *)k_fill1<WARPS, KV>, dev, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "fill shared memory");
     if (dry) return CIH_OK;
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fill1<WARPS>, WARPS * 32, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fill1<WARPS, KV>, WARPS * 32, smem);
     per_sm = std::max(per_sm, 1);
     if (b.launch_ctas > 0) per_sm = std::min(per_sm, b.launch_ctas);
     const int64_t want = (r1 - r0 + WARPS - 1) / WARPS;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm, want));
     count_launches(1);
-    k_fill1<WARPS><<<grid, WARPS * 32, smem, st>>>(b.dev, rowptr, F, W, r0, r1, b.dev_status);
+    k_fill1<WARPS, KV><<<grid, WARPS * 32, smem, st>>>(b.dev, rowptr, F, W, r0, r1, b.dev_status);
     e = cudaGetLastError();
     return e == cudaSuccess ? CIH_OK : cuda_fail(e, "fill launch");
 }
 
+int launch_fill1(const cih_basis &b, int kv, const int64_t *rowptr, const FillArgs &F, const FillWork &W, cudaStream_t st, bool dry,
+                 int64_t r0, int64_t r1)
+{
+    if (b.launch_warps == 8)
+        return kv == 1 ? launch_fill1_w<8, 1>(b, rowptr, F, W, st, dry, r0, r1)
+             : kv == 2 ? launch_fill1_w<8, 2>(b, rowptr, F, W, st, dry, r0, r1) : launch_fill1_w<8, 4>(b, rowptr, F, W, st, dry, r0, r1);
+    return kv == 1 ? launch_fill1_w<16, 1>(b, rowptr, F, W, st, dry, r0, r1)
+         : kv == 2 ? launch_fill1_w<16, 2>(b, rowptr, F, W, st, dry, r0, r1) : launch_fill1_w<16, 4>(b, rowptr, F, W, st, dry, r0, r1);
+}
+
+int launch_prep(const cih_basis &b, int kv, const FillArgs &F, const FillWork &W, cudaStream_t st)
+{
+    const int64_t warps = b.dev.n_sqrow + b.s[0].n_sd + b.s[1].n_sd;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8, 152 * 16));
+    count_launches(1);
+    if (kv == 1) k_fill_prep<1><<<grid, 256, 0, st>>>(b.dev, F, W, b.dev_status);
+    else if (kv == 2) k_fill_prep<2><<<grid, 256, 0, st>>>(b.dev, F, W, b.dev_status);
+    else k_fill_prep<4><<<grid, 256, 0, st>>>(b.dev, F, W, b.dev_status);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? CIH_OK : cuda_fail(e, "fill preparation");
+}
+
 }  // namespace
 
-size_t fill_work_floats(const cih_basis &b)
-{
-    // k_fill1 takes 32-bit byte offsets and keeps at most 32 particles of a species
-    const int64_t most = (int64_t)1 << 32;
-    for (int s = 0; s < 2; ++s)
-        if (b.fw_total[s] * 8 >= most || b.n1_total[s] * 8 >= most) return 0;
-    if (b.sq_total * 4 >= most || b.dev.A - 1 > 32 || b.dev.nZ[0] > 32 || b.dev.nZ[1] > 32 || b.dim == 0) return 0;
-    return (size_t)(2 * (b.s[0].n_sd + b.s[1].n_sd) + 2 * (b.fw_total[0] + b.fw_total[1]) + b.sq_total);
-}
+size_t fill_work_floats(const cih_basis &b) { return fill1_fits(b, 1) ? work_floats(b, 1) : 0; }
 
 int fill_prepare(const cih_basis &b, double hw, const float *tbme, const double *esp, const double *t1, float *work,
                  cudaStream_t st)
@@ -1435,12 +1544,7 @@ int fill_prepare(const cih_basis &b, double hw, const float *tbme, const double 
     F.tb_si = 1;
     F.esp = esp;
     F.t1 = t1;
-    const int64_t warps = b.dev.n_sqrow + b.s[0].n_sd + b.s[1].n_sd;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8, 152 * 16));
-    count_launches(1);
-    k_fill_prep<<<grid, 256, 0, st>>>(b.dev, F, work_at(b, work), b.dev_status);
-    const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? CIH_OK : cuda_fail(e, "fill preparation");
+    return launch_prep(b, 1, F, work_at(b, work, 1, 0, 1), st);
 }
 
 int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, const float *tbme, bool interleaved,
@@ -1451,28 +1555,25 @@ int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, con
     FillArgs F{K, hw, tbme, interleaved ? 1 : b.layout.total, interleaved ? (int64_t)K : 1, vec4, em && K > 1 ? 1 : 0,
                esp, col, val, sharded ? 1 : 0, r0, t1};
     const int64_t rend = r1 < 0 ? b.dim : r1;
-    float *own = nullptr;
-    if (K == 1 && !work && prepare && rend - r0 >= kPrepareMin && (rend - r0) * kPrepareShare >= b.dim) {
-        const size_t n = fill_work_floats(b);
-        if (n > 0 && cudaMallocFromPoolAsync((void **)&own, n * sizeof(float), b.pool, st) != cudaSuccess) {
-            (void)cudaGetLastError();
-            own = nullptr;
+    if (K == 1 && work && b.dim > 0 && rend > r0)
+        return launch_fill1(b, 1, rowptr, F, work_at(b, const_cast<float *>(work), 1, 0, 1), st, false, r0, rend);
+    const int kv = K == 1 ? 1 : K == 2 ? 2 : 4;                // sets of one pass
+    if (K < kFillSets && !work && prepare && rend - r0 >= kPrepareMin && (rend - r0) * kPrepareShare >= b.dim && fill1_fits(b, kv)) {
+        float *own = nullptr;
+        if (cudaMallocFromPoolAsync((void **)&own, work_floats(b, kv) * sizeof(float), b.pool, st) == cudaSuccess) {
+            int rc = CIH_OK;
+            for (int k0 = 0; k0 < K && !rc; k0 += kv) {
+                const int ks = std::min(kv, K - k0), v = ks == 1 ? 1 : ks == 2 ? 2 : 4;
+                const FillWork W = work_at(b, own, v, k0, ks);
+                rc = launch_prep(b, v, F, W, st);
+                if (!rc) rc = launch_fill1(b, v, rowptr, F, W, st, false, r0, rend);
+            }
+            cudaFreeAsync(own, st);
+            return rc;
         }
-        if (own) {
-            const int rc = fill_prepare(b, hw, tbme, esp, t1, own, st);
-            if (rc) { cudaFreeAsync(own, st); return rc; }
-            work = own;
-        }
+        (void)cudaGetLastError();
     }
-    if (K != 1 || !work) return launch_rows<1>(b, rowptr, nullptr, F, GradArgs{}, st, false, r0, r1);
-    int rc = CIH_OK;
-    if (b.dim > 0 && rend > r0) {
-        const FillWork W = work_at(b, const_cast<float *>(work));
-        rc = b.launch_warps == 8 ? launch_fill1<8>(b, rowptr, F, W, st, false, r0, rend)
-                                 : launch_fill1<16>(b, rowptr, F, W, st, false, r0, rend);
-    }
-    if (own) cudaFreeAsync(own, st);
-    return rc;
+    return launch_rows<1>(b, rowptr, nullptr, F, GradArgs{}, st, false, r0, r1);
 }
 
 int prepare_rows(const cih_basis &b, int K)
@@ -1484,9 +1585,7 @@ int prepare_rows(const cih_basis &b, int K)
     int rc = launch_rows<0>(b, nullptr, nullptr, F, G, nullptr, true);
     if (!rc) rc = launch_rows<1>(b, nullptr, nullptr, F, G, nullptr, true);
     if (!rc) rc = launch_rows<2>(b, nullptr, nullptr, F, G, nullptr, true);
-    if (!rc && K == 1 && fill_work_floats(b) > 0)
-        rc = b.launch_warps == 8 ? launch_fill1<8>(b, nullptr, F, FillWork{}, nullptr, true, 0, 0)
-                                 : launch_fill1<16>(b, nullptr, F, FillWork{}, nullptr, true, 0, 0);
+    if (!rc && K == 1 && fill_work_floats(b) > 0) rc = launch_fill1(b, 1, nullptr, F, FillWork{}, nullptr, true, 0, 0);
     return rc;
 }
 

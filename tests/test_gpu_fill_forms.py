@@ -60,6 +60,32 @@ def test_prepared_fill(cih, space, energies):
     assert np.all(np.abs(got - val_o) <= 1e-5 * (np.abs(val_o) + 1.0))
 
 
+@pytest.mark.parametrize("space", [(3, 3, 2, 0), (4, 4, 2, 0), (2, 6, 3, 4), (4, 0, 6, 0)])
+@pytest.mark.parametrize("K", [2, 3, 4, 5, 7])
+def test_few_sets(cih, space, K):
+    """Fewer than eight sets: passes of up to four sets through the working copy.
+    Each set has the bits of its own one-set fill, in every layout and from
+    shards of a few rows."""
+    B = cih.Basis(*space)
+    T = torch.from_numpy(synth.tbme_tables(B.tbme_len, range(K))).cuda()
+    e = torch.from_numpy(synth.single_particle_energies(sum(B.n_orb), 3)).cuda()
+    rowptr, nnz = B.count()
+    col, val = B.fill(rowptr, nnz, T, e_sp=e)
+    for k in range(K):
+        c1, v1 = B.fill(rowptr, nnz, T[k], e_sp=e)
+        assert torch.equal(c1, col) and torch.equal(v1[0], val[k])
+    til = cih.tbme_interleave(T)
+    c2, v2 = B.fill_interleaved(rowptr, nnz, til, K, e_sp=e)
+    c3, v3 = B.fill_batched(rowptr, nnz, til, K, e_sp=e)
+    assert torch.equal(c2, col) and torch.equal(v2, val)
+    assert torch.equal(c3, col) and torch.equal(v3.t(), val)
+    step = max(1, B.dim // 30)
+    parts = [B.fill_rows(rowptr, r, min(B.dim, r + step), T, e_sp=e) for r in range(0, B.dim, step)]
+    assert torch.equal(torch.cat([c for c, _ in parts]), col)
+    assert torch.equal(torch.cat([v for _, v in parts], dim=1), val)
+    B.check()
+
+
 def test_prepared_fill_in_a_graph(cih):
     """The working copy of a captured fill belongs to the graph: replays read the
     table anew."""
