@@ -16,6 +16,14 @@ namespace cih {
 
 constexpr int kMaxWords = 4;              // <= 256 orbitals per species
 constexpr int kLevels = 8;                // oscillator levels of a species: Nmax <= 7 with 256 orbitals
+// Walk order of the one-set kernels: the rows of up to kWalkRun proton sub-dets
+// with the same neutron range side by side, so that the warps of a CTA read one
+// neutron's lists together instead of each its own from L2.  Fill at 4+4 Nmax=6
+// 7.00 -> 5.77 ms (8 sub-dets: 6.03), 5+6 Nmax=4 1.87 -> 1.81; where the lists of the
+// rows in flight are in L2 anyway it gains nothing (48,917 rows 117 -> 127 us), hence
+// the least number of rows.
+constexpr int kWalkRun = 16;
+constexpr int64_t kWalkRows = 1 << 19;
 constexpr uint64_t kPoolKeep = 1ull << 30; // bytes the library pool keeps after a Lanczos call
 constexpr int kSortTile = 4096;           // longest neighbour list the sort handles
 
@@ -86,6 +94,7 @@ struct DevBasis {
     int32_t A;                 // particles
     int32_t nZ[2];             // particles per species
     const int32_t *row_p;      // row -> proton sub-det
+    const int2 *walk;          // place in the walk of the one-set kernels -> (proton sub-det, row), or null: row order
     const ProtonRec *prec;
     const NeutronRec *nrec;
     // Groups of p's later one-moves q > p with equal (class, N): every member

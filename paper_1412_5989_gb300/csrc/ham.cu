@@ -1126,8 +1126,11 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
     const int64_t gw = (blockIdx.x * (int64_t)kThreads + tid) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * kThreads) >> 5;
 
-    for (int64_t row = r0 + gw; row < r1; row += nw) {
-        const int p = B.row_p[row];
+    const bool walk = B.walk && r0 == 0 && r1 == B.dim;         // (a range of rows is taken in row order)
+    for (int64_t place = r0 + gw; place < r1; place += nw) {
+        const int2 at_row = walk ? B.walk[place] : make_int2(B.row_p[place], (int)place);
+        const int p = at_row.x;
+        const int64_t row = at_row.y;
         const ProtonRec PR = B.prec[p];
         const int n = (int)(row - PR.colb);
         const NeutronRec NR = B.nrec[n];

@@ -379,13 +379,24 @@ __global__ void k_neutron_rec(DevSpecies SN, NeutronRec *rec)
         rec[n] = NeutronRec{SN.n1_off[n], SN.fw_off[n], (int32_t)(SN.fw_off[n + 1] - SN.fw_off[n]), SN.n1_self[n], SN.N[n], 0};
 }
 
-__global__ void k_row_p(int64_t np, const int64_t *rowbase, int32_t *row_p)
+// row -> proton sub-det, and (walk not null) the order the one-set kernels take
+// the rows in: inside each aligned run of kWalkRun proton sub-dets those with the
+// same neutron range go side by side, n by n.  One warp per p.
+__global__ void k_row_p(int64_t np, const int64_t *rowbase, const int32_t *nb, const int32_t *nc, int32_t *row_p, int2 *walk)
 {
     int lane = threadIdx.x & 31;
     int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t p = warp; p < np; p += nwarps)
-        for (int64_t r = rowbase[p] + lane; r < rowbase[p + 1]; r += 32) row_p[r] = (int32_t)p;
+    for (int64_t p = warp; p < np; p += nwarps) {
+        const int64_t r0 = rowbase[p], r1 = rowbase[p + 1];
+        for (int64_t r = r0 + lane; r < r1; r += 32) row_p[r] = (int32_t)p;
+        if (!walk) continue;
+        int64_t g0 = p, g1 = p + 1;                            // p's neighbours in the run with its range
+        while (g0 > p / kWalkRun * kWalkRun && nb[g0 - 1] == nb[p] && nc[g0 - 1] == nc[p]) --g0;
+        while (g1 < np && g1 < (p / kWalkRun + 1) * kWalkRun && nb[g1] == nb[p] && nc[g1] == nc[p]) ++g1;
+        for (int64_t r = r0 + lane; r < r1; r += 32)
+            walk[rowbase[g0] + (r - r0) * (g1 - g0) + (p - g0)] = make_int2((int)p, (int)r);
+    }
 }
 
 // Single-pass forward lists: sub-det x at rank r of a class [cb, ce) of size
@@ -1031,6 +1042,7 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
         const int g0 = (int)std::min<int64_t>((np + 255) / 256 + 1, 65535);
         int64_t *goff;
         int32_t *row_p;
+        int2 *walk = nullptr;
         uint8_t *occp;
         int32_t *occc;
         int2 *l1;
@@ -1038,7 +1050,7 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
         if ((rc = dev_alloc(b, &goff, np + 1)) || (rc = dev_alloc(b, &row_p, b.dim)) ||
             (rc = dev_alloc(b, &occp, (size_t)np * std::max(b.s[0].Z, 1))) ||
             (rc = dev_alloc(b, &occc, (size_t)np * std::max(b.s[0].Z, 1))) || (rc = dev_alloc(b, &l1, L[0].tot[1])) ||
-            (rc = dev_alloc(b, &prec, np)))
+            (rc = dev_alloc(b, &prec, np)) || (b.dim >= kWalkRows && (rc = dev_alloc(b, &walk, b.dim))))
             return rc;
         const int grid = grid_for(np);
         const SpeciesBuild &SB = b.sbuild[0];
@@ -1048,7 +1060,7 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
                 k_groups<decltype(w)::value, 0><<<grid, 256, 0, st>>>(SB, b.dev, goff, nullptr, nullptr);
                 k_occ<decltype(w)::value><<<g0, 256, 0, st>>>(SB, b.s[0].Z, b.dev.code[0], occp, occc);
             });
-            k_row_p<<<grid, 256, 0, st>>>(np, b.dev.rowbase, row_p);
+            k_row_p<<<grid, 256, 0, st>>>(np, b.dev.rowbase, b.dev.nb, b.dev.nc, row_p, walk);
         }
         if ((rc = exclusive_scan_i64(goff, np, b.scan_scratch, b.scan_scratch_len, st))) return rc;
         int64_t *total = pin.p + 6;
@@ -1072,6 +1084,7 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
             b.n1_total[t] = L[t].tot[1];
         }
         b.dev.row_p = row_p;
+        b.dev.walk = walk;
         b.dev.grp = grp;
         b.dev.l1 = l1;
         b.dev.prec = prec;
