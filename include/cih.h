@@ -373,7 +373,9 @@ int cih_ham_upper_sumsq(cih_basis_h h, const int64_t *rowptr_dev, int64_t r0, in
  *   fixed-point sums hold |g_t| < 128 and |g_t| <= 2 ||psi||^2); grad_dev: K x tbme_len double (device, caller-owned,
  *   overwritten).
  * Scratch: K x tbme_len int64 and K x dim int64, library-allocated for the
- * call.  Errors: CIH_ERR_ARG, CIH_ERR_NOMEM, CIH_ERR_CUDA. */
+ * call; with K = 1 and at least 2^19 rows also dim int64 and two int64 per pn
+ * table entry where the pool gives them (else the call runs without, with the
+ * same bits).  Errors: CIH_ERR_ARG, CIH_ERR_NOMEM, CIH_ERR_CUDA. */
 int cih_ham_tbme_grad(cih_basis_h h, const int64_t *rowptr_dev, int32_t K,
                       const double *psi_dev, double *grad_dev, void *stream);
 

@@ -247,7 +247,9 @@ int batch_solve(cih_instance_t *inst, int n, double hw, int nev, int max_iter, d
                 if (e != cudaSuccess) return fail(CIH_ERR_NOMEM, "batch: adjoint scratch");
                 e = cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * ng, st);
                 int g = e == cudaSuccess ? CIH_OK : cuda_fail(e, "batch: adjoint clear");
-                if (!g) g = launch_grad(b, rowptr[i], inst[i].K, psi[i], acc, st);
+                // (the faster form where its scratch stays within the instance's)
+                const bool pairs = 8 * ng + 8 * (int64_t)inst[i].K * b.dim + (int64_t)grad_pairs_bytes(b) <= plan[i].scratch;
+                if (!g) g = launch_grad(b, rowptr[i], inst[i].K, psi[i], acc, st, pairs);
                 if (!g) g = launch_grad_finish(ng, acc, inst[i].grad_dev, st);
                 cudaFreeAsync(acc, st);
                 if (g) return g;

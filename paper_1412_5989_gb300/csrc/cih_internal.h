@@ -320,8 +320,12 @@ int launch_interleave(int K, int64_t len, const float *in, float *out, cudaStrea
 // one-time set-up of the row kernels a call with K sets would launch (shared-
 // memory limits), so that launches made during a stream capture only launch
 int prepare_rows(const cih_basis &b, int K);
+// one vector over a large basis takes a faster form that needs grad_pairs_bytes()
+// more scratch (0: does not apply), unless pairs is false or the pool has no room;
+// both forms give the same bits
+size_t grad_pairs_bytes(const cih_basis &b);
 int launch_grad(const cih_basis &b, const int64_t *rowptr, int K, const double *psi,
-                unsigned long long *acc, cudaStream_t st);
+                unsigned long long *acc, cudaStream_t st, bool pairs = true);
 int launch_grad_finish(int64_t n, const unsigned long long *acc, double *grad, cudaStream_t st);
 
 // generic device scans (scan.cu)

@@ -158,6 +158,10 @@ constexpr int kLaneSets = 16;     // from this many sets on, multi-term sums run
 // in a tree).  From eight on the row kernel's element-major paths write whole lines.
 constexpr int kFillSets = 8;
 constexpr int64_t kPrepareShare = 24, kPrepareMin = 4096;
+// Rows from which one vector's adjoint takes the form of k_grad_pairs + k_grad1
+// (row kernel / this form: 48,917 rows 156 / 205 us, 143,792 rows 396 / 389,
+// 197,822 rows 676 / 681, 814,092 rows 2,898 / 2,319, 2.2 M rows 8,082 / 6,200)
+constexpr int64_t kGradPairsMin = 1 << 19;
 constexpr int kSlowCap = 64;
 constexpr int kMaxA = 64;
 constexpr int kPairCap = kMaxA * (kMaxA - 1) / 2;
@@ -1305,6 +1309,258 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
     }
 }
 
+// ---- adjoint of one vector
+//
+// Every sum here is of integers, so its parts may be added in any grouping:
+//   own species   an element that moves one species only (two-moves; the
+//                 own-species spectators of one-moves; the own part of the
+//                 diagonal) uses the same table entry whatever the other species
+//                 does.  k_grad_pairs sums psi psi over the common partners of
+//                 each forward pair (two contiguous runs of psi) and adds once
+//                 per pair instead of once per row: a tenth of all adds;
+//   the rest      (pn moves, and the other species' terms of one-moves and of
+//                 the diagonal) k_grad1 adds per row.
+// For the neutrons the vector is copied neutron-major, so that their runs are
+// contiguous too.  k_grad1 adds into the pn groups as full squares (folded at the
+// end): the entries of a proton move and one neutron orbital are contiguous there,
+// and the limit is the number of 32-byte sectors of the atomic adds (4+4 Nmax=6:
+// 8.1 ms in the row kernel, 7.7 into the packed triangles, 6.2 into the squares).
+
+// The partners of the sub-dets of species s: other-species sub-dets beg[x] ..
+// beg[x] + lev[x * NL + l] - 1 pair with every same-class sub-det of level l (a
+// prefix of the class, ascending in N); cnt[x] is x's own count.
+struct Partners {
+    const int32_t *beg[2], *lev[2];
+    const int64_t *base[2];                // first place of x's run in the vector of its species' order
+    const long long *psi[2];               // the vector proton-major (as given) and neutron-major
+};
+
+__global__ void k_partners(DevBasis B, SpeciesBuild S0, SpeciesBuild S1, int s, int twoM, int32_t *beg, int32_t *lev, int64_t *cnt)
+{
+    const DevSpecies &X = B.sp[s];
+    const SpeciesBuild &Sx = s ? S1 : S0, &So = s ? S0 : S1;
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < X.n_sd; x += gridDim.x * blockDim.x) {
+        const int M = twoM - Sx.M2[x], par = (B.Nlim - Sx.N[x]) & 1;
+        auto below = [&](int par_, int N) {                  // sub-dets ordered (2M, parity, N) before (M, par_, N)
+            int lo = 0, hi = So.n_sd;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1, m = So.M2[mid], q = So.N[mid], r = q & 1;
+                if (m != M ? m < M : r != par_ ? r < par_ : q < N) lo = mid + 1; else hi = mid;
+            }
+            return lo;
+        };
+        const int b0 = below(par, -1), px = (Sx.N[x] - X.N0) & 1;
+        beg[x] = b0;
+        for (int l = 0; l < X.NL; ++l) {
+            const int c = below(par, B.Nlim - (X.N0 + 2 * l + px) + 1) - b0;
+            lev[x * X.NL + l] = c > 0 ? c : 0;
+            if (l == (Sx.N[x] - X.N0) >> 1) cnt[x] = c;
+        }
+    }
+}
+
+// out[base[n] + p - beg[n]] = psi[row of (p, n)]
+__global__ void k_psi_neutron_major(DevBasis B, const int32_t *beg, const int64_t *base, const long long *psi, long long *out)
+{
+    for (int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; row < B.dim; row += (int64_t)gridDim.x * blockDim.x) {
+        const int p = B.row_p[row], n = (int)(row - B.prec[p].colb);
+        out[base[n] + p - beg[n]] = psi[row];
+    }
+}
+
+// One block per sub-det x (the lowest ones have thousands of pairs with hundreds
+// of partners), eight lanes per forward pair (x, y): the sum over their common
+// partners of psi psi, added to the pair's table entry (two-move) or to its
+// own-species spectator entries (one-move).
+__global__ void __launch_bounds__(256) k_grad_pairs(DevBasis B, Partners Pt, unsigned long long *acc, int *status)
+{
+    const int tid = threadIdx.x, lane = tid & 31, li = tid & 7;
+    const int64_t n0 = B.sp[0].n_sd, n1 = n0 + B.sp[1].n_sd;
+    for (int64_t t = blockIdx.x; t < n1; t += gridDim.x) {
+        const int s = t < n0 ? 0 : 1;
+        const DevSpecies S = s ? B.sp[1] : B.sp[0];
+        const int64_t x = t - (s ? n0 : 0), f0 = S.fw_off[x];
+        const int Z = s ? B.nZ[1] : B.nZ[0], len = (int)(S.fw_off[x + 1] - f0), two = S.fw_lev[x * S.NL + S.NL - 1];
+        const uint8_t *occ = (s ? B.occ[1] : B.occ[0]) + x * Z;
+        const int32_t *lev = (s ? Pt.lev[1] : Pt.lev[0]) + x * S.NL;
+        const int64_t *base = s ? Pt.base[1] : Pt.base[0];
+        const long long *psi = s ? Pt.psi[1] : Pt.psi[0], *px = psi + base[x];
+        const int nb = s ? 0 : B.nb[x];
+        if (tid < 32) {                                         // own part of the diagonal: weight 1, every partner of x
+            const int c = (int)(base[x + 1] - base[x]);
+            long long sum = 0;
+            for (int i = lane; i < c; i += 32) sum += __mul64hi(px[i], px[i]) >> 2;
+            for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+            for (int l = lane; l < Z * (Z - 1) / 2; l += 32) {
+                int i, j, sg;
+                int64_t idx;
+                pair_of(l, Z, i, j);
+                const int a = S.orb_base + occ[i], b = S.orb_base + occ[j];
+                if (tbme_at(B, nullptr, a, b, a, b, idx, sg)) atomicAdd(acc + idx, (unsigned long long)(sg < 0 ? -sum : sum));
+                else if (atomicOr(status, 1) == 0) { status[2] = a | (b << 16); status[3] = 1; }
+            }
+        }
+        for (int e0 = 0; e0 < len; e0 += 32) {
+            const int e = e0 + (tid >> 3);
+            const bool on = e < len;
+            long long sum = 0;
+            int tb = 0;
+            if (on) {
+                const int2 rc = S.fw_rec[f0 + e];
+                tb = S.fw_tb[f0 + e];
+                const long long *py = psi + (s ? base[rc.x] : (int64_t)(rc.x + nb));
+                const int c = lev[rc.y >> 24];
+                for (int i = li; i < c; i += 8) sum += __mul64hi(px[i], py[i]) >> 1;
+            }
+            for (int d = 4; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+            if (!on) continue;
+            if (e < two) {
+                if (li == 0) atomicAdd(acc + (tb >> 1), (unsigned long long)(tb & 1 ? -sum : sum));
+                continue;
+            }
+            const int code = ~tb, a = S.orb_base + (code & 0xFF), c = S.orb_base + ((code >> 8) & 0xFF);
+            for (int i = li; i < Z; i += 8) {
+                const int k = S.orb_base + occ[i];
+                if (k == a) continue;
+                int64_t idx;
+                int sg;
+                if (tbme_at(B, nullptr, a, k, c, k, idx, sg))
+                    atomicAdd(acc + idx, (unsigned long long)(((code >> 16) & 1) != (sg < 0) ? -sum : sum));
+                else if (atomicOr(status, 1) == 0) {
+                    status[2] = a | (c << 16);
+                    status[3] = 2 | (k << 8);
+                }
+            }
+        }
+    }
+}
+
+// acc of the table entries of the pn groups += the squares' entries: (u, v) and
+// (v, u) are one; one warp per row of a square
+__global__ void __launch_bounds__(256) k_grad_fold(DevBasis B, const unsigned long long *sq, unsigned long long *acc)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t t = warp; t < B.n_sqrow; t += nw) {
+        const int r = B.sqrow[t], k = r >> 16, u = r & 0xFFFF;
+        const int2 g = B.pn_k[k];
+        const int n = g.y;
+        const unsigned long long *s = sq + B.pn_kq[k].x;
+        unsigned long long *o = acc + g.x + (int64_t)u * n - ((int64_t)u * (u - 1)) / 2 - u;
+        for (int v = u + lane; v < n; v += 32) {
+            unsigned long long x = s[(int64_t)u * n + v];
+            if (v > u) x += s[(int64_t)v * n + u];
+            o[v] += x;
+        }
+    }
+}
+
+// The walk of k_fill1 without places: every (member, neutron move) pair of the
+// row's groups, and the other species' terms of its one-moves and diagonal.
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
+k_grad1(DevBasis B, const long long *psi, unsigned long long *acc)
+{
+    constexpr int kThreads = WARPS * 32;
+    extern __shared__ __align__(16) unsigned char sb[];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const unsigned lt = (1u << lane) - 1, le = (2u << lane) - 1u;
+    const DevSpecies &SP = B.sp[0];
+    const int T = B.pn_T, Zp = B.nZ[0], Zn = B.nZ[1];
+    int2 *KG = sptr<int2>(sb, f1::kg);
+    int16_t *S = sptr<int16_t>(sb, f1::S<WARPS>);
+    for (int i = tid; i < SP.n_orb * T; i += kThreads) S[i] = B.pn_s[i];
+    for (int i = tid; i < 64; i += kThreads) KG[i] = B.pn_kq[i];
+    __syncthreads();
+    unsigned char *wb = sb + f1::warp0 + wid * f1::w_size;
+    int4 *w_seg = sptr<int4>(wb, f1::w_seg);
+    int *w_s0 = sptr<int>(wb, f1::w_ext);
+    int *w_op = sptr<int>(wb, f1::w_op), *w_on = sptr<int>(wb, f1::w_on);
+    const int P = term_lanes(Zp, Zn), sub = lane / P, li = lane % P, per = 32 / P;
+    const int64_t gw = (blockIdx.x * (int64_t)kThreads + tid) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * kThreads) >> 5;
+    auto add = [&](int l1, int n1, long long q) {
+        const int idx = pn_square_at(KG, S, T, l1, n1);
+        atomicAdd(acc + idx, (unsigned long long)(((l1 >> 16) ^ (n1 >> 26)) & 1 ? -q : q));
+    };
+    for (int64_t place = gw; place < B.dim; place += nw) {
+        const int2 at_row = B.walk ? B.walk[place] : make_int2(B.row_p[place], (int)place);
+        const int p = at_row.x;
+        const int64_t row = at_row.y;
+        const ProtonRec PR = B.prec[p];
+        const int n = (int)(row - PR.colb);
+        const NeutronRec NR = B.nrec[n];
+        const long long pr = psi[row];
+        const int16_t *dirn = B.dir + (int64_t)n * B.dir_len;
+        const int cA1 = max(0, dirn[PR.dirA] - NR.self);
+        if (lane < Zp) w_op[lane] = B.occ_code[0][(int64_t)p * Zp + lane];
+        if (lane < Zn) w_on[lane] = B.occ_code[1][(int64_t)n * Zn + lane];
+        const unsigned l1o = (unsigned)PR.l1 * 8u, n1o = (unsigned)NR.n1 * 8u;
+        __syncwarp();
+        {                                                       // diagonal, w = 1
+            const long long q = __mul64hi(pr, pr) >> 2;
+            for (int i = sub; i < Zp; i += per)
+                if (li < Zn) add(w_op[i], w_on[li], q);
+        }
+        int c1 = 0;                                             // proton one-moves with n kept
+        for (int g0 = 0; g0 < PR.ng; g0 += 32) {
+            int4 gr = make_int4(0, 0, 0, 0);
+            if (g0 + lane < PR.ng) gr = B.grp[PR.g0 + g0 + lane];
+            const int n1c = (unsigned)gr.x >> 16, s0 = dirn[gr.y & 0xFFFF], len = dirn[(unsigned)gr.y >> 16] - s0;
+            if (g0 == 0) c1 = __reduce_add_sync(0xffffffffu, (gr.w & 0xFF) > NR.N ? n1c : 0);
+            const int npn = n1c * len;
+            int ipn = npn;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, ipn, d);
+                if (lane >= d) ipn += o;
+            }
+            const int Tpn = __shfl_sync(0xffffffffu, ipn, 31), st = ipn - npn;
+            const unsigned ne = __ballot_sync(0xffffffffu, npn > 0);
+            if (npn > 0) {
+                const int j = __popc(ne & lt);
+                w_seg[j] = make_int4(st, (int)(0xFFFFFFFFu / (unsigned)len), gr.x & 0xFFFF, len);
+                w_s0[j] = s0;
+            }
+            __syncwarp();
+            int before = -1;
+            for (int w0 = 0; w0 < Tpn; w0 += 32 * kW) {         // as in k_fill1
+                int2 q[kW], ent[kW];
+                long long v[kW];
+#pragma unroll
+                for (int u = 0; u < kW; ++u) {
+                    const int w = w0 + 32 * u;
+                    const unsigned mk = __reduce_or_sync(0xffffffffu, npn > 0 && (unsigned)(st - w) < 32u ? 1u << (st - w) : 0u);
+                    const int j = before + __popc(mk & le), e = min(w + lane, Tpn - 1);
+                    before += __popc(mk);
+                    const int4 sg4 = w_seg[j];
+                    const int rel = e - sg4.x;
+                    int qi = (int)__umulhi((unsigned)rel, (unsigned)sg4.y), k = rel - qi * sg4.w;   // at most one short
+                    if (k >= sg4.w) { ++qi; k -= sg4.w; }
+                    q[u] = at_byte<int2>(B.l1, l1o + (unsigned)(sg4.z + qi) * 8u);
+                    ent[u] = at_byte<int2>(B.n1p, n1o + (unsigned)(w_s0[j] + k) * 8u);
+                }
+#pragma unroll
+                for (int u = 0; u < kW; ++u) v[u] = __ldg(psi + (q[u].x + ent[u].x));
+#pragma unroll
+                for (int u = 0; u < kW; ++u)
+                    if (w0 + 32 * u + lane < Tpn) add(q[u].y, ent[u].y, __mul64hi(pr, v[u]) >> 1);
+            }
+            __syncwarp();
+        }
+        for (int t0 = 0; t0 < cA1 + c1; t0 += per) {            // one-moves: P lanes an element
+            const int t = t0 + sub;
+            if (t >= cA1 + c1) continue;
+            const bool neu = t < cA1;
+            const int2 m = neu ? B.n1p[NR.n1 + NR.self + t] : B.l1[PR.l1 + t - cA1];
+            if (li >= (neu ? Zp : Zn)) continue;
+            const long long q = __mul64hi(pr, psi[neu ? PR.colb + m.x : m.x + n]) >> 1;
+            add(neu ? w_op[li] : m.y, neu ? m.y : w_on[li], q);
+        }
+        __syncwarp();
+    }
+}
+
 // Count pass: for row (p, n), 1 for the diagonal + n's forward same-class
 // neighbours inside p's range + the sum over p's groups of members x segment
 // length (+ members and two-moves where n itself is a partner).  Equal to the
@@ -1602,54 +1858,146 @@ int launch_interleave(int K, int64_t len, const float *in, float *out, cudaStrea
     return e == cudaSuccess ? CIH_OK : cuda_fail(e, "interleave");
 }
 
-// psi_fix[i] = psi[i] * 2^61 rounded; |psi| >= 4 cannot be held and sets status bit 32
-__global__ void k_psi_fix(int64_t n, const double *psi, long long *psi_fix, int *status)
+// psi_fix[i] = psi[i] * 2^61 rounded; |psi| >= 4 cannot be held and sets status
+// bit 32.  Grid (blocks, K); part[k * gridDim.x + block] = this block's share of
+// ||psi_k||^2.
+__global__ void __launch_bounds__(256) k_psi_fix(int64_t dim, const double *psi, long long *psi_fix, double *part, int *status)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double v = psi[i];
-        if (!(fabs(v) < 4.0)) {
+    __shared__ double red[8];
+    const double *v = psi + (int64_t)blockIdx.y * dim;
+    long long *o = psi_fix + (int64_t)blockIdx.y * dim;
+    double s = 0.0;
+    for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < dim; i += gridDim.x * 256ll) {
+        const double x = v[i];
+        s += x * x;
+        if (!(fabs(x) < 4.0)) {
             atomicOr(status, 32);
-            psi_fix[i] = 0;
+            o[i] = 0;
         } else {
-            psi_fix[i] = __double2ll_rn(v * kPsiScale);
+            o[i] = __double2ll_rn(x * kPsiScale);
         }
     }
-}
-
-// ||psi_k||^2 of each set, one block per set: above 1 + 1e-6 sets status bit 32
-// (|g_t| <= 2 ||psi||^2 must stay below the 2^7 the 2^-56 accumulators hold)
-__global__ void __launch_bounds__(1024) k_psi_norm(int64_t dim, const double *psi, int *status)
-{
-    __shared__ double part[32];
-    const double *v = psi + (int64_t)blockIdx.x * dim;
-    double s = 0.0;
-    for (int64_t i = threadIdx.x; i < dim; i += blockDim.x) s += v[i] * v[i];
     for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        s = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.0;
-        for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-        if (threadIdx.x == 0 && !(s <= 1.0 + 1e-6)) atomicOr(status, 32);
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) s += red[w];
+        part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = s;
     }
 }
 
+// ||psi_k||^2 above 1 + 1e-6 sets status bit 32 (|g_t| <= 2 ||psi||^2 must stay
+// below the 2^7 the 2^-56 accumulators hold); one warp per set
+__global__ void k_psi_norm(int parts, const double *part, int *status)
+{
+    double s = 0.0;
+    for (int i = threadIdx.x; i < parts; i += 32) s += part[(int64_t)blockIdx.x * parts + i];
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    if (threadIdx.x == 0 && !(s <= 1.0 + 1e-6)) atomicOr(status, 32);
+}
+
+namespace {
+
+template <int WARPS>
+int launch_grad1_w(const cih_basis &b, const long long *psi, unsigned long long *acc, cudaStream_t st)
+{
+    const size_t smem = (size_t)f1::S<WARPS> + ((size_t)b.dev.sp[0].n_orb * b.dev.pn_T * 2 + 15) / 16 * 16;
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaError_t e = raise_smem_limit((const void *)k_grad1<WARPS>, dev, (int)smem);
+    if (e != cudaSuccess) return cuda_fail(e, "adjoint shared memory");
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grad1<WARPS>, WARPS * 32, smem);
+    per_sm = std::max(per_sm, 1);
+    if (b.launch_ctas > 0) per_sm = std::min(per_sm, b.launch_ctas);
+    const int64_t want = (b.dim + WARPS - 1) / WARPS;
+    count_launches(1);
+    k_grad1<WARPS><<<(int)std::min<int64_t>((int64_t)sms * per_sm, want), WARPS * 32, smem, st>>>(b.dev, psi, acc);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? CIH_OK : cuda_fail(e, "adjoint launch");
+}
+
+}  // namespace
+
+size_t grad_pairs_bytes(const cih_basis &b)
+{
+    if (b.dim < kGradPairsMin || fill_work_floats(b) == 0) return 0;
+    const DevBasis &D = b.dev;
+    const int64_t np = b.s[0].n_sd, nn = b.s[1].n_sd;
+    // 8-byte arrays: neutron-major vector, neutron run starts, proton counts, scan
+    // scratch, pn squares; then 4-byte: first partners and level counts
+    return 8 * (size_t)(b.dim + (nn + 1) + np + scan_scratch_needed(nn) + b.sq_total) +
+           4 * (size_t)(np * (1 + D.sp[0].NL) + nn * (1 + D.sp[1].NL));
+}
+
+namespace {
+
+// one vector in the form of k_grad_pairs + k_grad1; 1: not this form (few rows, no
+// memory for its scratch, or a shape outside k_grad1's)
+int launch_grad1(const cih_basis &b, const long long *fix, unsigned long long *acc, cudaStream_t st)
+{
+    const size_t bytes = grad_pairs_bytes(b);
+    if (bytes == 0) return 1;
+    const DevBasis &D = b.dev;
+    const int64_t np = b.s[0].n_sd, nn = b.s[1].n_sd, ns = scan_scratch_needed(nn);
+    int64_t *buf = nullptr;
+    if (cudaMallocFromPoolAsync((void **)&buf, bytes, b.pool, st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 1;
+    }
+    long long *psin = reinterpret_cast<long long *>(buf);
+    int64_t *basen = buf + b.dim, *cntp = basen + nn + 1, *scan = cntp + np;
+    unsigned long long *sq = reinterpret_cast<unsigned long long *>(scan + ns);
+    int32_t *begp = reinterpret_cast<int32_t *>(sq + b.sq_total), *levp = begp + np, *begn = levp + np * D.sp[0].NL, *levn = begn + nn;
+    count_launches(4);
+    k_partners<<<(int)((np + 127) / 128), 128, 0, st>>>(D, b.sbuild[0], b.sbuild[1], 0, b.space.twoM, begp, levp, cntp);
+    k_partners<<<(int)((nn + 127) / 128), 128, 0, st>>>(D, b.sbuild[0], b.sbuild[1], 1, b.space.twoM, begn, levn, basen);
+    int rc = exclusive_scan_i64(basen, nn, scan, ns, st);
+    if (!rc) {
+        k_psi_neutron_major<<<(int)std::min<int64_t>((b.dim + 255) / 256, 152 * 16), 256, 0, st>>>(D, begn, basen, fix, psin);
+        const Partners Pt{{begp, begn}, {levp, levn}, {D.rowbase, basen}, {fix, psin}};
+        k_grad_pairs<<<(int)std::min<int64_t>(np + nn, 152 * 32), 256, 0, st>>>(D, Pt, acc, b.dev_status);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) rc = cuda_fail(e, "adjoint pairs");
+    }
+    cudaMemsetAsync(sq, 0, sizeof(unsigned long long) * b.sq_total, st);
+    if (!rc) rc = b.launch_warps == 8 ? launch_grad1_w<8>(b, fix, sq, st) : launch_grad1_w<16>(b, fix, sq, st);
+    if (!rc && b.dev.n_sqrow > 0) {
+        count_launches(1);
+        k_grad_fold<<<std::min((b.dev.n_sqrow + 7) / 8, 152 * 16), 256, 0, st>>>(D, sq, acc);
+    }
+    cudaFreeAsync(buf, st);
+    return rc;
+}
+
+}  // namespace
+
 int launch_grad(const cih_basis &b, const int64_t *rowptr, int K, const double *psi,
-                unsigned long long *acc, cudaStream_t st)
+                unsigned long long *acc, cudaStream_t st, bool pairs)
 {
     const int64_t n = (int64_t)K * b.dim;
     if (n == 0) return CIH_OK;
+    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>((b.dim + 1023) / 1024, 152 * 8));
     long long *fix = nullptr;
-    cudaError_t e = cudaMallocFromPoolAsync((void **)&fix, sizeof(long long) * n, b.pool, st);
+    cudaError_t e = cudaMallocFromPoolAsync((void **)&fix, sizeof(long long) * n + sizeof(double) * (size_t)parts * K, b.pool, st);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return fail(CIH_ERR_NOMEM, "adjoint: fixed-point vector");
     }
+    double *part = reinterpret_cast<double *>(fix + n);
     count_launches(2);
-    k_psi_norm<<<K, 1024, 0, st>>>(b.dim, psi, b.dev_status);
-    k_psi_fix<<<(int)std::min<int64_t>((n + 255) / 256, 152 * 16), 256, 0, st>>>(n, psi, fix, b.dev_status);
-    GradArgs G{K, fix, acc};
-    const int rc = launch_rows<2>(b, rowptr, nullptr, FillArgs{}, G, st);
+    for (int k0 = 0; k0 < K; k0 += 32768) {                  // (grid.y is limited)
+        const int kc = std::min(K - k0, 32768);
+        k_psi_fix<<<dim3(parts, kc), 256, 0, st>>>(b.dim, psi + (int64_t)k0 * b.dim, fix + (int64_t)k0 * b.dim,
+                                                   part + (int64_t)k0 * parts, b.dev_status);
+    }
+    k_psi_norm<<<K, 32, 0, st>>>(parts, part, b.dev_status);
+    int rc = K == 1 && pairs ? launch_grad1(b, fix, acc, st) : 1;
+    if (rc == 1) {
+        const GradArgs G{K, fix, acc};
+        rc = launch_rows<2>(b, rowptr, nullptr, FillArgs{}, G, st);
+    }
     cudaFreeAsync(fix, st);
     return rc;
 }
