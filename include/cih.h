@@ -225,8 +225,8 @@ int cih_ham_fill_batched(cih_basis_h h, const int64_t *rowptr_dev, int32_t K, do
  * with the host copies inside the call): the K two-body tables are copied
  * host -> device, the count pass and scan run, the row pointers come back
  * (one synchronisation, which gives nnz), then the fill runs in 8 row chunks
- * of about equal nonzero counts while a second stream copies each finished
- * chunk's columns and values device -> host.
+ * (the first ones small, so that the copies start early) while a second stream
+ * copies each finished chunk's columns and values device -> host.
  *   tbme_host: K x tbme_len float (set-major); e_sp_host: NULL or
  *   n_orb_p + n_orb_n double; rowptr_host: dim + 1 int64; col_host:
  *   capacity int32; val_host: K x capacity float, the values of set k at

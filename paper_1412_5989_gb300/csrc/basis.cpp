@@ -102,8 +102,9 @@ struct Enumerator {
 };
 
 template <class Fn>
-void parallel_tops(int ntop, Fn &&fn)
+void parallel_tops(int ntop, bool serial, Fn &&fn)
 {
+    if (serial) { for (int t = 0; t < ntop; ++t) fn(t); return; }
     unsigned hw = std::max(1u, std::min(4u, std::thread::hardware_concurrency()));
     if (const char *e = std::getenv("CIH_THREADS")) hw = (unsigned)std::max(1, std::atoi(e));
     int nt = (int)std::min<unsigned>(hw, (unsigned)std::max(ntop / 4, 1));
@@ -240,7 +241,7 @@ void write_subdets(Species &s, SubdetCount &C, const std::vector<char> &keep_key
     s.bits.assign((size_t)total * kMaxWords, 0);
     s.N.assign(total, 0);
     s.M2.assign(total, 0);
-    parallel_tops(ntop, [&](int t) {
+    parallel_tops(ntop, small_host(total), [&](int t) {
         uint64_t w[kMaxWords] = {0, 0, 0, 0};
         const int a = C.tops[t];
         w[a >> 6] |= 1ull << (a & 63);
@@ -442,7 +443,8 @@ int build_host_species(const cih_space_t &sp, cih_basis &b)
 
     // the two species are independent: count them side by side
     SubdetCount cnt[2];
-    side_by_side([&]() { count_subdets(b.s[0], cnt[0]); }, [&]() { count_subdets(b.s[1], cnt[1]); });
+    side_by_side([&]() { count_subdets(b.s[0], cnt[0]); }, [&]() { count_subdets(b.s[1], cnt[1]); },
+                 b.s[0].n_orb + b.s[1].n_orb <= 100);            // (a table of few orbitals)
     tm.mark("count p and n");
 
     // appearing buckets: those with a partner bucket of the other species
@@ -467,10 +469,13 @@ int build_host_species(const cih_space_t &sp, cih_basis &b)
                              appears(cnt[t].M2_of(k), cnt[t].N_of(k), sp.twoM, b.Nlim, minN, mspan);
         }
     }
+    int64_t subsets = 0;
+    for (int t = 0; t < 2; ++t)
+        for (int64_t c : cnt[t].total) subsets += c;
     side_by_side([&]() { write_subdets(b.s[0], cnt[0], keep[0]); },
-                 [&]() { write_subdets(b.s[1], cnt[1], keep[1]); });
+                 [&]() { write_subdets(b.s[1], cnt[1], keep[1]); }, small_host(subsets));
     tm.mark("appearing sub-dets written");
-    side_by_side([&]() { make_classes(b.s[0]); }, [&]() { make_classes(b.s[1]); });
+    side_by_side([&]() { make_classes(b.s[0]); }, [&]() { make_classes(b.s[1]); }, small_host(b.s[0].n_sd + b.s[1].n_sd));
     tm.mark("appearing filter + classes");
     return CIH_OK;
 }

@@ -24,6 +24,7 @@ constexpr int kLevels = 8;                // oscillator levels of a species: Nma
 // the least number of rows.
 constexpr int kWalkRun = 16;
 constexpr int64_t kWalkRows = 1 << 19;
+constexpr int64_t kPrepareMin = 4096;     // rows from which a fill of few sets prepares a working copy (ham.cu)
 constexpr uint64_t kPoolKeep = 1ull << 30; // bytes the library pool keeps after a Lanczos call
 constexpr int kSortTile = 4096;           // longest neighbour list the sort handles
 
@@ -243,10 +244,22 @@ struct cih_basis {
 
 namespace cih {
 
-// f0() here and f1() on a second thread; an exception of either is rethrown
+// Host work on this many sub-dets is done in the calling thread: starting and
+// joining a thread takes some 50 us (a set-up used 13; whole set-up with 4,096 /
+// 10,000 / 20,000 / 50,000 as the limit: 14,072 sub-dets 1.46 / 0.96 / 1.03 / 1.05
+// ms, 18,648 1.94 / 1.53 / 1.51 / 1.66, 54,201 2.09 / 2.08 / 1.93 / 2.13).
+inline bool small_host(int64_t n_sd) { return n_sd <= 16384; }
+
+// f0() here and f1() on a second thread (after it when `serial`); an exception
+// of either is rethrown
 template <class F0, class F1>
-inline void side_by_side(F0 &&f0, F1 &&f1)
+inline void side_by_side(F0 &&f0, F1 &&f1, bool serial = false)
 {
+    if (serial) {
+        f0();
+        f1();
+        return;
+    }
     std::exception_ptr e1;
     std::thread th([&]() {
         try {

@@ -157,7 +157,7 @@ constexpr int kLaneSets = 16;     // from this many sets on, multi-term sums run
 // from the tables, where a one-move gathered ten entries per set and reduced them
 // in a tree).  From eight on the row kernel's element-major paths write whole lines.
 constexpr int kFillSets = 8;
-constexpr int64_t kPrepareShare = 24, kPrepareMin = 4096;
+constexpr int64_t kPrepareShare = 24;
 // Rows from which one vector's adjoint takes the form of k_grad_pairs + k_grad1
 // (row kernel / this form: 48,917 rows 156 / 205 us, 143,792 rows 396 / 389,
 // 197,822 rows 676 / 681, 814,092 rows 2,898 / 2,319, 2.2 M rows 8,082 / 6,200)

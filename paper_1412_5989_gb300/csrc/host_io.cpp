@@ -25,7 +25,11 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
         bufs.push_back(*p);
         return true;
     };
+    // ends of the row chunks in 64ths of the nonzeros
+    constexpr int kChunks = 8;
+    static const int kChunkEnd[kChunks] = {1, 4, 10, 20, 31, 42, 53, 64};
     cudaStream_t cs = nullptr;
+    cudaEvent_t counted = nullptr;
     std::vector<cudaEvent_t> evs;
     int rc = CIH_OK;
     float *tbme_d = nullptr;
@@ -44,7 +48,25 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
     if (esp_h) cudaMemcpyAsync(esp_d, esp_h, sizeof(double) * n_orb, cudaMemcpyHostToDevice, st);
     if ((rc = launch_count(b, rowptr_d, st)) || (rc = launch_scan(b, rowptr_d, st))) goto done;
     e = cudaMemcpyAsync(rowptr_h, rowptr_d, sizeof(int64_t) * (dim + 1), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&counted, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(counted, st);
+    if (e != cudaSuccess) { rc = cuda_fail(e, "build_host: row pointers"); goto done; }
+    // what does not need the count runs while it does: one set's working copy of
+    // the table (prepared once for all chunks), the copy stream and its events
+    if (K == 1 && dim >= kPrepareMin && fill_work_floats(b) > 0 && alloc((void **)&work, sizeof(float) * fill_work_floats(b)) &&
+        (rc = fill_prepare(b, hw, tbme_d, esp_d, nullptr, work, st)))
+        goto done;
+    e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+    if (e != cudaSuccess) { cs = nullptr; rc = cuda_fail(e, "build_host: copy stream"); goto done; }
+    for (int c = 0; c < kChunks; ++c) {
+        cudaEvent_t ev;
+        if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) {
+            rc = cuda_fail(e, "build_host: event");
+            goto done;
+        }
+        evs.push_back(ev);
+    }
+    e = cudaEventSynchronize(counted);
     if (e != cudaSuccess) { rc = cuda_fail(e, "build_host: row pointers"); goto done; }
     nnz = rowptr_h[dim];
     if (nnz_out) *nnz_out = nnz;
@@ -58,31 +80,21 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
         rc = fail(CIH_ERR_NOMEM, "build_host: device matrix");
         goto done;
     }
-    // one set: the fill's working copy of the table, prepared once for all chunks
-    if (K == 1 && fill_work_floats(b) > 0 && alloc((void **)&work, sizeof(float) * fill_work_floats(b)) &&
-        (rc = fill_prepare(b, hw, tbme_d, esp_d, nullptr, work, st)))
-        goto done;
     tm.mark_sync("device matrix allocated", st);
-    e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-    if (e != cudaSuccess) { cs = nullptr; rc = cuda_fail(e, "build_host: copy stream"); goto done; }
     {
-        // row chunks of about equal nonzero counts; chunk c's copies wait for its fill
-        const int C = (int)std::max<int64_t>(1, std::min<int64_t>(8, dim));
+        // row chunks; chunk c's copies wait for its fill.  The fill is four to five
+        // times faster than the link, so the first chunks are small (the copies
+        // start early) and each is filled while the one before it is copied.
+        const int C = (int)std::max<int64_t>(1, std::min<int64_t>(kChunks, dim));
         std::vector<int64_t> rb(C + 1, dim);
         rb[0] = 0;
         for (int c = 1; c < C; ++c)
-            rb[c] = std::lower_bound(rowptr_h, rowptr_h + dim + 1, nnz * c / C) - rowptr_h;
+            rb[c] = std::lower_bound(rowptr_h, rowptr_h + dim + 1, nnz * kChunkEnd[c - 1] / 64) - rowptr_h;
         for (int c = 0; c < C && !rc; ++c) {
-            const int64_t r0 = std::min(rb[c], dim), r1 = std::max(r0, std::min(rb[c + 1], dim));
-            if ((rc = launch_fill(b, rowptr_d, K, hw, tbme_d, false, false, esp_d, col_d, val_d, st, r0, r1, false,
-                                  nullptr, work)))
+            const int64_t r0 = std::min(rb[c], dim), r1 = c == C - 1 ? dim : std::max(r0, std::min(rb[c + 1], dim));
+            if ((rc = launch_fill(b, rowptr_d, K, hw, tbme_d, false, false, esp_d, col_d, val_d, st, r0, r1, false, nullptr, work)))
                 break;
-            cudaEvent_t ev;
-            if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) {
-                rc = cuda_fail(e, "build_host: event");
-                break;
-            }
-            evs.push_back(ev);
+            const cudaEvent_t ev = evs[c];
             cudaEventRecord(ev, st);
             cudaStreamWaitEvent(cs, ev, 0);
             const int64_t e0 = rowptr_h[r0], e1 = rowptr_h[r1];
@@ -105,6 +117,7 @@ done:
     e = cudaStreamSynchronize(st);
     if (!rc && e != cudaSuccess) rc = cuda_fail(e, "build_host");
     for (cudaEvent_t ev : evs) cudaEventDestroy(ev);
+    if (counted) cudaEventDestroy(counted);
     if (cs) cudaStreamDestroy(cs);
     return rc;
 }

@@ -569,6 +569,44 @@ int upload(cih_basis &b, T **p, const std::vector<T> &h, cudaStream_t st)
     return CIH_OK;
 }
 
+// Small host arrays travel to the device together: one allocation and one copy
+// for all that are added before flush() (a separate copy of each costs about as
+// much host time as a kernel launch; a basis has some forty).  The pointers are
+// set by flush(); arrays above kPackMost go by themselves.
+struct Packer {
+    static constexpr size_t kPackMost = 1 << 16;
+    cih_basis &b;
+    cudaStream_t st;
+    std::vector<unsigned char> host;
+    std::vector<std::pair<void **, size_t>> at;
+    int rc = CIH_OK;
+
+    Packer(cih_basis &b_, cudaStream_t s) : b(b_), st(s) {}
+    template <class T>
+    void add(T **p, const std::vector<T> &h)
+    {
+        if (rc) return;
+        if (h.size() * sizeof(T) > kPackMost) {
+            rc = upload(b, p, h, st);
+            return;
+        }
+        const size_t o = (host.size() + 255) / 256 * 256;
+        host.resize(o + std::max<size_t>(h.size() * sizeof(T), 1));
+        if (!h.empty()) std::memcpy(host.data() + o, h.data(), h.size() * sizeof(T));
+        at.push_back({(void **)p, o});
+    }
+    int flush()
+    {
+        if (rc || at.empty()) return rc;
+        unsigned char *d;
+        if ((rc = upload(b, &d, host, st))) return rc;
+        for (auto &x : at) *x.first = d + x.second;
+        at.clear();
+        host.clear();
+        return CIH_OK;
+    }
+};
+
 int grid_for(int64_t warps)
 {
     int dev = 0, sms = 148;
@@ -587,6 +625,17 @@ void with_words(int W, Fn &&fn)
     else fn(std::integral_constant<int, 4>());
 }
 
+// species t: host arrays (built for both species side by side), then their
+// upload and the one-move hash table
+struct SpeciesHost {
+    std::vector<uint64_t> bits;
+    std::vector<int8_t> N, oN;
+    std::vector<int16_t> M2, om2;
+    std::vector<int32_t> cls_end, cb, ce, cls_of;
+    std::vector<int64_t> class_stage;         // staged forward lists: first slot of each class
+    int64_t fw_stage = 0;                     // and their total
+};
+
 // Neighbour lists of one species, in three phases so that both species'
 // kernels queue back to back and the host work in between overlaps them:
 //   1. staged forward and one-move passes, their counts scanned, list totals
@@ -603,7 +652,7 @@ struct Lists {
 };
 
 template <int W>
-int lists_phase1(cih_basis &b, int t, SpeciesBuild &S, Lists &L, cudaStream_t st)
+int lists_phase1(cih_basis &b, int t, SpeciesBuild &S, const SpeciesHost &H, Lists &L, cudaStream_t st)
 {
     const Species &hs = b.s[t];
     const int64_t n = L.n = S.n_sd;
@@ -613,19 +662,9 @@ int lists_phase1(cih_basis &b, int t, SpeciesBuild &S, Lists &L, cudaStream_t st
     if ((rc = dev_alloc(b, &L.scratch, L.ns))) return rc;
     L.grid = grid_for(n);
     // staging: forward lists by class triangle, one-move lists by fixed slots
-    std::vector<int32_t> cls_of(std::max<int64_t>(n, 1));
-    std::vector<int64_t> class_stage(std::max<size_t>(hs.cls_begin.size(), 1));
-    int64_t fw_stage = 0;
-    for (size_t c = 0; c < hs.cls_begin.size(); ++c) {
-        const int64_t m = hs.cls_end[c] - hs.cls_begin[c];
-        class_stage[c] = fw_stage;
-        fw_stage += m * (m - 1) / 2;
-        for (int64_t x = hs.cls_begin[c]; x < hs.cls_end[c]; ++x) cls_of[x] = (int32_t)c;
-    }
     L.cap1 = std::max(1, hs.Z * std::max(0, hs.n_orb - hs.Z));
     if (L.cap1 > kSortTile) return fail(CIH_ERR_UNSUPPORTED, "one-move lists longer than the sort tile");
-    if ((rc = upload(b, &L.d_cls_of, cls_of, st)) || (rc = upload(b, &L.d_class_stage, class_stage, st)) ||
-        (rc = dev_alloc(b, &L.fw_st, fw_stage)) || (rc = dev_alloc(b, &L.n1_st, (size_t)n * L.cap1)))
+    if ((rc = dev_alloc(b, &L.fw_st, H.fw_stage)) || (rc = dev_alloc(b, &L.n1_st, (size_t)n * L.cap1)))
         return rc;
     if (n > 0) {
         count_launches(2);
@@ -687,15 +726,6 @@ int lists_phase3(cih_basis &b, int t, SpeciesBuild &S, Lists &L, cudaStream_t st
     return CIH_OK;
 }
 
-// species t: host arrays (built for both species side by side), then their
-// upload and the one-move hash table
-struct SpeciesHost {
-    std::vector<uint64_t> bits;
-    std::vector<int8_t> N, oN;
-    std::vector<int16_t> M2, om2;
-    std::vector<int32_t> cls_end, cb, ce;
-};
-
 void species_prep(const cih_basis &b, int t, SpeciesHost &H)
 {
     const int W = b.W;
@@ -711,21 +741,44 @@ void species_prep(const cih_basis &b, int t, SpeciesHost &H)
     H.ce.assign(s.cls_end.begin(), s.cls_end.end());
     H.oN.assign(s.oN.begin(), s.oN.end());
     H.om2.assign(s.om2.begin(), s.om2.end());
+    H.cls_of.resize(std::max<int64_t>(s.n_sd, 1));
+    H.class_stage.resize(std::max<size_t>(s.cls_begin.size(), 1));
+    for (size_t c = 0; c < s.cls_begin.size(); ++c) {
+        const int64_t m = s.cls_end[c] - s.cls_begin[c];
+        H.class_stage[c] = H.fw_stage;
+        H.fw_stage += m * (m - 1) / 2;
+        for (int64_t x = s.cls_begin[c]; x < s.cls_end[c]; ++x) H.cls_of[x] = (int32_t)c;
+    }
 }
 
-int species_upload(cih_basis &b, int t, const SpeciesHost &H, cudaStream_t st)
+int species_upload(cih_basis &b, int t, const SpeciesHost &H, Lists &L, cudaStream_t st)
 {
     const int W = b.W;
     const Species &s = b.s[t];
     int rc;
     uint64_t *d_bits; int8_t *d_N; int16_t *d_M2; int32_t *d_cls_end, *d_cb, *d_ce;
     int8_t *d_oN; int16_t *d_om2;
-    if ((rc = upload(b, &d_bits, H.bits, st)) || (rc = upload(b, &d_N, H.N, st)) ||
-        (rc = upload(b, &d_M2, H.M2, st)) || (rc = upload(b, &d_cls_end, H.cls_end, st)) ||
-        (rc = upload(b, &d_cb, H.cb, st)) ||
-        (rc = upload(b, &d_ce, H.ce, st)) || (rc = upload(b, &d_oN, H.oN, st)) ||
-        (rc = upload(b, &d_om2, H.om2, st)))
-        return rc;
+    int32_t *d_upto;
+    int maxN = 0;
+    for (int a = 0; a < s.n_orb; ++a) maxN = std::max(maxN, s.oN[a]);
+    std::vector<int32_t> upto(maxN + 1, 0);
+    for (int a = 0; a < s.n_orb; ++a) upto[s.oN[a]] += 1;
+    for (int k = 1; k <= maxN; ++k) upto[k] += upto[k - 1];
+    for (int a = 1; a < s.n_orb; ++a)
+        if (s.oN[a] < s.oN[a - 1]) return fail(CIH_ERR_UNSUPPORTED, "orbitals not ordered by shell");
+    Packer up(b, st);
+    up.add(&d_bits, H.bits);
+    up.add(&d_N, H.N);
+    up.add(&d_M2, H.M2);
+    up.add(&d_cls_end, H.cls_end);
+    up.add(&d_cb, H.cb);
+    up.add(&d_ce, H.ce);
+    up.add(&d_oN, H.oN);
+    up.add(&d_om2, H.om2);
+    up.add(&d_upto, upto);
+    up.add(&L.d_cls_of, H.cls_of);
+    up.add(&L.d_class_stage, H.class_stage);
+    if ((rc = up.flush())) return rc;
     DevSpecies &D = b.dev.sp[t];
     D.bits = d_bits;
     D.N = d_N;
@@ -753,15 +806,6 @@ int species_upload(cih_basis &b, int t, const SpeciesHost &H, cudaStream_t st)
         k_bits_T<<<grid_for(((int64_t)s.n_sd * W + 31) / 32), 256, 0, st>>>(s.n_sd, W, d_bits, bitsT);
     }
     S.bitsT = bitsT;
-    int maxN = 0;
-    for (int a = 0; a < s.n_orb; ++a) maxN = std::max(maxN, s.oN[a]);
-    std::vector<int32_t> upto(maxN + 1, 0);
-    for (int a = 0; a < s.n_orb; ++a) upto[s.oN[a]] += 1;
-    for (int k = 1; k <= maxN; ++k) upto[k] += upto[k - 1];
-    for (int a = 1; a < s.n_orb; ++a)
-        if (s.oN[a] < s.oN[a - 1]) return fail(CIH_ERR_UNSUPPORTED, "orbitals not ordered by shell");
-    int32_t *d_upto;
-    if ((rc = upload(b, &d_upto, upto, st))) return rc;
     S.orb_upto = d_upto;
     S.maxN = maxN;
     const int hg = (int)std::min<int64_t>((s.n_sd + 255) / 256 + 1, 65535);
@@ -781,18 +825,14 @@ int basis_tables_upload(cih_basis &b, cudaStream_t st)
     int32_t *d_nb, *d_nc, *d_pid, *d_gsize;
     int64_t *d_rowbase, *d_goff;
     int8_t *d_orbN;
-    if ((rc = upload(b, &d_nb, b.nb, st)) || (rc = upload(b, &d_nc, b.nc, st)) ||
-        (rc = upload(b, &d_rowbase, b.rowbase, st)) || (rc = upload(b, &d_orbN, orbN, st)) ||
-        (rc = upload(b, &d_pid, b.layout.pid, st)) || (rc = upload(b, &d_gsize, b.layout.gsize, st)) ||
-        (rc = upload(b, &d_goff, b.layout.goff, st)))
-        return rc;
-    b.dev.nb = d_nb;
-    b.dev.nc = d_nc;
-    b.dev.rowbase = d_rowbase;
-    b.dev.orbN = d_orbN;
-    b.dev.pid = d_pid;
-    b.dev.gsize = d_gsize;
-    b.dev.goff = d_goff;
+    Packer up(b, st);
+    up.add(&d_nb, b.nb);
+    up.add(&d_nc, b.nc);
+    up.add(&d_rowbase, b.rowbase);
+    up.add(&d_orbN, orbN);
+    up.add(&d_pid, b.layout.pid);
+    up.add(&d_gsize, b.layout.gsize);
+    up.add(&d_goff, b.layout.goff);
     b.dev.ngroups = (int32_t)b.layout.gsize.size();
     b.dev.n_p = (int32_t)b.s[0].n_sd;
     b.dev.ntot = ntot;
@@ -844,25 +884,39 @@ int basis_tables_upload(cih_basis &b, cudaStream_t st)
     b.sq_total = sq;
     b.dev.n_sqrow = (int32_t)sqrow.size();
     int2 *d_pk, *d_pq; int16_t *d_ps; uint16_t *d_orbs; uint8_t *d_pa; int32_t *d_sqrow, *d_pc, *d_nc2;
-    if ((rc = upload(b, &d_pq, pq, st)) || (rc = upload(b, &d_sqrow, sqrow, st)) || (rc = upload(b, &d_pc, pcode, st)) ||
-        (rc = upload(b, &d_nc2, ncode, st)))
-        return rc;
+    int16_t *d_obg, *d_obl; int32_t *d_obs, *d_obo;
+    up.add(&d_pq, pq);
+    up.add(&d_sqrow, sqrow);
+    up.add(&d_pc, pcode);
+    up.add(&d_nc2, ncode);
+    up.add(&d_pk, pk);
+    up.add(&d_ps, ps);
+    up.add(&d_orbs, orbs);
+    up.add(&d_pa, pa);
+    up.add(&d_obg, b.onebody.grp);
+    up.add(&d_obl, b.onebody.loc);
+    up.add(&d_obs, b.onebody.gsize);
+    up.add(&d_obo, b.onebody.goff);
+    if ((rc = up.flush())) return rc;
+    b.dev.nb = d_nb;
+    b.dev.nc = d_nc;
+    b.dev.rowbase = d_rowbase;
+    b.dev.orbN = d_orbN;
+    b.dev.pid = d_pid;
+    b.dev.gsize = d_gsize;
+    b.dev.goff = d_goff;
     b.dev.pn_kq = d_pq;
     b.dev.sqrow = d_sqrow;
     b.dev.code[0] = d_pc;
     b.dev.code[1] = d_nc2;
-    if ((rc = upload(b, &d_pk, pk, st)) || (rc = upload(b, &d_ps, ps, st)) || (rc = upload(b, &d_orbs, orbs, st)) ||
-        (rc = upload(b, &d_pa, pa, st)))
-        return rc;
     b.dev.pn_k = d_pk;
     b.dev.pn_a = d_pa;
     b.dev.pn_s = d_ps;
     b.dev.orbs = d_orbs;
-    int16_t *d_obg, *d_obl; int32_t *d_obs, *d_obo;
-    if ((rc = upload(b, &d_obg, b.onebody.grp, st)) || (rc = upload(b, &d_obl, b.onebody.loc, st)) ||
-        (rc = upload(b, &d_obs, b.onebody.gsize, st)) || (rc = upload(b, &d_obo, b.onebody.goff, st)))
-        return rc;
-    b.dev.ob_grp = d_obg; b.dev.ob_loc = d_obl; b.dev.ob_gsize = d_obs; b.dev.ob_goff = d_obo;
+    b.dev.ob_grp = d_obg;
+    b.dev.ob_loc = d_obl;
+    b.dev.ob_gsize = d_obs;
+    b.dev.ob_goff = d_obo;
     return CIH_OK;
 }
 
@@ -959,7 +1013,7 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
     //    pageable memory wait for their own stream only, so neither species'
     //    uploads wait for the other's kernels.
     SpeciesHost H[2];
-    side_by_side([&]() { species_prep(b, 0, H[0]); }, [&]() { species_prep(b, 1, H[1]); });
+    side_by_side([&]() { species_prep(b, 0, H[0]); }, [&]() { species_prep(b, 1, H[1]); }, small_host(b.s[0].n_sd + b.s[1].n_sd));
     SideStream side;
     if ((e = side.create()) != cudaSuccess) return cuda_fail(e, "side stream");
     const cudaStream_t ss[2] = {st, side.s};
@@ -968,8 +1022,8 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
     tm.mark("species host arrays");
     for (int t = 0; t < 2; ++t) {
         AllocOn on(b, ss[t]);
-        if ((rc = species_upload(b, t, H[t], ss[t]))) return rc;
-        with_words(W, [&](auto w) { rc = lists_phase1<decltype(w)::value>(b, t, b.sbuild[t], L[t], ss[t]); });
+        if ((rc = species_upload(b, t, H[t], L[t], ss[t]))) return rc;
+        with_words(W, [&](auto w) { rc = lists_phase1<decltype(w)::value>(b, t, b.sbuild[t], H[t], L[t], ss[t]); });
         if (rc) return rc;
     }
     tm.mark("species queued");
