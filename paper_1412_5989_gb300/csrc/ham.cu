@@ -57,7 +57,8 @@ struct FillArgs {
     int sharded;              // 1: col / val hold only the rows from shard_row on (positions
     int64_t shard_row;        //    relative to rowptr[shard_row], nnz = that shard's count)
     const double *t1;         // one-body table (OneBodyLayout) in place of the orbital energies, or null
-};
+    int split;                // the row kernel makes its sums in k_fill1's order (basis of kPrepareMin rows or
+};                            //   more, fewer than kFillSets sets): a fill's bits do not depend on its rows
 
 // The tables of up to four sets prepared for the fill (k_fill_prep), all in one
 // allocation, every entry the KV values of the sets together (KV = 1, 2 or 4):
@@ -502,8 +503,8 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
         nslow = 0;
         return;
     }
-    if (MODE == 1 && !EM && F.K < kFillSets) {
-        // few sets: an element's terms over the other species' particles (a lane
+    if (MODE == 1 && !EM && F.split) {
+        // k_fill1's order: an element's terms over the other species' particles (a lane
         // each, summed as a tree) and over its own species' spectators (loaded a
         // lane each, summed ascending after the one-body term): the sums of k_fill1
         const int Zp = B.nZ[0], Zn = B.nZ[1], gsz = term_lanes(Zp, Zn), per = 32 / gsz;
@@ -745,8 +746,8 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
                 if (lane == 0 && rowlen > 0) R.col[0] = (int32_t)row;
                 __syncwarp();
             }
-            const bool split = MODE == 1 && !EM && F.K < kFillSets;
-            if (split) {                                     // the sums and their order of k_fill1
+            const bool split = MODE == 1 && !EM && F.split;
+            if (split) {                                     // k_fill1's order
                 const int P = term_lanes(Zpro, Zneu), sub = lane / P, j = lane % P;
                 for (int k = 0; k < (K1 ? 1 : F.K); ++k) {
                     DF acc = df_of(0.f);
@@ -1812,7 +1813,7 @@ int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, con
 {
     const int vec4 = interleaved && K % 4 == 0 && ((uintptr_t)tbme & 15) == 0 && (!em || ((uintptr_t)val & 15) == 0);
     FillArgs F{K, hw, tbme, interleaved ? 1 : b.layout.total, interleaved ? (int64_t)K : 1, vec4, em && K > 1 ? 1 : 0,
-               esp, col, val, sharded ? 1 : 0, r0, t1};
+               esp, col, val, sharded ? 1 : 0, r0, t1, K < kFillSets && b.dim >= kPrepareMin ? 1 : 0};
     const int64_t rend = r1 < 0 ? b.dim : r1;
     if (K == 1 && work && b.dim > 0 && rend > r0)
         return launch_fill1(b, 1, rowptr, F, work_at(b, const_cast<float *>(work), 1, 0, 1), st, false, r0, rend);
