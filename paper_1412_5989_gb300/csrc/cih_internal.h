@@ -158,9 +158,11 @@ struct SpeciesBuild {
     int32_t n_sd, n_orb, Nsub_max;
     const int32_t *hash;        // open-addressing table of sub-det indices, -1 = empty
     uint32_t hash_mask;         // capacity - 1 (power of two)
-    const uint64_t *bitsT;      // W x n_sd: the bit strings word-major (coalesced scans)
+    const uint64_t *fold;       // exclusive or of the words of each bit string (W > 1)
     const int32_t *orb_upto;    // [N]: orbitals with shell <= N (orbitals are ordered by shell)
     int32_t maxN;               // highest orbital shell
+    const uint8_t *keep;        // [(2M + mtop) * (Nsub_max + 1) + N]: some sub-det has these
+    int32_t mtop;
 };
 
 // ---------------------------------------------------------------- host side

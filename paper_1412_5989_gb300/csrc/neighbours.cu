@@ -23,11 +23,21 @@ namespace {
 
 
 
+// (base is 256-byte aligned: strings of two and four words load 16 bytes at a time)
 template <int W>
 __device__ __forceinline__ void load_bits(const uint64_t *base, int64_t i, uint64_t (&o)[W])
 {
+    if constexpr (W == 1) {
+        o[0] = __ldg(base + i);
+    } else {
+        const ulonglong2 *b = reinterpret_cast<const ulonglong2 *>(base) + i * (W / 2);
 #pragma unroll
-    for (int w = 0; w < W; ++w) o[w] = base[i * W + w];
+        for (int w = 0; w < W / 2; ++w) {
+            const ulonglong2 v = __ldg(b + w);
+            o[2 * w] = v.x;
+            o[2 * w + 1] = v.y;
+        }
+    }
 }
 
 template <int W>
@@ -63,7 +73,8 @@ __device__ int find_subdet(const SpeciesBuild &S, const uint64_t (&yb)[W])
     for (uint32_t probe = 0; probe <= S.hash_mask; ++probe) {
         const int32_t x = S.hash[h];
         if (x < 0) return -1;
-        const uint64_t *xb = S.bits + (int64_t)x * W;
+        uint64_t xb[W];
+        load_bits<W>(S.bits, x, xb);
         bool eq = true;
 #pragma unroll
         for (int w = 0; w < W; ++w) eq &= xb[w] == yb[w];
@@ -71,6 +82,24 @@ __device__ int find_subdet(const SpeciesBuild &S, const uint64_t (&yb)[W])
         h = (h + 1) & S.hash_mask;
     }
     return -1;
+}
+
+// bit k of a string, and the string with bit k flipped (word selects instead of
+// indexed words, which would put the string into local memory)
+template <int W>
+__device__ __forceinline__ bool has_bit(const uint64_t (&x)[W], int k)
+{
+    uint64_t v = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) v = w == (k >> 6) ? x[w] : v;
+    return (v >> (k & 63)) & 1;
+}
+
+template <int W>
+__device__ __forceinline__ void flip_bit(uint64_t (&x)[W], int k)
+{
+#pragma unroll
+    for (int w = 0; w < W; ++w) x[w] ^= w == (k >> 6) ? 1ull << (k & 63) : 0ull;
 }
 
 template <int W>
@@ -174,10 +203,10 @@ __global__ void k_split(SpeciesBuild S, int base, int N0, int NL, const int32_t 
                     const int s1 = (count_below<W>(R, b1) + count_below<W>(R, d1)) & 1;
                     tb[slot] = ~(int32_t)(b1 | (d1 << 8) | (s1 << 16));
                 } else {
-                    int a1 = low_bit<W>(dx); dx[a1 >> 6] &= ~(1ull << (a1 & 63));
-                    int a2 = low_bit<W>(dx);
-                    int c1 = low_bit<W>(dy); dy[c1 >> 6] &= ~(1ull << (c1 & 63));
-                    int c2 = low_bit<W>(dy);
+                    const int a1 = low_bit<W>(dx), c1 = low_bit<W>(dy);
+                    flip_bit<W>(dx, a1);
+                    flip_bit<W>(dy, c1);
+                    const int a2 = low_bit<W>(dx), c2 = low_bit<W>(dy);
                     int sg = (count_below<W>(R, a1) + count_below<W>(R, a2) + count_below<W>(R, c1) + count_below<W>(R, c2)) & 1;
                     int32_t e1 = pid[(base + a1) * ntot + base + a2], e2 = pid[(base + c1) * ntot + base + c2];
                     if (e1 < 0 || e2 < 0 || ((e1 ^ e2) & (0xFFF << 16))) {
@@ -402,132 +431,204 @@ __global__ void k_row_p(int64_t np, const int64_t *rowbase, const int32_t *nb, c
 // Single-pass forward lists: sub-det x at rank r of a class [cb, ce) of size
 // m has room for m - r - 1 entries at stage offset
 //   class_stage[c] + r (m - 1) - r (r - 1) / 2,
-// written in ascending order; cnt[x] gets the count.
+// written in ascending order; cnt[x] gets the count.  One warp per sub-det, lanes
+// over the later class members.  Strings of several words are first compared by
+// their words' exclusive or (S.fold): folding can only lower the count of
+// differing bits, so what it rejects (most) needs no full comparison; the rest
+// queues up in shared memory and is compared in full 32 at a time.  Bound by
+// the instructions of the comparisons: 288 us for a species of 4+4 Nmax=6 with
+// two words compared for every member, 192 us with one.
 template <int W>
-__global__ void k_forward_staged(SpeciesBuild S, const int32_t *cls_of, const int64_t *class_stage, int64_t *cnt,
-                                 int32_t *stage)
+__global__ void __launch_bounds__(256) k_forward_staged(SpeciesBuild S, const int32_t *cls_of, const int64_t *class_stage, int64_t *cnt,
+                                                        int32_t *stage)
 {
-    int lane = threadIdx.x & 31;
+    __shared__ int32_t queue[8][64];
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1;
+    int32_t *q = queue[threadIdx.x >> 5];
     int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t x = warp; x < S.n_sd; x += nwarps) {
         uint64_t bx[W];
         load_bits<W>(S.bits, x, bx);
+        uint64_t fx = 0;
+#pragma unroll
+        for (int w = 0; w < W; ++w) fx ^= bx[w];
         const int c = cls_of[x];
         const int64_t cb = S.cls_begin[c], m = S.cls_endc[c] - cb, r = x - cb;
         int32_t *out = stage + class_stage[c] + r * (m - 1) - r * (r - 1) / 2;
         const int end = S.cls_end[x];
         int64_t pos = 0;
-        for (int y0 = (int)x + 1; y0 < end; y0 += 32) {
-            const int y = y0 + lane;
+        int nq = 0;
+        auto compare = [&](int n) {                            // the first n queued members
             bool hit = false;
-            if (y < end) {                               // word-major copy: the warp's reads coalesce
+            int y = 0;
+            if (lane < n) {
+                y = q[lane];
+                uint64_t by[W];
+                load_bits<W>(S.bits, y, by);
                 int d = 0;
 #pragma unroll
-                for (int w = 0; w < W; ++w) d += __popcll(bx[w] ^ S.bitsT[(int64_t)w * S.n_sd + y]);
+                for (int w = 0; w < W; ++w) d += __popcll(bx[w] ^ by[w]);
                 hit = d <= 4;
             }
             const unsigned msk = __ballot_sync(0xffffffffu, hit);
-            if (hit) out[pos + __popc(msk & ((1u << lane) - 1))] = y;
+            if (hit) out[pos + __popc(msk & lt)] = y;
             pos += __popc(msk);
+        };
+#pragma unroll 2
+        for (int y0 = (int)x + 1; y0 < end; y0 += 32) {
+            const int y = y0 + lane;
+            const bool near = y < end && __popcll(fx ^ (W == 1 ? __ldg(S.bits + y) : __ldg(S.fold + y))) <= 4;
+            const unsigned msk = __ballot_sync(0xffffffffu, near);
+            if (W == 1) {                                      // the fold is the string
+                if (near) out[pos + __popc(msk & lt)] = y;
+                pos += __popc(msk);
+                continue;
+            }
+            if (near) q[nq + __popc(msk & lt)] = y;
+            nq += __popc(msk);
+            __syncwarp();
+            if (nq >= 32) {
+                compare(32);
+                nq -= 32;
+                __syncwarp();
+                const int32_t k = lane < nq ? q[32 + lane] : 0;
+                __syncwarp();
+                if (lane < nq) q[lane] = k;
+                __syncwarp();
+            }
         }
+        if (nq > 0) compare(nq);
         if (lane == 0) cnt[x] = pos;
+        __syncwarp();
     }
 }
 
-// bitsT[w * n + x] = bits[x * W + w]
-__global__ void k_bits_T(int64_t n, int W, const uint64_t *bits, uint64_t *bitsT)
+// fold[x] = exclusive or of the words of x's bit string
+__global__ void k_fold(int64_t n, int W, const uint64_t *bits, uint64_t *fold)
 {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n * W; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t x = t / W;
-        const int w = (int)(t - x * W);
-        bitsT[(int64_t)w * n + x] = bits[t];
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
+        uint64_t f = 0;
+        for (int w = 0; w < W; ++w) f ^= bits[x * W + w];
+        fold[x] = f;
     }
 }
 
 // Single-pass one-move lists: each sub-det writes its moves (unsorted) into
-// a slot of `cap` entries; cnt[x] gets the count.
+// a slot of `cap` entries; cnt[x] gets the count.  One warp per sub-det: the
+// moves (r, a) whose image has the (2M, N) of some sub-det (S.keep; about one in
+// four does) queue up in shared memory, and the hash look-ups, two dependent
+// reads each, run for 32 of them at a time: 343 us a species at 4+4 Nmax=6 with a
+// look-up for every free target orbital, most lanes idle, 269 us so.
+constexpr int kMoveQueue = 64;
+
 template <int W>
-__global__ void k_onemove_staged(SpeciesBuild S, int cap, int64_t *cnt, int32_t *stage)
+__global__ void __launch_bounds__(256) k_onemove_staged(SpeciesBuild S, int cap, int64_t *cnt, int32_t *stage)
 {
-    int lane = threadIdx.x & 31;
+    __shared__ uint16_t queue[8][kMoveQueue];
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1;
+    uint16_t *q = queue[threadIdx.x >> 5];
     int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t x = warp; x < S.n_sd; x += nwarps) {
         uint64_t bx[W];
         load_bits<W>(S.bits, x, bx);
-        const int Nx = S.N[x];
+        const int Nx = S.N[x], Mx = S.M2[x];
         int32_t *out = stage + x * (int64_t)cap;
-        int pos = 0;
+        int pos = 0, nq = 0;
+        auto look_up = [&](int n) {                            // the first n queued moves
+            int found = -1;
+            if (lane < n) {
+                const int r = q[lane] & 0xFF, a = q[lane] >> 8;
+                uint64_t yb[W];
+#pragma unroll
+                for (int v = 0; v < W; ++v) yb[v] = bx[v];
+                flip_bit<W>(yb, r);
+                flip_bit<W>(yb, a);
+                found = find_subdet<W>(S, yb);
+            }
+            const unsigned msk = __ballot_sync(0xffffffffu, found >= 0);
+            if (found >= 0) out[pos + __popc(msk & lt)] = found;
+            pos += __popc(msk);
+        };
+#pragma unroll
         for (int w = 0; w < W; ++w) {
             uint64_t occ = bx[w];
             while (occ) {
                 const int r = w * 64 + __ffsll((long long)occ) - 1;
                 occ &= occ - 1;
-                const int Nr = S.oN[r];
+                const int Nr = S.oN[r], Mr = S.om2[r];
                 // targets a with Nx - Nr + N_a <= Nsub_max: a prefix of the shell-ordered orbitals
                 const int lim = S.Nsub_max - Nx + Nr;
                 const int aend = lim < 0 ? 0 : lim >= S.maxN ? S.n_orb : S.orb_upto[lim];
                 for (int a0 = 0; a0 < aend; a0 += 32) {
                     const int a = a0 + lane;
-                    int found = -1;
-                    if (a < aend && !((bx[a >> 6] >> (a & 63)) & 1) && Nx - Nr + S.oN[a] <= S.Nsub_max) {
-                        uint64_t yb[W];
-#pragma unroll
-                        for (int v = 0; v < W; ++v) yb[v] = bx[v];
-                        yb[r >> 6] &= ~(1ull << (r & 63));
-                        yb[a >> 6] |= 1ull << (a & 63);
-                        found = find_subdet<W>(S, yb);
+                    bool ok = false;
+                    if (a < aend && !has_bit<W>(bx, a)) {
+                        const int Ny = Nx - Nr + S.oN[a], k = Mx - Mr + S.om2[a] + S.mtop;
+                        ok = Ny >= 0 && Ny <= S.Nsub_max && k >= 0 && k <= 2 * S.mtop && S.keep[k * (S.Nsub_max + 1) + Ny];
                     }
-                    const unsigned msk = __ballot_sync(0xffffffffu, found >= 0);
-                    if (found >= 0) out[pos + __popc(msk & ((1u << lane) - 1))] = found;
-                    pos += __popc(msk);
+                    const unsigned msk = __ballot_sync(0xffffffffu, ok);
+                    if (ok) q[nq + __popc(msk & lt)] = (uint16_t)(r | a << 8);
+                    nq += __popc(msk);
+                    __syncwarp();
+                    if (nq >= 32) {
+                        look_up(32);
+                        nq -= 32;
+                        __syncwarp();
+                        const uint16_t m = lane < nq ? q[32 + lane] : 0;
+                        __syncwarp();
+                        if (lane < nq) q[lane] = m;
+                        __syncwarp();
+                    }
                 }
             }
         }
+        if (nq > 0) look_up(nq);
         if (lane == 0) cnt[x] = pos;
+        __syncwarp();
     }
 }
 
-// one block per list: bitonic sort of the staged moves in shared memory,
-// written compact at off[x]
-__global__ void k_onemove_compact_sort(int64_t n, int cap, const int64_t *off, const int32_t *stage, int32_t *out)
+// the staged moves sorted (ascending), written compact at off[x]: one warp per
+// list, bitonic in shared memory (tile entries a warp, a power of two >= cap).  The
+// lists have some 100 entries: a block to each waited at its barriers, 280 us a
+// species at 4+4 Nmax=6 against 143 us.
+__global__ void __launch_bounds__(256) k_onemove_compact_sort(int64_t n, int cap, int tile, const int64_t *off, const int32_t *stage,
+                                                              int32_t *out)
 {
-    __shared__ int32_t sh[kSortTile];
-    for (int64_t x = blockIdx.x; x < n; x += gridDim.x) {
+    extern __shared__ int32_t sort_sh[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int32_t *sh = sort_sh + wid * tile;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t x = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; x < n; x += nw) {
         const int64_t o = off[x];
         const int len = (int)(off[x + 1] - o);
         const int32_t *in = stage + x * (int64_t)cap;
-        if (len <= 32) {                          // small lists: one warp, insertion by rank
-            if (threadIdx.x < 32) {
-                const int32_t v = threadIdx.x < len ? in[threadIdx.x] : INT32_MAX;
-                int rank = 0;
-                for (int j = 0; j < len; ++j) {
-                    const int32_t u = __shfl_sync(0xffffffffu, v, j);
-                    rank += (u < v);
-                }
-                if ((int)threadIdx.x < len) out[o + rank] = v;
-            }
+        if (len <= 32) {                          // small lists: place by rank
+            const int32_t v = lane < len ? in[lane] : INT32_MAX;
+            int rank = 0;
+            for (int j = 0; j < len; ++j) rank += __shfl_sync(0xffffffffu, v, j) < v;
+            if (lane < len) out[o + rank] = v;
             continue;
         }
-        int P = 1;
+        int P = 64;
         while (P < len) P <<= 1;
-        for (int i = threadIdx.x; i < P; i += blockDim.x) sh[i] = i < len ? in[i] : INT32_MAX;
-        __syncthreads();
+        for (int i = lane; i < P; i += 32) sh[i] = i < len ? in[i] : INT32_MAX;
+        __syncwarp();
         for (int k = 2; k <= P; k <<= 1)
             for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < P; i += blockDim.x) {
-                    const int l = i ^ j;
-                    if (l > i) {
-                        const bool up = (i & k) == 0;
-                        const int32_t a = sh[i], c = sh[l];
-                        if ((a > c) == up) { sh[i] = c; sh[l] = a; }
-                    }
+                for (int t = lane; t < P / 2; t += 32) {       // pair t: i without bit j, and i | j
+                    const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1)), l = i | j;
+                    const int32_t a = sh[i], c = sh[l];
+                    if ((a > c) == ((i & k) == 0)) { sh[i] = c; sh[l] = a; }
                 }
-                __syncthreads();
+                __syncwarp();
             }
-        for (int i = threadIdx.x; i < len; i += blockDim.x) out[o + i] = sh[i];
-        __syncthreads();
+        for (int i = lane; i < len; i += 32) out[o + i] = sh[i];
+        __syncwarp();
     }
 }
 
@@ -634,6 +735,8 @@ struct SpeciesHost {
     std::vector<int32_t> cls_end, cb, ce, cls_of;
     std::vector<int64_t> class_stage;         // staged forward lists: first slot of each class
     int64_t fw_stage = 0;                     // and their total
+    std::vector<uint8_t> keep;                // (2M + mtop, N): some sub-det has it
+    int mtop = 0;
 };
 
 // Neighbour lists of one species, in three phases so that both species'
@@ -686,7 +789,14 @@ int lists_phase2(cih_basis &b, int t, SpeciesBuild &S, Lists &L, cudaStream_t st
     if ((rc = dev_alloc(b, &L.n1, L.tot[1])) || (rc = dev_alloc(b, &self, n))) return rc;
     if (n > 0) {
         count_launches(2);
-        k_onemove_compact_sort<<<(int)std::min<int64_t>(n, 65535), 256, 0, st>>>(n, L.cap1, L.cnt_n1, L.n1_st, L.n1);
+        int tile = 64;
+        while (tile < L.cap1) tile <<= 1;
+        const int wpb = std::min(8, 32768 / tile);              // at most 128 KB of shared memory a block
+        const size_t sh = sizeof(int32_t) * (size_t)tile * wpb;
+        const cudaError_t e = cudaFuncSetAttribute(k_onemove_compact_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 << 10);
+        if (e != cudaSuccess) return cuda_fail(e, "sort shared memory");
+        k_onemove_compact_sort<<<(int)std::min<int64_t>((n + wpb - 1) / wpb, 152 * 16), 32 * wpb, sh, st>>>(n, L.cap1, tile, L.cnt_n1,
+                                                                                                          L.n1_st, L.n1);
         k_n1_self<<<L.grid, 256, 0, st>>>(n, L.cnt_n1, L.n1, self);
     }
     dev_free(b, L.n1_st);
@@ -741,6 +851,9 @@ void species_prep(const cih_basis &b, int t, SpeciesHost &H)
     H.ce.assign(s.cls_end.begin(), s.cls_end.end());
     H.oN.assign(s.oN.begin(), s.oN.end());
     H.om2.assign(s.om2.begin(), s.om2.end());
+    for (int m : s.cls_M2) H.mtop = std::max(H.mtop, std::abs(m));
+    H.keep.assign((size_t)(2 * H.mtop + 1) * (s.Nsub_max + 1), 0);
+    for (int64_t i = 0; i < s.n_sd; ++i) H.keep[(size_t)(s.M2[i] + H.mtop) * (s.Nsub_max + 1) + s.N[i]] = 1;
     H.cls_of.resize(std::max<int64_t>(s.n_sd, 1));
     H.class_stage.resize(std::max<size_t>(s.cls_begin.size(), 1));
     for (size_t c = 0; c < s.cls_begin.size(); ++c) {
@@ -759,6 +872,7 @@ int species_upload(cih_basis &b, int t, const SpeciesHost &H, Lists &L, cudaStre
     uint64_t *d_bits; int8_t *d_N; int16_t *d_M2; int32_t *d_cls_end, *d_cb, *d_ce;
     int8_t *d_oN; int16_t *d_om2;
     int32_t *d_upto;
+    uint8_t *d_keep;
     int maxN = 0;
     for (int a = 0; a < s.n_orb; ++a) maxN = std::max(maxN, s.oN[a]);
     std::vector<int32_t> upto(maxN + 1, 0);
@@ -776,6 +890,7 @@ int species_upload(cih_basis &b, int t, const SpeciesHost &H, Lists &L, cudaStre
     up.add(&d_oN, H.oN);
     up.add(&d_om2, H.om2);
     up.add(&d_upto, upto);
+    up.add(&d_keep, H.keep);
     up.add(&L.d_cls_of, H.cls_of);
     up.add(&L.d_class_stage, H.class_stage);
     if ((rc = up.flush())) return rc;
@@ -799,14 +914,18 @@ int species_upload(cih_basis &b, int t, const SpeciesHost &H, Lists &L, cudaStre
         return cuda_fail(cudaGetLastError(), "hash table");
     S.hash = table;
     S.hash_mask = cap - 1;
-    uint64_t *bitsT;
-    if ((rc = dev_alloc(b, &bitsT, std::max<size_t>((size_t)s.n_sd * W, 1)))) return rc;
-    if (s.n_sd > 0) {
-        count_launches(1);
-        k_bits_T<<<grid_for(((int64_t)s.n_sd * W + 31) / 32), 256, 0, st>>>(s.n_sd, W, d_bits, bitsT);
+    uint64_t *fold = nullptr;
+    if (W > 1) {
+        if ((rc = dev_alloc(b, &fold, s.n_sd))) return rc;
+        if (s.n_sd > 0) {
+            count_launches(1);
+            k_fold<<<(int)std::min<int64_t>((s.n_sd + 255) / 256, 65535), 256, 0, st>>>(s.n_sd, W, d_bits, fold);
+        }
     }
-    S.bitsT = bitsT;
+    S.fold = fold;
     S.orb_upto = d_upto;
+    S.keep = d_keep;
+    S.mtop = H.mtop;
     S.maxN = maxN;
     const int hg = (int)std::min<int64_t>((s.n_sd + 255) / 256 + 1, 65535);
     count_launches(1);
