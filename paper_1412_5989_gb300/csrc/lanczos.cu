@@ -88,37 +88,88 @@ struct RowRange {
 // Lanczos vectors have ||x|| = 1.  Each product, an FP32 pair, enters as its
 // rounded hi plus its rounded lo: at most one unit 2^-s of absolute error.
 
-// partial[blk] = this block's sum of the squares of the strictly-upper
-// values of all sets (a warp per row, lanes over (nonzero, set) pairs), in
-// double-float sums of the exact FP32-pair squares
-constexpr int kSumsqThreads = 1024;
+// partial[blk] = this block's sum of the squares of the strictly-upper values of
+// all sets, in double-float sums of the exact FP32-pair squares.  A warp takes R
+// rows at a time and streams their values, whatever row they are of, 512 at a
+// time: four float4 a lane, the next four in flight while these are summed; the K
+// values of a row's first element, the diagonal, are set to zero where they fall
+// into the stretch.  Bound by HBM and the latency at each change of rows.  A loop
+// over each row with one float a lane and load took, at 4+4 Nmax=6, 0.93 ms
+// (4.0 TB/s) against 0.82 ms, and at 64 sets of 3+4 Nmax=4 0.68 against 0.41 ms; runs of
+// equal length for all warps, found by a search, 0.23 ms there but 1.11 ms for one set.
+// R = 8 / K rows (at least one): 4 to 16 for one set are alike, 31 leave warps idle.
+// Blocks beyond gridDim.x have no part: their partials are zero.
+constexpr int kSumsqThreads = 1024, kSumsqGrid = 152;              // one block an SM, 32 warps
 __global__ void __launch_bounds__(kSumsqThreads) k_upper_sumsq(RowRange rr, int K, const int64_t *rowptr,
                                                                const float *vem, double *partial)
 {
     __shared__ double red[kSumsqThreads / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    DF acc = df_of(0.f);
-    for (int64_t i = rr.r0 + blockIdx.x * (int64_t)(blockDim.x >> 5) + wid; i < rr.r1;
-         i += (int64_t)gridDim.x * (blockDim.x >> 5)) {
-        const int64_t t1 = (rowptr[i + 1] - rr.base) * K;
-#pragma unroll 4
-        for (int64_t t = (rowptr[i] - rr.base + 1) * K + lane; t < t1; t += 32) {
-            const float v = vem[t];
-            const float p = v * v;
-            acc = df_add(acc, DF{p, fmaf(v, v, -p)});
+    const int64_t nw = (int64_t)gridDim.x * (kSumsqThreads / 32), w = blockIdx.x * (int64_t)(kSumsqThreads / 32) + wid;
+    const int64_t skip = ((uintptr_t)vem >> 2) & 3;                // floats by which vem is past a 16-byte boundary
+    const int R = max(1, 8 / K);
+    DF acc[4] = {df_of(0.f), df_of(0.f), df_of(0.f), df_of(0.f)};
+    for (int64_t i0 = rr.r0 + w * R; i0 < rr.r1; i0 += nw * R) {
+        const int64_t win = (rowptr[min(i0 + min(lane, R), rr.r1)] - rr.base) * K;      // row starts; lane R: the end
+        const int64_t lo = __shfl_sync(0xffffffffu, win, 0), hi = __shfl_sync(0xffffffffu, win, R);
+        auto load = [&](int64_t b, float4 (&x)[4]) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int64_t t = b + 128 * q + 4 * lane;
+                if (t >= lo && t + 4 <= hi) {
+                    x[q] = __ldcs(reinterpret_cast<const float4 *>(vem + t));
+                } else {
+                    x[q].x = t >= lo && t < hi ? vem[t] : 0.f;
+                    x[q].y = t + 1 >= lo && t + 1 < hi ? vem[t + 1] : 0.f;
+                    x[q].z = t + 2 >= lo && t + 2 < hi ? vem[t + 2] : 0.f;
+                    x[q].w = t + 3 >= lo && t + 3 < hi ? vem[t + 3] : 0.f;
+                }
+            }
+        };
+        float4 cur[4], next[4];
+        const int64_t b0 = ((lo + skip) & ~(int64_t)3) - skip;      // at a boundary, at most 3 before lo
+        load(b0, next);
+        for (int64_t b = b0; b < hi; b += 512) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cur[q] = next[q];
+            if (b + 512 < hi) load(b + 512, next);
+            unsigned in = __ballot_sync(0xffffffffu, lane < R && win + K > b && win < b + 512);
+            while (in) {                                            // diagonals inside the stretch
+                const int l = __ffs(in) - 1;
+                in &= in - 1;
+                const int d = (int)(__shfl_sync(0xffffffffu, win, l) - b) - 4 * lane;    // from this lane's first value
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if ((unsigned)(128 * q - d) < (unsigned)K) cur[q].x = 0.f;
+                    if ((unsigned)(128 * q + 1 - d) < (unsigned)K) cur[q].y = 0.f;
+                    if ((unsigned)(128 * q + 2 - d) < (unsigned)K) cur[q].z = 0.f;
+                    if ((unsigned)(128 * q + 3 - d) < (unsigned)K) cur[q].w = 0.f;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float v[4] = {cur[q].x, cur[q].y, cur[q].z, cur[q].w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float p = v[c] * v[c];
+                    acc[q] = df_add(acc[q], DF{p, fmaf(v[c], v[c], -p)});
+                }
+            }
         }
     }
+    DF sum = df_add(df_add(acc[0], acc[1]), df_add(acc[2], acc[3]));
     for (int d = 16; d > 0; d >>= 1) {
-        const DF o{__shfl_xor_sync(0xffffffffu, acc.hi, d), __shfl_xor_sync(0xffffffffu, acc.lo, d)};
-        acc = df_add(acc, o);
+        const DF o{__shfl_xor_sync(0xffffffffu, sum.hi, d), __shfl_xor_sync(0xffffffffu, sum.lo, d)};
+        sum = df_add(sum, o);
     }
-    if (lane == 0) red[wid] = (double)acc.hi + (double)acc.lo;
+    if (lane == 0) red[wid] = (double)sum.hi + (double)sum.lo;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
+        for (int k = 0; k < kSumsqThreads / 32; ++k) t += red[k];
         partial[blockIdx.x] = t;
     }
+    if (blockIdx.x == 0 && threadIdx.x >= gridDim.x && threadIdx.x < kSumsqBlocks) partial[threadIdx.x] = 0.0;
 }
 
 // sc = (2^s, 2^-s, 2^r, 2^-r) from the sum of squares F^2 (the kSumsqBlocks
@@ -232,14 +283,13 @@ __global__ void k_split(int64_t n, const double *x, const double *sc, float2 *xs
 // matrix is read with evict-first loads, so that its stream does not push x
 // and the accumulators out of L2 (with lanes over sets the same hint ran
 // slower).  Each block walks
-// one contiguous run of rows, so that rows of one proton sub-determinant
+// one contiguous run of `per` rows, so that rows of one proton sub-determinant
 // (which touch the same x and accumulator blocks) share its L1.
 template <int KS>
 __global__ void __launch_bounds__(kThreads, 4) k_spmv(RowRange rr, int K, const int64_t *rowptr, const int32_t *col, const float *vem,
-                       const float2 *xs, const float2 *xm, float2 *yrow, unsigned long long *yfix)
+                       const float2 *xs, const float2 *xm, float2 *yrow, unsigned long long *yfix, int64_t per)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t per = (rr.r1 - rr.r0 + gridDim.x - 1) / gridDim.x;
     const int64_t r0 = rr.r0 + blockIdx.x * per, r1 = min(rr.r1, r0 + per);
     const int wpb = blockDim.x >> 5;
     for (int64_t i = r0 + (threadIdx.x >> 5); i < r1; i += wpb) {
@@ -366,19 +416,40 @@ __global__ void k_shard_finish(int64_t n, const double *sc, double *yx, unsigned
     }
 }
 
+// Rows a block of the product takes, a multiple of its 8 warps.  Long runs share more
+// of L1, short ones leave the GPU less idle at the end, and the more sets, the
+// longer a row takes.  Measured, us a call, by rows a block (and, last, for 4,864
+// blocks of equal runs, whose 8 warps share 11, 30, 42 or 456 rows unevenly):
+//   one set:  4+4 Nmax=6   32: 5925  64: 5673  128: 5589  192: 5634   5998
+//             5+6 Nmax=4   32: 1457  64: 1414  128: 1432  192: 1472   1451
+//             4+4 Nmax=4   16:  325  32:  316   64:  322               314
+//   4 sets:   3+3 Nmax=6    8: 1072  16: 1053   32: 1110              1155
+//   8 sets:   5+6 Nmax=4    8: 6259  16: 6178   32: 6117   64: 6280   6912
+//   32 sets:  4+4 Nmax=4    8: 4986  16: 5139   32: 5512              5465
+//   64 sets:  3+4 Nmax=4    8: 1811  16: 1893   32: 2248              1975
+inline int64_t rows_per_block(int64_t rows, int K)
+{
+    const int64_t per = (rows + 4 * 4864 * (int64_t)K) / (8 * 4864 * (int64_t)K) * 8;
+    return std::max<int64_t>(8, std::min<int64_t>(per, std::max(16, 128 / K)));
+}
+
 // One product's k_spmv launch.  (Passes of 32 sets, to keep a share of the
 // randomly accessed vectors L2-resident at 64 sets, ran slower.)
 void launch_spmv(RowRange rr, int K, const int64_t *rowptr, const int32_t *col, const float *vem, const float2 *xs,
-                 const float2 *xm, float2 *yrow, unsigned long long *yfix, int gr, cudaStream_t st)
+                 const float2 *xm, float2 *yrow, unsigned long long *yfix, cudaStream_t st)
 {
+    const int64_t rows = rr.r1 - rr.r0, per = rows_per_block(rows, K);
+    const int64_t blocks = (rows + per - 1) / per;              // rows < 2^31: at most 2^28
+    if (blocks == 0) return;
+    const unsigned gr = (unsigned)blocks;
     count_launches(1);
-    if (K == 64) k_spmv<64><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
-    else if (K > 16) k_spmv<32><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
-    else if (K == 1) k_spmv<1><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
-    else if (K <= 2) k_spmv<2><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
-    else if (K <= 4) k_spmv<4><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
-    else if (K <= 8) k_spmv<8><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
-    else k_spmv<16><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix);
+    if (K == 64) k_spmv<64><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, per);
+    else if (K > 16) k_spmv<32><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, per);
+    else if (K == 1) k_spmv<1><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, per);
+    else if (K <= 2) k_spmv<2><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, per);
+    else if (K <= 4) k_spmv<4><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, per);
+    else if (K <= 8) k_spmv<8><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, per);
+    else k_spmv<16><<<gr, kThreads, 0, st>>>(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, per);
 }
 
 // ---- orthogonalisation: classical Gram-Schmidt twice, every sum in a fixed order
@@ -696,7 +767,6 @@ int lanczos(const cih_basis &b, const int64_t *rowptr, const int32_t *col, const
         if ((e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming)) != cudaSuccess) rc = cuda_fail(e, "lanczos: event");
     if (!rc && (e = prepare_dots(K)) != cudaSuccess) rc = cuda_fail(e, "lanczos: shared memory");
     const int g = grid_for(vstride);
-    const int gr = (int)std::max<int64_t>(1, std::min<int64_t>((r1 - r0 + 7) / 8, 152 * 32));
 
     // element-major values, the mirror scale and cleared accumulators (no host
     // synchronisation; a shard's scale comes from the whole matrix's norm)
@@ -717,14 +787,14 @@ int lanczos(const cih_basis &b, const int64_t *rowptr, const int32_t *col, const
         } else {
             cudaMemsetAsync(yfix, 0, sizeof(unsigned long long) * (size_t)vstride, st);
             count_launches(2);
-            k_upper_sumsq<<<kSumsqBlocks, kSumsqThreads, 0, st>>>(rr, K, rowptr, vem, partial);
+            k_upper_sumsq<<<kSumsqGrid, kSumsqThreads, 0, st>>>(rr, K, rowptr, vem, partial);
             k_mirror_scale<<<1, kSumsqBlocks, 0, st>>>(partial, K, nullptr, sc);
         }
     }
 
     // w = H v_j from the split of v_j
     auto spmv = [&]() -> int {
-        launch_spmv(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, gr, st);
+        launch_spmv(rr, K, rowptr, col, vem, xs, xm, yrow, yfix, st);
         if (!sh) {
             count_launches(1);
             k_sym_finish<<<g, kThreads, 0, st>>>(vstride, sc, yrow, w, yfix);
@@ -898,12 +968,11 @@ int ham_spmv(const cih_basis &b, const int64_t *rowptr, const int32_t *col, cons
         }
         cudaMemsetAsync(yfix, 0, sizeof(unsigned long long) * (size_t)n, st);
         count_launches(4);
-        k_upper_sumsq<<<kSumsqBlocks, kSumsqThreads, 0, st>>>(RowRange{0, dim, 0}, K, rowptr, vem, partial);
+        k_upper_sumsq<<<kSumsqGrid, kSumsqThreads, 0, st>>>(RowRange{0, dim, 0}, K, rowptr, vem, partial);
         launch_dots(kSumUnit, dim, K, 1, x, n, x, xpart, xn2, nullptr, nullptr, xf, nullptr, st);
         k_mirror_scale<<<1, kSumsqBlocks, 0, st>>>(partial, K, xn2, sc);
         k_split<<<grid_for(n), kThreads, 0, st>>>(n, x, sc, xs, xm);
-        const int gr = (int)std::min<int64_t>((dim + 7) / 8, 152 * 32);
-        launch_spmv(RowRange{0, dim, 0}, K, rowptr, col, vem, xs, xm, yrow, yfix, gr, st);
+        launch_spmv(RowRange{0, dim, 0}, K, rowptr, col, vem, xs, xm, yrow, yfix, st);
         k_sym_finish<<<grid_for(n), kThreads, 0, st>>>(n, sc, yrow, y, yfix);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "spmv kernels");
@@ -943,7 +1012,7 @@ int upper_sumsq(const cih_basis &b, const int64_t *rowptr, int64_t r0, int64_t r
         k_vals_em<<<grid_for(nnz * K), kThreads, 0, st>>>(K, nnz, val, vem);
     }
     count_launches(1);
-    k_upper_sumsq<<<kSumsqBlocks, kSumsqThreads, 0, st>>>(RowRange{r0, r1, ends[0]}, K, rowptr, vem, partial);
+    k_upper_sumsq<<<kSumsqGrid, kSumsqThreads, 0, st>>>(RowRange{r0, r1, ends[0]}, K, rowptr, vem, partial);
     std::vector<double> hp(kSumsqBlocks);
     e = cudaMemcpyAsync(hp.data(), partial, sizeof(double) * kSumsqBlocks, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
