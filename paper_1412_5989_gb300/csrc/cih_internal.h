@@ -24,7 +24,6 @@ constexpr int kLevels = 8;                // oscillator levels of a species: Nma
 // the least number of rows.
 constexpr int kWalkRun = 16;
 constexpr int64_t kWalkRows = 1 << 19;
-constexpr int64_t kPrepareMin = 4096;     // rows from which a fill of few sets prepares a working copy (ham.cu)
 constexpr uint64_t kPoolKeep = 1ull << 30; // bytes the library pool keeps after a Lanczos call
 constexpr int kSortTile = 4096;           // longest neighbour list the sort handles
 
@@ -315,12 +314,12 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
 // kernels (ham.cu)
 int launch_count(const cih_basis &b, int64_t *rowptr, cudaStream_t st);
 int launch_scan(const cih_basis &b, int64_t *rowptr, cudaStream_t st);
-// With one set (set-major) a fill over many rows first prepares a working copy
-// of the table (fill_prepare) in fill_work_floats() floats of device memory:
-// `work` when the caller gives it (already prepared), else allocated for the call
-// on the stream (unless prepare is false); without it (no memory, few rows) the
-// fill reads the table itself, with the same results.  fill_work_floats is 0 where that form does
-// not apply.
+// A fill of few sets of a large basis first prepares a working copy of the table
+// (fill_prepare; one set: fill_work_floats() floats of device memory): `work` when the
+// caller gives it (one set, already prepared), else allocated for the call on the
+// stream (unless prepare is false); without it (no memory, few of the rows) the fill
+// reads the table itself, with the same results.  fill_work_floats is 0 where that
+// form does not apply.
 size_t fill_work_floats(const cih_basis &b);
 int fill_prepare(const cih_basis &b, double hw, const float *tbme, const double *esp, const double *t1, float *work,
                  cudaStream_t st);

@@ -57,8 +57,8 @@ struct FillArgs {
     int sharded;              // 1: col / val hold only the rows from shard_row on (positions
     int64_t shard_row;        //    relative to rowptr[shard_row], nnz = that shard's count)
     const double *t1;         // one-body table (OneBodyLayout) in place of the orbital energies, or null
-    int split;                // the row kernel makes its sums in k_fill1's order (basis of kPrepareMin rows or
-};                            //   more, fewer than kFillSets sets): a fill's bits do not depend on its rows
+    int split;                // the row kernel makes its sums in k_fill1's order (fill_splits): a fill's bits
+};                            //   do not depend on its rows
 
 // The tables of up to four sets prepared for the fill (k_fill_prep), all in one
 // allocation, every entry the KV values of the sets together (KV = 1, 2 or 4):
@@ -148,16 +148,15 @@ __device__ __forceinline__ long long psi_prod(const long long *psi, int64_t i, i
 // starts at c + j (len + 1) + t, len being the level's segment.
 
 constexpr int kLaneSets = 16;     // from this many sets on, multi-term sums run with lanes over sets
-// A one-set fill prepares a working copy when it covers at least kPrepareMin rows
-// and 1 / kPrepareShare of the basis.  Measured with / without: 800 rows 25 / 21
-// us, 2,104 rows 26 / 23, 7,916 rows 37 / 41, 8,500 rows 35 / 45, 48,917 rows 113
-// / 167; at 4+4 Nmax=6 (2.2 M rows) a 1/15 share 600 / 1,130, 1/32 355 / 515, 1/64
-// 228 / 257, at 4+4 Nmax=4 a 1/17 share 55 / 59, 1/32 44 / 32.
-// Fills of fewer than kFillSets sets go through the working copy, one, two or four
-// sets a pass (three sets at 5+6 Nmax=4 with a one-body table: 2.91 ms, 6.57 ms
-// from the tables, where a one-move gathered ten entries per set and reduced them
-// in a tree).  From eight on the row kernel's element-major paths write whole lines.
+// Fills of fewer than kFillSets sets of a basis that fill_splits names go through a
+// working copy of the table, one, two or four sets a pass (three sets at 5+6 Nmax=4
+// with a one-body table: 2.91 ms, 6.57 ms from the tables, where a one-move
+// gathered ten entries per set and reduced them in a tree).  From eight sets on the row
+// kernel's element-major paths write whole lines.
 constexpr int kFillSets = 8;
+// Of such a basis, rows fewer than 1 / kPrepareShare are filled from the table.
+// Measured with / without the copy: at 4+4 Nmax=6 (2.2 M rows) a 1/15 share 600 / 1,130
+// us, 1/32 355 / 515, 1/64 228 / 257; at 4+4 Nmax=4 a 1/17 share 55 / 59, 1/32 44 / 32.
 constexpr int64_t kPrepareShare = 24;
 // Rows from which one vector's adjoint takes the form of k_grad_pairs + k_grad1
 // (row kernel / this form: 48,917 rows 156 / 205 us, 143,792 rows 396 / 389,
@@ -1789,9 +1788,29 @@ int launch_prep(const cih_basis &b, int kv, const FillArgs &F, const FillWork &W
     return e == cudaSuccess ? CIH_OK : cuda_fail(e, "fill preparation");
 }
 
+// Whether fills of K sets of this basis go through the working copy, and so make
+// their sums in its order (rows that do not pay for it in the row kernel, slower
+// there than in the order of the terms: a quarter for one set, more for several).
+// A copy costs its two launches and its entries once; each row gains.  Several sets
+// gain more a row; from five on there are two passes, and the values of
+// five to seven sets of an element, written by both, share their lines.  Measured
+// against the row kernel without this order, by rows and entries of a copy a row:
+//   one set: 4,945 rows, 50 entries 0.76x; 8,500, 15 0.95x; 13,162, 85 0.93x; 17,769,
+//     170 0.90x; 14,502, 12 1.17x; 17,040, 61 1.22x; 23,907, 54 1.07x; 39,421, 94 1.14x
+//   two, four: 4,945, 50 0.85x, 0.91x; 6,758, 425 0.88x, 0.98x; 8,500, 15 1.12x, 1.13x;
+//     10,753, 51 1.15x, 1.21x; 17,769, 170 1.06x, 1.04x
+//   seven, set-major and element-major: 23,907, 54 1.11x, 0.84x; 36,498, 18 1.31x, 0.97x;
+//     165,736, 82 1.36x, 0.93x; 48,917, 35 1.54x, 1.04x; 143,792, 18 1.98x, 1.15x
+bool fill_splits(const cih_basis &b, int K)
+{
+    const int64_t rows = K == 1 ? 16384 : K <= 4 ? 8192 : 40960, entries = K == 1 ? 128 : K <= 4 ? 192 : 64;
+    return K < kFillSets && b.dim >= rows && fill1_fits(b, K == 1 ? 1 : K == 2 ? 2 : 4) &&
+           (int64_t)work_floats(b, 1) <= entries * b.dim;
+}
+
 }  // namespace
 
-size_t fill_work_floats(const cih_basis &b) { return fill1_fits(b, 1) ? work_floats(b, 1) : 0; }
+size_t fill_work_floats(const cih_basis &b) { return fill_splits(b, 1) ? work_floats(b, 1) : 0; }
 
 int fill_prepare(const cih_basis &b, double hw, const float *tbme, const double *esp, const double *t1, float *work,
                  cudaStream_t st)
@@ -1813,12 +1832,12 @@ int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, con
 {
     const int vec4 = interleaved && K % 4 == 0 && ((uintptr_t)tbme & 15) == 0 && (!em || ((uintptr_t)val & 15) == 0);
     FillArgs F{K, hw, tbme, interleaved ? 1 : b.layout.total, interleaved ? (int64_t)K : 1, vec4, em && K > 1 ? 1 : 0,
-               esp, col, val, sharded ? 1 : 0, r0, t1, K < kFillSets && b.dim >= kPrepareMin ? 1 : 0};
+               esp, col, val, sharded ? 1 : 0, r0, t1, fill_splits(b, K) ? 1 : 0};
     const int64_t rend = r1 < 0 ? b.dim : r1;
     if (K == 1 && work && b.dim > 0 && rend > r0)
         return launch_fill1(b, 1, rowptr, F, work_at(b, const_cast<float *>(work), 1, 0, 1), st, false, r0, rend);
     const int kv = K == 1 ? 1 : K == 2 ? 2 : 4;                // sets of one pass
-    if (K < kFillSets && !work && prepare && rend - r0 >= kPrepareMin && (rend - r0) * kPrepareShare >= b.dim && fill1_fits(b, kv)) {
+    if (F.split && !work && prepare && rend > r0 && (rend - r0) * kPrepareShare >= b.dim) {
         float *own = nullptr;
         if (cudaMallocFromPoolAsync((void **)&own, work_floats(b, kv) * sizeof(float), b.pool, st) == cudaSuccess) {
             int rc = CIH_OK;

@@ -15,8 +15,9 @@ pytestmark = pytest.mark.gpu
 
 SPACES = [(3, 0, 4, 1), (0, 4, 3, 0), (1, 1, 5, 0), (1, 4, 3, 1), (4, 1, 3, 1), (2, 6, 2, 0), (6, 2, 2, 0), (3, 3, 2, 4),
           (2, 2, 5, 0), (5, 6, 1, 1), (9, 3, 1, 0), (1, 0, 5, 1), (2, 3, 0, 1),
-          # from 4,096 rows on the copy is prepared
-          (4, 4, 2, 0), (1, 2, 7, 1), (2, 6, 3, 4), (6, 2, 3, 4), (2, 2, 6, 4), (0, 4, 6, 0), (4, 0, 6, 0)]
+          (4, 4, 2, 0), (1, 2, 7, 1), (2, 6, 3, 4), (6, 2, 3, 4), (2, 2, 6, 4), (0, 4, 6, 0), (4, 0, 6, 0),
+          # large enough for the copy to be prepared
+          (3, 3, 4, 0), (2, 5, 4, 1), (5, 2, 4, 1)]
 
 
 @pytest.fixture(scope="module")
@@ -60,12 +61,14 @@ def test_prepared_fill(cih, space, energies):
     assert np.all(np.abs(got - val_o) <= 1e-5 * (np.abs(val_o) + 1.0))
 
 
-@pytest.mark.parametrize("space", [(3, 3, 2, 0), (4, 4, 2, 0), (2, 6, 3, 4), (4, 0, 6, 0)])
+@pytest.mark.parametrize("space", [(3, 3, 2, 0), (4, 4, 2, 0), (2, 6, 3, 4), (4, 0, 6, 0), (4, 5, 2, 1), (3, 3, 4, 0),
+                                   (3, 4, 4, 1)])
 @pytest.mark.parametrize("K", [2, 3, 4, 5, 7])
 def test_few_sets(cih, space, K):
     """Fewer than eight sets: passes of up to four sets through the working copy.
-    Each set has the bits of its own one-set fill, in every layout and from
-    shards of a few rows."""
+    The bits are the same in every layout and from shards of a few rows; where the
+    copy is prepared for these sets and not for one, or the other way round, a
+    set's sums have another order than its own one-set fill's."""
     B = cih.Basis(*space)
     T = torch.from_numpy(synth.tbme_tables(B.tbme_len, range(K))).cuda()
     e = torch.from_numpy(synth.single_particle_energies(sum(B.n_orb), 3)).cuda()
@@ -73,7 +76,10 @@ def test_few_sets(cih, space, K):
     col, val = B.fill(rowptr, nnz, T, e_sp=e)
     for k in range(K):
         c1, v1 = B.fill(rowptr, nnz, T[k], e_sp=e)
-        assert torch.equal(c1, col) and torch.equal(v1[0], val[k])
+        assert torch.equal(c1, col)
+        if B.dim < 8192:
+            assert torch.equal(v1[0], val[k])
+        assert bool(((v1[0] - val[k]).abs() <= 1e-6 * (val[k].abs() + 1.0)).all())
     til = cih.tbme_interleave(T)
     c2, v2 = B.fill_interleaved(rowptr, nnz, til, K, e_sp=e)
     c3, v3 = B.fill_batched(rowptr, nnz, til, K, e_sp=e)
@@ -89,7 +95,7 @@ def test_few_sets(cih, space, K):
 def test_prepared_fill_in_a_graph(cih):
     """The working copy of a captured fill belongs to the graph: replays read the
     table anew."""
-    B = cih.Basis(4, 4, 2, 0)
+    B = cih.Basis(3, 3, 4, 0)
     rowptr, nnz = B.count()
     T = torch.from_numpy(synth.tbme_table(B.tbme_len, 1)).cuda()
     col, val = B.fill(rowptr, nnz, T)
