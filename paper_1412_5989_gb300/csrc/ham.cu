@@ -127,7 +127,7 @@ __device__ __forceinline__ long long psi_prod(const long long *psi, int64_t i, i
 
 // ---------------------------------------------------------------- row kernel
 //
-// Warps walk rows independently (grid-stride); a CTA shares the pn index
+// Warps walk rows independently (next_row); a CTA shares the pn index
 // tables in shared memory.  For row (p, n):
 //   diagonal  - the warp sums the one-body energies and every occupied pair
 //               (lanes over pairs, double-float reduction);
@@ -154,6 +154,7 @@ constexpr int kLaneSets = 16;     // from this many sets on, multi-term sums run
 // gathered ten entries per set and reduced them in a tree).  From eight sets on the row
 // kernel's element-major paths write whole lines.
 constexpr int kFillSets = 8;
+constexpr int kTakeRuns = 4;      // runs of rows a CTA from which its warps take them from a counter (next_row)
 // Of such a basis, rows fewer than 1 / kPrepareShare are filled from the table.
 // Measured with / without the copy: at 4+4 Nmax=6 (2.2 M rows) a 1/15 share 600 / 1,130
 // us, 1/32 355 / 515, 1/64 228 / 257; at 4+4 Nmax=4 a 1/17 share 55 / 59, 1/32 44 / 32.
@@ -602,6 +603,28 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
     nslow = 0;
 }
 
+// The rows of a CTA are the runs of WARPS rows blockIdx.x, blockIdx.x + gridDim.x,
+// ... of its range; its warps take them one by one, the first run without asking,
+// the rest from a counter in shared memory (WARPS before the first call).  Rows differ
+// in length, and a warp's rows, at fixed distances, alike: with every warp taking its
+// own, the longest warp had 1.8 times the mean at 3+4 Nmax=4 (11 rows each), 1.4 at
+// 4+4 Nmax=4, 1.1 at 4+4 Nmax=6.  us, own rows / taken: one-set fill 132 / 119, 306 /
+// 290, 5,770 / 5,610 there; adjoint at 4+4 Nmax=4 375 / 344; 64 sets at 3+4 Nmax=4 849 /
+// 668.  Up to kTakeRuns runs the counter costs what it gains (5+5 Nmax=2, 14,502 rows,
+// eight sets: 199 / 207).
+template <int WARPS>
+__device__ __forceinline__ int64_t first_row(int64_t r0, int wid) { return r0 + (int64_t)blockIdx.x * WARPS + wid; }
+
+template <int WARPS>
+__device__ __forceinline__ int64_t next_row(int64_t row, int64_t r0, int64_t r1, int *counter, int lane)
+{
+    const int64_t run = (int64_t)gridDim.x * WARPS;             // rows of one run of every CTA
+    if (r1 - r0 <= kTakeRuns * run) return row + run;
+    int t = lane == 0 ? atomicAdd(counter, 1) : 0;
+    t = __shfl_sync(0xffffffffu, t, 0);
+    return r0 + (t / WARPS) * run + (int64_t)blockIdx.x * WARPS + t % WARPS;
+}
+
 template <int MODE, bool K1, int WARPS, int EM>
 __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
 k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs Gr, int64_t r0, int64_t r1,
@@ -617,6 +640,9 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
     const int T = B.pn_T;
     int2 *KG = sptr<int2>(sb, sm::kg);
     int16_t *XS = sptr<int16_t>(sb, sm::S<WARPS>);
+    __shared__ int taken;
+    if (tid == 0) taken = WARPS;
+    if (MODE == 0) __syncthreads();
     if (MODE != 0) {
         for (int i = tid; i < SP.n_orb * T; i += kThreads) XS[i] = B.pn_s[i];
         for (int i = tid; i < 64; i += kThreads) KG[i] = B.pn_k[i];
@@ -652,8 +678,6 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
     int32_t *w_spos = sptr<int32_t>(wb, sm::w_spos), *w_scol = sptr<int32_t>(wb, sm::w_scol);
     uint32_t *w_scode = sptr<uint32_t>(wb, sm::w_scode);
     int16_t *w_occ = sptr<int16_t>(wb, sm::w_occ);
-    const int64_t gw = (blockIdx.x * (int64_t)kThreads + tid) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * kThreads) >> 5;
     const int Zpro = B.nZ[0], Zneu = B.nZ[1];
     // K sets, element-major values: warp-cooperative value writes
     // (EM: the launcher chose this instantiation because F.em, F.vec4 and
@@ -661,7 +685,7 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
     // compile without these paths, and these without theirs)
     constexpr bool coop = MODE == 1 && !K1 && EM;
 
-    for (int64_t row = r0 + gw; row < r1; row += nw) {
+    for (int64_t row = first_row<WARPS>(r0, wid); row < r1; row = next_row<WARPS>(row, r0, r1, &taken, lane)) {
         const int p = B.row_p[row];
         const ProtonRec PR = B.prec[p];
         const int n = (int)(row - PR.colb);
@@ -1083,10 +1107,11 @@ constexpr int kW = 2;             // pn windows of 32 elements in flight in k_fi
 // one-moves and the diagonal the prepared own-species sum plus the terms over
 // the other species.  Reading the table itself in every row (pair lookups, a
 // gather per spectator) took 364 us at 4+4 Nmax=4 and 8.5 ms at 4+4 Nmax=6;
-// this form 298 us and 7.1 ms with its preparation.  At 3+3 Nmax=6 it issues
-// 5.6 warp instructions per stored nonzero (64 % of the issue slots; 10.9 before
-// the groups); the pn loop is 60 % of the time, waiting on L2 for the members,
-// moves and values of its windows.
+// this form 298 us and 7.1 ms with its preparation, and, with rows of 16 proton
+// sub-dets side by side and rows taken by next_row, 281 us and 5.6 ms.  At 3+3
+// Nmax=6 it issues 6.1 warp instructions per stored nonzero (70 % of the issue slots;
+// 10.9 before the groups); the pn loop is 60 % of the time, waiting on L2 for the
+// members, moves and values of its windows.
 template <int WARPS, int KV>
 __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
 k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, int64_t r1, int *status)
@@ -1099,6 +1124,8 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
     const int T = B.pn_T, Zp = B.nZ[0], Zn = B.nZ[1];
     int2 *KQ = sptr<int2>(sb, f1::kg);
     int16_t *S = sptr<int16_t>(sb, f1::S<WARPS>);
+    __shared__ int taken;
+    if (tid == 0) taken = WARPS;
     for (int i = tid; i < SP.n_orb * T; i += kThreads) S[i] = B.pn_s[i];
     for (int i = tid; i < 64; i += kThreads) KQ[i] = B.pn_kq[i];
     __syncthreads();
@@ -1127,11 +1154,9 @@ k_fill1(DevBasis B, const int64_t *rowptr, FillArgs F, FillWork W, int64_t r0, i
             if (KV == 1 || u < W.ks) __stcs(val + e * es + u * kst, __int_as_float(__float_as_int(v.v[u]) ^ sm));
     };
     const int P = term_lanes(Zp, Zn), sub = lane / P, li = lane % P, per = 32 / P;
-    const int64_t gw = (blockIdx.x * (int64_t)kThreads + tid) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * kThreads) >> 5;
 
     const bool walk = B.walk && r0 == 0 && r1 == B.dim;         // (a range of rows is taken in row order)
-    for (int64_t place = r0 + gw; place < r1; place += nw) {
+    for (int64_t place = first_row<WARPS>(r0, wid); place < r1; place = next_row<WARPS>(place, r0, r1, &taken, lane)) {
         const int2 at_row = walk ? B.walk[place] : make_int2(B.row_p[place], (int)place);
         const int p = at_row.x;
         const int64_t row = at_row.y;
@@ -1469,6 +1494,8 @@ k_grad1(DevBasis B, const long long *psi, unsigned long long *acc)
     const int T = B.pn_T, Zp = B.nZ[0], Zn = B.nZ[1];
     int2 *KG = sptr<int2>(sb, f1::kg);
     int16_t *S = sptr<int16_t>(sb, f1::S<WARPS>);
+    __shared__ int taken;
+    if (tid == 0) taken = WARPS;
     for (int i = tid; i < SP.n_orb * T; i += kThreads) S[i] = B.pn_s[i];
     for (int i = tid; i < 64; i += kThreads) KG[i] = B.pn_kq[i];
     __syncthreads();
@@ -1477,13 +1504,11 @@ k_grad1(DevBasis B, const long long *psi, unsigned long long *acc)
     int *w_s0 = sptr<int>(wb, f1::w_ext);
     int *w_op = sptr<int>(wb, f1::w_op), *w_on = sptr<int>(wb, f1::w_on);
     const int P = term_lanes(Zp, Zn), sub = lane / P, li = lane % P, per = 32 / P;
-    const int64_t gw = (blockIdx.x * (int64_t)kThreads + tid) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * kThreads) >> 5;
     auto add = [&](int l1, int n1, long long q) {
         const int idx = pn_square_at(KG, S, T, l1, n1);
         atomicAdd(acc + idx, (unsigned long long)(((l1 >> 16) ^ (n1 >> 26)) & 1 ? -q : q));
     };
-    for (int64_t place = gw; place < B.dim; place += nw) {
+    for (int64_t place = first_row<WARPS>(0, wid); place < B.dim; place = next_row<WARPS>(place, 0, B.dim, &taken, lane)) {
         const int2 at_row = B.walk ? B.walk[place] : make_int2(B.row_p[place], (int)place);
         const int p = at_row.x;
         const int64_t row = at_row.y;
