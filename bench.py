@@ -546,7 +546,7 @@ def run_ours(args, rank, world, local_rank):
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_source": f"{peak_kind} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"
                 if peak_kind == "measured" else "fallback 6.8 TB/s",
-                "kernel": "k_rows<W,1,K1> (fill)" if K == 1 else f"k_rows<W,1> (batched fill, K={K})",
+                "kernel": "k_fill_prep + k_fill1 (fill)" if K == 1 else f"k_rows<W,1> (batched fill, K={K})",
                 "algorithmic_bytes_per_launch": nnz_s * bytes_per_nnz,
                 "traffic": fill_traffic(kernel_source_sha()) if (args.workload == "4p4n_nmax6" and K == 1
                                                                   and not sharded) else None,
