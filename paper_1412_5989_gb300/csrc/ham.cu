@@ -1967,7 +1967,7 @@ int launch_grad1_w(const cih_basis &b, const long long *psi, unsigned long long 
 
 size_t grad_pairs_bytes(const cih_basis &b)
 {
-    if (b.dim < kGradPairsMin || fill_work_floats(b) == 0) return 0;
+    if (b.dim < kGradPairsMin || !fill1_fits(b, 1)) return 0;
     const DevBasis &D = b.dev;
     const int64_t np = b.s[0].n_sd, nn = b.s[1].n_sd;
     // 8-byte arrays: neutron-major vector, neutron run starts, proton counts, scan
