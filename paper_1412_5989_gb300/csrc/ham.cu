@@ -30,6 +30,7 @@
 // spectators k in R in ascending combined order.  Proton and neutron moves
 // of a pn element factorise (the cross-species counts cancel in pairs).
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <map>
 #include <mutex>
@@ -57,8 +58,8 @@ struct FillArgs {
     int sharded;              // 1: col / val hold only the rows from shard_row on (positions
     int64_t shard_row;        //    relative to rowptr[shard_row], nnz = that shard's count)
     const double *t1;         // one-body table (OneBodyLayout) in place of the orbital energies, or null
-    int split;                // the row kernel makes its sums in k_fill1's order (fill_splits): a fill's bits
-};                            //   do not depend on its rows
+    float tol_one, tol_diag;  // split order (fill_splits): see near_tie
+};
 
 // The tables of up to four sets prepared for the fill (k_fill_prep), all in one
 // allocation, every entry the KV values of the sets together (KV = 1, 2 or 4):
@@ -155,10 +156,6 @@ constexpr int kLaneSets = 16;     // from this many sets on, multi-term sums run
 // kernel's element-major paths write whole lines.
 constexpr int kFillSets = 8;
 constexpr int kTakeRuns = 4;      // runs of rows a CTA from which its warps take them from a counter (next_row)
-// Of such a basis, rows fewer than 1 / kPrepareShare are filled from the table.
-// Measured with / without the copy: at 4+4 Nmax=6 (2.2 M rows) a 1/15 share 600 / 1,130
-// us, 1/32 355 / 515, 1/64 228 / 257; at 4+4 Nmax=4 a 1/17 share 55 / 59, 1/32 44 / 32.
-constexpr int64_t kPrepareShare = 24;
 // Rows from which one vector's adjoint takes the form of k_grad_pairs + k_grad1
 // (row kernel / this form: 48,917 rows 156 / 205 us, 143,792 rows 396 / 389,
 // 197,822 rows 676 / 681, 814,092 rows 2,898 / 2,319, 2.2 M rows 8,082 / 6,200)
@@ -394,16 +391,152 @@ __device__ __forceinline__ DF diag_own(const DevBasis &B, const int2 *lg, const 
     return warp_sum(acc, 32);
 }
 
+// k_fill1 makes the sums of several terms in another order than the row kernel: per
+// species, then together.  A double-float sum of terms that do not fit its 48 bits
+// depends on the order by an amount far below the FP32 result's last bit, so the
+// rounded results differ only where the sum lies that close to the middle of two
+// floats (near_tie) and is not exact (exact_sum).  Those sums, some in ten thousand,
+// the row kernel makes again in k_fill1's order on the bases whose fills of all rows
+// go through k_fill1 (SPLIT): a fill's bits do not depend on its rows, on scratch or
+// on a capture.  (All of them in that order cost a quarter of the time with one
+// set, 40 % with seven.)
+//
+// How close: with u = 2^-24 and T the sum of the terms' magnitudes below a
+// df_add, its operands' low parts are at most 2 u T and its own error (two rounded
+// additions, and the fast two-sum where the high parts cancel) at most 12 u^2 T, so
+// an order in which no term goes through more than D additions errs by at most
+// 12 D u^2 T, and two orders differ by the sum of theirs (split_tolerances); 16 instead
+// of 12 also covers the rounding of T and of the test itself.
+
+// whether a sum within tol x mag of s may round to another float (NaN: yes)
+__device__ __forceinline__ bool near_tie(DF s, float mag, float tol)
+{
+    const float r = df_round(s), e = mag * tol;
+    return !(s.hi + (s.lo + e) == r && s.hi + (s.lo - e) == r);
+}
+
+// Whether every sum of the terms, in any order, is exact: the terms are multiples of
+// g = the last bit of the smallest (at least 2^-24 of it), so with T <= 2^46 g a
+// partial sum's high part has a last bit of at most 2^23 g, and the low parts
+// stay integers below 2^24.  (Of the sums of some seven FP32 numbers of the same
+// size a few per cent are exactly half-way.)
+__device__ __forceinline__ bool exact_sum(float mag, unsigned least)
+{
+    return mag < 1e38f && (least == 0xFFFFFFFFu || mag * 2.384185791015625e-7f <= __uint_as_float(least + 1u));
+}
+
+// Of the terms of a sum: the sum of their magnitudes, and the bits less one of the
+// smallest magnitude (zeros, whose bits less one are the largest number, do not count).
+struct TermSizes {
+    float sum = 0.f;
+    unsigned least = 0xFFFFFFFFu;
+    __device__ __forceinline__ void add(float t)
+    {
+        sum += fabsf(t);
+        least = min(least, (__float_as_uint(t) & 0x7FFFFFFFu) - 1u);
+    }
+    __device__ __forceinline__ void over(int width)              // of the lanes of a group together
+    {
+        for (int d = width >> 1; d > 0; d >>= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, d, width);
+            least = min(least, __shfl_xor_sync(0xffffffffu, least, d, width));
+        }
+    }
+};
+
+// The sums of a row again in k_fill1's order.  The diagonal: the pn pairs, and each
+// species' own part.  A one-move: its terms over the other species' particles (a lane
+// each, summed as a tree) and over its own species' spectators (loaded a lane each,
+// summed ascending after the one-body term).  A call of its own at the row's end, so
+// that the rows without such sums keep their registers; w_occ, w_lev: the row's.
+__device__ __noinline__ void split_row(const DevBasis &B, const int2 *lg, const FillArgs &F, int64_t row, const int16_t *w_occ,
+                                       const int4 *w_lev, float *val, int64_t es, int64_t ks, int *status)
+{
+    const int lane = threadIdx.x & 31, nbase = B.sp[1].orb_base;
+    const DevSpecies &SP = B.sp[0], &SN = B.sp[1];
+    const int Zp = B.nZ[0], Zn = B.nZ[1], gsz = term_lanes(Zp, Zn), i = lane % gsz;
+    const ProtonRec PR = B.prec[B.row_p[row]];
+    const int n = (int)(row - PR.colb);
+    const NeutronRec NR = B.nrec[n];
+    const int cA1 = max(0, B.dir[(int64_t)n * B.dir_len + PR.dirA] - NR.self);
+    int c1 = 0;                                                 // proton one-moves with n kept
+    if (lane < PR.ng) {
+        const int4 gr = B.grp[PR.g0 + lane];
+        if ((gr.w & 0xFF) > NR.N) c1 = (unsigned)gr.x >> 16;
+    }
+    c1 = __reduce_add_sync(0xffffffffu, c1);
+    __syncwarp();                                               // after the row's first values
+    for (int k = 0; k < F.K; ++k) {
+        DF acc = df_of(0.f);
+        for (int x = lane / gsz; x < Zp; x += 32 / gsz) {
+            if (i >= Zn) continue;
+            const int a = w_occ[x], c = w_occ[Zp + i];
+            int64_t idx;
+            int sg;
+            if (tbme_at(B, lg, a, c, a, c, idx, sg)) {
+                const float v = __ldg(F.tbme + (int64_t)k * F.tb_sk + idx * F.tb_si);
+                acc = df_add(acc, df_of(sg < 0 ? -v : v));
+            }
+        }
+        acc = warp_sum(acc, 32);
+        const DF dp = diag_own(B, lg, F, k, Zp, [&](int x) { return (int)w_occ[x]; }, status);
+        const DF dn = diag_own(B, lg, F, k, Zn, [&](int x) { return (int)w_occ[Zp + x]; }, status);
+        if (lane == 0) val[(int64_t)k * ks] = df_round(df_add(acc, df_add(dp, dn)));
+    }
+    for (int t0 = 0; t0 < cA1 + c1; t0 += 32 / gsz) {
+        const int t = t0 + lane / gsz;
+        const bool act = t < cA1 + c1, neu = t < cA1;
+        int e = 0, code = 0;
+        if (act && neu) {
+            const int64_t sl = NR.fw + NR.fwlen - 1 - t;
+            e = 1 + t + (SN.fw_rec[sl].y & 0xFFFFFF);
+            code = ~SN.fw_tb[sl];
+        } else if (act) {
+            const int64_t sl = PR.fw + PR.fwlen - 1 - (t - cA1);
+            const int o = SP.fw_rec[sl].y;
+            const int4 lv = w_lev[o >> 24];
+            e = lv.x + (t - cA1) * lv.y + (o & 0xFFFFFF) + lv.z;
+            code = ~SP.fw_tb[sl];
+        }
+        const int base = neu ? nbase : 0, a = base + (code & 0xFF), c = base + ((code >> 8) & 0xFF);
+        const int own0 = neu ? Zp : 0, nown = (neu ? Zn : Zp) - 1, oth0 = neu ? 0 : Zp, noth = neu ? Zp : Zn;
+        int ia = 0;                                             // a's place among its species
+        for (int x = 0; x <= nown; ++x) ia += (w_occ[own0 + x] < a);
+        const bool ho = act && i < noth, hs = act && i < nown;
+        const int ko = ho ? w_occ[oth0 + i] : 0, kx = hs ? w_occ[own0 + i + (i >= ia ? 1 : 0)] : 0;
+        int64_t xo = 0, xs = 0;
+        int go = 1, gs = 1;
+        const bool oko = ho && tbme_at(B, lg, a, ko, c, ko, xo, go), oks = hs && tbme_at(B, lg, a, kx, c, kx, xs, gs);
+        const DF one = act ? onebody_term(B, F, a, c, status) : df_of(0.f);
+        for (int k = 0; k < F.K; ++k) {
+            const float *tk = F.tbme + (int64_t)k * F.tb_sk;
+            float to = oko ? __ldg(tk + xo * F.tb_si) : 0.f, ts = oks ? __ldg(tk + xs * F.tb_si) : 0.f;
+            if (go < 0) to = -to;
+            if (gs < 0) ts = -ts;
+            const DF v = warp_sum(df_of(to), gsz);
+            DF own = one;
+            for (int x = 0; x < gsz; ++x) {
+                const float y = __shfl_sync(0xffffffffu, ts, x, gsz);
+                if (x < nown) own = df_add(own, df_of(y));
+            }
+            if (act && i == 0) {
+                const float r = df_round(df_add(v, own));
+                val[(int64_t)e * es + (int64_t)k * ks] = (code >> 16) & 1 ? -r : r;
+            }
+        }
+    }
+}
+
 // Deferred one-move elements of a row: lanes over (element, spectator)
 // pairs, groups of the next power of two >= A-1 lanes, segmented sum (from
 // kLaneSets sets on: one element at a time, lanes over sets).
 // The queue holds row-relative positions, columns and packed moves
 // (bra-only a, ket-only c, sign, neutron flag in bit 31).
-template <int MODE, bool K1, int EM>
+template <int MODE, bool K1, int EM, bool SPLIT>
 __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, const FillArgs &F, const GradArgs &Gr,
                                            int *status, const int16_t *w_occ, const int32_t *w_spos,
                                            const int32_t *w_scol, const uint32_t *w_scode, int &nslow,
-                                           const RowOut &R)
+                                           const RowOut &R, bool &again)
 {
     const int lane = threadIdx.x & 31;
     const int A = B.A, nbase = B.sp[1].orb_base;
@@ -503,53 +636,6 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
         nslow = 0;
         return;
     }
-    if (MODE == 1 && !EM && F.split) {
-        // k_fill1's order: an element's terms over the other species' particles (a lane
-        // each, summed as a tree) and over its own species' spectators (loaded a
-        // lane each, summed ascending after the one-body term): the sums of k_fill1
-        const int Zp = B.nZ[0], Zn = B.nZ[1], gsz = term_lanes(Zp, Zn), per = 32 / gsz;
-        for (int e0 = 0; e0 < ns; e0 += per) {
-            const int e = e0 + lane / gsz, i = lane % gsz;
-            const bool act = e < ns;
-            const uint32_t code = act ? w_scode[e] : 0;
-            const bool neu = (code >> 31) != 0;
-            const int base = neu ? nbase : 0;
-            const int a = base + (int)(code & 0xFF), c = base + (int)((code >> 8) & 0xFF);
-            const int own0 = neu ? Zp : 0, nown = (neu ? Zn : Zp) - 1, oth0 = neu ? 0 : Zp, noth = neu ? Zp : Zn;
-            int ia = 0;                                             // a's place among its species
-            for (int x = 0; x <= nown; ++x) ia += (w_occ[own0 + x] < a);
-            const bool ho = act && i < noth, hs = act && i < nown;
-            const int ko = ho ? w_occ[oth0 + i] : 0, ks = hs ? w_occ[own0 + i + (i >= ia ? 1 : 0)] : 0;
-            int64_t xo = 0, xs = 0;
-            int go = 1, gs = 1;
-            const bool oko = !ho || tbme_at(B, lg, a, ko, c, ko, xo, go), oks = !hs || tbme_at(B, lg, a, ks, c, ks, xs, gs);
-            if ((!oko || !oks) && atomicOr(status, 1) == 0) {
-                status[2] = a | (c << 16);
-                status[3] = 2 | ((oko ? ks : ko) << 8);
-            }
-            const DF one = act ? onebody_term(B, F, a, c, status) : df_of(0.f);
-            for (int kk = 0; kk < (K1 ? 1 : F.K); ++kk) {
-                const float *tk = F.tbme + (int64_t)kk * F.tb_sk;
-                float to = 0.f, ts = 0.f;
-                if (ho && oko) { to = __ldg(tk + xo * F.tb_si); if (go < 0) to = -to; }
-                if (hs && oks) { ts = __ldg(tk + xs * F.tb_si); if (gs < 0) ts = -ts; }
-                const DF v = warp_sum(df_of(to), gsz);
-                DF own = one;
-                for (int x = 0; x < gsz; ++x) {
-                    const float y = __shfl_sync(0xffffffffu, ts, x, gsz);
-                    if (x < nown) own = df_add(own, df_of(y));
-                }
-                if (act && i == 0) {
-                    const float r = df_round(df_add(v, own));
-                    if (kk == 0) R.col[w_spos[e]] = w_scol[e];
-                    R.val[(int64_t)w_spos[e] * R.es + (int64_t)kk * R.ks] = (code >> 16) & 1 ? -r : r;
-                }
-            }
-        }
-        __syncwarp();
-        nslow = 0;
-        return;
-    }
     int gsz = 1;
     while (gsz < sp_n) gsz <<= 1;
     const int per = 32 / gsz;
@@ -584,12 +670,25 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
                     const float t = __ldg(F.tbme + (int64_t)kk * F.tb_sk + idx * F.tb_si);
                     v = df_of(sg < 0 ? -t : t);
                 }
+                const float term = v.hi;
                 v = df_add(t1v, v);
                 v = warp_sum(v, gsz);
                 if (act && i == 0) {
                     if (kk == 0) R.col[eo] = (int32_t)colj;
                     const float r = df_round(v);
                     R.val[(int64_t)eo * R.es + (int64_t)kk * R.ks] = sgn ? -r : r;
+                }
+                if (SPLIT) {
+                    TermSizes z;
+                    z.add(term);
+                    float mag = fabsf(t1v.hi) + __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(z.sum))) * (float)sp_n;
+                    const bool near = act && i == 0 && near_tie(v, mag, F.tol_one);
+                    if (__any_sync(0xffffffffu, near)) {          // look closer: the element's own terms
+                        z.add(t1v.hi);
+                        z.add(t1v.lo);
+                        z.over(gsz);
+                        again |= near && near_tie(v, z.sum, F.tol_one) && !exact_sum(z.sum, z.least);
+                    }
                 }
             } else if (has && ok) {
                 const long long q =
@@ -625,10 +724,9 @@ __device__ __forceinline__ int64_t next_row(int64_t row, int64_t r0, int64_t r1,
     return r0 + (t / WARPS) * run + (int64_t)blockIdx.x * WARPS + t % WARPS;
 }
 
-template <int MODE, bool K1, int WARPS, int EM>
-__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
-k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs Gr, int64_t r0, int64_t r1,
-       int *status)
+template <int MODE, bool K1, int WARPS, int EM, bool SPLIT>
+__device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowptr, int64_t *counts, const FillArgs &F, const GradArgs &Gr,
+                                          int64_t r0, int64_t r1, int *status)
 {
     constexpr int kThreads = WARPS * 32;
     extern __shared__ __align__(16) unsigned char sb[];
@@ -703,6 +801,7 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
             R.val = F.val + r0 * R.es;
         }
         int nslow = 0;
+        bool again = false;                                     // SPLIT: a sum of the row may depend on the order
 
         // ---- diagonal: occupied orbitals (combined, ascending), then all pairs
         if (MODE != 0) {
@@ -769,35 +868,9 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
                 if (lane == 0 && rowlen > 0) R.col[0] = (int32_t)row;
                 __syncwarp();
             }
-            const bool split = MODE == 1 && !EM && F.split;
-            if (split) {                                     // k_fill1's order
-                const int P = term_lanes(Zpro, Zneu), sub = lane / P, j = lane % P;
-                for (int k = 0; k < (K1 ? 1 : F.K); ++k) {
-                    DF acc = df_of(0.f);
-                    for (int i = sub; i < Zpro; i += 32 / P) {
-                        if (j >= Zneu) continue;
-                        const int a = w_occ[i], c = w_occ[Zpro + j];
-                        int64_t idx;
-                        int sg;
-                        if (tbme_at(B, lg, a, c, a, c, idx, sg)) {
-                            const float v = __ldg(F.tbme + (int64_t)k * F.tb_sk + idx * F.tb_si);
-                            acc = df_add(acc, df_of(sg < 0 ? -v : v));
-                        } else if (atomicOr(status, 1) == 0) {
-                            status[2] = a | (c << 16);
-                            status[3] = 1;
-                        }
-                    }
-                    acc = warp_sum(acc, 32);
-                    const DF dp = diag_own(B, lg, F, k, Zpro, [&](int i) { return (int)w_occ[i]; }, status);
-                    const DF dn = diag_own(B, lg, F, k, Zneu, [&](int i) { return (int)w_occ[Zpro + i]; }, status);
-                    if (lane == 0 && rowlen > 0) {
-                        if (k == 0) R.col[0] = (int32_t)row;
-                        R.val[(int64_t)k * R.ks] = df_round(df_add(acc, df_add(dp, dn)));
-                    }
-                }
-            }
-            for (int k = 0; k < (kset || split ? 0 : K1 ? 1 : MODE == 1 ? F.K : Gr.K); ++k) {
+            for (int k = 0; k < (kset ? 0 : K1 ? 1 : MODE == 1 ? F.K : Gr.K); ++k) {
                 DF acc = df_of(0.f);
+                TermSizes z;
                 for (int l = lane; l < npairs; l += 32) {
                     const int a = w_occ[pi[l]], c = w_occ[pj[l]];
                     int64_t idx;
@@ -809,6 +882,7 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
                     if (MODE == 1) {
                         const float v = __ldg(F.tbme + (int64_t)k * F.tb_sk + idx * F.tb_si);
                         acc = df_add(acc, df_of(sg < 0 ? -v : v));
+                        if (SPLIT) z.add(v);
                     } else {                                     // w = 1 on the diagonal
                         const long long q = psi_prod(Gr.psi + (int64_t)k * B.dim, row, row) >> 2;
                         atomicAdd(Gr.acc + (int64_t)k * B.tbme_len + idx, (unsigned long long)(sg < 0 ? -q : q));
@@ -819,11 +893,22 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
                     for (int i = lane; i < A; i += 32) {
                         const float2 q = e1[w_occ[i]];
                         acc = df_add(acc, DF{q.x, q.y});
+                        if (SPLIT) {
+                            z.add(q.x);
+                            z.add(q.y);
+                        }
                     }
                     acc = warp_sum(acc, 32);
                     if (lane == 0 && rowlen > 0) {
                         if (k == 0) R.col[0] = (int32_t)row;
                         R.val[(int64_t)k * R.ks] = df_round(acc);
+                    }
+                    if (SPLIT) {
+                        const float most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(z.sum)));
+                        if (__any_sync(0xffffffffu, rowlen > 0 && near_tie(acc, 32.f * most, F.tol_diag))) {
+                            z.over(32);
+                            again |= near_tie(acc, z.sum, F.tol_diag) && !exact_sum(z.sum, z.least);
+                        }
                     }
                 }
             }
@@ -856,7 +941,7 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
             for (int t0 = 0; t0 < cA1; t0 += 32) {
                 const int t = t0 + lane, c = min(32, cA1 - t0);
                 if (nslow + c > kSlowCap)
-                    flush_slow<MODE, K1, EM>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R);
+                    flush_slow<MODE, K1, EM, SPLIT>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R, again);
                 if (lane < c) {
                     const int sl = NR.fwlen - 1 - t;
                     const int2 rc = rec[sl];
@@ -891,6 +976,7 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
             const int Tall = __shfl_sync(0xffffffffu, itot, 31), Tpn = __shfl_sync(0xffffffffu, ipn, 31);
             if (MODE == 1 && pos + Tall > rowlen) {
                 if (lane == 0) atomicOr(status, 2);
+                rowlen = -1;                                    // (no second look at an incomplete row)
                 break;
             }
             const int at0 = pos + itot - tot, st = ipn - npn, f1 = gr.x & 0xFFFF;
@@ -932,7 +1018,7 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
             for (int t0 = 0; t0 < c1; t0 += 32) {
                 const int t = t0 + lane, cc = min(32, c1 - t0);
                 if (nslow + cc > kSlowCap)
-                    flush_slow<MODE, K1, EM>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R);
+                    flush_slow<MODE, K1, EM, SPLIT>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R, again);
                 if (lane < cc) {
                     const int2 q = l1row[t];
                     const int o = recp[PR.fwlen - 1 - t].y;
@@ -976,10 +1062,29 @@ k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs 
             __syncwarp();
             pos += Tall;
         }
-        if (MODE != 0 && nslow > 0) flush_slow<MODE, K1, EM>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R);
+        if (MODE != 0 && nslow > 0) flush_slow<MODE, K1, EM, SPLIT>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R, again);
+        if (SPLIT && __any_sync(0xffffffffu, again && rowlen > 0)) split_row(B, lg, F, row, w_occ, w_lev, R.val, R.es, R.ks, status);
         if (MODE == 0 && lane == 0) counts[row] = pos;
         __syncwarp();
     }
+}
+
+// Two forms of the same kernel: with grid-constant parameters ptxas spills less for one
+// set (20 bytes against 24, 36 against 40 with SPLIT), but the loops over sets run slower
+// (64 sets of 3+4 Nmax=3, set-major: 780 us against 646).
+template <int MODE, bool K1, int WARPS, int EM, bool SPLIT = false>
+__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
+k_rows(DevBasis B, const int64_t *rowptr, int64_t *counts, FillArgs F, GradArgs Gr, int64_t r0, int64_t r1, int *status)
+{
+    walk_rows<MODE, K1, WARPS, EM, SPLIT>(B, rowptr, counts, F, Gr, r0, r1, status);
+}
+
+template <int MODE, bool K1, int WARPS, int EM, bool SPLIT = false>
+__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS)
+k_rows_const(const __grid_constant__ DevBasis B, const int64_t *rowptr, int64_t *counts, const __grid_constant__ FillArgs F, GradArgs Gr,
+             int64_t r0, int64_t r1, int *status)
+{
+    walk_rows<MODE, K1, WARPS, EM, SPLIT>(B, rowptr, counts, F, Gr, r0, r1, status);
 }
 
 // The working copy of the tables (FillWork): warps over the rows of the pn
@@ -1673,7 +1778,13 @@ int launch_rows_w(const cih_basis &b, const int64_t *rowptr, int64_t *counts, co
         // element-major K sets: warp-cooperative writes; 64 is the batched configuration's set count
         if (em) return F.K == 64 ? go(k_rows<MODE, false, WARPS, 64>) : go(k_rows<MODE, false, WARPS, 1>);
     }
-    if constexpr (MODE != 0) {
+    if constexpr (MODE == 1) {
+        if (F.tol_one > 0.f) return k1 ? go(k_rows_const<MODE, true, WARPS, 0, true>) : go(k_rows_const<MODE, false, WARPS, 0, true>);
+    }
+    if constexpr (MODE == 1) {
+        if (k1) return go(k_rows_const<MODE, true, WARPS, 0>);
+    }
+    if constexpr (MODE == 2) {
         if (k1) return go(k_rows<MODE, true, WARPS, 0>);
     }
     return go(k_rows<MODE, false, WARPS, 0>);
@@ -1813,24 +1924,44 @@ int launch_prep(const cih_basis &b, int kv, const FillArgs &F, const FillWork &W
     return e == cudaSuccess ? CIH_OK : cuda_fail(e, "fill preparation");
 }
 
-// Whether fills of K sets of this basis go through the working copy, and so make
-// their sums in its order (rows that do not pay for it in the row kernel, slower
-// there than in the order of the terms: a quarter for one set, more for several).
-// A copy costs its two launches and its entries once; each row gains.  Several sets
+// Whether a fill of K sets of `rows` of the rows goes through the working copy.  A copy
+// costs its two launches and its entries once; each row gains.  Several sets
 // gain more a row; from five on there are two passes, and the values of
 // five to seven sets of an element, written by both, share their lines.  Measured
-// against the row kernel without this order, by rows and entries of a copy a row:
+// against the row kernel, by rows and entries of a copy a row:
 //   one set: 4,945 rows, 50 entries 0.76x; 8,500, 15 0.95x; 13,162, 85 0.93x; 17,769,
 //     170 0.90x; 14,502, 12 1.17x; 17,040, 61 1.22x; 23,907, 54 1.07x; 39,421, 94 1.14x
 //   two, four: 4,945, 50 0.85x, 0.91x; 6,758, 425 0.88x, 0.98x; 8,500, 15 1.12x, 1.13x;
 //     10,753, 51 1.15x, 1.21x; 17,769, 170 1.06x, 1.04x
 //   seven, set-major and element-major: 23,907, 54 1.11x, 0.84x; 36,498, 18 1.31x, 0.97x;
 //     165,736, 82 1.36x, 0.93x; 48,917, 35 1.54x, 1.04x; 143,792, 18 1.98x, 1.15x
-bool fill_splits(const cih_basis &b, int K)
+// A part of the rows by the same rule for its own rows, with two to four sets from
+// 12,288 rows on (the copy covers all sub-dets, so few rows pay for many entries).
+// Over some 500 parts (halves to fiftieths) of 20 bases, mean time over the better
+// way's by this rule / always / never through the copy: one set 1.006 / 1.33 / 1.02, two
+// 1.04 / 1.23 / 1.14, four 1.03 / 1.37 / 1.09, seven 1.02 / 1.81 / 1.04.
+bool copy_pays(const cih_basis &b, int K, int64_t rows)
 {
-    const int64_t rows = K == 1 ? 16384 : K <= 4 ? 8192 : 40960, entries = K == 1 ? 128 : K <= 4 ? 192 : 64;
-    return K < kFillSets && b.dim >= rows && fill1_fits(b, K == 1 ? 1 : K == 2 ? 2 : 4) &&
-           (int64_t)work_floats(b, 1) <= entries * b.dim;
+    const int64_t least = K == 1 ? 16384 : K > 4 ? 40960 : rows == b.dim ? 8192 : 12288, entries = K == 1 ? 128 : K <= 4 ? 192 : 64;
+    return K < kFillSets && rows >= least && fill1_fits(b, K == 1 ? 1 : K == 2 ? 2 : 4) &&
+           (int64_t)work_floats(b, 1) <= entries * rows;
+}
+// Whether the fills of all rows of K sets go through the copy, and so the sums of
+// every fill are those of its order (SPLIT)
+bool fill_splits(const cih_basis &b, int K) { return copy_pays(b, K, b.dim); }
+
+// additions a term goes through, in the row kernel's order and in k_fill1's together,
+// for a one-move and for the diagonal, x 16 u^2
+void split_tolerances(const cih_basis &b, FillArgs &F)
+{
+    auto lg = [](int x) { int l = 0; while (1 << l < x) ++l; return l; };
+    auto warps = [](int x) { return (x + 31) / 32; };
+    const int A = b.dev.A, Zp = b.dev.nZ[0], Z = std::max(Zp, b.dev.nZ[1]), P = std::min(lg(Z), 5);
+    const int one = 1 + lg(A - 1) + std::max(Z - 1, P) + 1;
+    const int pn = warps(Zp << P) + 5, own = warps(Z * (Z - 1) / 2) + warps(Z) + 5 + 1;
+    const int diag = warps(A * (A - 1) / 2) + warps(A) + 5 + std::max(pn, own) + 1;
+    F.tol_one = std::ldexp((float)one, 4 - 48);
+    F.tol_diag = std::ldexp((float)diag, 4 - 48);
 }
 
 }  // namespace
@@ -1857,12 +1988,14 @@ int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, con
 {
     const int vec4 = interleaved && K % 4 == 0 && ((uintptr_t)tbme & 15) == 0 && (!em || ((uintptr_t)val & 15) == 0);
     FillArgs F{K, hw, tbme, interleaved ? 1 : b.layout.total, interleaved ? (int64_t)K : 1, vec4, em && K > 1 ? 1 : 0,
-               esp, col, val, sharded ? 1 : 0, r0, t1, fill_splits(b, K) ? 1 : 0};
+               esp, col, val, sharded ? 1 : 0, r0, t1, 0.f, 0.f};
+    const bool split = fill_splits(b, K);
+    if (split) split_tolerances(b, F);
     const int64_t rend = r1 < 0 ? b.dim : r1;
     if (K == 1 && work && b.dim > 0 && rend > r0)
         return launch_fill1(b, 1, rowptr, F, work_at(b, const_cast<float *>(work), 1, 0, 1), st, false, r0, rend);
     const int kv = K == 1 ? 1 : K == 2 ? 2 : 4;                // sets of one pass
-    if (F.split && !work && prepare && rend > r0 && (rend - r0) * kPrepareShare >= b.dim) {
+    if (split && !work && prepare && copy_pays(b, K, rend - r0)) {
         float *own = nullptr;
         if (cudaMallocFromPoolAsync((void **)&own, work_floats(b, kv) * sizeof(float), b.pool, st) == cudaSuccess) {
             int rc = CIH_OK;
