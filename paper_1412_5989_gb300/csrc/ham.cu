@@ -34,6 +34,7 @@
 #include <cstdlib>
 #include <map>
 #include <mutex>
+#include <type_traits>
 
 #include "cih_internal.h"
 #include "ham_common.cuh"
@@ -108,6 +109,13 @@ __device__ __forceinline__ DF onebody_term(const DevBasis &B, const FillArgs &F,
     const double t = F.t1[k];
     const float hi = (float)t;
     return DF{hi, (float)(t - (double)hi)};
+}
+
+// The elements that a CTA of k_rows fills (row_parts): 1 the diagonal, 2 the neutron
+// moves, 4 the proton moves with the neutrons kept, 8 the pn elements.
+__device__ __forceinline__ int row_part()
+{
+    return gridDim.y == 1 ? 15 : gridDim.y == 2 ? 3 << (2 * blockIdx.y) : blockIdx.y == 0 ? 3 : 2 << blockIdx.y;
 }
 
 struct GradArgs {
@@ -198,6 +206,34 @@ __device__ __forceinline__ DF warp_sum(DF v, int width)
         v = df_add(v, o);
     }
     return v;
+}
+
+// warp_sum of several sums side by side (a step of one hides the other's latency)
+template <int U>
+__device__ __forceinline__ void warp_sums(DF (&v)[U], int width)
+{
+    for (int d = width >> 1; d > 0; d >>= 1)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const DF o{__shfl_xor_sync(0xffffffffu, v[u].hi, d, width), __shfl_xor_sync(0xffffffffu, v[u].lo, d, width)};
+            v[u] = df_add(v[u], o);
+        }
+}
+
+// sums(width, k) for the sets k .. k + width - 1 of K, four at a time, the last one or
+// two as two: the sums of an element side by side, its table entries looked up once.
+// (us, one set at a time / two / four: four sets of 3+3 Nmax=2 31.4 / 27.2 / 25.2, eight
+// sets of 3+4 Nmax=3 160 / 136 / 118; two sets of 2,000 rows of 4+4 Nmax=4 39.6 / 34.4 / 39.6.)
+template <bool K1, class Sums>
+__device__ __forceinline__ void over_sets(int K, Sums &&sums)
+{
+    if (K1) {
+        sums(std::integral_constant<int, 1>(), 0);
+        return;
+    }
+    int k = 0;
+    for (; k + 2 < K; k += 4) sums(std::integral_constant<int, 4>(), k);
+    if (k < K) sums(std::integral_constant<int, 2>(), k);
 }
 
 // Row output view: column and value pointers at the row's first element;
@@ -430,10 +466,16 @@ __device__ __forceinline__ bool exact_sum(float mag, unsigned least)
 struct TermSizes {
     float sum = 0.f;
     unsigned least = 0xFFFFFFFFu;
+    __device__ __forceinline__ void smaller(float t) { least = min(least, (__float_as_uint(t) & 0x7FFFFFFFu) - 1u); }
     __device__ __forceinline__ void add(float t)
     {
         sum += fabsf(t);
-        least = min(least, (__float_as_uint(t) & 0x7FFFFFFFu) - 1u);
+        smaller(t);
+    }
+    __device__ __forceinline__ void most(float t)                // the same term of another set
+    {
+        sum = fmaxf(sum, fabsf(t));
+        smaller(t);
     }
     __device__ __forceinline__ void over(int width)              // of the lanes of a group together
     {
@@ -454,7 +496,7 @@ __device__ __noinline__ void split_row(const DevBasis &B, const int2 *lg, const 
 {
     const int lane = threadIdx.x & 31, nbase = B.sp[1].orb_base;
     const DevSpecies &SP = B.sp[0], &SN = B.sp[1];
-    const int Zp = B.nZ[0], Zn = B.nZ[1], gsz = term_lanes(Zp, Zn), i = lane % gsz;
+    const int Zp = B.nZ[0], Zn = B.nZ[1], gsz = term_lanes(Zp, Zn), i = lane % gsz, part = row_part();
     const ProtonRec PR = B.prec[B.row_p[row]];
     const int n = (int)(row - PR.colb);
     const NeutronRec NR = B.nrec[n];
@@ -466,7 +508,7 @@ __device__ __noinline__ void split_row(const DevBasis &B, const int2 *lg, const 
     }
     c1 = __reduce_add_sync(0xffffffffu, c1);
     __syncwarp();                                               // after the row's first values
-    for (int k = 0; k < F.K; ++k) {
+    for (int k = 0; k < (part & 1 ? F.K : 0); ++k) {
         DF acc = df_of(0.f);
         for (int x = lane / gsz; x < Zp; x += 32 / gsz) {
             if (i >= Zn) continue;
@@ -483,9 +525,10 @@ __device__ __noinline__ void split_row(const DevBasis &B, const int2 *lg, const 
         const DF dn = diag_own(B, lg, F, k, Zn, [&](int x) { return (int)w_occ[Zp + x]; }, status);
         if (lane == 0) val[(int64_t)k * ks] = df_round(df_add(acc, df_add(dp, dn)));
     }
-    for (int t0 = 0; t0 < cA1 + c1; t0 += 32 / gsz) {
+    const int first = part & 2 ? 0 : cA1, last = part & 4 ? cA1 + c1 : cA1;
+    for (int t0 = first; t0 < last; t0 += 32 / gsz) {
         const int t = t0 + lane / gsz;
-        const bool act = t < cA1 + c1, neu = t < cA1;
+        const bool act = t < last, neu = t < cA1;
         int e = 0, code = 0;
         if (act && neu) {
             const int64_t sl = NR.fw + NR.fwlen - 1 - t;
@@ -663,34 +706,50 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
         }
         // the one-body term t_ac (one per element: added by its group's first lane)
         const DF t1v = (MODE == 1 && act && i == 0) ? onebody_term(B, F, a, c, status) : df_of(0.f);
-        for (int kk = 0; kk < (K1 ? 1 : MODE == 1 ? F.K : Gr.K); ++kk) {
-            if (MODE == 1) {
-                DF v = df_of(0.f);
-                if (has && ok) {
-                    const float t = __ldg(F.tbme + (int64_t)kk * F.tb_sk + idx * F.tb_si);
-                    v = df_of(sg < 0 ? -t : t);
+        if (MODE == 1) {
+            TermSizes z;                                        // SPLIT: of the lane's terms, all sets together
+            bool near = false;
+            auto sums = [&](auto width, int k0) {               // the sets from k0 on
+                constexpr int U = decltype(width)::value;
+                DF v[U];
+                unsigned most = 0;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    float t = 0.f;
+                    if (has && ok && (K1 || k0 + u < F.K)) t = __ldg(F.tbme + (int64_t)(k0 + u) * F.tb_sk + idx * F.tb_si);
+                    if (SPLIT) {
+                        z.most(t);
+                        most = max(most, __float_as_uint(t) & 0x7FFFFFFFu);
+                    }
+                    v[u] = df_of(sg < 0 ? -t : t);
                 }
-                const float term = v.hi;
-                v = df_add(t1v, v);
-                v = warp_sum(v, gsz);
-                if (act && i == 0) {
-                    if (kk == 0) R.col[eo] = (int32_t)colj;
-                    const float r = df_round(v);
-                    R.val[(int64_t)eo * R.es + (int64_t)kk * R.ks] = sgn ? -r : r;
-                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[u] = df_add(t1v, v[u]);
+                warp_sums<U>(v, gsz);
                 if (SPLIT) {
-                    TermSizes z;
-                    z.add(term);
-                    float mag = fabsf(t1v.hi) + __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(z.sum))) * (float)sp_n;
-                    const bool near = act && i == 0 && near_tie(v, mag, F.tol_one);
-                    if (__any_sync(0xffffffffu, near)) {          // look closer: the element's own terms
-                        z.add(t1v.hi);
-                        z.add(t1v.lo);
-                        z.over(gsz);
-                        again |= near && near_tie(v, z.sum, F.tol_one) && !exact_sum(z.sum, z.least);
+                    const float mag = fabsf(t1v.hi) + __uint_as_float(__reduce_max_sync(0xffffffffu, most)) * (float)sp_n;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) near |= (K1 || k0 + u < F.K) && near_tie(v[u], mag, F.tol_one);
+                }
+                if (act && i == 0) {
+                    if (k0 == 0) R.col[eo] = (int32_t)colj;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const float r = df_round(v[u]);
+                        if (K1 || k0 + u < F.K) R.val[(int64_t)eo * R.es + (int64_t)(k0 + u) * R.ks] = sgn ? -r : r;
                     }
                 }
-            } else if (has && ok) {
+            };
+            over_sets<K1>(K1 ? 1 : F.K, sums);
+            if (SPLIT && __any_sync(0xffffffffu, near && act && i == 0)) {
+                z.add(t1v.hi);
+                z.add(t1v.lo);
+                z.over(gsz);
+                again |= near && act && i == 0 && !exact_sum(z.sum, z.least);
+            }
+        } else {
+            for (int kk = 0; kk < (K1 ? 1 : Gr.K); ++kk) {
+                if (!has || !ok) continue;
                 const long long q =
                     (K1 ? __mul64hi(R.psir, Gr.psi[colj]) : psi_prod(Gr.psi + (int64_t)kk * B.dim, R.row, colj)) >> 1;
                 const bool neg = (sgn != 0) != (sg < 0);
@@ -809,6 +868,8 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
                 w_occ[i] = i < Zpro ? (int16_t)B.occ[0][(int64_t)p * Zpro + i]
                                     : (int16_t)(nbase + B.occ[1][(int64_t)n * Zneu + (i - Zpro)]);
             __syncwarp();
+        }
+        if (MODE == 2 || (MODE == 1 && (row_part() & 1))) {
             const uint8_t *pi = sptr<uint8_t>(sb, sm::pi), *pj = sptr<uint8_t>(sb, sm::pj);
             const bool kset = MODE == 1 && !K1 && F.K >= kLaneSets && npairs <= kSlowCap;
             if (kset) {
@@ -868,9 +929,12 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
                 if (lane == 0 && rowlen > 0) R.col[0] = (int32_t)row;
                 __syncwarp();
             }
-            for (int k = 0; k < (kset ? 0 : K1 ? 1 : MODE == 1 ? F.K : Gr.K); ++k) {
-                DF acc = df_of(0.f);
+            auto sums = [&](auto width, int k0) {               // the sets from k0 on
+                constexpr int U = decltype(width)::value;
+                DF acc[U];
                 TermSizes z;
+#pragma unroll
+                for (int u = 0; u < U; ++u) acc[u] = df_of(0.f);
                 for (int l = lane; l < npairs; l += 32) {
                     const int a = w_occ[pi[l]], c = w_occ[pj[l]];
                     int64_t idx;
@@ -880,38 +944,57 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
                         continue;
                     }
                     if (MODE == 1) {
-                        const float v = __ldg(F.tbme + (int64_t)k * F.tb_sk + idx * F.tb_si);
-                        acc = df_add(acc, df_of(sg < 0 ? -v : v));
-                        if (SPLIT) z.add(v);
+                        float m = 0.f;
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            const float v = K1 || k0 + u < F.K ? __ldg(F.tbme + (int64_t)(k0 + u) * F.tb_sk + idx * F.tb_si) : 0.f;
+                            acc[u] = df_add(acc[u], df_of(sg < 0 ? -v : v));
+                            if (SPLIT) {
+                                m = fmaxf(m, fabsf(v));
+                                z.smaller(v);
+                            }
+                        }
+                        if (SPLIT) z.sum += m;
                     } else {                                     // w = 1 on the diagonal
-                        const long long q = psi_prod(Gr.psi + (int64_t)k * B.dim, row, row) >> 2;
-                        atomicAdd(Gr.acc + (int64_t)k * B.tbme_len + idx, (unsigned long long)(sg < 0 ? -q : q));
+                        const long long q = psi_prod(Gr.psi + (int64_t)k0 * B.dim, row, row) >> 2;
+                        atomicAdd(Gr.acc + (int64_t)k0 * B.tbme_len + idx, (unsigned long long)(sg < 0 ? -q : q));
                     }
                 }
                 if (MODE == 1) {
                     const float2 *e1 = sptr<float2>(sb, sm::e1);
                     for (int i = lane; i < A; i += 32) {
                         const float2 q = e1[w_occ[i]];
-                        acc = df_add(acc, DF{q.x, q.y});
+#pragma unroll
+                        for (int u = 0; u < U; ++u) acc[u] = df_add(acc[u], DF{q.x, q.y});
                         if (SPLIT) {
                             z.add(q.x);
                             z.add(q.y);
                         }
                     }
-                    acc = warp_sum(acc, 32);
+                    warp_sums<U>(acc, 32);
                     if (lane == 0 && rowlen > 0) {
-                        if (k == 0) R.col[0] = (int32_t)row;
-                        R.val[(int64_t)k * R.ks] = df_round(acc);
+                        if (k0 == 0) R.col[0] = (int32_t)row;
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (K1 || k0 + u < F.K) R.val[(int64_t)(k0 + u) * R.ks] = df_round(acc[u]);
                     }
                     if (SPLIT) {
-                        const float most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(z.sum)));
-                        if (__any_sync(0xffffffffu, rowlen > 0 && near_tie(acc, 32.f * most, F.tol_diag))) {
+                        const float mag = 32.f * __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(z.sum)));
+                        bool near = false;
+#pragma unroll
+                        for (int u = 0; u < U; ++u) near |= (K1 || k0 + u < F.K) && near_tie(acc[u], mag, F.tol_diag);
+                        if (__any_sync(0xffffffffu, near)) {      // look closer
                             z.over(32);
-                            again |= near_tie(acc, z.sum, F.tol_diag) && !exact_sum(z.sum, z.least);
+#pragma unroll
+                            for (int u = 0; u < U; ++u)
+                                again |= (K1 || k0 + u < F.K) && near_tie(acc[u], z.sum, F.tol_diag) && !exact_sum(z.sum, z.least);
                         }
                     }
                 }
-            }
+            };
+            if (MODE == 2)
+                for (int k = 0; k < (K1 ? 1 : Gr.K); ++k) sums(std::integral_constant<int, 1>(), k);
+            else if (!kset) over_sets<K1>(K1 ? 1 : F.K, sums);
         }
 
         // ---- A: same-class forward neutron neighbours inside p's range
@@ -922,7 +1005,7 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
             if (lane == 0) atomicOr(status, 2);
             continue;
         }
-        if (MODE != 0) {
+        if (MODE == 2 || (MODE == 1 && (row_part() & 2))) {
             const int2 *rec = SN.fw_rec + NR.fw;
             const int32_t *tbl = SN.fw_tb + NR.fw;
             for (int t0 = 0; t0 < cA2; t0 += 32) {
@@ -991,8 +1074,8 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
             int c1 = 0, c2 = 0;
             if (g0 == 0) {                                      // own-class groups come first, at most 32
                 if (gr.w) w_lev[((B.Nlim - (gr.w & 0xFF) + 1) - SP.N0) >> 1] = make_int4(c, len + 1, ins, 0);
-                c1 = __reduce_add_sync(0xffffffffu, self * n1c);
-                c2 = __reduce_add_sync(0xffffffffu, self * gr.z);
+                c1 = MODE == 2 || (row_part() & 4) ? __reduce_add_sync(0xffffffffu, self * n1c) : 0;
+                c2 = MODE == 2 || (row_part() & 4) ? __reduce_add_sync(0xffffffffu, self * gr.z) : 0;
             }
             __syncwarp();
             // pp two-moves: a prefix of p's list
@@ -1036,7 +1119,7 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
             // segment are the quotient and remainder by the segment length.
             const unsigned le = (2u << lane) - 1u;                 // bits 0..lane
             int before = 0;                                        // groups started before the window
-            for (int w0 = 0; w0 < Tpn; w0 += 32) {
+            for (int w0 = MODE == 2 || (row_part() & 8) ? 0 : Tpn; w0 < Tpn; w0 += 32) {
                 const unsigned mk = __reduce_or_sync(0xffffffffu, npn > 0 && st >= w0 && st < w0 + 32 ? 1u << (st - w0) : 0u);
                 const int e = w0 + lane;
                 int at = 0, idx = 0, sg = 0;
@@ -1747,6 +1830,13 @@ cudaError_t raise_smem_limit(const void *kern, int dev, int bytes)
     return e;
 }
 
+// Parts that the elements of a row are filled in, a CTA each: the diagonal and the
+// neutron moves; the proton moves; the pn elements (the last two together where two
+// parts are all that the GPU holds at once).  The chain of one warp that fills a row
+// takes most of the time of a fill of few rows, whose CTAs leave SMs idle.  us, one
+// part / three: 800 rows of 3+3 Nmax=2 16.4 / 12.3 with one set, 20.5 / 14.3 with four.
+inline int row_parts(int64_t ctas, int64_t held) { return 3 * ctas <= held ? 3 : 2 * ctas <= held ? 2 : 1; }
+
 template <int MODE, int WARPS>
 int launch_rows_w(const cih_basis &b, const int64_t *rowptr, int64_t *counts, const FillArgs &F, const GradArgs &G,
                   cudaStream_t st, bool dry, int64_t r0, int64_t r1)
@@ -1766,8 +1856,9 @@ int launch_rows_w(const cih_basis &b, const int64_t *rowptr, int64_t *counts, co
         if (b.launch_ctas > 0) per_sm = std::min(per_sm, b.launch_ctas);
         const int64_t want = (r1 - r0 + WARPS - 1) / WARPS;
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm, want));
+        const int parts = MODE == 1 ? row_parts(want, (int64_t)sms * per_sm) : 1;
         count_launches(1);
-        kern<<<grid, WARPS * 32, smem, st>>>(D, rowptr, counts, F, G, r0, r1, b.dev_status);
+        kern<<<dim3(grid, parts), WARPS * 32, smem, st>>>(D, rowptr, counts, F, G, r0, r1, b.dev_status);
         ee = cudaGetLastError();
         return ee == cudaSuccess ? CIH_OK : cuda_fail(ee, "row kernel launch");
     };
@@ -1930,7 +2021,8 @@ int launch_prep(const cih_basis &b, int kv, const FillArgs &F, const FillWork &W
 // five to seven sets of an element, written by both, share their lines.  Measured
 // against the row kernel, by rows and entries of a copy a row:
 //   one set: 4,945 rows, 50 entries 0.76x; 8,500, 15 0.95x; 13,162, 85 0.93x; 17,769,
-//     170 0.90x; 14,502, 12 1.17x; 17,040, 61 1.22x; 23,907, 54 1.07x; 39,421, 94 1.14x
+//     170 0.90x; 10,817, 34 1.12x; 14,502, 12 1.17x; 15,448, 78 0.90x; 17,040, 61 1.22x;
+//     23,907, 54 1.07x; 39,421, 94 1.14x
 //   two, four: 4,945, 50 0.85x, 0.91x; 6,758, 425 0.88x, 0.98x; 8,500, 15 1.12x, 1.13x;
 //     10,753, 51 1.15x, 1.21x; 17,769, 170 1.06x, 1.04x
 //   seven, set-major and element-major: 23,907, 54 1.11x, 0.84x; 36,498, 18 1.31x, 0.97x;
@@ -1942,7 +2034,8 @@ int launch_prep(const cih_basis &b, int kv, const FillArgs &F, const FillWork &W
 // 1.04 / 1.23 / 1.14, four 1.03 / 1.37 / 1.09, seven 1.02 / 1.81 / 1.04.
 bool copy_pays(const cih_basis &b, int K, int64_t rows)
 {
-    const int64_t least = K == 1 ? 16384 : K > 4 ? 40960 : rows == b.dim ? 8192 : 12288, entries = K == 1 ? 128 : K <= 4 ? 192 : 64;
+    const int64_t least = K == 1 ? 10240 : K > 4 ? 40960 : rows == b.dim ? 8192 : 12288;
+    const int64_t entries = K == 1 ? (rows < 16384 ? 40 : 128) : K <= 4 ? 192 : 64;
     return K < kFillSets && rows >= least && fill1_fits(b, K == 1 ? 1 : K == 2 ? 2 : 4) &&
            (int64_t)work_floats(b, 1) <= entries * rows;
 }
