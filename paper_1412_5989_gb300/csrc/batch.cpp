@@ -216,19 +216,19 @@ int batch_solve(cih_instance_t *inst, int n, double hw, int nev, int max_iter, d
                 !mem.get((void **)&psi[i], 8 * K * std::max<int64_t>(inst[i].basis->dim, 1)))
                 return fail(CIH_ERR_NOMEM, "batch: wave arrays");
         }
-        // working copies for the one-set fills where the wave leaves room for
+        // working copies for the fills of few sets where the wave leaves room for
         // them (taken here: an allocation inside the capture would be the graph's)
         std::vector<float *> work(n, nullptr);
         int64_t room = avail;
         for (int i : w) room -= plan[i].resident;
         for (int i : w) {
-            const size_t f = inst[i].K == 1 ? fill_work_floats(*inst[i].basis) : 0;
+            const size_t f = fill_work_floats(*inst[i].basis, inst[i].K);
             if (f == 0 || (int64_t)(f * sizeof(float)) > room || !fills.get((void **)&work[i], f * sizeof(float))) continue;
             room -= (int64_t)(f * sizeof(float));
         }
         rc = fan_out(st, w, br, true, [&](int i, cudaStream_t s) {
             const cih_instance_t &x = inst[i];
-            const int r = work[i] ? fill_prepare(*x.basis, hw, x.tbme_dev, x.e_sp_dev, nullptr, work[i], s) : CIH_OK;
+            const int r = work[i] ? fill_prepare(*x.basis, x.K, hw, x.tbme_dev, x.e_sp_dev, nullptr, work[i], s) : CIH_OK;
             return r ? r : launch_fill(*x.basis, rowptr[i], x.K, hw, x.tbme_dev, false, false, x.e_sp_dev, col[i], val[i], s,
                                        0, -1, false, nullptr, work[i], false);
         });

@@ -314,14 +314,14 @@ int upload_and_build_neighbours(cih_basis &b, cudaStream_t st, const std::functi
 // kernels (ham.cu)
 int launch_count(const cih_basis &b, int64_t *rowptr, cudaStream_t st);
 int launch_scan(const cih_basis &b, int64_t *rowptr, cudaStream_t st);
-// A fill of few sets of a large basis first prepares a working copy of the table
-// (fill_prepare; one set: fill_work_floats() floats of device memory): `work` when the
-// caller gives it (one set, already prepared), else allocated for the call on the
-// stream (unless prepare is false); without it (no memory, few of the rows) the fill
-// reads the table itself, with the same results.  fill_work_floats is 0 where that
-// form does not apply.
-size_t fill_work_floats(const cih_basis &b);
-int fill_prepare(const cih_basis &b, double hw, const float *tbme, const double *esp, const double *t1, float *work,
+// A fill of few sets of a large basis first prepares a working copy of the tables
+// (fill_prepare, for several fills of the same tables: fill_work_floats(K) floats of device
+// memory, set-major tables): `work` when the caller gives it, already prepared, else
+// allocated for the call on the stream (unless prepare is false); without it (no
+// memory, few of the rows) the fill reads the tables themselves, with the same
+// results.  fill_work_floats is 0 where that form does not apply.
+size_t fill_work_floats(const cih_basis &b, int K);
+int fill_prepare(const cih_basis &b, int K, double hw, const float *tbme, const double *esp, const double *t1, float *work,
                  cudaStream_t st);
 // interleaved: tables element-major (len x K); em: values element-major (nnz x K)
 // sharded: col / val hold only rows r0 .. r1 - 1 (positions relative to rowptr[r0]);

@@ -2059,20 +2059,47 @@ void split_tolerances(const cih_basis &b, FillArgs &F)
 
 }  // namespace
 
-size_t fill_work_floats(const cih_basis &b) { return fill_splits(b, 1) ? work_floats(b, 1) : 0; }
+namespace {
 
-int fill_prepare(const cih_basis &b, double hw, const float *tbme, const double *esp, const double *t1, float *work,
+// fn(first set, sets, values of an entry) for the passes of a fill of K sets
+template <class Fn>
+int over_passes(int K, Fn &&fn)
+{
+    const int kv = K == 1 ? 1 : K == 2 ? 2 : 4;
+    int rc = CIH_OK;
+    for (int k0 = 0; k0 < K && !rc; k0 += kv) {
+        const int ks = std::min(kv, K - k0);
+        rc = fn(k0, ks, ks == 1 ? 1 : ks == 2 ? 2 : 4);
+    }
+    return rc;
+}
+
+}  // namespace
+
+size_t fill_work_floats(const cih_basis &b, int K)
+{
+    size_t n = 0;
+    if (!fill_splits(b, K)) return 0;
+    over_passes(K, [&](int, int, int v) { n += work_floats(b, v); return CIH_OK; });
+    return n;
+}
+
+int fill_prepare(const cih_basis &b, int K, double hw, const float *tbme, const double *esp, const double *t1, float *work,
                  cudaStream_t st)
 {
     FillArgs F{};
-    F.K = 1;
+    F.K = K;
     F.hw = hw;
     F.tbme = tbme;
     F.tb_sk = b.layout.total;
     F.tb_si = 1;
     F.esp = esp;
     F.t1 = t1;
-    return launch_prep(b, 1, F, work_at(b, work, 1, 0, 1), st);
+    return over_passes(K, [&](int k0, int ks, int v) {
+        const int rc = launch_prep(b, v, F, work_at(b, work, v, k0, ks), st);
+        work += work_floats(b, v);
+        return rc;
+    });
 }
 
 int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, const float *tbme, bool interleaved,
@@ -2085,19 +2112,21 @@ int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, con
     const bool split = fill_splits(b, K);
     if (split) split_tolerances(b, F);
     const int64_t rend = r1 < 0 ? b.dim : r1;
-    if (K == 1 && work && b.dim > 0 && rend > r0)
-        return launch_fill1(b, 1, rowptr, F, work_at(b, const_cast<float *>(work), 1, 0, 1), st, false, r0, rend);
-    const int kv = K == 1 ? 1 : K == 2 ? 2 : 4;                // sets of one pass
+    if (split && work && rend > r0)
+        return over_passes(K, [&](int k0, int ks, int v) {
+            const FillWork W = work_at(b, const_cast<float *>(work), v, k0, ks);
+            work += work_floats(b, v);
+            return launch_fill1(b, v, rowptr, F, W, st, false, r0, rend);
+        });
     if (split && !work && prepare && copy_pays(b, K, rend - r0)) {
         float *own = nullptr;
-        if (cudaMallocFromPoolAsync((void **)&own, work_floats(b, kv) * sizeof(float), b.pool, st) == cudaSuccess) {
-            int rc = CIH_OK;
-            for (int k0 = 0; k0 < K && !rc; k0 += kv) {
-                const int ks = std::min(kv, K - k0), v = ks == 1 ? 1 : ks == 2 ? 2 : 4;
+        const size_t bytes = work_floats(b, K == 1 ? 1 : K == 2 ? 2 : 4) * sizeof(float);        // of the largest pass
+        if (cudaMallocFromPoolAsync((void **)&own, bytes, b.pool, st) == cudaSuccess) {
+            const int rc = over_passes(K, [&](int k0, int ks, int v) {
                 const FillWork W = work_at(b, own, v, k0, ks);
-                rc = launch_prep(b, v, F, W, st);
-                if (!rc) rc = launch_fill1(b, v, rowptr, F, W, st, false, r0, rend);
-            }
+                const int r = launch_prep(b, v, F, W, st);
+                return r ? r : launch_fill1(b, v, rowptr, F, W, st, false, r0, rend);
+            });
             cudaFreeAsync(own, st);
             return rc;
         }
@@ -2115,7 +2144,8 @@ int prepare_rows(const cih_basis &b, int K)
     int rc = launch_rows<0>(b, nullptr, nullptr, F, G, nullptr, true);
     if (!rc) rc = launch_rows<1>(b, nullptr, nullptr, F, G, nullptr, true);
     if (!rc) rc = launch_rows<2>(b, nullptr, nullptr, F, G, nullptr, true);
-    if (!rc && K == 1 && fill_work_floats(b) > 0) rc = launch_fill1(b, 1, nullptr, F, FillWork{}, nullptr, true, 0, 0);
+    if (!rc && fill_work_floats(b, K) > 0)
+        rc = over_passes(K, [&](int, int, int v) { return launch_fill1(b, v, nullptr, F, FillWork{}, nullptr, true, 0, 0); });
     return rc;
 }
 

@@ -53,8 +53,8 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
     if (e != cudaSuccess) { rc = cuda_fail(e, "build_host: row pointers"); goto done; }
     // what does not need the count runs while it does: one set's working copy of
     // the table (prepared once for all chunks), the copy stream and its events
-    if (K == 1 && fill_work_floats(b) > 0 && alloc((void **)&work, sizeof(float) * fill_work_floats(b)) &&
-        (rc = fill_prepare(b, hw, tbme_d, esp_d, nullptr, work, st)))
+    if (K == 1 && fill_work_floats(b, 1) > 0 && alloc((void **)&work, sizeof(float) * fill_work_floats(b, 1)) &&
+        (rc = fill_prepare(b, 1, hw, tbme_d, esp_d, nullptr, work, st)))
         goto done;
     e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e != cudaSuccess) { cs = nullptr; rc = cuda_fail(e, "build_host: copy stream"); goto done; }
