@@ -51,10 +51,13 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&counted, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(counted, st);
     if (e != cudaSuccess) { rc = cuda_fail(e, "build_host: row pointers"); goto done; }
-    // what does not need the count runs while it does: one set's working copy of
-    // the table (prepared once for all chunks), the copy stream and its events
-    if (K == 1 && fill_work_floats(b, 1) > 0 && alloc((void **)&work, sizeof(float) * fill_work_floats(b, 1)) &&
-        (rc = fill_prepare(b, 1, hw, tbme_d, esp_d, nullptr, work, st)))
+    // what does not need the count runs while it does: the working copy of the
+    // tables (prepared once for all chunks), the copy stream and its events.  From five
+    // sets on a copy is two passes, and the link is slower than the row kernel (us,
+    // with / without a copy: 3+4 Nmax=4, one set 522 / 558, four 1,114 / 1,137, seven 1,780 /
+    // 1,748; 4+4 Nmax=4 1,420 / 1,430, 3,343 / 3,352, 5,353 / 5,306)
+    if (K <= 4 && fill_work_floats(b, K) > 0 && alloc((void **)&work, sizeof(float) * fill_work_floats(b, K)) &&
+        (rc = fill_prepare(b, K, hw, tbme_d, esp_d, nullptr, work, st)))
         goto done;
     e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e != cudaSuccess) { cs = nullptr; rc = cuda_fail(e, "build_host: copy stream"); goto done; }
@@ -76,7 +79,14 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
                                         std::to_string(capacity));
         goto done;
     }
-    if (!alloc((void **)&col_d, sizeof(int32_t) * (size_t)nnz) || !alloc((void **)&val_d, sizeof(float) * (size_t)K * nnz)) {
+    // the matrix comes before the working copy where the device has no room for both
+    while (!((col_d || alloc((void **)&col_d, sizeof(int32_t) * (size_t)nnz)) &&
+             alloc((void **)&val_d, sizeof(float) * (size_t)K * nnz)) && work) {
+        bufs.erase(std::find(bufs.begin(), bufs.end(), (void *)work));
+        cudaFreeAsync(work, st);
+        work = nullptr;
+    }
+    if (!val_d) {
         rc = fail(CIH_ERR_NOMEM, "build_host: device matrix");
         goto done;
     }
@@ -92,7 +102,7 @@ int build_host(cih_basis &b, int K, double hw, const float *tbme_h, const double
             rb[c] = std::lower_bound(rowptr_h, rowptr_h + dim + 1, nnz * kChunkEnd[c - 1] / 64) - rowptr_h;
         for (int c = 0; c < C && !rc; ++c) {
             const int64_t r0 = std::min(rb[c], dim), r1 = c == C - 1 ? dim : std::max(r0, std::min(rb[c + 1], dim));
-            if ((rc = launch_fill(b, rowptr_d, K, hw, tbme_d, false, false, esp_d, col_d, val_d, st, r0, r1, false, nullptr, work)))
+            if ((rc = launch_fill(b, rowptr_d, K, hw, tbme_d, false, false, esp_d, col_d, val_d, st, r0, r1, false, nullptr, work, false)))
                 break;
             const cudaEvent_t ev = evs[c];
             cudaEventRecord(ev, st);
