@@ -145,11 +145,17 @@ int cih_ham_count(cih_basis_h h, int64_t *rowptr_dev, int64_t *nnz_out, void *st
  * FP32.  For the few dozen terms of one element this is the exact sum in all
  * but pathological cancellations, so the stored value agrees with the FP64
  * sum rounded to FP32 within 1e-5 (|value| + 1) (in practice bit for bit).
- * With K < 8 and at least 4,096 rows the call takes stream-ordered
- * scratch from the library's pool for a working copy of the tables (87 MB a set at
- * 4+4 Nmax=6, for at most four sets; inside a stream capture the allocation becomes
- * part of the graph); without it the fill reads the tables itself, with the same
- * results.
+ * With K < 8 and many rows (from 10,240 on with one set, 8,192 with two to four,
+ * 40,960 with five to seven, if the copy has few entries a row) the call takes
+ * stream-ordered scratch from the library's pool for a working copy of the tables (158 MB a
+ * set at 4+4 Nmax=6, for at most four sets); without it, for fewer rows, and inside a
+ * stream capture (a captured fill is one kernel node and allocates nothing) the fill
+ * reads the tables itself, with the same bits.
+ * Bits: a set's values do not depend on the rows filled, on scratch or on a
+ * capture.  They may depend on K in the last bit of a multi-term value (the
+ * order of its sum): the sets of a fill with K < 16 have the bits of their own
+ * one-set fills on bases below 8,192 rows, and wherever one and K sets go by the same
+ * of the above ways for all rows.
  * Errors: CIH_ERR_ARG (K < 1, NULL arrays), CIH_ERR_CUDA. */
 int cih_ham_fill(cih_basis_h h, const int64_t *rowptr_dev, int32_t K, double hbar_omega,
                  const float *tbme_dev, const double *e_sp_dev,

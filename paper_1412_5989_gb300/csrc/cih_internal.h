@@ -318,7 +318,7 @@ int launch_scan(const cih_basis &b, int64_t *rowptr, cudaStream_t st);
 // (fill_prepare, for several fills of the same tables: fill_work_floats(K) floats of device
 // memory, set-major tables): `work` when the caller gives it, already prepared, else
 // allocated for the call on the stream (unless prepare is false); without it (no
-// memory, few of the rows) the fill reads the tables themselves, with the same
+// memory, few of the rows, a captured stream) the fill reads the tables themselves, with the same
 // results.  fill_work_floats is 0 where that form does not apply.
 size_t fill_work_floats(const cih_basis &b, int K);
 int fill_prepare(const cih_basis &b, int K, double hw, const float *tbme, const double *esp, const double *t1, float *work,

@@ -486,13 +486,18 @@ struct TermSizes {
     }
 };
 
-// The sums of a row again in k_fill1's order.  The diagonal: the pn pairs, and each
+// Which sums of a row split_row makes: the diagonal, and the one-moves (neutrons first)
+// whose number's block of `per` is, modulo 31, a bit.
+constexpr unsigned kSplitDiagonal = 1u << 31;
+__device__ __forceinline__ unsigned split_block(int t, int per) { return 1u << (t / per % 31); }
+
+// Sums of a row again in k_fill1's order.  The diagonal: the pn pairs, and each
 // species' own part.  A one-move: its terms over the other species' particles (a lane
 // each, summed as a tree) and over its own species' spectators (loaded a lane each,
 // summed ascending after the one-body term).  A call of its own at the row's end, so
 // that the rows without such sums keep their registers; w_occ, w_lev: the row's.
-__device__ __noinline__ void split_row(const DevBasis &B, const int2 *lg, const FillArgs &F, int64_t row, const int16_t *w_occ,
-                                       const int4 *w_lev, float *val, int64_t es, int64_t ks, int *status)
+__device__ __noinline__ void split_row(const DevBasis &B, const int2 *lg, const FillArgs &F, int64_t row, unsigned which,
+                                       const int16_t *w_occ, const int4 *w_lev, float *val, int64_t es, int64_t ks, int *status)
 {
     const int lane = threadIdx.x & 31, nbase = B.sp[1].orb_base;
     const DevSpecies &SP = B.sp[0], &SN = B.sp[1];
@@ -508,7 +513,7 @@ __device__ __noinline__ void split_row(const DevBasis &B, const int2 *lg, const 
     }
     c1 = __reduce_add_sync(0xffffffffu, c1);
     __syncwarp();                                               // after the row's first values
-    for (int k = 0; k < (part & 1 ? F.K : 0); ++k) {
+    for (int k = 0; k < (which & kSplitDiagonal ? F.K : 0); ++k) {
         DF acc = df_of(0.f);
         for (int x = lane / gsz; x < Zp; x += 32 / gsz) {
             if (i >= Zn) continue;
@@ -526,9 +531,12 @@ __device__ __noinline__ void split_row(const DevBasis &B, const int2 *lg, const 
         if (lane == 0) val[(int64_t)k * ks] = df_round(df_add(acc, df_add(dp, dn)));
     }
     const int first = part & 2 ? 0 : cA1, last = part & 4 ? cA1 + c1 : cA1;
+    int per = 32;                                               // flush_slow's
+    while (per > 1 && per * (B.A - 1) > 32) per >>= 1;
     for (int t0 = first; t0 < last; t0 += 32 / gsz) {
         const int t = t0 + lane / gsz;
-        const bool act = t < last, neu = t < cA1;
+        const bool act = t < last && (which & split_block(t, per)), neu = t < cA1;
+        if (!__any_sync(0xffffffffu, act)) continue;
         int e = 0, code = 0;
         if (act && neu) {
             const int64_t sl = NR.fw + NR.fwlen - 1 - t;
@@ -579,7 +587,7 @@ template <int MODE, bool K1, int EM, bool SPLIT>
 __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, const FillArgs &F, const GradArgs &Gr,
                                            int *status, const int16_t *w_occ, const int32_t *w_spos,
                                            const int32_t *w_scol, const uint32_t *w_scode, int &nslow,
-                                           const RowOut &R, bool &again)
+                                           const RowOut &R, int &flushed, unsigned &again)
 {
     const int lane = threadIdx.x & 31;
     const int A = B.A, nbase = B.sp[1].orb_base;
@@ -741,11 +749,12 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
                 }
             };
             over_sets<K1>(K1 ? 1 : F.K, sums);
-            if (SPLIT && __any_sync(0xffffffffu, near && act && i == 0)) {
+            near = near && act && i == 0;
+            if (SPLIT && __any_sync(0xffffffffu, near)) {
                 z.add(t1v.hi);
                 z.add(t1v.lo);
                 z.over(gsz);
-                again |= near && act && i == 0 && !exact_sum(z.sum, z.least);
+                if (near && !exact_sum(z.sum, z.least)) again |= split_block(flushed + e, per);
             }
         } else {
             for (int kk = 0; kk < (K1 ? 1 : Gr.K); ++kk) {
@@ -758,6 +767,7 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
         }
     }
     __syncwarp();
+    if (SPLIT) flushed += ns;
     nslow = 0;
 }
 
@@ -860,7 +870,7 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
             R.val = F.val + r0 * R.es;
         }
         int nslow = 0;
-        bool again = false;                                     // SPLIT: a sum of the row may depend on the order
+        unsigned again = 0;                                     // SPLIT: sums of the row that may depend on the order
 
         // ---- diagonal: occupied orbitals (combined, ascending), then all pairs
         if (MODE != 0) {
@@ -987,7 +997,8 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
                             z.over(32);
 #pragma unroll
                             for (int u = 0; u < U; ++u)
-                                again |= (K1 || k0 + u < F.K) && near_tie(acc[u], z.sum, F.tol_diag) && !exact_sum(z.sum, z.least);
+                                if ((K1 || k0 + u < F.K) && near_tie(acc[u], z.sum, F.tol_diag) && !exact_sum(z.sum, z.least))
+                                    again |= kSplitDiagonal;
                         }
                     }
                 }
@@ -1000,7 +1011,7 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
         // ---- A: same-class forward neutron neighbours inside p's range
         const int16_t *dirn = B.dir + (int64_t)n * B.dir_len;
         const int cA1 = max(0, dirn[PR.dirA] - NR.self), cA2 = SN.fw_lev[(int64_t)n * SN.NL + PR.levA];
-        int pos = 1 + cA1 + cA2;
+        int pos = 1 + cA1 + cA2, flushed = SPLIT && !(row_part() & 2) ? cA1 : 0;           // one-moves done (split_row's numbers)
         if (MODE == 1 && pos > rowlen) {
             if (lane == 0) atomicOr(status, 2);
             continue;
@@ -1024,7 +1035,7 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
             for (int t0 = 0; t0 < cA1; t0 += 32) {
                 const int t = t0 + lane, c = min(32, cA1 - t0);
                 if (nslow + c > kSlowCap)
-                    flush_slow<MODE, K1, EM, SPLIT>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R, again);
+                    flush_slow<MODE, K1, EM, SPLIT>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R, flushed, again);
                 if (lane < c) {
                     const int sl = NR.fwlen - 1 - t;
                     const int2 rc = rec[sl];
@@ -1101,7 +1112,7 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
             for (int t0 = 0; t0 < c1; t0 += 32) {
                 const int t = t0 + lane, cc = min(32, c1 - t0);
                 if (nslow + cc > kSlowCap)
-                    flush_slow<MODE, K1, EM, SPLIT>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R, again);
+                    flush_slow<MODE, K1, EM, SPLIT>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R, flushed, again);
                 if (lane < cc) {
                     const int2 q = l1row[t];
                     const int o = recp[PR.fwlen - 1 - t].y;
@@ -1145,8 +1156,11 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
             __syncwarp();
             pos += Tall;
         }
-        if (MODE != 0 && nslow > 0) flush_slow<MODE, K1, EM, SPLIT>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R, again);
-        if (SPLIT && __any_sync(0xffffffffu, again && rowlen > 0)) split_row(B, lg, F, row, w_occ, w_lev, R.val, R.es, R.ks, status);
+        if (MODE != 0 && nslow > 0) flush_slow<MODE, K1, EM, SPLIT>(B, lg, F, Gr, status, w_occ, w_spos, w_scol, w_scode, nslow, R, flushed, again);
+        if (SPLIT) {
+            again = __reduce_or_sync(0xffffffffu, rowlen > 0 ? again : 0);
+            if (again) split_row(B, lg, F, row, again, w_occ, w_lev, R.val, R.es, R.ks, status);
+        }
         if (MODE == 0 && lane == 0) counts[row] = pos;
         __syncwarp();
     }
@@ -2102,6 +2116,17 @@ int fill_prepare(const cih_basis &b, int K, double hw, const float *tbme, const 
     });
 }
 
+// Whether the stream is being captured: a graph with an allocation in it could not be a
+// child graph nor be instantiated twice, so a captured fill takes no scratch (the row
+// kernel, the same bits).
+static bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();
+    return true;
+}
+
 int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, const float *tbme, bool interleaved,
                 bool em, const double *esp, int32_t *col, float *val, cudaStream_t st, int64_t r0, int64_t r1,
                 bool sharded, const double *t1, const float *work, bool prepare)
@@ -2118,7 +2143,7 @@ int launch_fill(const cih_basis &b, const int64_t *rowptr, int K, double hw, con
             work += work_floats(b, v);
             return launch_fill1(b, v, rowptr, F, W, st, false, r0, rend);
         });
-    if (split && !work && prepare && copy_pays(b, K, rend - r0)) {
+    if (split && !work && prepare && copy_pays(b, K, rend - r0) && !capturing(st)) {
         float *own = nullptr;
         const size_t bytes = work_floats(b, K == 1 ? 1 : K == 2 ? 2 : 4) * sizeof(float);        // of the largest pass
         if (cudaMallocFromPoolAsync((void **)&own, bytes, b.pool, st) == cudaSuccess) {
