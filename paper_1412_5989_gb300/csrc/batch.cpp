@@ -128,10 +128,14 @@ int batch_solve(cih_instance_t *inst, int n, double hw, int nev, int max_iter, d
         inst[i].status = CIH_OK;
     }
     if (budget == 0) {
+        // free memory and the idle blocks of the library's pool, which serves the batch
         size_t fr = 0, tot = 0;
+        uint64_t reserved = 0, used = 0;
         cudaError_t e = cudaMemGetInfo(&fr, &tot);
+        if (e == cudaSuccess) e = cudaMemPoolGetAttribute(inst[0].basis->pool, cudaMemPoolAttrReservedMemCurrent, &reserved);
+        if (e == cudaSuccess) e = cudaMemPoolGetAttribute(inst[0].basis->pool, cudaMemPoolAttrUsedMemCurrent, &used);
         if (e != cudaSuccess) return cuda_fail(e, "batch: memory info");
-        budget = (int64_t)(0.9 * (double)fr);
+        budget = (int64_t)(0.9 * (double)(fr + (reserved > used ? reserved - used : 0)));
     }
     Branches br;
     if (br.make(n)) return cuda_fail(cudaGetLastError(), "batch: streams");
