@@ -3,7 +3,11 @@ sums through a working copy of the tables; a shard of few rows sums in the row
 kernel, which makes the sums that the order could change again in the other form's
 order.  Both are compared bit for bit, on tables for which the order matters.
 """
+import numpy as np
 import pytest
+
+import oracle
+from paper_1412_5989_gb300 import synth
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -45,7 +49,8 @@ def same(a, b):
 
 # space, set counts whose fills of all rows go through the copy
 SPACES = [((4, 5, 2, 1), (2, 3, 4)), ((3, 3, 4, 0), (1, 2, 3, 4)), ((5, 2, 4, 1), (1, 2, 3, 4)), ((3, 4, 4, 1), (1, 2, 3, 4, 5, 7)),
-          ((10, 3, 2, 1), (1, 2, 3, 4)), ((16, 3, 1, 1), (2, 3, 4))]
+          ((10, 3, 2, 1), (1, 2, 3, 4)), ((16, 3, 1, 1), (2, 3, 4)), ((1, 6, 4, 1), (2, 3, 4)), ((6, 1, 4, 1), (2, 3, 4)),
+          ((2, 2, 7, 0), (2, 3, 4))]
 
 
 @pytest.mark.parametrize("space,copied", SPACES)
@@ -66,6 +71,32 @@ def test_shards_same_bits(cih, space, copied, kind):
         assert cih.kernel_launches() - n0 == len(parts)          # shards of a fortieth: the row kernel
         assert torch.equal(torch.cat([c for c, _ in parts]), col)
         assert same(torch.cat([v for _, v in parts], dim=1), val)
+    B.check()
+
+
+@pytest.mark.parametrize("space", [(1, 6, 4, 1), (6, 1, 4, 1), (10, 3, 2, 1), (16, 3, 1, 1), (2, 2, 7, 0), (2, 3, 6, 1)])
+@pytest.mark.parametrize("onebody", [False, True])
+def test_copy_against_the_oracle(cih, space, onebody):
+    """Few particles of a species, many of one, many levels: every element of two sets."""
+    B = cih.Basis(*space)
+    S = oracle.Space(*space)
+    t = synth.tbme_tables(B.tbme_len, range(2))
+    T = torch.from_numpy(t).cuda()
+    rowptr, nnz = B.count()
+    n0 = cih.kernel_launches()
+    if onebody:
+        t1 = synth.onebody_table(B.onebody_len, 5) * 10.0
+        col, val = B.fill_onebody(rowptr, nnz, T, torch.from_numpy(t1).cuda())
+        S.set_onebody(t1)
+        e = None
+    else:
+        e = synth.single_particle_energies(sum(B.n_orb), 3)
+        col, val = B.fill(rowptr, nnz, T, e_sp=torch.from_numpy(e).cuda())
+    assert cih.kernel_launches() - n0 == 2
+    for k in range(2):
+        _, _, col_o, val_o = S.rows(np.arange(B.dim), t[k], esp=e)
+        np.testing.assert_array_equal(col.cpu().numpy(), col_o)
+        assert np.all(np.abs(val[k].cpu().numpy().astype(np.float64) - val_o) <= 1e-5 * (np.abs(val_o) + 1.0))
     B.check()
 
 
