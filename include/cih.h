@@ -411,8 +411,8 @@ typedef struct {
  *      lowest Ritz vectors (held for the wave), plus the Lanczos and adjoint
  *      scratch (held one instance at a time);
  *   3. instances are admitted in the given order into waves whose peak stays
- *      within hbm_budget bytes (0 = 90% of the free device memory at the
- *      call); an instance above the budget on its own gets CIH_ERR_CAPACITY
+ *      within hbm_budget bytes (0 = 90% of the free device memory and the
+ *      library pool's idle bytes at the call); an instance above the budget on its own gets CIH_ERR_CAPACITY
  *      and is skipped;
  *   4. per wave: the fills of all its instances as one CUDA graph launch
  *      (one branch per instance), then per instance the lowest nev

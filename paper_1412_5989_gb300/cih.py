@@ -386,8 +386,8 @@ class Basis:
         _ok(lib.cih_set_launch(self._h, warps_per_cta, ctas_per_sm), "set_launch")
 
     def set_count_mode(self, walk: bool):
-        """Count pass of this basis: walk the candidates (True) or sum the
-        count lists where the basis has them (False, the default)."""
+        """Count pass of this basis: the row kernel's walk (True) or the sum of
+        the groups' terms (False, the default)."""
         _ok(lib.cih_set_count_mode(self._h, int(bool(walk))), "set_count_mode")
 
     def autotune_fill(self, rowptr, nnz: int, tbme, hbar_omega: float = 20.0, e_sp=None, *, K: int | None = None,

@@ -21,9 +21,9 @@
 // and all residual bounds beta_m |z_m| from implicit-QR sweeps that rotate only
 // the last row of the eigenvector matrix; the lowest Ritz vector's coefficients by
 // inverse iteration.
-// Start of this form -> now, one GB300, whole solves: 800 rows 15.2 -> 4.0 ms;
-// 143,792 rows with gradient 87 -> 39 ms; 64 sets of 48,917 rows 492 -> 370 ms;
-// the uneven batch of 197,822 / 143,792 / 814,092 rows 645 -> 395 ms.
+// One GB300, whole solves: 800 rows 4.2 ms; 143,792 rows with set-up and gradient 37
+// ms; 64 sets of 48,917 rows 325 ms; the uneven batch of 197,822 / 143,792 / 814,092
+// rows 394 ms.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -99,7 +99,7 @@ struct RowRange {
 // equal length for all warps, found by a search, 0.23 ms there but 1.11 ms for one set.
 // R = 8 / K rows (at least one): 4 to 16 for one set are alike, 31 leave warps idle.
 // Blocks beyond gridDim.x have no part: their partials are zero.
-constexpr int kSumsqThreads = 1024, kSumsqGrid = 152;              // one block an SM, 32 warps
+constexpr int kSumsqThreads = 1024, kSumsqGrid = 152;              // one block on each of GB300's SMs, 32 warps
 __global__ void __launch_bounds__(kSumsqThreads) k_upper_sumsq(RowRange rr, int K, const int64_t *rowptr,
                                                                const float *vem, double *partial)
 {
@@ -248,7 +248,8 @@ __device__ __forceinline__ int round_i32(float x)
 // The mirrored product q (hi + lo, units 2^-s) as an integer: hi and lo each
 // rounded.  Below 2^50 hi splits exactly into A 2^30 + rem, |rem| <= 2^29 (A through
 // the float's own rounding at 1.5 2^23, rem by one FMA; from 2^24 on hi is an
-// integer, so rounding rem rounds hi), and |lo| <= 2^26: two 32-bit conversions
+// integer, so rounding rem rounds hi), and |lo| <= 1.5 2^26 (v x.y, and half the last
+// bit of hi): the sum of both fits 32 bits.  Two 32-bit conversions
 // and a wide multiply-add, some 16 instructions, where shifting the two mantissas
 // took about 40: a call of 64 sets at 3+4 Nmax=4 2.69 -> 2.44 ms, at 4+4 Nmax=4
 // 8.05 -> 7.33 ms; one set, bound by its atomic adds, unchanged.
@@ -279,7 +280,7 @@ __global__ void k_split(int64_t n, const double *x, const double *sc, float2 *xs
 
 // K > 16: lanes over sets, two per lane per pass; K <= 16 (KS = next power
 // of two): 32/KS lane groups split the row's nonzeros, four at a time per
-// group, and the groups' row sums are reduced at the end.  With K < 32 the
+// group, and the groups' row sums are reduced at the end, and the
 // matrix is read with evict-first loads, so that its stream does not push x
 // and the accumulators out of L2 (with lanes over sets the same hint ran
 // slower).  Each block walks
@@ -628,7 +629,9 @@ int dot_vecs(int nb, int K, int nvec)
     return std::max(4, std::min(kDotVecs, nb * nvec / 304 / 4 * 4));
 }
 
-// k_dots takes up to 66 KB of shared memory (set once per device; idempotent)
+// k_dots takes up to 66 KB of shared memory (set once per device; idempotent).  The set
+// count is fixed at compile time for 64 sets, the batched configuration, as in k_spmv (a
+// solve of 64 sets of 3+4 Nmax=4 takes 328 ms without, 325 with), and for one.
 cudaError_t prepare_dots(int K)
 {
     const int bytes = (int)sizeof(double) * kDotPad * kDotVecs;

@@ -1071,8 +1071,8 @@ struct PinnedTotals {
     }
 };
 
-// A second stream for the neutron species' list passes, which depend on the
-// proton species' only through the candidate table.  The destructor waits for
+// A second stream for the neutron species' list passes, which need nothing of the
+// proton species'.  The destructor waits for
 // it, so that no early return leaves its kernels running on buffers the basis
 // then frees.
 struct SideStream {
