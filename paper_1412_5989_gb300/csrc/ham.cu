@@ -594,7 +594,7 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
     __syncwarp();
     const int ns = nslow;
     const int sp_n = A - 1;
-    if (MODE == 1 && !K1 && F.K >= kLaneSets) {
+    if (MODE == 1 && !K1 && (EM > 1 || F.K >= kLaneSets)) {      // (EM > 1: 64 sets)
         // K sets: the table entries of 32 / (A - 1) elements at a time (lanes
         // over (element, spectator) pairs, so their lookups run together), then
         // per element lanes over sets sum them in spectator order
@@ -690,7 +690,7 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
     int gsz = 1;
     while (gsz < sp_n) gsz <<= 1;
     const int per = 32 / gsz;
-    for (int e0 = 0; e0 < ns; e0 += per) {
+    for (int e0 = 0; EM <= 1 && e0 < ns; e0 += per) {
         const int e = e0 + lane / gsz;
         const int i = lane % gsz;
         const bool act = e < ns;
@@ -756,9 +756,8 @@ __device__ __forceinline__ void flush_slow(const DevBasis &B, const int2 *lg, co
                 z.over(gsz);
                 if (near && !exact_sum(z.sum, z.least)) again |= split_block(flushed + e, per);
             }
-        } else {
+        } else if (has && ok) {
             for (int kk = 0; kk < (K1 ? 1 : Gr.K); ++kk) {
-                if (!has || !ok) continue;
                 const long long q =
                     (K1 ? __mul64hi(R.psir, Gr.psi[colj]) : psi_prod(Gr.psi + (int64_t)kk * B.dim, R.row, colj)) >> 1;
                 const bool neg = (sgn != 0) != (sg < 0);
@@ -953,59 +952,66 @@ __device__ __forceinline__ void walk_rows(const DevBasis &B, const int64_t *rowp
                         if (atomicOr(status, 1) == 0) { status[2] = a | (c << 16); status[3] = 1; }
                         continue;
                     }
-                    if (MODE == 1) {
-                        float m = 0.f;
+                    float m = 0.f;
 #pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            const float v = K1 || k0 + u < F.K ? __ldg(F.tbme + (int64_t)(k0 + u) * F.tb_sk + idx * F.tb_si) : 0.f;
-                            acc[u] = df_add(acc[u], df_of(sg < 0 ? -v : v));
-                            if (SPLIT) {
-                                m = fmaxf(m, fabsf(v));
-                                z.smaller(v);
-                            }
+                    for (int u = 0; u < U; ++u) {
+                        const float v = K1 || k0 + u < F.K ? __ldg(F.tbme + (int64_t)(k0 + u) * F.tb_sk + idx * F.tb_si) : 0.f;
+                        acc[u] = df_add(acc[u], df_of(sg < 0 ? -v : v));
+                        if (SPLIT) {
+                            m = fmaxf(m, fabsf(v));
+                            z.smaller(v);
                         }
-                        if (SPLIT) z.sum += m;
-                    } else {                                     // w = 1 on the diagonal
-                        const long long q = psi_prod(Gr.psi + (int64_t)k0 * B.dim, row, row) >> 2;
-                        atomicAdd(Gr.acc + (int64_t)k0 * B.tbme_len + idx, (unsigned long long)(sg < 0 ? -q : q));
+                    }
+                    if (SPLIT) z.sum += m;
+                }
+                const float2 *e1 = sptr<float2>(sb, sm::e1);
+                for (int i = lane; i < A; i += 32) {
+                    const float2 q = e1[w_occ[i]];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) acc[u] = df_add(acc[u], DF{q.x, q.y});
+                    if (SPLIT) {
+                        z.add(q.x);
+                        z.add(q.y);
                     }
                 }
-                if (MODE == 1) {
-                    const float2 *e1 = sptr<float2>(sb, sm::e1);
-                    for (int i = lane; i < A; i += 32) {
-                        const float2 q = e1[w_occ[i]];
+                warp_sums<U>(acc, 32);
+                if (lane == 0 && rowlen > 0) {
+                    if (k0 == 0) R.col[0] = (int32_t)row;
 #pragma unroll
-                        for (int u = 0; u < U; ++u) acc[u] = df_add(acc[u], DF{q.x, q.y});
-                        if (SPLIT) {
-                            z.add(q.x);
-                            z.add(q.y);
-                        }
-                    }
-                    warp_sums<U>(acc, 32);
-                    if (lane == 0 && rowlen > 0) {
-                        if (k0 == 0) R.col[0] = (int32_t)row;
+                    for (int u = 0; u < U; ++u)
+                        if (K1 || k0 + u < F.K) R.val[(int64_t)(k0 + u) * R.ks] = df_round(acc[u]);
+                }
+                if (SPLIT) {
+                    const float mag = 32.f * __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(z.sum)));
+                    bool near = false;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) near |= (K1 || k0 + u < F.K) && near_tie(acc[u], mag, F.tol_diag);
+                    if (__any_sync(0xffffffffu, near)) {      // look closer
+                        z.over(32);
 #pragma unroll
                         for (int u = 0; u < U; ++u)
-                            if (K1 || k0 + u < F.K) R.val[(int64_t)(k0 + u) * R.ks] = df_round(acc[u]);
-                    }
-                    if (SPLIT) {
-                        const float mag = 32.f * __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(z.sum)));
-                        bool near = false;
-#pragma unroll
-                        for (int u = 0; u < U; ++u) near |= (K1 || k0 + u < F.K) && near_tie(acc[u], mag, F.tol_diag);
-                        if (__any_sync(0xffffffffu, near)) {      // look closer
-                            z.over(32);
-#pragma unroll
-                            for (int u = 0; u < U; ++u)
-                                if ((K1 || k0 + u < F.K) && near_tie(acc[u], z.sum, F.tol_diag) && !exact_sum(z.sum, z.least))
-                                    again |= kSplitDiagonal;
-                        }
+                            if ((K1 || k0 + u < F.K) && near_tie(acc[u], z.sum, F.tol_diag) && !exact_sum(z.sum, z.least))
+                                again |= kSplitDiagonal;
                     }
                 }
             };
-            if (MODE == 2)
-                for (int k = 0; k < (K1 ? 1 : Gr.K); ++k) sums(std::integral_constant<int, 1>(), k);
-            else if (!kset) over_sets<K1>(K1 ? 1 : F.K, sums);
+            if constexpr (MODE == 2) {
+                for (int k = 0; k < (K1 ? 1 : Gr.K); ++k) {
+                    for (int l = lane; l < npairs; l += 32) {
+                        const int a = w_occ[pi[l]], c = w_occ[pj[l]];
+                        int64_t idx;
+                        int sg;
+                        if (!tbme_at(B, lg, a, c, a, c, idx, sg)) {
+                            if (atomicOr(status, 1) == 0) { status[2] = a | (c << 16); status[3] = 1; }
+                            continue;
+                        }
+                        const long long q = psi_prod(Gr.psi + (int64_t)k * B.dim, row, row) >> 2;    // w = 1 on the diagonal
+                        atomicAdd(Gr.acc + (int64_t)k * B.tbme_len + idx, (unsigned long long)(sg < 0 ? -q : q));
+                    }
+                }
+            } else if (!kset) {
+                over_sets<K1>(K1 ? 1 : F.K, sums);
+            }
         }
 
         // ---- A: same-class forward neutron neighbours inside p's range
@@ -2168,6 +2174,11 @@ int prepare_rows(const cih_basis &b, int K)
     G.K = K;
     int rc = launch_rows<0>(b, nullptr, nullptr, F, G, nullptr, true);
     if (!rc) rc = launch_rows<1>(b, nullptr, nullptr, F, G, nullptr, true);
+    if (!rc && fill_splits(b, K)) {                          // (a fill without room for its copy)
+        FillArgs S = F;
+        split_tolerances(b, S);
+        rc = launch_rows<1>(b, nullptr, nullptr, S, G, nullptr, true);
+    }
     if (!rc) rc = launch_rows<2>(b, nullptr, nullptr, F, G, nullptr, true);
     if (!rc && fill_work_floats(b, K) > 0)
         rc = over_passes(K, [&](int, int, int v) { return launch_fill1(b, v, nullptr, F, FillWork{}, nullptr, true, 0, 0); });
