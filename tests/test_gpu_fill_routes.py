@@ -66,6 +66,10 @@ def test_shards_same_bits(cih, space, copied, kind):
         n0 = cih.kernel_launches()
         col, val = B.fill(rowptr, nnz, t, e_sp=e)
         assert (cih.kernel_launches() - n0 > 1) == (K in copied)
+        if K == 1:
+            one = [B.fill(rowptr, nnz, T[k], e_sp=e)[1][0] for k in range(7)]
+        if K < 8 and (1 in copied) == (K in copied):                # the same way for one set: the same bits
+            assert all(same(val[k], one[k]) for k in range(K))
         n0 = cih.kernel_launches()
         parts = [B.fill_rows(rowptr, r, min(B.dim, r + step), t, e_sp=e) for r in range(0, B.dim, step)]
         assert cih.kernel_launches() - n0 == len(parts)          # shards of a fortieth: the row kernel
